@@ -4,16 +4,24 @@
 //    offset array) is written to the workspace - the step Sec. 4 performs first.
 // 2. decompress_kernel: persistent; each warp takes its chunks by ticket (one atomic add each; no
 //    ordering constraint remains).  Each warp has one record buffer: the cp.async of its
-//    next record starts as soon as the current one has been expanded into the plane buffer;
-//    offsets are loaded one step earlier still.  Decoding a record:
+//    next record starts as soon as the current one has been read; offsets are loaded one step
+//    earlier still.  Decoding a record:
 //      a. header and flags; a walk over the sparse rows' bitmaps gives every row's
-//         position; sparse rows are expanded into their 128-byte plane slots,
-//      b. runs of dense rows are copied into their slots (16-byte funnel-shifted moves), all
-//         plane words are gathered into registers from fixed slot addresses, two 32x32
-//         transposes give Z, unzigzag + warp scan give G (inverse Eq. 5), Case 1 divides by
-//         10^alpha (correctly rounded) and Case 2 undoes the zigzag of the IEEE bits
-//         (inverse Eq. 4),
-//      c. values are staged (swizzled) and written with coalesced 16-byte stores.
+//         position; sparse rows are expanded into 128-byte slots,
+//      b. every plane's row is read where it lies (dense: unaligned in the record; sparse: its
+//         slot), 32 planes at a time; the planes, shifted down one and XORed with plane 0, go
+//         through 32x32 transposes, which gives the unzigzagged deltas at once; a warp scan gives
+//         G (inverse Eq. 5), Case 1 divides by 10^alpha (correctly rounded) and Case 2 undoes the
+//         zigzag of the IEEE bits (inverse Eq. 4),
+//      c. whole 32-byte sectors per lane (aligned FP64) or staged, coalesced stores.
+// What bounds it: latency and integer issue together (FP64 segments: ALU pipe 55 %, L1 data pipe
+// 53 %, issue 51 % of cycles at 16 warps per SM; HBM 40 %).  Reading the dense rows in place
+// instead of copying them to a plane buffer took the kernel from 4302 to 2880 warp instructions
+// per FP64 chunk and its shared memory from 17.6 to 13.6 KB per warp (12 to 16 warps per SM).
+// Measured, 2^26 segment values (both launches): FP64 420 -> 322 us, FP32 216 -> 152 us; Case-1
+// FP64 of 40 M values in 1025-value chunks 547 -> 307 us.  Slower, and left out: a TMA bulk copy of
+// the record on an mbarrier (-1 %), tickets for groups of 4 to 8 chunks (-7 to -15 %: the window of
+// memory in use grows with the group), more registers with fewer warps (144: -6 %).
 // Every read of a record is bounds-checked against its size; a malformed record sets
 // FALCON_ERR_CORRUPT and writes nothing.
 #include "falcon.h"
@@ -23,33 +31,45 @@ namespace falcon {
 
 namespace {
 
-// Per-warp buffers of a value kind: one record at a 0..15 byte phase + 16 readable bytes (an
-// FP64 record is at most 19 + 64 * 144 = 9235 bytes, an FP32 one 11 + 32 * 144 = 4619, an FP16
-// one 7 + 16 * 144 = 2311: every row sparse without a zero byte, bitmap + 128 bytes), then W
-// plane slots of 128 bytes and 64 u16 sparse-byte totals.  The narrow kinds' smaller buffers
-// let more warps stay resident.
+// Shared memory: a 144-byte row of zeros per CTA (what planes >= w read), then per warp
+//   - one record at a 0..15 byte phase + 16 readable bytes (an FP64 record is at most
+//     19 + 64 * 144 = 9235 bytes, an FP32 one 11 + 32 * 144 = 4619, an FP16 one 7 + 16 * 144 = 2311:
+//     every row sparse without a zero byte, bitmap + 128 bytes),
+//   - 128-byte slots for the expanded sparse rows of 32 planes at a time (FP64 runs its two
+//     halves one after the other through the same slots), later the staging of a chunk whose
+//     output is not 32-byte aligned,
+//   - where each of those 32 planes' rows lies: (word address, bit shift) pairs.
+// Dense rows are read where they lie in the record, so no plane buffer is kept: 13.6 KB per FP64
+// warp instead of 17.6 KB, 16 resident warps per SM instead of 12.
+constexpr uint32_t kZeroBytes = 144;
 template <int D> struct DecLayout {
-    static constexpr int kBuf = D == kD64 ? 9280 : (D == kD32 ? 4672 : 2368);
-    static constexpr int kPlane = Traits<D>::W * 128 + 128;
-    static constexpr int kWarpBytes = kBuf + kPlane;
+    static constexpr uint32_t kBuf = D == kD64 ? 9280 : (D == kD32 ? 4672 : 2368);
+    static constexpr uint32_t kRows = Traits<D>::W < 32 ? Traits<D>::W : 32;
+    static constexpr uint32_t kSlots = kRows * 128;
+    static constexpr uint32_t kTab = 32 * 8;
+    static constexpr uint32_t kWarpBytes = kBuf + kSlots + kTab;
 };
+
+// The 32-bit word at any byte offset of the CTA's dynamic shared memory.
+__device__ __forceinline__ uint32_t lds_any(const uint8_t *smem, uint32_t off) {
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(smem + (off & ~3u));
+    return __funnelshift_r(w[0], w[1], off * 8u);           // the shift counts modulo 32
+}
+__device__ __forceinline__ uint32_t bswap(uint32_t x) { return __byte_perm(x, 0u, 0x0123); }
 
 // Byte-permute selector that spreads a lane's compacted non-zero bytes over its four row
 // bytes, by bitmap nibble n: row byte i (nibble bit 3 - i) takes the next compacted byte if
-// the bit is set, else a zero byte (selector 4, the zero operand).
-__shared__ uint32_t s_expand_sel[16];
-
-__device__ __forceinline__ void init_expand_sel() {
-    if (threadIdx.x < 16) {
-        const uint32_t n = threadIdx.x;
-        uint32_t sel = 0, r = 0;
-        for (int i = 0; i < 4; ++i) {
-            if ((n >> (3 - i)) & 1u) sel |= (r++) << (4 * i);
-            else sel |= 4u << (4 * i);
-        }
-        s_expand_sel[n] = sel;
+// the bit is set, else a zero byte (selector 4, the zero operand).  Lane l keeps the selector of
+// nibble l & 15, so one shuffle looks it up.
+__device__ __forceinline__ uint32_t expand_sel(uint32_t n) {
+    uint32_t sel = 0, r = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if ((n >> (3 - i)) & 1u) sel |= (r++) << (4 * i);
+        else sel |= 4u << (4 * i);
     }
-}        // one record buffer, one plane buffer
+    return sel;
+}
 
 // fl(fl(g) / 10^a) with IEEE FP64 operations, as the decoder defines it for any g; the hot
 // path takes div_pow10_exact for |g| < 2^53 (every g an encoder writes: |g| < 10^15).
@@ -60,39 +80,26 @@ __device__ __forceinline__ float div_pow10(int32_t g, int a) {
     return __fdiv_rn(__int2float_rn(g), __uint_as_float(FALCON_P10_F32[a - FALCON_P10_F32_LO]));
 }
 
-// number of set bits of a 4-bit value, with plain integer operations
-__device__ __forceinline__ uint32_t nibble_count(uint32_t n) {
-    const uint32_t x = n - ((n >> 1) & 5u);
-    return (x & 3u) + (x >> 2);
-}
-
-__device__ __forceinline__ const Job &job_of(const Job *jobs, int njobs, const Job &single, uint64_t t) {
-    return (jobs == nullptr) ? single : jobs[find_job(jobs, njobs, t)];
-}
-
-// Offset (within the stream) and size of the record of ticket t: the loads are issued early
-// (locate), the offset is added up when the record is fetched (resolve).
+// A chunk to decode and where its record lies.  The loads are unconditional (a ticket past the
+// last chunk reads the last chunk's words), so nothing waits for them before the record is fetched.
 struct Loc {
-    uint64_t t;
-    uint64_t rec_off;
+    const Job *job;
+    uint64_t c;                                   // chunk of the job
+    uint64_t off;                                 // record position from the stream's first record
     uint32_t size;
-    ChunkPos pos;
 };
 
-__device__ __forceinline__ Loc locate(const Job *jobs, int njobs, const Job &single, uint64_t t, int lane) {
-    const Job &job = job_of(jobs, njobs, single, t);
-    const uint64_t c = t - job.chunk_begin;
+// Forms for one job (a single stream) read it from shared memory; the either-dtype form finds
+// the ticket's job in the table.
+template <bool kTable>
+__device__ __forceinline__ Loc locate(const Job *jobs, int njobs, const Job &single, uint64_t t, uint64_t total_chunks) {
     Loc l;
-    l.t = t;
-    l.pos = load_pos(reinterpret_cast<const uint32_t *>(job.in + 32), job.flags, c, lane);
-    l.size = l.pos.size;
-    l.rec_off = 0;
+    t = t < total_chunks ? t : total_chunks - 1u;
+    l.job = kTable ? jobs + find_job(jobs, njobs, t) : &single;
+    l.c = kTable ? t - l.job->chunk_begin : t;
+    l.off = l.job->flags[l.c];
+    l.size = reinterpret_cast<const uint32_t *>(l.job->in + 32)[l.c];
     return l;
-}
-
-__device__ __forceinline__ void resolve(const Job *jobs, int njobs, const Job &single, Loc &l) {
-    const Job &job = job_of(jobs, njobs, single, l.t);
-    l.rec_off = 32ull + 4ull * job.nchunks + resolve_pos(l.pos);
 }
 
 // Largest valid record of a chunk of m values: header, flags, and w = W rows of at most
@@ -102,54 +109,199 @@ __device__ __forceinline__ uint32_t max_record(uint32_t m, uint32_t dtype) {
     return 3u + W / 8u + W / 8u + W * (chunk_cols(m) / 8u + chunk_cols(m) / 64u);
 }
 
-// Starts the cp.async of a record into rbuf; returns false if its location is invalid.
-__device__ __forceinline__ bool issue_record(const Job &job, const Loc &l, uint8_t *rbuf, int lane) {
-    const uint64_t c = l.t - job.chunk_begin;
-    const uint64_t first = c * (uint64_t)job.block;
+// A record in (or on its way to) the warp's buffer: its chunk, size and 16-byte phase there.
+struct Rec {
+    const Job *job;
+    uint64_t c;
+    uint32_t size;
+    uint32_t phase;                               // kBadRecord: its location is invalid
+};
+constexpr uint32_t kBadRecord = 16u;
+
+// Starts the cp.async of a located record into rbuf.
+__device__ __forceinline__ Rec issue_record(const Loc &l, uint8_t *rbuf, int lane) {
+    const Job &job = *l.job;
+    const uint64_t rec_off = 32ull + 4ull * job.nchunks + l.off;
+    const uint64_t first = l.c * (uint64_t)job.block;
+    const uint32_t size = l.size;
     const uint32_t m = (uint32_t)((job.n - first) < job.block ? (job.n - first) : job.block);
     const uint32_t z1b = job.dtype == 0 ? 8u : (job.dtype == 1 ? 4u : 2u);
-    if (l.size < 3u + z1b || l.size > max_record(m, job.dtype) || l.rec_off + l.size > job.in_bytes) return false;
-    const uint8_t *gsrc = job.in + l.rec_off;
+    if (size < 3u + z1b || size > max_record(m, job.dtype) || rec_off + size > job.in_bytes)
+        return {l.job, l.c, size, kBadRecord};
+    const uint8_t *gsrc = job.in + rec_off;
     const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(gsrc) & 15u);
     const uint8_t *gbase = gsrc - sh;                       // >= job.in (16-byte aligned)
     const uint8_t *gend = job.in + job.in_bytes;
-    const uint32_t units = (sh + l.size + 15u) / 16u;
+    const uint32_t units = (sh + size + 15u) / 16u;
     const uint32_t base = smem_addr(rbuf);
-    for (uint32_t u = lane; u < units; u += 32) {
-        const uint8_t *src = gbase + 16u * u;
-        if (src + 16 <= gend) cp_async16(base + 16u * u, src);
-        else
-            for (uint32_t b = 0; b < 16u && src + b < gend; ++b) rbuf[16u * u + b] = src[b];
+    // only the stream's last unit may reach past its end
+    const uint32_t whole = gbase + 16u * units <= gend ? units : units - 1u;
+#pragma unroll 4
+    for (uint32_t u = lane; u < whole; u += 32) cp_async16(base + 16u * u, gbase + 16u * u);
+    if (whole < units) {
+        const uint32_t b = 16u * whole + (uint32_t)lane;
+        if (lane < 16 && gbase + b < gend) rbuf[b] = gbase[b];
     }
-    return true;
+    return {l.job, l.c, size, sh};
 }
 
-// Copies len bytes from any byte address of a shared buffer to a 16-byte aligned one in
-// another buffer: one 16-byte store per lane and unit, built from two aligned 16-byte loads
-// and funnel shifts, then the tail bytes singly.  The source buffer has 16 readable bytes past
-// the copied bytes.
-__device__ __forceinline__ void copy_to_planes(uint8_t *dst, const uint8_t *src, uint32_t len, int lane) {
-    const uintptr_t sa = reinterpret_cast<uintptr_t>(src);
-    const uint32_t off = (uint32_t)(sa & 15u), k0 = off >> 2, sb = (off & 3u) * 8u;
-    const uint4 *S = reinterpret_cast<const uint4 *>(sa - off);
-    const uint32_t units = len >> 4;
-    for (uint32_t u = (uint32_t)lane; u < units; u += 32) {
-        const uint4 a = S[u], b = S[u + 1];
-        uint4 o;
-        switch (k0) {
-            case 0: o = make_uint4(__funnelshift_r(a.x, a.y, sb), __funnelshift_r(a.y, a.z, sb), __funnelshift_r(a.z, a.w, sb), __funnelshift_r(a.w, b.x, sb)); break;
-            case 1: o = make_uint4(__funnelshift_r(a.y, a.z, sb), __funnelshift_r(a.z, a.w, sb), __funnelshift_r(a.w, b.x, sb), __funnelshift_r(b.x, b.y, sb)); break;
-            case 2: o = make_uint4(__funnelshift_r(a.z, a.w, sb), __funnelshift_r(a.w, b.x, sb), __funnelshift_r(b.x, b.y, sb), __funnelshift_r(b.y, b.z, sb)); break;
-            default: o = make_uint4(__funnelshift_r(a.w, b.x, sb), __funnelshift_r(b.x, b.y, sb), __funnelshift_r(b.y, b.z, sb), __funnelshift_r(b.z, b.w, sb)); break;
+// Where the rows of up to 32 planes lie (Sec. 3.3).  `rows`: the planes that exist (low bits),
+// `dense` the dense ones among them; `cur`: shared-memory offset of the top plane's row, moved to
+// the end of the last row.  Sparse rows are walked top to bottom (each one's length is known only
+// from its bitmap) and expanded into their 128-byte slots; then lane p writes plane p's place.
+// Per sparse row the lane reads the 32 bitmap bits of its 8-lane group: the groups' counts meet in
+// one byte-packed OR reduction, whose prefix is one multiply, and the lane's non-zero bytes are
+// one unaligned word, spread by one byte permute.  No position is checked: a row takes at most
+// 16 + 128 bytes, so every read stays in the record buffer whatever the bytes say, and the caller's
+// size check rejects a malformed record before anything is stored.
+struct RowLane {                                  // per-lane constants of a chunk's row walk
+    uint32_t keep;                                // bitmap bits of this lane's group that exist
+    uint32_t before;                              // those of the lanes before this one
+    uint32_t seltab;                              // expand_sel(lane & 15)
+};
+__device__ __forceinline__ void place_rows(uint8_t *smem, uint32_t slots, uint32_t tab, uint32_t &cur, uint32_t rows,
+                                           uint32_t dense, uint32_t row_bytes, uint32_t bm_bytes, const RowLane &rl,
+                                           int lane) {
+    const uint32_t start = cur;
+    const uint32_t group = (uint32_t)lane >> 3, gshift = 8u * group, nshift = 28u - 4u * ((uint32_t)lane & 7u);
+    const uint32_t presel = group ? 0x443Fu + group : 0x4444u;
+    uint32_t sparse = rows & ~dense;
+    uint32_t sum = 0, mine = 0;                   // sparse bytes so far; above this lane's plane
+    uint32_t above = 32u - (uint32_t)__clz((int)rows);
+    // the row before: its two words, shift, selector and slot (its store waits for none of this
+    // row's loads; the first iteration stores zeros where the second puts the first row)
+    uint32_t w0 = 0, w1 = 0, wsh = 0, sel = 0x4444u;
+    uint8_t *slot = smem + slots + 128u * (31u - (uint32_t)__clz((int)sparse)) + 4u * lane;
+    const bool any = sparse != 0u;
+#pragma unroll 1
+    while (sparse) {
+        const uint32_t p = 31u - (uint32_t)__clz((int)sparse);
+        sparse ^= 1u << p;
+        cur += row_bytes * (above - 1u - p);      // the dense rows in between
+        above = p;
+        const uint32_t b = cur + 4u * group;
+        const uint32_t *bw = reinterpret_cast<const uint32_t *>(smem + (b & ~3u));
+        const uint32_t b0 = bw[0], b1 = bw[1];
+        *reinterpret_cast<uint32_t *>(slot) = __byte_perm(__funnelshift_r(w0, w1, wsh), 0u, sel);
+        const uint32_t W = bswap(__funnelshift_r(b0, b1, b * 8u)) & rl.keep;   // first row byte at bit 31
+        const uint32_t incl = __reduce_or_sync(kFull, (uint32_t)__popc(W) << gshift) * 0x01010101u;
+        const uint32_t total = incl >> 24;        // at most 128
+        const uint32_t at = cur + bm_bytes + __byte_perm(incl, 0u, presel) + (uint32_t)__popc(W & rl.before);
+        sel = __shfl_sync(kFull, rl.seltab, (int)(W >> nshift));
+        const uint32_t *aw = reinterpret_cast<const uint32_t *>(smem + (at & ~3u));
+        w0 = aw[0];
+        w1 = aw[1];
+        wsh = at * 8u;
+        slot = smem + slots + 128u * p + 4u * lane;
+        cur += bm_bytes + total;
+        sum += bm_bytes + total;
+        if ((uint32_t)lane < p) mine = sum;
+    }
+    if (any) *reinterpret_cast<uint32_t *>(slot) = __byte_perm(__funnelshift_r(w0, w1, wsh), 0u, sel);
+    cur += row_bytes * above;
+    const bool mine_dense = (dense >> lane) & 1u, exists = (rows >> lane) & 1u;
+    uint32_t a = start + row_bytes * (uint32_t)__popc((dense >> lane) >> 1) + mine;
+    a = mine_dense ? a : (exists ? slots + 128u * (uint32_t)lane : 0u);
+    *reinterpret_cast<uint2 *>(smem + tab + 8u * lane) = make_uint2(a & ~3u, a * 8u);
+}
+
+// This lane's word (row bytes 4 lane .. 4 lane + 3) of kN planes placed by place_rows.
+template <int kN>
+__device__ __forceinline__ void gather_rows(const uint8_t *smem, uint32_t tab, int lane, uint32_t (&r)[kN]) {
+    const uint8_t *mine = smem + 4 * lane;
+#pragma unroll
+    for (int i = 0; i < kN / 2; ++i) {
+        const uint4 e = *reinterpret_cast<const uint4 *>(smem + tab + 16 * i);
+        const uint32_t *x = reinterpret_cast<const uint32_t *>(mine + e.x), *y = reinterpret_cast<const uint32_t *>(mine + e.z);
+        r[2 * i] = __funnelshift_r(x[0], x[1], e.y);
+        r[2 * i + 1] = __funnelshift_r(y[0], y[1], e.w);
+    }
+}
+
+// 32 bytes to global memory with one store (32-byte aligned): a whole sector per lane.
+__device__ __forceinline__ void store32(void *dst, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
+
+// Values (four 16-byte words at a time) of a lane as 64-bit words.
+__device__ __forceinline__ uint64_t pair64(uint64_t const (&d)[32], int i) { return d[i]; }
+__device__ __forceinline__ uint64_t pair64(uint32_t const (&d)[32], int i) { return ((uint64_t)d[2 * i + 1] << 32) | d[2 * i]; }
+__device__ __forceinline__ uint64_t pair64(uint16_t const (&d)[32], int i) {
+    const uint32_t lo = (uint32_t)d[4 * i] | ((uint32_t)d[4 * i + 1] << 16);
+    const uint32_t hi = (uint32_t)d[4 * i + 2] | ((uint32_t)d[4 * i + 3] << 16);
+    return ((uint64_t)hi << 32) | lo;
+}
+
+// The chunk's m values (lane l holds 32 l .. 32 l + 31 in d, lane 31 value 1024 in vx) to dst.  A
+// whole FP64 chunk at a 32-byte aligned address: each lane stores its contiguous values in whole
+// sectors.  Otherwise they pass through the slots (swizzled; FP64 half the lanes at a time) and
+// leave as coalesced 16-byte units, or single values where dst is not 16-byte aligned.  (Whole
+// sectors against staging: FP64 segments 325 / 332 us, FP32 170 / 162 us, so FP32 and FP16, whose
+// values pass the slots once, always stage.)
+template <int D>
+__device__ __forceinline__ void store_values(uint8_t *dst, uint32_t m, uint8_t *slots,
+                                             const typename Traits<D>::U (&d)[32], typename Traits<D>::U vx, int lane) {
+    using T = Traits<D>;
+    using U = typename T::U;
+    constexpr int S = T::S, UN = T::UNITS, PER = 16 / S;
+    if (m > 1024u && lane == 31) *reinterpret_cast<U *>(dst + 1024 * S) = vx;
+    if (D == kD64 && m >= 1024u && (reinterpret_cast<uintptr_t>(dst) & 31u) == 0) {
+        uint8_t *mine = dst + lane * (32 * S);
+#pragma unroll
+        for (int i = 0; i < S; ++i)
+            store32(mine + 32 * i, pair64(d, 4 * i), pair64(d, 4 * i + 1), pair64(d, 4 * i + 2), pair64(d, 4 * i + 3));
+        return;
+    }
+    constexpr int kPasses = D == kD64 ? 2 : 1, kLanes = 32 / kPasses;
+    const bool al16 = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0;
+#pragma unroll 1
+    for (int pass = 0; pass < kPasses; ++pass) {
+        const uint32_t v0 = (uint32_t)(pass * kLanes * 32);
+        if (v0 >= m) break;
+        const uint32_t cnt = min(m - v0, (uint32_t)(kLanes * 32));
+        if (lane / kLanes == pass) {
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                const uint64_t lo = pair64(d, 2 * u), hi = pair64(d, 2 * u + 1);
+                *reinterpret_cast<uint4 *>(slots + ((lane % kLanes) * UN + unit_swizzle<D>(lane % kLanes, u)) * 16) =
+                    make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+            }
         }
-        *reinterpret_cast<uint4 *>(dst + 16u * u) = o;
+        __syncwarp();
+        uint8_t *out = dst + v0 * S;
+        uint32_t done = 0;
+        if (cnt == (uint32_t)(kLanes * 32)) {     // whole pass: fixed trip counts
+            if (al16) {
+#pragma unroll
+                for (int i = 0; i < kLanes * UN / 32; ++i) {
+                    const uint32_t q = 32u * i + lane;
+                    *reinterpret_cast<uint4 *>(out + 16u * q) = *reinterpret_cast<const uint4 *>(slots + phys_unit<D>(q) * 16u);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < kLanes; ++i) {
+                    const uint32_t e = 32u * i + lane;
+                    *reinterpret_cast<U *>(out + e * S) = *reinterpret_cast<const U *>(slots + phys_elem_byte<D>(e));
+                }
+            }
+            __syncwarp();
+            continue;
+        }
+        if (al16) {
+            const uint32_t nunits = cnt * S >> 4;
+#pragma unroll 4
+            for (uint32_t q = lane; q < nunits; q += 32)
+                *reinterpret_cast<uint4 *>(out + 16u * q) = *reinterpret_cast<const uint4 *>(slots + phys_unit<D>(q) * 16u);
+            done = nunits * PER;
+        }
+        // value 32 i + lane of the pass belongs to its lane i, unit lane / PER
+#pragma unroll 8
+        for (uint32_t e = done + lane; e < cnt; e += 32)
+            *reinterpret_cast<U *>(out + e * S) = *reinterpret_cast<const U *>(slots + phys_elem_byte<D>(e));
+        __syncwarp();
     }
-    const uint32_t tail = len & 15u;
-    if ((uint32_t)lane < tail) dst[16u * units + lane] = src[16u * units + lane];
 }
 
-// `next` starts the copy of the warp's next record into rbuf; it is called exactly once, as
-// soon as this record has been read completely.
 // A value's exact FP64 value, and its key in IEEE 754 totalOrder (for min / max of non-NaN values).
 __device__ __forceinline__ double value_f64(uint64_t b) { return __longlong_as_double((long long)b); }
 __device__ __forceinline__ double value_f64(uint32_t b) { return (double)__uint_as_float(b); }
@@ -159,89 +311,87 @@ __device__ __forceinline__ uint64_t order_key(double x) {
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
+// One chunk's record (in the warp's buffer at shared-memory offset wofs) to its values.  `next`
+// starts the copy of the warp's next record into the buffer; it is called exactly once, as soon as
+// this record has been read completely.
 // kAgg (analytics on compressed data): instead of storing the values, the warp adds them up
 // (NaN count, totalOrder min / max, their sum: each lane its 32 values in index order, then a
 // butterfly over the lanes, identical in every lane since FP addition commutes); the chunk's
 // sum goes to sums[c], the rest into the control block by atomics.
-template <int D, bool kAgg, class Next>
-__device__ void decode_chunk(const Job &job, const Loc &l, bool loc_ok, const uint8_t *rbuf, uint8_t *pbuf,
-                             int lane, Next &&next, Control *ctl) {
+template <int D, class L, bool kAgg, class Next>
+__device__ __forceinline__ void decode_chunk(const Rec &r0, uint8_t *smem, uint32_t wofs, uint32_t seltab, int lane,
+                                             Next &&next, Control *ctl) {
     using T = Traits<D>;
     using U = typename T::U;
-
-    const uint64_t c = l.t - job.chunk_begin;
+    const uint32_t slots = wofs + L::kBuf, tab = slots + L::kSlots;
+    const Job &job = *r0.job;
+    const uint64_t c = r0.c;
     const uint32_t B = job.block;
     const uint64_t first = c * (uint64_t)B;
     const uint32_t m = (uint32_t)((job.n - first) < B ? (job.n - first) : B);
     const uint32_t cols = chunk_cols(m);
-    const uint32_t nact = cols / 32u;
-    const uint32_t row_bytes = cols / 8u;
-    const uint32_t size = l.size;
-    const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(job.in + l.rec_off) & 15u);
-    const uint8_t *rec = rbuf + sh;
-    // plane p lives in slot W - 1 - p of pbuf: slot addresses are written planes + (63 - p) * 128
-    uint8_t *planes = pbuf - (64 - T::W) * 128;
-    uint16_t *rowpos = reinterpret_cast<uint16_t *>(pbuf + T::W * 128);
+    const uint32_t row_bytes = cols / 8u, bm_bytes = cols / 64u;
+    const uint32_t rec = wofs + (r0.phase & 15u);
 
-    // ---- a. header, flags, row positions; sparse rows expanded ---------------------------
-    bool bad = !loc_ok;
-    uint32_t alpha = 0, beta_hat = 0, w = 0, pos = 0;
-    U z1 = 0;
-    uint64_t dense_mask = 0;
-    if (!bad) {
-        alpha = rec[0];
-        beta_hat = rec[1];
+    // ---- a. header and flags ------------------------------------------------------------------
+    bool bad = r0.phase == kBadRecord;
+    const uint32_t h0 = lds_any(smem, rec);
+    const uint32_t alpha = h0 & 0xFFu, beta_hat = (h0 >> 8) & 0xFFu;
+    U z1;
+    if constexpr (D == kD64) z1 = ((uint64_t)lds_any(smem, rec + 6) << 32) | lds_any(smem, rec + 2);
+    else if constexpr (D == kD32) z1 = lds_any(smem, rec + 2);
+    else z1 = (uint16_t)(h0 >> 16);
+    const uint32_t w = smem[rec + 2 + T::Z1B];
+    const uint32_t hdr = 3u + T::Z1B + (w + 7u) / 8u;
+    if (w > (uint32_t)T::W || (m <= 1u && w != 0u) || hdr > r0.size) bad = true;
+    // the flags' last w bits, big-endian: bit p is plane p's
+    const uint32_t rows_lo = w >= 32u ? ~0u : (1u << w) - 1u;
+    const uint32_t dense_lo = bswap(lds_any(smem, rec + hdr - 4u)) & rows_lo;
+    RowLane rl;
+    {
+        const uint32_t nact = cols / 32u, g8 = (uint32_t)lane & ~7u;
+        const uint32_t have = nact > g8 ? min(nact - g8, 8u) : 0u;          // lanes of this group with row bytes
+        rl.keep = have ? 0xFFFFFFFFu << (32u - 4u * have) : 0u;
+        rl.before = (lane & 7) ? 0xFFFFFFFFu << (32u - 4u * ((uint32_t)lane & 7u)) : 0u;
+        rl.seltab = seltab;
+    }
+    uint32_t cur = rec + hdr;
+
+    // ---- b. every plane's row: placed, gathered (lane: 4 row bytes per plane), transposed -------
+    // The planes are transposed one row up (plane p at row p - 1) and XORed with plane 0, whose
+    // bits are the signs: that is the inverse zigzag of all values at once, one XOR per plane.
+    // Lanes past the row's bytes (tail chunks) gather stale bytes; their columns lie past the
+    // chunk's values, are never stored, and only feed the scan of later lanes.
+    U d[32];
+    uint32_t top0 = 0;                            // FP64: plane 32's word
+    if constexpr (D == kD64) {
+        if (!bad && w > 32u) {
+            const uint32_t rows_hi = w >= 64u ? ~0u : (1u << (w - 32u)) - 1u;
+            const uint32_t dense_hi = bswap(lds_any(smem, rec + hdr - 8u)) & rows_hi;
+            place_rows(smem, slots, tab, cur, rows_hi, dense_hi, row_bytes, bm_bytes, rl, lane);
+            __syncwarp();
+            uint32_t a[32];
+            {
+                uint32_t r[32];
+                gather_rows<32>(smem, tab, lane, r);
+                top0 = r[0];
 #pragma unroll
-        for (int i = 0; i < T::Z1B; ++i) z1 |= (U)rec[2 + i] << (8 * i);
-        w = rec[2 + T::Z1B];
-        const uint32_t flag_bytes = (w + 7u) / 8u;
-        pos = 3u + T::Z1B + flag_bytes;
-        if (w > (uint32_t)T::W || (m <= 1u && w != 0u) || pos > size) bad = true;
-        else
-            for (uint32_t i = 0; i < flag_bytes; ++i) dense_mask = (dense_mask << 8) | rec[3 + T::Z1B + i];
-    }
-    const bool active = (uint32_t)lane < nact;
-    const uint32_t bm_bytes = nact / 2u;
-    const uint32_t hdr = pos;
-    const uint64_t wmask = (w >= 64u) ? ~0ull : ((1ull << w) - 1ull);
-    // Sparse rows only (top to bottom): a sparse row's position is the header, the dense rows
-    // above it (row_bytes each) and the sparse rows above it.  Dense rows need no walk.  No
-    // position is checked here: a row takes at most 16 + 128 bytes, so every read stays in the
-    // record buffer whatever the bytes say, and the size check after the walk (every row's
-    // bytes add up to the record size) rejects a malformed record before anything is stored.
-    uint64_t sparse = bad ? 0ull : (~dense_mask & wmask);
-    uint32_t sparse_sum = 0, walked = 0;       // sparse rows above the current one
-#pragma unroll 1
-    while (sparse) {
-        const int p = 63 - __clzll((long long)sparse);
-        sparse &= ~(1ull << p);
-        // rows above p: w - 1 - p, of which `walked` are sparse
-        const uint32_t spos = hdr + row_bytes * (w - 1u - (uint32_t)p - walked) + sparse_sum;
-        ++walked;
-        uint32_t nib = 0;
-        if (active) {
-            const uint32_t byte = rec[spos + (lane >> 1)];
-            nib = (lane & 1) ? (byte & 0xFu) : (byte >> 4);
+                for (int i = 0; i < 31; ++i) a[i] = r[i + 1];
+                a[31] = 0;
+            }
+            transpose32(a);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) d[k] = (U)a[k ^ 7] << 32;
+            __syncwarp();
+        } else {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) d[k] = 0;
         }
-        const uint32_t cnt = nibble_count(nib);
-        const unsigned b0 = __ballot_sync(kFull, cnt & 1u);
-        const unsigned b1 = __ballot_sync(kFull, cnt & 2u);
-        const unsigned b2 = __ballot_sync(kFull, cnt & 4u);
-        const unsigned lt = (1u << lane) - 1u;
-        const uint32_t before = __popc(b0 & lt) + 2u * __popc(b1 & lt) + 4u * __popc(b2 & lt);
-        const uint32_t nnz = __reduce_add_sync(kFull, cnt);
-        // the lane's non-zero bytes start at record byte spos + bm_bytes + before: load the
-        // four bytes from there (two aligned words) and put each in its place with one byte
-        // permute (selector by the bitmap nibble)
-        const uint32_t qa = sh + spos + bm_bytes + before;
-        const uint32_t *wq = reinterpret_cast<const uint32_t *>(rbuf + (qa & ~3u));
-        const uint32_t word = __funnelshift_r(wq[0], wq[1], (qa & 3u) * 8u);
-        const uint32_t x = __byte_perm(word, 0u, s_expand_sel[nib]);
-        *reinterpret_cast<uint32_t *>(planes + (63 - p) * 128 + 4 * lane) = x;
-        sparse_sum += bm_bytes + nnz;
-        if (lane == 0) rowpos[p] = (uint16_t)sparse_sum;   // sparse bytes through row p
     }
-    if (!bad && hdr + row_bytes * (uint32_t)__popcll(dense_mask & wmask) + sparse_sum != size) bad = true;
+    if (!bad) {
+        place_rows(smem, slots, tab, cur, rows_lo, dense_lo, row_bytes, bm_bytes, rl, lane);
+        bad = cur - rec != r0.size;
+    }
     if (bad) {
         if (lane == 0) set_status(job.result, kErrCorrupt);
         __syncwarp();
@@ -249,127 +399,95 @@ __device__ void decode_chunk(const Job &job, const Loc &l, bool loc_ok, const ui
         return;
     }
     __syncwarp();
-
-    // ---- b. dense runs copied into the plane slots (plane p: slot 63 - p, 128 bytes, in
-    //      record order), then every plane word gathered with one aligned load ---------------
     {
-        uint64_t dm = dense_mask & wmask;
-#pragma unroll 1
-        while (dm) {
-            const int p = 63 - __clzll((long long)dm);
-            const uint64_t below = (p >= 63) ? ~0ull : ((2ull << p) - 1ull);
-            const uint64_t holes = ~dense_mask & below;
-            const int q = (row_bytes == 128u) ? (holes ? 64 - __clzll((long long)holes) : 0) : p;
-            const uint64_t above = (p >= 63) ? 0ull : (wmask & ~((2ull << p) - 1ull));
-            const uint64_t sp_above = ~dense_mask & above;
-            // sparse bytes above p: the running total at the lowest sparse row above p
-            const uint32_t sbytes = sp_above ? (uint32_t)rowpos[__ffsll((long long)sp_above) - 1] : 0u;
-            const uint32_t rp = hdr + row_bytes * (uint32_t)__popcll(dense_mask & above) + sbytes;
-            copy_to_planes(planes + (63 - p) * 128, rec + rp, (uint32_t)(p - q + 1) * row_bytes, lane);
-            dm &= (q > 0) ? ((1ull << q) - 1ull) : 0ull;
-        }
-    }
-    __syncwarp();
-    next();                                       // the record has been read
-    // Slots of planes >= w hold stale bytes: they are masked off after each transpose (bit p
-    // of every value), one AND per value instead of a select per word.  Lanes >= nact (tail
-    // chunks) gather stale words too; their columns lie past the chunk's values and are never
-    // stored, and they only feed the scan of later lanes.
-    auto plane_word = [&](int p) -> uint32_t {
-        return *reinterpret_cast<const uint32_t *>(planes + (63 - p) * 128 + 4 * lane);
-    };
-    U d[32];
-    if constexpr (D == 0) {
-        if (w > 32) {
-            uint32_t a[32];
+        constexpr int R = T::W < 32 ? T::W : 32;
+        uint32_t a[32], r[R];
+        gather_rows<R>(smem, tab, lane, r);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) a[i] = plane_word(i + 32);
-            transpose32(a);
-            const uint32_t keep = w >= 64 ? ~0u : ((1u << (w - 32)) - 1u);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] = (U)(a[k ^ 7] & keep) << 32;
-        } else {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] = 0;
-        }
-    }
-    {
-        uint32_t a[32];
-#pragma unroll
-        for (int p = 0; p < 32; ++p) a[p] = p < T::W ? plane_word(p) : 0u;    // FP16: 16 planes
+        for (int i = 0; i < 32; ++i) a[i] = i + 1 < R ? r[i + 1] ^ r[0] : (i + 1 == R ? top0 ^ r[0] : 0u);
+        __syncwarp();
+        next();                                   // the record has been read
         transpose32(a);
-        const uint32_t keep = w >= 32 ? ~0u : ((1u << w) - 1u);
-        if constexpr (D == 0) {
 #pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] |= (U)(a[k ^ 7] & keep);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] = (U)(a[k ^ 7] & keep);
+        for (int k = 0; k < 32; ++k) {
+            if constexpr (D == kD64) {
+                const uint32_t s = (uint32_t)((int32_t)(r[0] << (31 - (k ^ 7))) >> 31);
+                d[k] = ((uint64_t)((uint32_t)(d[k] >> 32) ^ s) << 32) | a[k ^ 7];
+            } else {
+                d[k] = (U)a[k ^ 7];
+            }
         }
     }
+    // ---- c. G (inverse Eq. 5): lane l's values 32 l .. 32 l + 31 -------------------------------
     U run = 0;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) { run += unzigzag(d[k]); d[k] = run; }
-    U lane_off;
-    if constexpr (D == 0) lane_off = warp_exclusive_u64(run, lane);
-    else lane_off = (U)warp_exclusive_u64((uint64_t)run, lane);
-    const U gbase = z1 + lane_off;               // G of value 32*lane + k + 1 = gbase + d[k]
-    const bool case1 = alpha <= (uint32_t)T::A_MAX && beta_hat <= (uint32_t)T::B_MAX;
-    if (case1) {
-        if constexpr (D == 0) {
-            // |g| >= 2^53 only in streams no encoder writes: then every value takes the FP64 path
-            bool big = false;
+    for (int k = 0; k < 32; ++k) run += d[k];
+    if constexpr (D == kD64) run = z1 + warp_exclusive_u64(run, lane);
+    else run = (U)(z1 + warp_exclusive_u32((uint32_t)run, lane));
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                const uint64_t gk = gbase + d[k];
-                big |= (gk + (1ull << 53)) > (1ull << 54);          // |g| > 2^53
-            }
-            if (__any_sync(kFull, big)) {
+    for (int k = 0; k < 32; ++k) {
+        const U t = d[k];
+        d[k] = run;
+        run += t;
+    }
+    U vx = run;                                   // lane 31: value 1024
+    // ---- d. values (inverse Eq. 4) ---------------------------------------------------------------
+    if (alpha <= (uint32_t)T::A_MAX && beta_hat <= (uint32_t)T::B_MAX) {
+        if constexpr (D == kD64) {
+            // every g fits 32 bits (|g| <= 2^31): the common case
+            uint32_t wide = 0;
+            auto hi = [](uint64_t g) { return (uint32_t)(g >> 32); };
+            auto sgn = [](uint32_t x) { return (uint32_t)((int32_t)x >> 31); };
 #pragma unroll
-                for (int k = 0; k < 32; ++k)
-                    d[k] = (U)__double_as_longlong(div_pow10((int64_t)(gbase + d[k]), (int)alpha));
+            for (int k = 0; k < 32; ++k) wide |= hi(d[k]) ^ sgn((uint32_t)d[k]);
+            wide |= hi(vx) ^ sgn((uint32_t)vx);
+            if (alpha <= (uint32_t)kDiv10NarrowMax && !__any_sync(kFull, wide)) {
+                const Div10Narrow q = div10_narrow_of((int)alpha);
+                auto conv = [&](uint32_t g) {
+                    const uint32_t s = sgn(g);
+                    return div_pow10_exact32((g ^ s) - s, s, q);
+                };
+#pragma unroll
+                for (int k = 0; k < 32; ++k) d[k] = conv((uint32_t)d[k]);
+                vx = conv((uint32_t)vx);
             } else {
+                uint32_t big = hi(vx) ^ sgn(hi(vx));
 #pragma unroll
-                for (int k = 0; k < 32; ++k) d[k] = div_pow10_exact((int64_t)(gbase + d[k]), (int)alpha);
+                for (int k = 0; k < 32; ++k) big |= hi(d[k]) ^ sgn(hi(d[k]));
+                if (__any_sync(kFull, big >= (1u << 21))) {       // some |g| > 2^53: only in streams no encoder writes
+#pragma unroll 1
+                    for (int i = 0; i < 32; ++i) {          // rolled (small code): the values rotate through d[0]
+                        const U v = (U)__double_as_longlong(div_pow10((int64_t)d[0], (int)alpha));
+#pragma unroll
+                        for (int k = 0; k < 31; ++k) d[k] = d[k + 1];
+                        d[31] = v;
+                    }
+                    vx = (U)__double_as_longlong(div_pow10((int64_t)vx, (int)alpha));
+                } else {
+                    const Div10 q = div10_of((int)alpha);
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) d[k] = div_pow10_exact((int64_t)d[k], q);
+                    vx = div_pow10_exact((int64_t)vx, q);
+                }
             }
         } else if constexpr (D == kD32) {
 #pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] = (U)__float_as_uint(div_pow10((int32_t)(gbase + d[k]), (int)alpha));
+            for (int k = 0; k < 32; ++k) d[k] = (U)__float_as_uint(div_pow10((int32_t)d[k], (int)alpha));
+            vx = (U)__float_as_uint(div_pow10((int32_t)vx, (int)alpha));
         } else {
             // fl16(g / 10^a) as fl16(fl32(g / 10^a)): exact for every 16-bit g and a <= 4 (the
             // second rounding never lands on a different value; checked for all 327,680 inputs)
             const float p = __uint_as_float(FALCON_P10_F32[alpha - FALCON_P10_F32_LO]);
+            auto conv = [&](U g) { return __half_as_ushort(__float2half_rn(__fdiv_rn((float)(int16_t)g, p))); };
 #pragma unroll
-            for (int k = 0; k < 32; ++k)
-                d[k] = __half_as_ushort(__float2half_rn(__fdiv_rn((float)(int16_t)(U)(gbase + d[k]), p)));
+            for (int k = 0; k < 32; ++k) d[k] = conv(d[k]);
+            vx = conv(vx);
         }
     } else {
 #pragma unroll
-        for (int k = 0; k < 32; ++k) d[k] = unzigzag((U)(gbase + d[k]));
+        for (int k = 0; k < 32; ++k) d[k] = unzigzag(d[k]);
+        vx = unzigzag(vx);
     }
-    U v0;
-    if (case1) {
-        if constexpr (D == 0) {
-            const uint64_t g1 = z1;
-            v0 = ((g1 + (1ull << 53)) > (1ull << 54)) ? (U)__double_as_longlong(div_pow10((int64_t)g1, (int)alpha))
-                                                       : div_pow10_exact((int64_t)g1, (int)alpha);
-        } else if constexpr (D == kD32) {
-            v0 = (U)__float_as_uint(div_pow10((int32_t)z1, (int)alpha));
-        } else {
-            v0 = __half_as_ushort(__float2half_rn(
-                __fdiv_rn((float)(int16_t)z1, __uint_as_float(FALCON_P10_F32[alpha - FALCON_P10_F32_LO]))));
-        }
-    } else {
-        v0 = unzigzag(z1);
-    }
-    // shift by one so that lane l holds values 32l .. 32l+31 (value 1024 stays in vx)
-    U carry = shfl_up_x(d[31], 1);
-    if (lane == 0) carry = v0;
-    const U vx = d[31];
-#pragma unroll
-    for (int k = 31; k > 0; --k) d[k] = d[k - 1];
-    d[0] = carry;
-    __syncwarp();                                 // plane words consumed
 
     if constexpr (kAgg) {
         // keys in the values' own width (IEEE order = unsigned order of the keys), widened to
@@ -402,7 +520,7 @@ __device__ void decode_chunk(const Job &job, const Loc &l, bool loc_ok, const ui
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum = __dadd_rn(sum, __shfl_xor_sync(kFull, sum, o));
         if (lane == 0) {
-            reinterpret_cast<double *>(job.flags + tile_count(job.nchunks))[c] = sum;
+            reinterpret_cast<double *>(job.flags + job.nchunks)[c] = sum;
             if (nan) atomicAdd(&ctl->agg[0], (unsigned long long)nan);
             if (kmax) {                           // some value was not a NaN
                 auto unkey = [&](U k) { return (k & SIGN) ? (U)(k & ABSM) : (U)~k; };
@@ -414,47 +532,42 @@ __device__ void decode_chunk(const Job &job, const Loc &l, bool loc_ok, const ui
         return;
     }
 
-    // ---- c. stage (swizzled) and store --------------------------------------------------------
-    constexpr int UN = T::UNITS;
-#pragma unroll
-    for (int u = 0; u < UN; ++u) {
-        uint4 q;
-        if constexpr (D == 0) {
-            q = make_uint4((uint32_t)d[2 * u], (uint32_t)((uint64_t)d[2 * u] >> 32),
-                           (uint32_t)d[2 * u + 1], (uint32_t)((uint64_t)d[2 * u + 1] >> 32));
-        } else if constexpr (D == kD32) {
-            q = make_uint4((uint32_t)d[4 * u], (uint32_t)d[4 * u + 1], (uint32_t)d[4 * u + 2], (uint32_t)d[4 * u + 3]);
-        } else {
-            q = make_uint4((uint32_t)d[8 * u] | ((uint32_t)d[8 * u + 1] << 16), (uint32_t)d[8 * u + 2] | ((uint32_t)d[8 * u + 3] << 16),
-                           (uint32_t)d[8 * u + 4] | ((uint32_t)d[8 * u + 5] << 16), (uint32_t)d[8 * u + 6] | ((uint32_t)d[8 * u + 7] << 16));
-        }
-        *reinterpret_cast<uint4 *>(pbuf + (lane * UN + unit_swizzle<D>(lane, u)) * 16) = q;
-    }
-    if (m > 1024u && lane == 31) *reinterpret_cast<U *>(pbuf + phys_elem_byte<D>(1024)) = vx;
-    __syncwarp();
-    uint8_t *dst = job.out + first * T::S;
-    const uint32_t nbytes = m * T::S;
-    uint32_t done = 0;
-    if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-        const uint32_t nunits = nbytes >> 4;
-        for (uint32_t q = lane; q < nunits; q += 32)
-            *reinterpret_cast<uint4 *>(dst + 16u * q) = *reinterpret_cast<const uint4 *>(pbuf + phys_unit<D>(q) * 16u);
-        done = (nunits * 16u) / T::S;
-    }
-    for (uint32_t e = done + lane; e < m; e += 32)
-        *reinterpret_cast<U *>(dst + (size_t)e * T::S) = *reinterpret_cast<const U *>(pbuf + phys_elem_byte<D>(e));
-    __syncwarp();
+    store_values<D>(job.out + first * T::S, m, smem + slots, d, vx, lane);
 }
 
 }  // namespace
 
-// Record offsets per 64-chunk tile (exclusive prefix of the u32 size array) of every job
-// into the first words of job.flags.
+// The position of every record (exclusive prefix of the u32 size array) of every job into the
+// first words of job.flags.  `parts` CTAs per job, each over its own share of the chunks: a CTA
+// adds up every size before its share first (at most 152 CTAs reading at most the whole array, from
+// L2), then scans its share 1024 chunks at a time, so no CTA waits for another.
 __global__ void __launch_bounds__(1024)
-offsets_kernel(const Job *__restrict__ jobs, Job single) {
+offsets_kernel(const Job *__restrict__ jobs, Job single, uint32_t parts) {
     __shared__ uint64_t warp_sums[33];
-    const Job &job = (jobs == nullptr) ? single : jobs[blockIdx.x];
-    (void)tile_prefix(reinterpret_cast<const uint32_t *>(job.in + 32), job.nchunks, job.flags, warp_sums);
+    const Job &job = (jobs == nullptr) ? single : jobs[blockIdx.x / parts];
+    const uint32_t part = blockIdx.x % parts;
+    const uint64_t nc = job.nchunks;
+    const uint64_t share = ((nc + parts - 1) / parts + 1023u) & ~1023ull;
+    const uint64_t begin = part * share, end = begin + share < nc ? begin + share : nc;
+    if (begin >= nc) return;
+    const uint32_t *sizes = reinterpret_cast<const uint32_t *>(job.in + 32);      // 16-byte aligned
+    uint64_t carry = 0;
+    if (begin > 0) {                              // begin is a multiple of 1024
+        const uint4 *q = reinterpret_cast<const uint4 *>(sizes);
+        uint64_t sum = 0;
+        for (uint64_t i = threadIdx.x; i < begin / 4u; i += 1024u) {
+            const uint4 x = __ldg(q + i);
+            sum += (uint64_t)x.x + x.y + x.z + x.w;
+        }
+        (void)block_exclusive_scan(sum, carry, warp_sums);
+    }
+    for (uint64_t b = begin; b < end; b += 1024u) {
+        const uint64_t c = b + threadIdx.x;
+        uint64_t total;
+        const uint64_t ex = block_exclusive_scan(c < end ? sizes[c] : 0u, total, warp_sums);
+        if (c < end) job.flags[c] = carry + ex;
+        carry += total;
+    }
 }
 
 // Forms by dtype: kDt = 0 (every job FP64), 1 (every job FP32), 2 (either, per job).
@@ -462,18 +575,21 @@ constexpr int kDtF64 = 0, kDtF32 = 1, kDtMixed = 2, kDtF16 = 3;
 // the value kind whose buffers a form needs (the either-dtype form: the largest)
 template <int kDt> constexpr int layout_kind() { return kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64); }
 
+// Registers: 128 (FP64, either-dtype: 16 warps per SM), 80 (FP32, FP16: 24 warps; 96 registers and
+// 20 warps: 1.3 % slower).  The aggregate forms keep FP64 sums as well and take 168.
 template <int kDt, bool kAgg = false>
-__global__ void __launch_bounds__(32 * kMaxDecompressWarps, 1)
+__global__ void __maxnreg__((kDt == kDtF32 || kDt == kDtF16) && !kAgg ? 80 : (kAgg ? 168 : 128))
 decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     using L = DecLayout<layout_kind<kDt>()>;
-    uint8_t *wbase = smem + warp * L::kWarpBytes;
-    uint8_t *pbuf = wbase + L::kBuf;
+    const uint32_t wofs = kZeroBytes + (uint32_t)warp * L::kWarpBytes;
+    uint8_t *wbase = smem + wofs;
+    const uint32_t seltab = expand_sel((uint32_t)lane & 15u);
     __shared__ Job s_single;                      // the single job, read from shared memory
     if (threadIdx.x == 0) s_single = single;
-    init_expand_sel();
+    if (threadIdx.x < kZeroBytes / 16u) reinterpret_cast<uint4 *>(smem)[threadIdx.x] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     const uint64_t gw = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp;
     const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
@@ -481,46 +597,36 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
         const Job &jb = (jobs != nullptr) ? jobs[j] : s_single;
         if (lane == 0) jb.result[0] = jb.n;
     }
-    // chunk tickets two deep: t is decoded, tn's record is fetched during t, tnn is located
-    uint64_t t = ticket_of(take_ticket(ctl, kTicketDecode, lane));
-    if (t >= total_chunks) return;
+    // chunk tickets two deep: while one chunk is decoded the next one's record is fetched, and the
+    // ticket of the one after that is on its way (read, and its position loads issued, when this
+    // chunk is done)
+    constexpr bool kTable = kDt == kDtMixed;
     uint64_t tn = ticket_of(take_ticket(ctl, kTicketDecode, lane));
-    Loc lc = locate(jobs, njobs, s_single, t, lane);
-    resolve(jobs, njobs, s_single, lc);
-    bool okc = issue_record(job_of(jobs, njobs, s_single, t), lc, wbase, lane);
+    if (tn >= total_chunks) return;
+    Rec rec = issue_record(locate<kTable>(jobs, njobs, s_single, tn, total_chunks), wbase, lane);
     cp_async_commit();
-    Loc ln{};
-    if (tn < total_chunks) ln = locate(jobs, njobs, s_single, tn, lane);
+    tn = ticket_of(take_ticket(ctl, kTicketDecode, lane));
+    Loc ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks);
     for (;;) {
-        const unsigned long long raw = tn < total_chunks ? take_ticket(ctl, kTicketDecode, lane) : 0ull;
-        uint64_t tnn = total_chunks;
-        bool okn = false;
-        Loc lnn{};
+        const unsigned long long raw = take_ticket(ctl, kTicketDecode, lane);
         cp_async_wait_none();                    // the current record has landed
         __syncwarp();
         // the next record goes into the same buffer once this one has been read
+        Rec rn{};
         auto next = [&]() {
-            if (tn < total_chunks) {
-                resolve(jobs, njobs, s_single, ln);
-                okn = issue_record(job_of(jobs, njobs, s_single, tn), ln, wbase, lane);
-                tnn = ticket_of(raw);
-                if (tnn < total_chunks) lnn = locate(jobs, njobs, s_single, tnn, lane);
-            }
+            if (tn < total_chunks) rn = issue_record(ln, wbase, lane);
             cp_async_commit();
         };
-        const Job &job = job_of(jobs, njobs, s_single, t);
-        if constexpr (kDt == kDtF64) decode_chunk<kD64, kAgg>(job, lc, okc, wbase, pbuf, lane, next, ctl);
-        else if constexpr (kDt == kDtF32) decode_chunk<kD32, kAgg>(job, lc, okc, wbase, pbuf, lane, next, ctl);
-        else if constexpr (kDt == kDtF16) decode_chunk<kD16, kAgg>(job, lc, okc, wbase, pbuf, lane, next, ctl);
-        else if (job.dtype == 0) decode_chunk<kD64, kAgg>(job, lc, okc, wbase, pbuf, lane, next, ctl);
-        else if (job.dtype == 1) decode_chunk<kD32, kAgg>(job, lc, okc, wbase, pbuf, lane, next, ctl);
-        else decode_chunk<kD16, kAgg>(job, lc, okc, wbase, pbuf, lane, next, ctl);
+        if constexpr (kDt == kDtF64) decode_chunk<kD64, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
+        else if constexpr (kDt == kDtF32) decode_chunk<kD32, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
+        else if constexpr (kDt == kDtF16) decode_chunk<kD16, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
+        else if (rec.job->dtype == 0) decode_chunk<kD64, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
+        else if (rec.job->dtype == 1) decode_chunk<kD32, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
+        else decode_chunk<kD16, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
         if (tn >= total_chunks) break;
-        t = tn;
-        tn = tnn;
-        lc = ln;
-        okc = okn;
-        ln = lnn;
+        rec = rn;
+        tn = ticket_of(raw);
+        ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks);
     }
     cp_async_wait_none();
 }
@@ -528,7 +634,7 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
 int decompress_grid(uint64_t total_chunks) {
     const int w = g_cta_warps[1];
     return persistent_grid_size(reinterpret_cast<const void *>(decompress_kernel<kDtMixed>), w,
-                                w * DecLayout<kD64>::kWarpBytes,
+                                (int)(kZeroBytes + w * DecLayout<kD64>::kWarpBytes),
                                 g_ctas_per_sm[1], total_chunks);
 }
 
@@ -540,7 +646,7 @@ __global__ void __launch_bounds__(1024)
 aggregate_finish_kernel(Job single, Control *ctl, falcon_stats *out) {
     __shared__ double part[1024];
     const uint64_t nc = single.nchunks;
-    const double *sums = reinterpret_cast<const double *>(single.flags + tile_count(nc));
+    const double *sums = reinterpret_cast<const double *>(single.flags + nc);
     const uint64_t c0 = nc * threadIdx.x / 1024u, c1 = nc * (threadIdx.x + 1u) / 1024u;
     double s = -0.0;
     for (uint64_t c = c0; c < c1; ++c) s = __dadd_rn(s, sums[c]);
@@ -568,15 +674,25 @@ namespace {
 template <int kDt, bool kAgg = false>
 void launch_decode(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, Control *ctl,
                    cudaStream_t stream) {
-    const int w = g_cta_warps[1], smem = w * DecLayout<layout_kind<kDt>()>::kWarpBytes;
+    const int w = g_cta_warps[1], smem = (int)(kZeroBytes + w * DecLayout<layout_kind<kDt>()>::kWarpBytes);
     const int grid = persistent_grid_size(reinterpret_cast<const void *>(decompress_kernel<kDt, kAgg>), w, smem,
                                           g_ctas_per_sm[1], total_chunks);
     decompress_kernel<kDt, kAgg><<<grid, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
 }
 }  // namespace
 
+// One CTA per 1024 chunks up to 152 for a single stream; a table's many jobs get one each.
+static void launch_offsets(const Job *d_jobs, int njobs, const Job &single, cudaStream_t stream) {
+    uint32_t parts = 1;
+    if (d_jobs == nullptr) {
+        const uint64_t steps = (single.nchunks + 1023u) / 1024u;
+        parts = steps < 1u ? 1u : (steps > 152u ? 152u : (uint32_t)steps);
+    }
+    offsets_kernel<<<(unsigned)njobs * parts, 1024, 0, stream>>>(d_jobs, single, parts);
+}
+
 cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cudaStream_t stream) {
-    offsets_kernel<<<1, 1024, 0, stream>>>(nullptr, single);
+    launch_offsets(nullptr, 1, single, stream);
     if (single.nchunks > 0) {
         if (single.dtype == 0) launch_decode<kDtF64, true>(nullptr, 1, single, single.nchunks, ctl, stream);
         else if (single.dtype == 1) launch_decode<kDtF32, true>(nullptr, 1, single, single.nchunks, ctl, stream);
@@ -588,7 +704,7 @@ cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cud
 
 cudaError_t launch_decompress(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks,
                               Control *ctl, cudaStream_t stream) {
-    offsets_kernel<<<(d_jobs != nullptr) ? njobs : 1, 1024, 0, stream>>>(d_jobs, single);
+    launch_offsets(d_jobs, njobs, single, stream);
     if (d_jobs != nullptr) launch_decode<kDtMixed>(d_jobs, njobs, single, total_chunks, ctl, stream);
     else if (single.dtype == 0) launch_decode<kDtF64>(d_jobs, njobs, single, total_chunks, ctl, stream);
     else if (single.dtype == 1) launch_decode<kDtF32>(d_jobs, njobs, single, total_chunks, ctl, stream);

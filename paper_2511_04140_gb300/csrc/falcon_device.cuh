@@ -154,17 +154,15 @@ __device__ __forceinline__ uint64_t warp_exclusive_u64(uint64_t v, int lane) {
     return incl - v;
 }
 
-// number of zero bytes of a 32-bit word (exact)
-__device__ __forceinline__ int zero_bytes(uint32_t x) {
-    uint32_t y = (x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu;
-    y = ~(y | x | 0x7F7F7F7Fu);
-    return __popc(y);
-}
-// 4-bit mask, bit (3-i) set iff byte i of x is non-zero
-__device__ __forceinline__ uint32_t nonzero_nibble(uint32_t x) {
-    uint32_t y = (x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu;
-    y = (y | x) & 0x80808080u;          // bit 8i+7 set iff byte i != 0
-    return ((y >> 4) & 8u) | ((y >> 13) & 4u) | ((y >> 22) & 2u) | ((y >> 31) & 1u);
+// the same for a 32-bit lane value
+__device__ __forceinline__ uint32_t warp_exclusive_u32(uint32_t v, int lane) {
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    return incl - v;
 }
 
 // --------------------------------------------------------------------------------------
@@ -513,39 +511,67 @@ __device__ __forceinline__ uint16_t case1_g(uint16_t u, int a) {
     return (uint16_t)((u >> 15) ? (0u - N) : N);
 }
 
-// fl(g / 10^a), correctly rounded (nearest, ties to even), for |g| < 2^53 and 0 <= a <= 22, in
+// fl(g / 10^a), correctly rounded (nearest, ties to even), for |g| <= 2^53 and 0 <= a <= 22, in
 // integer arithmetic (the inverse of Eq. 4, Case 1).  g / 10^a = (g / 5^a) 2^-a and the
 // scaling by 2^-a is exact (no result is subnormal), so the work is one correctly rounded
 // division by 5^a: with G = |g| normalised to [2^63, 2^64), d = floor(log2 5^a) and the
-// reciprocal R = floor(2^(64+d) / 5^a), T = mulhi(G, R) is floor(G 2^d / 5^a) or one less
-// (division by an invariant integer, Granlund and Montgomery, PLDI 1994); the remainder,
-// below 2 * 5^a, is exact in 64-bit arithmetic and corrects T.  T has 63 or 64 significant
-// bits; its top 53 bits, the next bit and a sticky bit (lower bits or a non-zero remainder)
-// round to the IEEE significand.  Returns the bits of the double.
-__device__ __forceinline__ uint64_t div_pow10_exact(int64_t g, int a) {
-    if (g == 0) return 0;
+// reciprocal R = floor(2^(64+d) / 5^a), T = mulhi(G, R) is floor(Q) or one less, Q = G 2^d / 5^a
+// (division by an invariant integer, Granlund and Montgomery, PLDI 1994).  (a = 0: R = 2^64 - 1
+// gives T = G - 1.)  Q has 63 or 64 integer bits, of which 10 or 11 lie below the 53-bit result.
+// A tie cannot occur (a 54-bit quotient times 5^a exceeds 2^53 or a = 0 and g fits), so Q rounds up
+// iff Q's dropped part is at least half: T's next bit decides, except when T's dropped bits are
+// one below half, where the remainder G 2^d - T 5^a (below 2 * 5^a, exact modulo 2^64) says
+// whether floor(Q) is T + 1.  That happens for one value in 1024 to 2048, so its two products are
+// off the common path.
+struct Div10 {
+    uint64_t R, D;                                // reciprocal, 5^a
+    int d, e0;                                    // floor(log2 5^a), exponent of T's unit
+};
+__device__ __forceinline__ Div10 div10_of(int a) {
+    const int d = FALCON_LOG2_POW5[a];
+    return {a > 0 ? FALCON_RECIP5[a] : ~0ull, FALCON_POW5[a], d, 11 - d - a + 52 + 1022};
+}
+// bits of the double T-or-T+1 rounds to; s = the shift that normalised |g|
+__device__ __forceinline__ uint64_t div10_round(uint64_t G, uint64_t T, int s, const Div10 &q) {
+    const uint32_t lz = (uint32_t)(~T >> 63);     // T has 63 or 64 significant bits
+    const uint64_t Tn = T << lz;
+    uint32_t up = ((uint32_t)Tn >> 10) & 1u;
+    if (((((uint32_t)Tn) & 0x7FFu) | lz) == 0x3FFu) up = (G << q.d) - T * q.D >= q.D;
+    // the significand's leading one adds one to the biased exponent field, a carry another
+    return ((uint64_t)(uint32_t)(q.e0 - (int)lz - s) << 52) + (Tn >> 11) + up;
+}
+__device__ __forceinline__ uint64_t div_pow10_exact(int64_t g, const Div10 &q) {
     const uint64_t sign = (uint64_t)g & 0x8000000000000000ull;
     const uint64_t ag = g < 0 ? 0ull - (uint64_t)g : (uint64_t)g;
     const int s = __clzll((long long)ag);
-    const uint64_t G = ag << s;
-    uint64_t T = G, r = 0;
-    int d = 0;
-    if (a > 0) {
-        d = FALCON_LOG2_POW5[a];
-        const uint64_t D = FALCON_POW5[a];
-        T = __umul64hi(G, FALCON_RECIP5[a]);
-        r = (G << d) - T * D;                   // true remainder in [0, 2 D): exact mod 2^64
-        if (r >= D) { r -= D; ++T; }
-    }
-    const int lz = __clzll((long long)T);       // 0 or 1
+    const uint64_t G = ag << (s & 63);
+    const uint64_t v = div10_round(G, __umul64hi(G, q.R), s, q) | sign;
+    return ag ? v : 0;
+}
+// The same for |g| < 2^32 and a <= 17, given as |g| and a sign word (top bit), with a 96-bit
+// reciprocal and no remainder: T = floor(Q - e) with e < 2^-32, and Q, a multiple of 1 / 5^a that is
+// never a tie, lies at least 2^9 / 5^a > 2^-32 from the point where rounding changes, so T's next
+// bit decides.  (Q an integer: T = Q - 1 rounds alike, as above.)
+struct Div10Narrow {
+    uint32_t r0, r1, r2;                          // 2^(96+d) / 5^a, low word first
+    int e0;
+};
+constexpr int kDiv10NarrowMax = 17;
+__device__ __forceinline__ Div10Narrow div10_narrow_of(int a) {
+    const uint64_t r = a > 0 ? FALCON_RECIP5[a] : ~0ull;
+    return {FALCON_RECIP5_LO[a], (uint32_t)r, (uint32_t)(r >> 32), 11 - (int)FALCON_LOG2_POW5[a] - a + 52 + 1022 - 32};
+}
+__device__ __forceinline__ uint64_t div_pow10_exact32(uint32_t ag, uint32_t sgn, const Div10Narrow &q) {
+    const int s = __clz((int)ag);
+    const uint32_t G = ag << (s & 31);
+    const uint64_t lo = (uint64_t)G * q.r1 + __umulhi(G, q.r0);
+    const uint64_t T = (uint64_t)G * q.r2 + (uint32_t)(lo >> 32);
+    const uint32_t lz = (uint32_t)(~T >> 63);
     const uint64_t Tn = T << lz;
-    uint64_t mant = Tn >> 11;
-    const uint32_t rest = (uint32_t)Tn & 0x7FFu;
-    const bool sticky = (rest & 0x3FFu) != 0u || r != 0;
-    if ((rest & 0x400u) && (sticky || (mant & 1ull))) ++mant;
-    int e2 = 11 - lz - d - s - a;               // the value is mant * 2^e2
-    if (mant == (1ull << 53)) { mant >>= 1; ++e2; }
-    return sign | ((uint64_t)(e2 + 52 + 1023) << 52) | (mant & 0x000FFFFFFFFFFFFFull);
+    const uint64_t M = (Tn >> 11) + (((uint32_t)Tn >> 10) & 1u);
+    const uint32_t top = ((uint32_t)(q.e0 - (int)lz - s) << 20) + (uint32_t)(M >> 32);
+    const uint64_t v = ((uint64_t)(top | (sgn & 0x80000000u)) << 32) | (uint32_t)M;
+    return ag ? v : 0;
 }
 
 __device__ __forceinline__ void set_status(unsigned long long *result, uint32_t code) {
@@ -569,80 +595,6 @@ __device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t &t
     total = warp_sums[32];
     __syncthreads();
     return r;
-}
-
-// Exclusive prefix of a stream's u32 size array per 64-chunk tile, into tile_off[0 ..
-// tile_count(nc)) (one 1024-thread block, thread t owning tile t of each step of 1024 tiles).
-// Returns the total of all sizes (every thread).  A warp whose 32 tiles are all whole reads
-// their 8 KB of sizes coalesced (16-byte unit 32 k + lane, i.e. tiles 2k and 2k + 1 in the
-// two half-warps) and adds each tile up with half-warp shuffles in 32-bit arithmetic; a step
-// in which some 16-byte unit adds up to 2^26 or more (only in a malformed stream) falls back
-// to 64-bit sums per thread.
-__device__ __forceinline__ uint64_t tile_prefix(const uint32_t *sizes, uint64_t nc, unsigned long long *tile_off,
-                                                uint64_t *warp_sums) {
-    const uint64_t ntiles = tile_count(nc);
-    const uint64_t full_tiles = nc / kTile;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint64_t carry = 0;
-    for (uint64_t b = 0; b < ntiles; b += 1024) {
-        const uint64_t tile = b + threadIdx.x;
-        const uint64_t wt0 = b + 32u * (uint64_t)warp;
-        uint64_t sum = 0;
-        bool done = false;
-        if (wt0 + 32u <= full_tiles) {
-            const uint4 *q = reinterpret_cast<const uint4 *>(sizes + wt0 * kTile);
-            uint32_t mine = 0;
-            bool big = false;
-#pragma unroll 4
-            for (int k = 0; k < 16; ++k) {
-                const uint4 x = q[32 * k + lane];
-                const uint64_t s64 = (uint64_t)x.x + x.y + x.z + x.w;
-                big |= s64 >= (1ull << 26);
-                uint32_t s = (uint32_t)s64;
-                s += __shfl_xor_sync(kFull, s, 8);
-                s += __shfl_xor_sync(kFull, s, 4);
-                s += __shfl_xor_sync(kFull, s, 2);
-                s += __shfl_xor_sync(kFull, s, 1);
-                const uint32_t lo = __shfl_sync(kFull, s, 0), hi = __shfl_sync(kFull, s, 16);
-                if (lane == 2 * k) mine = lo;
-                if (lane == 2 * k + 1) mine = hi;
-            }
-            done = !__any_sync(kFull, big);
-            sum = mine;
-        }
-        if (!done && tile < ntiles) {
-            sum = 0;
-            const uint64_t c0 = tile * kTile;
-            const uint64_t c1 = (c0 + kTile <= nc) ? c0 + kTile : nc;
-            for (uint64_t c = c0; c < c1; ++c) sum += sizes[c];
-        }
-        uint64_t total;
-        const uint64_t ex = carry + block_exclusive_scan(sum, total, warp_sums);
-        if (tile < ntiles) tile_off[tile] = ex;
-        carry += total;
-    }
-    return carry;
-}
-
-// Where chunk c's record starts (relative to the first record): its tile's offset plus the
-// sizes of the earlier chunks of the tile.  load_pos issues the loads (every lane), resolve_pos
-// adds them up (warp-collective) once they are needed, so their latency can be hidden.
-struct ChunkPos {
-    uint64_t tile;
-    uint32_t s0, s1, size;
-};
-__device__ __forceinline__ ChunkPos load_pos(const uint32_t *sizes, const unsigned long long *tile_off, uint64_t c,
-                                             int lane) {
-    const uint64_t t0 = c & ~(kTile - 1);
-    ChunkPos p;
-    p.tile = tile_off[c / kTile];
-    p.size = sizes[c];
-    p.s0 = (t0 + (uint64_t)lane < c) ? sizes[t0 + lane] : 0u;
-    p.s1 = (t0 + 32u + (uint64_t)lane < c) ? sizes[t0 + 32u + lane] : 0u;
-    return p;
-}
-__device__ __forceinline__ uint64_t resolve_pos(const ChunkPos &p) {
-    return p.tile + __reduce_add_sync(kFull, p.s0 + p.s1);       // a tile holds < 2^20 bytes
 }
 
 // Finds the job that owns global ticket t (jobs sorted by chunk_begin).

@@ -58,8 +58,8 @@ constexpr size_t kControlBytes = 256;   // control block region (keeps flags 256
 
 // Workspace words of a job: compression keeps two per chunk (the analysis results and the
 // dense-row mask), then one per 64-chunk tile and one per 4096-chunk group (the sums of their
-// record sizes, which the analysis adds up); decompression keeps the record offset of each tile
-// in the first words.
+// record sizes, which the analysis adds up); decompression keeps the record offset of each chunk
+// in the first words (the aggregate its chunk sums in the next).
 // value kinds of the stream format: 0 FP64, 1 FP32, 2 FP16 (binary16)
 inline bool dtype_valid(int dtype) { return dtype >= 0 && dtype <= 2; }
 inline size_t dtype_bytes(int dtype) { return dtype == 0 ? 8 : (dtype == 1 ? 4 : 2); }
@@ -77,7 +77,7 @@ cudaError_t launch_compress(const Job *d_jobs, int njobs, const Job &single,
 cudaError_t launch_decompress(const Job *d_jobs, int njobs, const Job &single,
                               uint64_t total_chunks, Control *ctl, cudaStream_t stream);
 // analytics on compressed data: the decode without the stores, then the aggregate into
-// d_stats (falcon_stats); the chunk sums go into job.flags after the tile offsets
+// d_stats (falcon_stats); the chunk sums go into job.flags after the chunk offsets
 cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cudaStream_t stream);
 
 // Status of the arguments of a compression call (dtype, block size, pointers, alignment,

@@ -65,6 +65,27 @@ FALCON_TABLE_QUAL uint64_t FALCON_RECIP5[23] = {
     0xf1c90080baf72cb1ull, /* 5^22 */
 };
 
+FALCON_TABLE_QUAL uint32_t FALCON_RECIP5_LO[18] = {
+    0xffffffffu, /* 5^0 */
+    0xccccccccu, /* 5^1 */
+    0x3d70a3d7u, /* 5^2 */
+    0x645a1cacu, /* 5^3 */
+    0xd3c36113u, /* 5^4 */
+    0x0fcf80dcu, /* 5^5 */
+    0xa63f9a49u, /* 5^6 */
+    0x3d329076u, /* 5^7 */
+    0xfdc20d2bu, /* 5^8 */
+    0x31680a88u, /* 5^9 */
+    0xb573440eu, /* 5^10 */
+    0xf78f69a5u, /* 5^11 */
+    0xf93f87b7u, /* 5^12 */
+    0x2865a5f2u, /* 5^13 */
+    0x538484c1u, /* 5^14 */
+    0x0f9d3701u, /* 5^15 */
+    0x4c2ebe68u, /* 5^16 */
+    0x09befeb9u, /* 5^17 */
+};
+
 FALCON_TABLE_QUAL uint64_t FALCON_POW5_NORM[23] = {
     0x8000000000000000ull, /* 5^0 */
     0xa000000000000000ull, /* 5^1 */

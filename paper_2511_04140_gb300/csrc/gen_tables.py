@@ -4,6 +4,8 @@ rational arithmetic (Python's Fraction -> float conversion rounds exactly once).
   FALCON_POW5[a]          5^a for a = 0..22 (exact integers)
   FALCON_RECIP5[a]        floor(2^(64 + d) / 5^a) with d = floor(log2 5^a), a = 1..22 (a 64-bit
                           reciprocal in [2^63, 2^64); entry 0 unused)
+  FALCON_RECIP5_LO[a]     the next 32 bits of 2^(64 + d) / 5^a, a = 0..17 (entry 0: all ones, the
+                          96-bit reciprocal below 2^96)
   FALCON_LOG2_POW5[a]     d = floor(log2 5^a)
   FALCON_POW5_NORM[a]     5^a << (63 - d): 5^a with its top bit at bit 63
   FALCON_P10_F64[k - LO]  bits of fl64(10^k), k in [-30, 22]
@@ -64,6 +66,9 @@ def main():
     out += ["};", "", "FALCON_TABLE_QUAL uint64_t FALCON_RECIP5[23] = {"]
     out += [f"    0x{(0 if a == 0 else (1 << (64 + (5 ** a).bit_length() - 1)) // 5 ** a):016x}ull, /* 5^{a} */"
             for a in range(23)]
+    out += ["};", "", "FALCON_TABLE_QUAL uint32_t FALCON_RECIP5_LO[18] = {"]
+    out += [f"    0x{(0xFFFFFFFF if a == 0 else ((1 << (96 + (5 ** a).bit_length() - 1)) // 5 ** a) & 0xFFFFFFFF):08x}u, /* 5^{a} */"
+            for a in range(18)]
     out += ["};", "", "FALCON_TABLE_QUAL uint64_t FALCON_POW5_NORM[23] = {"]
     out += [f"    0x{(5 ** a) << (64 - (5 ** a).bit_length()):016x}ull, /* 5^{a} */" for a in range(23)]
     out += ["};", "", "FALCON_TABLE_QUAL uint8_t FALCON_LOG2_POW5[23] = {"]
