@@ -1,27 +1,35 @@
 // Falcon compression (Sec. 3 of the paper; the work of Alg. 3 CmpKernel) for sm_103a, as
 // two launches, neither of which waits on another warp:
 //   1. analyse: each warp takes its chunks by ticket (its one shared-memory value buffer
-//      receives the next chunk by cp.async, swizzled, as soon as the Case decision is done)
+//      receives the next chunk by cp.async, swizzled, as soon as the current one is in registers)
 //      and computes
-//      - the lane's 32 values, specials (R1) and the chunk maximum,
-//      - Case 1 / Case 2 of Eq. 4: the smallest decimal place alpha_max at which every value
-//        passes Alg. 2's test, in exact integer arithmetic (q_test); FP32 checks Alg. 2's
-//        early stops where they are possible,
-//      - G (Eq. 4), Z (Eq. 5) and the bit width w in registers,
-//      - the non-zero bytes of every row (Sec. 3.3 lambda) from ORs of 8-column groups,
-//        without forming the bit planes, sparse/dense per row, the record size, which goes
+//      - specials (R1) and the largest magnitude from three-input maxima and minima of the values'
+//        magnitudes,
+//      - Case 1 / Case 2 of Eq. 4, out of line over the staged values: the smallest decimal place
+//        alpha_max at which every value passes Alg. 2's test, in exact integer arithmetic (q_test,
+//        test_g); FP32 checks Alg. 2's early stops where they are possible; Case 1 leaves G in the
+//        values' place,
+//      - the ORs of |Z| (Eq. 5) over 8-column groups, the bit width w, and from those ORs,
+//        transposed across the warp, the non-zero bytes of every row (Sec. 3.3 lambda) without
+//        forming the bit planes; sparse/dense per row; the record size, which goes
 //        into the stream's size array and is added to its 64-chunk tile's and 4096-chunk
-//        group's sums (the size synchronisation of Sec. 3.4), and alpha, beta_hat, w and the
+//        group's sums (the size synchronisation of Sec. 3.4); alpha, beta_hat, w and the
 //        dense-row mask, which go into the workspace;
 //   2. emit: each chunk's record offset from those sums, the values again (straight from
-//      global memory: FP64 with the next chunk prefetched into L2, FP32 and FP16 with the
-//      next chunk's values loaded into registers during the current record), G, Z and the
-//      bit planes (32x32 register transposes, one 32-bit word per plane: 4 row bytes per
-//      lane) from the kept
-//      alpha and w, the record assembled in shared memory at the output's 16-byte phase, in
-//      place of the plane words it consumes, and sent to its offset with one TMA bulk copy;
+//      global memory, a whole sector per lane and load, not kept in L1: FP64 with the next chunk
+//      prefetched into L2, FP32 and FP16 with the next chunk's values loaded into registers during
+//      the current record), G, the deltas' bit planes (32x32 register transposes, one 32-bit word per
+//      plane: 4 row bytes per lane), zigzagged by one XOR with the sign plane, through 128-byte slots
+//      into the record, assembled in shared memory at the output's 16-byte phase and sent to
+//      its offset with one TMA bulk copy;
 //      the warp of each job's first chunk writes the header and the stream length and checks
 //      the capacity.
+// Both are bound by integer issue (FP64 segments: ALU pipe 59 % and 66 % of active cycles, 1559 and
+// 3018 warp instructions per chunk, against 1801 and 3590 with ballots and reductions per sparse row,
+// per-value zigzags and bit-sliced counts).  2^26 segment values: FP64 520 -> 453 us, FP32 270 -> 242 us;
+// Case-1 FP64 of 40 M values in 1025-value chunks 622 -> 453 us.  Slower, and left out: two copies of the
+// row code (FP64 485 us: instruction fetch), a transpose shared by both halves in a loop (475 us), dense
+// rows moved in 16-byte units (FP64 461, FP32 238 us), values kept in L1 (483 us).
 // The paper resolves offsets inside one launch with a decoupled look-back; with about 1800
 // resident warps on a GB300 the waits of that look-back took half of every warp's time, while
 // the analysis recomputed by the emit launch costs less.
@@ -36,95 +44,128 @@ namespace falcon {
 namespace {
 
 constexpr int kBuf = 8288;                  // one chunk of values / one record (+32 readable)
-constexpr int kScratch = 128;
-constexpr int kAnalyseWarpBytes = kBuf + kScratch;  // analysis: one value buffer
+constexpr int kAnalyseWarpBytes = kBuf;     // analysis: one value buffer
 
-// The emit launch's per-warp plane / record buffer: plane p's words at
-// kPlOff + (W-1-p)*128 + 4*lane.  The record is assembled in place, from byte 0, as the planes
-// are consumed top-down: an adaptive or dense row takes at most the 128 bytes of its slot, so
-// the record never overtakes the plane read next with kPlOff = 48.  Every-row-sparse records
-// (Sec. 5.4.2 ablation) may take 16 + 128 bytes per row and use the wide layout, whose plane
-// slots start past 16 bytes of growth per row.
-template <bool kWide> struct EmitLayout {
-    static constexpr int kPlOff = kWide ? 1072 : 48;
-    static constexpr int kBytes = kPlOff + 64 * 128 + 32;          // + 32 readable past any slot
+// The emit launch's per-warp buffers: the record, assembled at the output's 16-byte phase, and
+// 128-byte slots for the rows of 32 planes at a time, top plane first (FP64 runs its two halves one
+// after the other through the same slots).  A row takes at most 128 bytes of the record, 16 more in
+// an every-row-sparse one (Sec. 5.4.2 ablation, the wide layout).
+template <int D, bool kWide> struct EmitLayout {
+    static constexpr uint32_t W = Traits<D>::W;
+    static constexpr uint32_t kRec = (3u + Traits<D>::Z1B + W / 8u + W * (kWide ? 144u : 128u) + 15u + 15u) / 16u * 16u;
+    static constexpr uint32_t kRows = W < 32u ? W : 32u;
+    static constexpr uint32_t kBytes = kRec + kRows * 128u + 16u;         // + 16 readable past any slot
 };
 
-// Copies len bytes from src to dst inside a warp buffer, dst + 14 <= src (the move goes
-// down): unaligned head and tail bytes singly, the 16-byte aligned middle of the
-// destination with one 16-byte store per lane and iteration, its source taken from two
-// aligned 16-byte loads and funnel shifts.  In every iteration all lanes read before any
-// lane writes, and later iterations read strictly above earlier writes, so the overlapping
-// move is safe.  The buffer has 32 readable bytes past any source byte.
-__device__ __forceinline__ uint32_t fsr(uint32_t lo, uint32_t hi, uint32_t s) { return __funnelshift_r(lo, hi, s); }
-
-__device__ __forceinline__ void smem_move_down(uint8_t *buf, uint32_t dst, uint32_t src, uint32_t len, int lane) {
-    const uint32_t head = min((16u - (dst & 15u)) & 15u, len);
-    uint32_t hb = 0;
-    if ((uint32_t)lane < head) hb = buf[src + lane];
-    __syncwarp();
-    if ((uint32_t)lane < head) buf[dst + lane] = (uint8_t)hb;
-    __syncwarp();
-    const uint32_t D = dst + head, S = src + head;
-    const uint32_t units = (len - head) >> 4;
-    const uint32_t off = S & 15u, k0 = off >> 2, sb = (off & 3u) * 8u;
-    const uint32_t Sa = S - off;
-    for (uint32_t u0 = 0; u0 < units; u0 += 32) {
-        const uint32_t u = u0 + lane;
-        uint4 o = make_uint4(0, 0, 0, 0);
-        if (u < units) {
-            const uint4 a = *reinterpret_cast<const uint4 *>(buf + Sa + 16u * u);
-            const uint4 b = *reinterpret_cast<const uint4 *>(buf + Sa + 16u * u + 16u);
-            switch (k0) {
-                case 0: o = make_uint4(fsr(a.x, a.y, sb), fsr(a.y, a.z, sb), fsr(a.z, a.w, sb), fsr(a.w, b.x, sb)); break;
-                case 1: o = make_uint4(fsr(a.y, a.z, sb), fsr(a.z, a.w, sb), fsr(a.w, b.x, sb), fsr(b.x, b.y, sb)); break;
-                case 2: o = make_uint4(fsr(a.z, a.w, sb), fsr(a.w, b.x, sb), fsr(b.x, b.y, sb), fsr(b.y, b.z, sb)); break;
-                default: o = make_uint4(fsr(a.w, b.x, sb), fsr(b.x, b.y, sb), fsr(b.y, b.z, sb), fsr(b.z, b.w, sb)); break;
-            }
-        }
-        __syncwarp();
-        if (u < units) *reinterpret_cast<uint4 *>(buf + D + 16u * u) = o;
-    }
-    __syncwarp();
-    const uint32_t tail = (len - head) & 15u;
-    const uint32_t T0 = units * 16u;
-    uint32_t tb = 0;
-    if ((uint32_t)lane < tail) tb = buf[S + T0 + lane];
-    __syncwarp();
-    if ((uint32_t)lane < tail) buf[D + T0 + lane] = (uint8_t)tb;
-    __syncwarp();
-}
-
-// non-zero nibble of x (bit 3 - i set iff byte i is non-zero): the bytes' high-bit flags
-// gathered into the top byte by one multiply
-__device__ __forceinline__ uint32_t nz_nibble(uint32_t x) {
-    const uint32_t y = (((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
-    return ((y >> 7) * 0x08040201u) >> 24 & 0xFu;
-}
-
-// Sparse row (Sec. 3.3) written with byte stores at byte offset P of the warp buffer:
-// a bitmap of nact/2 bytes (bit 7 of byte 0 = row byte 0), then the non-zero row bytes.
-// Returns the row's length.
-__device__ __forceinline__ uint32_t sparse_row(uint8_t *buf, uint32_t P, uint32_t x, int lane, uint32_t nact) {
-    const bool active = (uint32_t)lane < nact;
-    const uint32_t nib = active ? nz_nibble(x) : 0u;
-    const uint32_t nib_next = __shfl_down_sync(kFull, nib, 1);
-    if (active && !(lane & 1)) buf[P + (lane >> 1)] = (uint8_t)((nib << 4) | nib_next);
-    const uint32_t cnt = __popc(nib);
-    const unsigned b0 = __ballot_sync(kFull, cnt & 1u);
-    const unsigned b1 = __ballot_sync(kFull, cnt & 2u);
-    const unsigned b2 = __ballot_sync(kFull, cnt & 4u);
-    const unsigned lt = (1u << lane) - 1u;
-    const uint32_t before = __popc(b0 & lt) + 2u * __popc(b1 & lt) + 4u * __popc(b2 & lt);
-    const uint32_t total = __reduce_add_sync(kFull, cnt);
-    uint32_t q = P + nact / 2u + before;
+// Byte-permute selector that moves a word's non-zero bytes to its front, by nibble n (bit 3 - i: byte
+// i is non-zero).  Lane l keeps the selector of nibble l & 15, so one shuffle looks it up.
+__device__ __forceinline__ uint32_t compact_sel(uint32_t n) {
+    uint32_t sel = 0x4444u, r = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const uint32_t byte = (x >> (8 * i)) & 0xFFu;
-        if (active && byte) buf[q++] = (uint8_t)byte;
+        if ((n >> (3 - i)) & 1u) {
+            sel = (sel & ~(15u << (4 * r))) | ((uint32_t)i << (4 * r));
+            ++r;
+        }
     }
-    __syncwarp();
-    return nact / 2u + total;
+    return sel;
+}
+
+// non-zero nibble of x (bit 3 - i set iff byte i is non-zero): the bytes' high-bit flags moved to
+// bits 32..35 by one high multiply
+__device__ __forceinline__ uint32_t nz_nibble(uint32_t x) {
+    const uint32_t y = (((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
+    return __umulhi(y, 0x10080402u) & 15u;
+}
+
+// inclusive prefix sum over the warp (the shuffle's own predicate says which lanes add)
+__device__ __forceinline__ uint32_t warp_inclusive(uint32_t v) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        asm volatile("{\n\t.reg .b32 t;\n\t.reg .pred p;\n\tshfl.sync.up.b32 t|p, %0, %1, 0, -1;\n\t@p add.u32 %0, %0, t;\n\t}"
+                     : "+r"(v)
+                     : "r"(o));
+    return v;
+}
+
+// Copies a run of rows (len bytes, a multiple of 8) from 4-byte aligned src to any byte address
+// dst: one aligned word per lane, built from two words and a funnel shift; the unaligned head and tail
+// bytes singly.
+__device__ __forceinline__ void copy_rows(uint8_t *dst, const uint8_t *src, uint32_t len, int lane) {
+    const uint32_t head = (0u - (uint32_t)reinterpret_cast<uintptr_t>(dst)) & 3u;
+    const uint32_t tail = (len - head) & 3u;
+    if ((uint32_t)lane < head) dst[lane] = src[lane];
+    if ((uint32_t)lane < tail) dst[len - tail + lane] = src[len - tail + lane];
+    const uint32_t words = (len - head) >> 2, sb = head * 8u;
+    const uint32_t *s = reinterpret_cast<const uint32_t *>(src) + lane;
+    uint32_t *d = reinterpret_cast<uint32_t *>(dst + head) + lane;
+#pragma unroll 4
+    for (uint32_t j = (uint32_t)lane; j < words; j += 32u, s += 32, d += 32) *d = __funnelshift_r(s[0], s[1], sb);
+}
+
+// The rows of up to 32 planes (Sec. 3.3) from their slots into the record.  `rows`: the planes that
+// exist (low bits), `dense` the dense ones among them; `cur`: record position of the top plane's row,
+// moved to the end of the last.  Plane p's row is in slot 31 - p.
+// Sparse rows go four at a time: their nibbles in the bytes of one word, so one shuffle serves four
+// bitmaps, and their byte counts in the bytes of another, so one prefix scan serves four rows (a
+// row has at most 128 non-zero bytes); what used to be a chain of ballots and reductions per row
+// has four rows' work to overlap.  Then runs of dense rows are copied.
+__device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, uint32_t &cur, uint32_t rows,
+                                          uint32_t dense, uint32_t row_bytes, uint32_t bm_bytes, uint32_t seltab, int lane) {
+    const uint32_t start = cur;
+    const bool maps = !(lane & 1) && (uint32_t)lane < 2u * bm_bytes;      // this lane stores a bitmap byte
+    uint32_t sparse = rows & ~dense;
+    uint32_t sum = 0, mine = 0;                   // sparse bytes so far; above this lane's plane
+    uint32_t above = 32u - (uint32_t)__clz((int)rows);
+    uint8_t *bm = rec + (lane >> 1);
+#pragma unroll 1
+    while (sparse) {
+        uint32_t p[4], x[4], nibs = 0;
+        bool have[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            have[i] = sparse != 0u;
+            p[i] = have[i] ? 31u - (uint32_t)__clz((int)sparse) : 0u;
+            sparse &= ~(1u << p[i]);
+            x[i] = *reinterpret_cast<const uint32_t *>(slots + 128u * (31u - p[i]) + 4u * lane);
+            if (i > 0) x[i] = have[i] ? x[i] : 0u;
+            nibs |= nz_nibble(x[i]) << (8 * i);
+        }
+        uint32_t c = nibs - ((nibs >> 1) & 0x05050505u);             // set bits of every nibble
+        c = (c & 0x03030303u) + ((c >> 2) & 0x03030303u);
+        const uint32_t incl = warp_inclusive(c);
+        const uint32_t tot = __shfl_sync(kFull, incl, 31), excl = incl - c;
+        const uint32_t pair = (nibs << 4) | __shfl_down_sync(kFull, nibs, 1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t gap = have[i] ? row_bytes * (above - 1u - p[i]) : 0u;   // the dense rows in between
+            const uint32_t len = have[i] ? bm_bytes + ((tot >> (8 * i)) & 255u) : 0u;
+            const uint32_t at = cur + gap;
+            above = have[i] ? p[i] : above;
+            cur = at + len;
+            sum += len;
+            if (have[i] && (uint32_t)lane < p[i]) mine = sum;
+            if (have[i] && maps) bm[at] = (uint8_t)(pair >> (8 * i));
+            const uint32_t packed = __byte_perm(x[i], 0u, __shfl_sync(kFull, seltab, (int)(nibs >> (8 * i))));
+            const uint32_t n = (c >> (8 * i)) & 7u;
+            uint8_t *q = rec + at + bm_bytes + ((excl >> (8 * i)) & 255u);
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (n > (uint32_t)t) q[t] = (uint8_t)(packed >> (8 * t));
+        }
+    }
+    cur += row_bytes * above;
+    const uint32_t place = start + row_bytes * (uint32_t)__popc((dense >> lane) >> 1) + mine;   // of dense plane `lane`
+    uint32_t dm = dense;
+#pragma unroll 1
+    while (dm) {
+        // a run of dense rows p, p-1, ..., q: contiguous in the slots when rows are 128 bytes long
+        const uint32_t p = 31u - (uint32_t)__clz((int)dm);
+        const uint32_t holes = ~dm & ((2u << p) - 1u);
+        const uint32_t q = row_bytes == 128u ? 32u - (uint32_t)__clz((int)holes) : p;
+        copy_rows(rec + __shfl_sync(kFull, place, (int)p), slots + 128u * (31u - p), (p - q + 1u) * row_bytes, lane);
+        dm &= (1u << q) - 1u;
+    }
 }
 
 // value k of this lane from the swizzled staging buffer
@@ -136,8 +177,18 @@ __device__ __forceinline__ typename Traits<D>::U lane_value(const uint8_t *buf, 
     return *reinterpret_cast<const U *>(buf + (lane * UN + unit_swizzle<D>(lane, k / PER)) * 16 + (k % PER) * Traits<D>::S);
 }
 
-// Every value of the chunk (the lane's 32 in v, value 1024 of a 1025-value chunk in vx)
-// passes Alg. 2's test at a.  Values past m are +0, which passes.
+// A tail chunk's staged values past the m-th repeat it: Eq. 5's pad columns (R11) are zero because
+// their G are equal, and every test over 1024 values answers as over the m.
+template <int D>
+__device__ __forceinline__ void pad_values(uint8_t *buf, uint32_t m, int lane) {
+    if (m >= 1024u) return;
+    using U = typename Traits<D>::U;
+    const U last = read_elem<D>(buf, m - 1u);
+#pragma unroll 1
+    for (uint32_t e = m + (uint32_t)lane; e < 1024u; e += 32) *reinterpret_cast<U *>(buf + phys_elem_byte<D>(e)) = last;
+    __syncwarp();
+}
+
 // Every value of the chunk passes Alg. 2's test at a; the values are re-read from the staging
 // buffer (index >= m: not a value).  A failing decimal place usually fails on every lane's
 // first value already, so those 32 are tested first.
@@ -153,27 +204,97 @@ __device__ __forceinline__ bool all_pass(const uint8_t *buf, int lane, uint32_t 
     return __all_sync(kFull, ok);
 }
 
+// Test and g of one value at decimal place a together (Eq. 4, Case 1): g = round(v 10^a) from one
+// 64-bit high product, then the exact distance |m 5^a - g 2^F| against 5^a / 2, modulo 2^64 (exact
+// while F <= 62, since g lies within one of v 10^a; smaller values take q_test).  Below a power of
+// two the interval is half as wide, which changes nothing: there m 5^a = 2^52 5^a, and its distance
+// to a multiple of 2^F is 0 or at least 2^52 > 5^a / 2.
+struct Case1At {                                  // constants of a decimal place
+    uint64_t p5, norm;                            // 5^a, 5^a with its top bit at bit 63
+    int f0, sh0;                                  // F = f0 - exponent field, shift = F + sh0
+    int a;
+};
+__device__ __forceinline__ Case1At case1_at(int a) {
+    return {FALCON_POW5[a], FALCON_POW5_NORM[a], 1075 - a, 10 - (int)FALCON_LOG2_POW5[a], a};
+}
+__device__ __forceinline__ uint64_t test_g(uint64_t u, const Case1At &c, bool &ok) {
+    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
+    const int F = c.f0 - (int)((hi >> 20) & 0x7FFu);
+    const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+    uint64_t N = case1_round(m, c.norm, F + c.sh0);
+    bool pass;
+    if (F > 62 || F <= 0) {
+        pass = q_test(u, c.a);
+        if ((u << 1) == 0) N = 0;
+    } else {
+        const uint64_t lim = c.p5 >> 1;
+        pass = (m * c.p5 - (N << F)) + lim <= 2u * lim;
+    }
+    ok &= pass;
+    return (hi >> 31) ? 0ull - N : N;
+}
+template <class U> __device__ __forceinline__ U test_g_narrow(U u, int a, bool &ok) {
+    ok &= q_test(u, a);
+    return case1_g(u, a);
+}
+
+// all_pass that leaves every value's g in the staging buffer in its place (rolled: small code).
+template <int D>
+__device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, int a) {
+    using U = typename Traits<D>::U;
+    constexpr int UN = Traits<D>::UNITS, PER = 32 / UN;
+    bool ok = true;
+    Case1At c{};
+    if constexpr (D == kD64) c = case1_at(a);
+    auto one = [&](U u, uint32_t i) {
+        bool pass = true;
+        U g;
+        if constexpr (D == kD64) g = test_g(u, c, pass);
+        else g = test_g_narrow(u, a, pass);
+        ok &= pass || i >= m;
+        return g;
+    };
+    if (m > 1024u && lane == 31) {
+        U *e = reinterpret_cast<U *>(buf + phys_elem_byte<D>(1024));
+        *e = one(*e, 1024);
+    }
+#pragma unroll 1
+    for (int u = 0; u < UN; ++u) {
+        uint4 *q = reinterpret_cast<uint4 *>(buf + (lane * UN + unit_swizzle<D>(lane, u)) * 16);
+        union { uint4 w; U e[PER]; } x;
+        x.w = *q;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) x.e[k] = one(x.e[k], 32u * lane + u * PER + k);
+        *q = x.w;
+    }
+    return __all_sync(kFull, ok);
+}
+
 // Smallest a in [0, atop] at which every value passes the round-trip test, or -1 (Case 2).
 // For chunks of valid values the predicate is monotone in a (Thm 4 with Thm 3), and its
 // smallest true point is the largest decimal place of the values; a failure at atop means
 // some value is an exception or needs alpha > atop.  Each lane's first value is tested at
 // atop (a failure settles Case 2), then its own decimal place is found; the warp's maximum
-// is a lower bound, and for most chunks the answer: one all-value test confirms it.
-// Otherwise the answer lies above it (test atop, then bisect).  Out of line, reading the
-// staged values: few chunks get here, and the hot path of the others stays small.
+// is a lower bound, and for most chunks the answer: one all-value test confirms it (`lb_ok`: the
+// caller has already made it).  Otherwise the answer lies above it (test atop, then bisect).
 template <int D>
-__device__ __noinline__ int search_alpha(const uint8_t *buf, int lane, uint32_t m, typename Traits<D>::U vx,
-                                         int atop) {
+__device__ __forceinline__ int alpha_bound(const uint8_t *buf, int lane, uint32_t m, int atop) {
     using U = typename Traits<D>::U;
     const U v0 = 32u * lane < m ? lane_value<D>(buf, lane, 0) : (U)0;
     if (!__all_sync(kFull, q_test(v0, atop))) return -1;
     int a0 = 0;
 #pragma unroll 1
     while (a0 < atop && !q_test(v0, a0)) ++a0;
-    const int lb = (int)__reduce_max_sync(kFull, (uint32_t)a0);
-    int lo = lb, hi = atop;                     // the answer, if any, lies in [lo, hi]
+    return (int)__reduce_max_sync(kFull, (uint32_t)a0);
+}
+// the answer above a lower bound that failed
+template <int D>
+__device__ __forceinline__ int alpha_above(const uint8_t *buf, int lane, uint32_t m, typename Traits<D>::U vx,
+                                           int lb, int atop) {
+    if (lb >= atop) return -1;
+    int lo = lb + 1, hi = atop;                 // the answer, if any, lies in [lo, hi]
     bool hi_ok = false;                         // all_pass(hi) is known to hold
-    int a = lb;
+    int a = atop;
 #pragma unroll 1
     for (;;) {
         const bool ok = all_pass<D>(buf, lane, m, vx, a);
@@ -185,7 +306,7 @@ __device__ __noinline__ int search_alpha(const uint8_t *buf, int lane, uint32_t 
             lo = a + 1;
         }
         if (hi_ok && lo >= hi) return hi;
-        a = hi_ok ? ((lo + hi) >> 1) : atop;    // lo <= a < hi once atop has passed
+        a = (lo + hi) >> 1;                     // lo <= a < hi once atop has passed
     }
 }
 
@@ -223,19 +344,15 @@ __device__ __forceinline__ int first_pass(uint16_t u, int atop) { return first_p
 // True if some value of the chunk stops early (the chunk then takes Case 2); alpha is the
 // search's alpha_max, at which every value round-trips.
 template <int D>
-__device__ __forceinline__ bool early_stop(const uint8_t *buf, int lane, uint32_t m, const typename Traits<D>::U (&v)[32],
-                                           typename Traits<D>::U vx, bool has_vx, typename Traits<D>::U vmax,
-                                           int alpha) {
+__device__ __forceinline__ bool early_stop(const uint8_t *buf, int lane, uint32_t m, typename Traits<D>::U vx,
+                                           bool has_vx, typename Traits<D>::U vmax, int alpha) {
     if (!may_stop_early(vmax, alpha)) return false;
-    uint32_t cand = 0;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) cand |= (uint32_t)(32u * lane + k < m && may_stop_early(v[k], alpha)) << k;
     bool bad = has_vx && may_stop_early(vx, alpha) && first_pass(vx, alpha) < 0;
 #pragma unroll 1
-    while (cand) {
-        const int k = __ffs(cand) - 1;
-        cand &= cand - 1;
-        bad |= first_pass(lane_value<D>(buf, lane, k), alpha) < 0;
+    for (int k = 0; k < 32; ++k) {
+        if (32u * lane + k >= m) break;
+        const typename Traits<D>::U u = lane_value<D>(buf, lane, k);
+        if (may_stop_early(u, alpha)) bad |= first_pass(u, alpha) < 0;
     }
     return __any_sync(kFull, bad);
 }
@@ -303,6 +420,106 @@ __device__ __noinline__ int alpha_elf(const uint8_t *buf, int lane, uint32_t m, 
     return all_pass<D>(buf, lane, m, vx, amax) ? amax : -1;
 }
 
+// Case 1's alpha_max of a chunk that may be Case 1 (no special value, the test value passes at
+// atop), or -1.  On success the staging buffer holds G (Eq. 4) in place of the values, otherwise
+// the values.
+template <int D>
+__device__ __forceinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, int e_max, int atop,
+                                           typename Traits<D>::U vmax, bool elf) {
+    using T = Traits<D>;
+    using U = typename T::U;
+    const bool has_vx = m > 1024u && lane == 31;
+    const U vx = has_vx ? read_elem<D>(buf, 1024) : (U)0;
+    int alpha;
+    if (elf) {
+        alpha = alpha_elf<D>(buf, lane, m, vx, has_vx, e_max);
+        if (alpha < 0) return -1;
+    } else {
+        alpha = alpha_bound<D>(buf, lane, m, atop);
+        if (alpha < 0) return -1;
+        if constexpr (D == kD64) {               // no value can stop early (Thm 4)
+            if (pass_to_g<D>(buf, lane, m, alpha)) return alpha;
+            __syncwarp();
+            stage_values_async<D>(src, m, buf, lane);        // the values again
+            cp_async_commit();
+            cp_async_wait_none();
+            __syncwarp();
+            pad_values<D>(buf, m, lane);
+            alpha = alpha_above<D>(buf, lane, m, vx, alpha, atop);
+        } else {
+            if (!all_pass<D>(buf, lane, m, vx, alpha)) alpha = alpha_above<D>(buf, lane, m, vx, alpha, atop);
+            // FP32 (R14), FP16 (R18): below beta_hat = B_MAX no value can stop early
+            // (see early_stop), so Alg. 2 value by value gives the same alpha_max
+            if (alpha >= 0 && alpha + e_max + 1 == T::B_MAX && early_stop<D>(buf, lane, m, vx, has_vx, vmax, alpha))
+                alpha = -1;
+        }
+        if (alpha < 0) return -1;
+    }
+    (void)pass_to_g<D>(buf, lane, m, alpha);
+    return alpha;
+}
+
+// Classification of a chunk's magnitudes: FP64 by a key that keeps the top 25 bits of the high word
+// and carries the value's index below, FP32 and FP16 by the magnitude itself.
+template <int D> struct Mag {
+    using U = typename Traits<D>::U;
+    static constexpr U ABS = (U)((U)~(U)0 >> 1);                 // every bit but the sign
+    static constexpr uint32_t kExpAll = D == kD64 ? 0x7FF00000u : (D == kD32 ? 0x7F800000u : 0x7C00u);
+    static constexpr uint32_t kExpOne = D == kD64 ? 0x00100000u : (D == kD32 ? 0x00800000u : 0x0400u);
+    static __device__ __forceinline__ uint32_t key(U u, uint32_t k) {
+        if constexpr (D == kD64) return ((uint32_t)(u >> 32) & 0x7FFFFFC0u) | k;
+        else return (uint32_t)(u & ABS);
+    }
+};
+
+// Case decision (Eq. 4) of a chunk whose keys have maximum `top` (kmax: this lane's) and, if
+// `low`, some value with a zero exponent field.  Returns alpha_max | beta_hat << 8, alpha_max = 31
+// in Case 2; the staging buffer holds G on a Case 1 return, the values otherwise.  Out of line,
+// over the staged values, with none of them in registers: the code of the rarer decisions stays out
+// of the hot path's instruction stream.
+constexpr int kCase2 = 31;
+template <int D>
+__device__ __noinline__ int case_decision(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, uint32_t kmax,
+                                          uint32_t top, bool low, bool elf) {
+    using T = Traits<D>;
+    using U = typename T::U;
+    constexpr U ABS = Mag<D>::ABS;
+    constexpr int kNone = kCase2 | (T::B_SENT << 8);
+    if (low) {                                    // +0 or a special value (-0, subnormal)
+        bool s = m > 1024u && lane == 31 && is_special(read_elem<D>(buf, 1024));
+#pragma unroll 4
+        for (int k = 0; k < 32; ++k) s |= is_special(lane_value<D>(buf, lane, k));
+        if (__any_sync(kFull, s)) return kNone;
+    }
+    // the largest magnitude (FP64: one that shares its key's top bits)
+    U vmax;
+    if constexpr (D == kD64) {
+        const uint32_t owner = __ffs(__ballot_sync(kFull, kmax == top)) - 1u;
+        vmax = top < 64u ? 0 : read_elem<D>(buf, 32u * owner + (top & 63u)) & ABS;
+    } else {
+        vmax = (U)top;
+    }
+    if (vmax == 0) return 0;                      // every value is +0, and its G
+    if (!log10_in_range(vmax)) return kNone;
+    int e_max = floor_log10(vmax);
+    if constexpr (D == kD64) {
+        // a power of ten between vmax and a larger value with the same key bits?
+        const uint32_t p = (uint32_t)(FALCON_P10_F64[e_max + 1 - FALCON_P10_F64_LO] >> 32);
+        if (((p ^ top) & 0x7FFFFFC0u) == 0) {
+            U x = m > 1024u ? read_elem<D>(buf, 1024) & ABS : (U)0;
+#pragma unroll 4
+            for (int k = 0; k < 32; ++k) x = max(x, (U)(lane_value<D>(buf, lane, k) & ABS));
+            e_max = floor_log10(warp_max_x(x));
+        }
+    }
+    const int atop = min(T::A_MAX, T::B_MAX - 1 - e_max);
+    // quick rejection: Alg. 2's round trip on the largest magnitude first (the test reads
+    // only |v|, so it runs on vmax itself, the same in every lane)
+    if (!elf && (atop < 0 || !q_test(vmax, atop))) return kNone;
+    const int alpha = case1_alpha<D>(src, buf, lane, m, e_max, atop, vmax, elf);
+    return alpha < 0 ? kNone : alpha | ((alpha + e_max + 1) << 8);
+}
+
 __device__ __forceinline__ void issue_chunk(const Job *jobs, int njobs, const Job &single, uint64_t t,
                                             uint8_t *buf, int lane) {
     const Job &job = (jobs == nullptr) ? single : jobs[find_job(jobs, njobs, t)];
@@ -325,177 +542,101 @@ __device__ __forceinline__ unsigned long long pack_meta(int alpha_byte, int beta
     return (unsigned long long)(((uint32_t)alpha_byte << 12) | ((uint32_t)beta_hat << 7) | (uint32_t)w) << kMetaShift;
 }
 
-// G (Eq. 4) and Z (Eq. 5) in place: v[k] becomes Z of column 32 lane + k, pad columns (R11)
-// are zero; alpha < 0 means Case 2.  Returns z_1 (every lane).
-template <int D>
-__device__ __forceinline__ typename Traits<D>::U to_z(typename Traits<D>::U (&v)[32],
-                                                        typename Traits<D>::U vx, int alpha, uint32_t m,
-                                                        int lane) {
-    using U = typename Traits<D>::U;
-    U gx;
-    if (alpha >= 0) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = case1_g(v[k], alpha);
-        gx = case1_g(vx, alpha);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = zigzag(v[k]);
-        gx = zigzag(vx);
-    }
-    const U z1 = shfl_x(v[0], 0);
-    U nxt = shfl_down_x(v[0], 1);
-    if (lane == 31) nxt = gx;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        const U hi = (k < 31) ? v[k + 1] : nxt;
-        v[k] = zigzag((U)(hi - v[k]));          // v now holds Z of columns 32*lane + k
-    }
-    // pad columns (R11): column c holds z_{c+2}, a pad when c + 1 >= m.  A full chunk of 1024
-    // values has one (the last column of lane 31), 1025 values none; only tail chunks take the
-    // general loop.
-    if (m == 1024u) {
-        if (lane == 31) v[31] = 0;
-    } else if (m < 1024u && 32u * lane + 32u >= m) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-            if (32u * lane + k + 1u >= m) v[k] = 0;
-    }
-    return z1;
-}
-
-// bit j of a nibble moved to bit 0 of byte j
-__device__ __forceinline__ uint32_t spread_nibble(uint32_t n) { return (n * 0x00204081u) & 0x01010101u; }
-
+// the sign of a delta, as a mask
+__device__ __forceinline__ uint64_t sign_mask(uint64_t x) { return (uint64_t)((int64_t)x >> 63); }
+__device__ __forceinline__ uint32_t sign_mask(uint32_t x) { return (uint32_t)((int32_t)x >> 31); }
+__device__ __forceinline__ uint16_t sign_mask(uint16_t x) { return (uint16_t)((int32_t)(int16_t)x >> 15); }
 
 // Launch 1, one chunk: everything up to the record size (see the file comment).  `next`
 // starts the copy of the warp's next chunk into buf; it is called once, as soon as the
 // staged values are no longer read (after the Case decision).
 template <int D, class Next>
-__device__ void analyse_chunk(const Job &job, uint64_t c, const uint8_t *buf, uint8_t *scratch, int lane,
-                              Next &&next) {
+__device__ __forceinline__ void analyse_chunk(const Job &job, uint64_t c, uint8_t *buf, int lane, Next &&next) {
     using T = Traits<D>;
     using U = typename T::U;
-    constexpr U ABS = (U)((U)~(U)0 >> 1);          // every bit but the sign (~ promotes uint16 to int)
     const uint32_t B = job.block;
     const uint64_t first = c * (uint64_t)B;
     const uint32_t m = (uint32_t)((job.n - first) < B ? (job.n - first) : B);
 
-    // ---- 1. values, specials, maximum ------------------------------------------------------
-    U v[32];
-    read_own<D>(buf, lane, m, v);
-    U vx = 0;                                   // value 1024 of a 1025-value chunk
-    if (m > 1024u && lane == 31) vx = read_elem<D>(buf, 1024);
-    bool sp;
-    U vmax;
-    if constexpr (D == 0) {
-        // on 32-bit halves: special <=> exponent field all zeros (value != +0) or all ones
-        uint32_t hmax = 0;
-        bool s = false;
-        auto cls = [&](uint64_t u) {
-            const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u, ha = hi & 0x7FFFFFFFu;
-            s |= (ha - 0x00100000u >= 0x7FE00000u) && ((hi | lo) != 0u);
-            hmax = ha > hmax ? ha : hmax;
-        };
-        cls(vx);
+    // ---- 1. Case decision (Eq. 4) -----------------------------------------------------------
+    // Three-input maxima and minima over the keys settle the special values: exponent all ones iff
+    // the maximum says so; a zero exponent field (rare but for zeros) is looked at again.
+    pad_values<D>(buf, m, lane);
+    constexpr int UN = T::UNITS, PER = 32 / UN;
+    uint32_t kmax = 0, kmin = ~0u;
+#pragma unroll 4
+    for (int u = 0; u < UN; ++u) {
+        union { uint4 w; U e[PER]; } x;
+        x.w = *reinterpret_cast<const uint4 *>(buf + (lane * UN + unit_swizzle<D>(lane, u)) * 16);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) cls(v[k]);
-        sp = __any_sync(kFull, s);
-        const uint32_t H = __reduce_max_sync(kFull, hmax);
-        uint32_t lmax = 0;
-        auto lo_of = [&](uint64_t u) {
-            if (((uint32_t)(u >> 32) & 0x7FFFFFFFu) == H) lmax = (uint32_t)u > lmax ? (uint32_t)u : lmax;
-        };
-        lo_of(vx);
-#pragma unroll
-        for (int k = 0; k < 32; ++k) lo_of(v[k]);
-        vmax = ((uint64_t)H << 32) | __reduce_max_sync(kFull, lmax);
-    } else {
-        sp = is_special(vx);
-        vmax = vx & ABS;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            sp |= is_special(v[k]);
-            const U a = v[k] & ABS;
-            vmax = a > vmax ? a : vmax;
+        for (int k = 0; k < PER; k += 2) {
+            const uint32_t a = Mag<D>::key(x.e[k], u * PER + k), b = Mag<D>::key(x.e[k + 1], u * PER + k + 1);
+            kmax = __vimax3_u32(kmax, a, b);
+            kmin = __vimin3_u32(kmin, a, b);
         }
-        sp = __any_sync(kFull, sp);
-        vmax = warp_max_x(vmax);
     }
+    if (m > 1024u && lane == 31) {
+        const uint32_t a = Mag<D>::key(read_elem<D>(buf, 1024), 32);
+        kmax = max(kmax, a);
+        kmin = min(kmin, a);
+    }
+    const uint32_t top = __reduce_max_sync(kFull, kmax);
+    const bool low = __any_sync(kFull, kmin < Mag<D>::kExpOne);
+    int alpha = kCase2, beta_hat = T::B_SENT;
+    if (top < Mag<D>::kExpAll) {
+        const int r = case_decision<D>(job.in + first * T::S, buf, lane, m, kmax, top, low, job.variant == kVariantElf);
+        alpha = r & 31;
+        beta_hat = r >> 8;
+        __syncwarp();
+    }
+    const bool case1 = alpha != kCase2;
 
-    // ---- 2. Case decision (Eq. 4) -----------------------------------------------------------
-    int alpha = -1;                             // -1: Case 2
-    int beta_hat = T::B_SENT;
-    if (!sp) {
-        if (vmax == 0) {
-            alpha = 0;
-            beta_hat = 0;
-        } else if (log10_in_range(vmax)) {
-            const int e_max = floor_log10(vmax);
-            const int atop = min(T::A_MAX, T::B_MAX - 1 - e_max);
-            if (job.variant == kVariantElf) {
-                alpha = alpha_elf<D>(buf, lane, m, vx, m > 1024u && lane == 31, e_max);
-            } else if (atop >= 0) {
-                // quick rejection: Alg. 2 on the largest magnitude first.  The test reads
-                // only |v|, so it runs on vmax itself, the same in every lane.
-                bool fail;
-                if constexpr (D == kD64) fail = !q_test(vmax, atop);
-                else fail = first_pass(vmax, atop) < 0;
-                if (!fail) {
-                    alpha = search_alpha<D>(buf, lane, m, vx, atop);
-                    // FP32 (R14), FP16 (R18): below beta_hat = B_MAX no value can stop early
-                    // (see early_stop), so Alg. 2 value by value gives the same alpha_max
-                    if constexpr (D != kD64) {
-                        if (alpha >= 0 && alpha + e_max + 1 == T::B_MAX &&
-                            early_stop<D>(buf, lane, m, v, vx, m > 1024u && lane == 31, vmax, alpha))
-                            alpha = -1;
-                    }
-                }
-            }
-            if (alpha >= 0) beta_hat = alpha + e_max + 1;
-        }
-    }
+    // ---- 2. G ---------------------------------------------------------------------------------
+    U v[32];
+    read_own<D>(buf, lane, v);
+    U vx = m > 1024u && lane == 31 ? read_elem<D>(buf, 1024) : v[31];        // no further value: no further delta
     __syncwarp();
     next();                                     // the staged values have been read
+    if (!case1) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) v[k] = zigzag(v[k]);
+        vx = zigzag(vx);
+    }
 
-    // ---- 3. G, Z, w (from the ORs of 8-column groups that step 4 uses) -------------------------
-    (void)to_z<D>(v, vx, alpha, m, lane);
+    // ---- 3. |Z| by 8-column groups, w -----------------------------------------------------------
+    U nxt = shfl_down_x(v[0], 1);
+    if (lane == 31) nxt = vx;
+    // OR of the Z of columns 8 i .. 8 i + 7: Z = (x ^ s) << 1 | (s & 1) for the delta x with sign s
     U o[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        U x = v[8 * i];
+        U mag = 0, neg = 0;
 #pragma unroll
-        for (int j = 1; j < 8; ++j) x |= v[8 * i + j];
-        o[i] = x;
+        for (int k = 8 * i; k < 8 * i + 8; ++k) {
+            const U x = (U)((k < 31 ? v[k + 1] : nxt) - v[k]);
+            const U s = sign_mask(x);
+            mag |= x ^ s;
+            neg |= s;
+        }
+        o[i] = (U)((U)(mag << 1) | (neg & 1u));
     }
     const U zor = warp_or_x((U)(o[0] | o[1] | o[2] | o[3]));
     const int w = zor ? ((D == 0) ? 64 - __clzll((long long)zor) : 32 - __clz((int)zor)) : 0;
 
     // ---- 4. non-zero bytes per row, without forming the bit planes ----------------------------
     // This lane's four bytes of row p cover its columns 8i .. 8i + 7 (i = 0..3); byte i is
-    // non-zero iff bit p is set in o[i], the OR of those columns' Z.  The four bits of every
-    // plane are added bit-sliced (count = b0 + 2 b1 + 4 b2) and spread into byte fields,
-    // planes 4g .. 4g + 3 in the bytes of one word, which is added over the warp and stored, one
-    // g at a time (a rolled loop: its code stays small).
+    // non-zero iff bit p is set in o[i].  Transposed across the warp, lane p holds which lanes'
+    // byte i of row p is non-zero, and four population counts give the row's total.
     const uint32_t cols = chunk_cols(m);
     const uint32_t row_bytes = cols / 8u;
-    constexpr int PW = T::W < 32 ? 32 : T::W;  // planes the 32-bit words hold (FP16: 16 of them zero)
+    const LaneTranspose lt = lane_transpose_of(lane);
+    uint32_t nz[2] = {0, 0};                    // of planes `lane` and `lane + 32`
 #pragma unroll
-    for (int h = 0; h < PW / 32; ++h) {
-        const uint32_t o0 = (uint32_t)((uint64_t)o[0] >> (32 * h)), o1 = (uint32_t)((uint64_t)o[1] >> (32 * h));
-        const uint32_t o2 = (uint32_t)((uint64_t)o[2] >> (32 * h)), o3 = (uint32_t)((uint64_t)o[3] >> (32 * h));
-        const uint32_t x1 = o0 ^ o1, x2 = o2 ^ o3, c1 = o0 & o1, c2 = o2 & o3;
-        uint32_t b0 = x1 ^ x2, b1 = c1 ^ c2 ^ (x1 & x2), b2 = c1 & c2;
-#pragma unroll 2
-        for (int g = 0; g < (T::W < 32 ? T::W / 4 : 8); ++g) {
-            const uint32_t word = spread_nibble(b0 & 15u) | (spread_nibble(b1 & 15u) << 1) | (spread_nibble(b2 & 15u) << 2);
-            const uint32_t sum = __reduce_add_sync(kFull, word);
-            if (lane == 0) reinterpret_cast<uint32_t *>(scratch)[8 * h + g] = sum;
-            b0 >>= 4;
-            b1 >>= 4;
-            b2 >>= 4;
-        }
+    for (int h = 0; h < (D == kD64 ? 2 : 1); ++h) {
+        if (h == 1 && w <= 32) break;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) nz[h] += __popc(lane_transpose((uint32_t)((uint64_t)o[i] >> (32 * h)), lt));
     }
-    __syncwarp();
 
     // ---- 5. storage choice (Sec. 3.3) and record size ------------------------------------------
     // the ablations of Sec. 5.4.2 force one scheme for every row
@@ -503,15 +644,13 @@ __device__ void analyse_chunk(const Job &job, uint64_t c, const uint8_t *buf, ui
     uint32_t cost = 0;
     bool dense_lo = false, dense_hi = false;
     if (lane < w) {                              // plane `lane`
-        const uint32_t nz = scratch[lane];
-        const bool sparse = all_sparse || (!all_dense && (row_bytes - nz) > cols / 64u);   // tie -> dense (R10)
-        cost += sparse ? cols / 64u + nz : row_bytes;
+        const bool sparse = all_sparse || (!all_dense && (row_bytes - nz[0]) > cols / 64u);   // tie -> dense (R10)
+        cost += sparse ? cols / 64u + nz[0] : row_bytes;
         dense_lo = !sparse;
     }
     if (D == 0 && lane + 32 < w) {                  // plane `lane + 32`
-        const uint32_t nz = scratch[lane + 32];
-        const bool sparse = all_sparse || (!all_dense && (row_bytes - nz) > cols / 64u);
-        cost += sparse ? cols / 64u + nz : row_bytes;
+        const bool sparse = all_sparse || (!all_dense && (row_bytes - nz[1]) > cols / 64u);
+        cost += sparse ? cols / 64u + nz[1] : row_bytes;
         dense_hi = !sparse;
     }
     const uint32_t body = __reduce_add_sync(kFull, cost);
@@ -520,7 +659,7 @@ __device__ void analyse_chunk(const Job &job, uint64_t c, const uint8_t *buf, ui
     const uint32_t size = 3u + T::Z1B + ((uint32_t)w + 7u) / 8u + body;
     if (lane == 0) {
         reinterpret_cast<uint32_t *>(job.out + 32)[c] = size;
-        job.flags[c] = pack_meta(alpha >= 0 ? alpha : T::A_SENT, beta_hat, w);
+        job.flags[c] = pack_meta(case1 ? alpha : T::A_SENT, beta_hat, w);
         job.flags[job.nchunks + c] = dense_mask;
         unsigned long long *tsum = job.flags + 2 * job.nchunks;
         atomicAdd(tsum + c / kTile, (unsigned long long)size);
@@ -528,14 +667,43 @@ __device__ void analyse_chunk(const Job &job, uint64_t c, const uint8_t *buf, ui
     }
 }
 
-// Lane reads its 32 values (indices 32 lane + k) from global memory, 16 bytes at a time when
-// the chunk is whole and 16-byte aligned; indices >= m read as +0.
+// 32 bytes (one sector) from global memory with one load, 32-byte aligned.
+__device__ __forceinline__ void load32(const void *p, uint64_t (&x)[4]) {
+    asm volatile("ld.global.nc.L1::no_allocate.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(x[0]), "=l"(x[1]), "=l"(x[2]), "=l"(x[3])
+                 : "l"(p));
+}
+
+// Lane reads its 32 values (indices 32 lane + k; indices >= m read as the last value) from global
+// memory: 16 bytes at a time when the chunk is whole and 16-byte aligned.  A whole FP64 chunk at 8
+// modulo 16 (`window`: the 16-byte units around it lie inside the input) reads the lane's 17 aligned
+// units and takes the values one half later, instead of 32 loads of 8 bytes.
 template <int D>
-__device__ __forceinline__ void load_own(const uint8_t *src, int lane, uint32_t m, typename Traits<D>::U (&v)[32]) {
+__device__ __forceinline__ void load_own(const uint8_t *src, bool window, int lane, uint32_t m,
+                                         typename Traits<D>::U (&v)[32]) {
     using U = typename Traits<D>::U;
     constexpr int UN = Traits<D>::UNITS;
     constexpr int PER = 32 / UN;
-    if (m >= 1024u && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+    const bool al16 = (reinterpret_cast<uintptr_t>(src) & 15u) == 0;
+    if (D != kD16 && m >= 1024u && (reinterpret_cast<uintptr_t>(src) & 31u) == 0) {
+        const uint8_t *mine = src + lane * (32 * Traits<D>::S);
+#pragma unroll
+        for (int u = 0; u < Traits<D>::S; ++u) {
+            uint64_t x[4];
+            load32(mine + 32 * u, x);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                if constexpr (D == kD64) {
+                    v[4 * u + h] = x[h];
+                } else if constexpr (D == kD32) {
+                    v[8 * u + 2 * h] = (U)x[h];
+                    v[8 * u + 2 * h + 1] = (U)(x[h] >> 32);
+                }
+            }
+        }
+        return;
+    }
+    if (m >= 1024u && al16) {
         const uint4 *q4 = reinterpret_cast<const uint4 *>(src) + lane * UN;
 #pragma unroll
         for (int u = 0; u < UN; ++u) {
@@ -557,13 +725,20 @@ __device__ __forceinline__ void load_own(const uint8_t *src, int lane, uint32_t 
                 v[PER * u + 3] = q.w;
             }
         }
-    } else {
-        const U *e = reinterpret_cast<const U *>(src);
+    } else if (D == kD64 && window) {
+        const uint4 *q4 = reinterpret_cast<const uint4 *>(src - 8) + lane * UN;
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            const uint32_t i = 32u * (uint32_t)lane + (uint32_t)k;
-            v[k] = i < m ? __ldg(e + i) : (U)0;
+        for (int u = 0; u < UN + 1; ++u) {
+            const uint4 q = __ldg(q4 + u);
+            if (u > 0) v[u > 0 ? 2 * u - 1 : 0] = (U)(((uint64_t)q.y << 32) | q.x);
+            if (u < UN) v[u < UN ? 2 * u : 0] = (U)(((uint64_t)q.w << 32) | q.z);
         }
+    } else {
+        const U *e = reinterpret_cast<const U *>(src) + 32 * lane;
+        const U last = __ldg(reinterpret_cast<const U *>(src) + (m - 1u));
+        const int have = (int)m - 32 * lane;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) v[k] = k < have ? __ldg(e + k) : last;
     }
 }
 
@@ -587,8 +762,10 @@ __device__ __forceinline__ void load_chunk(const Job &job, uint64_t c, int lane,
     const uint64_t first = c * (uint64_t)job.block;
     const uint32_t m = (uint32_t)((job.n - first) < job.block ? (job.n - first) : job.block);
     const uint8_t *src = job.in + first * Traits<D>::S;
-    load_own<D>(src, lane, m, v);
-    vx = (m > 1024u && lane == 31) ? __ldg(reinterpret_cast<const U *>(src) + 1024) : (U)0;
+    const bool window = D == kD64 && m >= 1024u && src - 8 >= job.in &&
+                        src + (m + 1u) * 8u <= job.in + job.n * 8u && (reinterpret_cast<uintptr_t>(src) & 15u) == 8u;
+    load_own<D>(src, window, lane, m, v);
+    vx = (m > 1024u && lane == 31) ? __ldg(reinterpret_cast<const U *>(src) + 1024) : v[31];
 }
 
 // Launch 2, one chunk: G, Z and the plane words again (alpha and w from the analysis), then
@@ -598,94 +775,114 @@ __device__ __forceinline__ void load_chunk(const Job &job, uint64_t c, int lane,
 // as soon as the plane words are in shared memory (the register loads then complete while
 // this record is assembled); otherwise the values are loaded here and `next` does nothing.
 template <int D, bool kWide, bool kPre, class Next>
-__device__ void emit_chunk(const Job &job, uint64_t c, uint8_t *buf, int lane, unsigned long long meta,
-                           unsigned long long dense, uint32_t size, uint64_t rel,
-                           typename Traits<D>::U (&v)[32], typename Traits<D>::U &vx, Next &&next) {
-    constexpr int kPlOff = EmitLayout<kWide>::kPlOff;
+__device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *buf, uint32_t seltab, int lane,
+                                           uint32_t meta_hi, uint64_t dense, uint32_t size, uint64_t rel,
+                                           typename Traits<D>::U (&v)[32], typename Traits<D>::U &vx, Next &&next) {
     using T = Traits<D>;
     using U = typename T::U;
+    using L = EmitLayout<D, kWide>;
     const uint32_t B = job.block;
     const uint64_t first = c * (uint64_t)B;
     const uint32_t m = (uint32_t)((job.n - first) < B ? (job.n - first) : B);
     const uint64_t data_start = 32ull + 4ull * job.nchunks;
-    const uint32_t mb = (uint32_t)(meta >> kMetaShift);
+    const uint32_t mb = meta_hi >> (kMetaShift - 32);
     const int alpha_byte = (int)(mb >> 12), beta_hat = (int)((mb >> 7) & 31u), w = (int)(mb & 127u);
-    const int alpha = alpha_byte == T::A_SENT ? -1 : alpha_byte;
     const uint64_t rec_off = data_start + rel;
     if (rec_off + size > job.out_cap) {          // the job's first chunk reports the capacity error
         next();
         return;
     }
 
-    // ---- G, Z and the plane words in shared memory --------------------------------------------
+    // ---- G (Eq. 4) and its deltas (Eq. 5) -------------------------------------------------------
     if constexpr (!kPre) load_chunk<D>(job, c, lane, v, vx);
-    const U z1 = to_z<D>(v, vx, alpha, m, lane);
-    if (lane == 0) bulk_wait_read();             // the previous record has left the buffer
-    __syncwarp();
-    // half h of the values holds planes 32 h .. 32 h + 31 (the high half only when w > 32)
+    if (alpha_byte != T::A_SENT) {
 #pragma unroll
-    for (int h = 0; h < ((D == 0) ? 2 : 1); ++h) {
-        if (h == 1 && w <= 32) break;
-        uint32_t a[32];
+        for (int k = 0; k < 32; ++k) v[k] = case1_g(v[k], alpha_byte);
+        vx = case1_g(vx, alpha_byte);
+    } else {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) a[j] = (uint32_t)((uint64_t)v[j ^ 7] >> (32 * h));
-        transpose32(a);
-        uint8_t *dst = buf + kPlOff + (T::W - 1 - 32 * h) * 128 + 4 * lane;
-#pragma unroll
-        for (int p = 0; p < (T::W < 32 ? T::W : 32); ++p) *reinterpret_cast<uint32_t *>(dst - p * 128) = a[p];
+        for (int k = 0; k < 32; ++k) v[k] = zigzag(v[k]);
+        vx = zigzag(vx);
     }
-    __syncwarp();
-    next();                                     // v and vx are free
+    const U z1 = shfl_x(v[0], 0);
+    U nxt = shfl_down_x(v[0], 1);
+    if (lane == 31) nxt = vx;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v[k] = (U)((k < 31 ? v[k + 1] : nxt) - v[k]);
 
+    // ---- planes (Sec. 3.3) and record -----------------------------------------------------------
+    // The zigzag is done on the planes: plane p of Z is plane p - 1 of the deltas XOR their sign
+    // plane, plane 0 is the sign plane (one XOR per plane instead of five operations per value).
+    // Half h of the deltas holds planes 32 h .. 32 h + 31; with w <= 32 every delta fits 32 bits and
+    // its sign is bit 31, otherwise it is bit 63.
     const uint32_t cols = chunk_cols(m);
-    const uint32_t nact = cols / 32u;
-    const uint32_t row_bytes = cols / 8u;
-    const uint64_t dense_mask = dense;
-    const uint32_t flag_bytes = ((uint32_t)w + 7u) / 8u;
-    const uint32_t hdr = 3u + T::Z1B + flag_bytes;
-    struct { int alpha_byte, beta_hat; uint64_t z1; } pd{alpha_byte, beta_hat, (uint64_t)z1};
+    const uint32_t row_bytes = cols / 8u, bm_bytes = cols / 64u;
     uint8_t *gdst = job.out + rec_off;
     const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(gdst) & 15u);
-
-    // ---- 6. record in shared memory (in place of the consumed plane words), then global ------
-    // Row r (plane w-r) ends before byte 37 + 128 r of the buffer (37 + 144 r when every row
-    // is sparse, wide layout) while the plane read next starts at kPlOff + (64 - w + r) * 128
-    // >= kPlOff + 128 r: nothing unread is overwritten.
-    {
-        // header byte `lane` (branch-free: every lane computes its byte, lanes < hdr store it)
-        const int i = lane;
-        const uint32_t zb = (uint32_t)(pd.z1 >> ((8 * (i - 2)) & 63)) & 0xFFu;
-        const uint32_t fb = (uint32_t)(dense_mask >> ((8u * (flag_bytes - 1u - (uint32_t)(i - 3 - T::Z1B))) & 63u)) & 0xFFu;
-        uint32_t byte = i < 2 + T::Z1B ? zb : ((i == 2 + T::Z1B) ? (uint32_t)w : fb);
-        byte = i == 0 ? (uint32_t)pd.alpha_byte : (i == 1 ? (uint32_t)pd.beta_hat : byte);
-        if ((uint32_t)lane < hdr) buf[sh + i] = (uint8_t)byte;
-    }
-    __syncwarp();
+    const uint32_t flag_bytes = ((uint32_t)w + 7u) / 8u;
+    const uint32_t hdr = 3u + T::Z1B + flag_bytes;
+    uint8_t *slots = buf + L::kRec - (32u - L::kRows) * 128u;         // plane p of a half: 128 (31 - p) further
+    uint8_t *dst = slots + 31 * 128 + 4 * lane;                      // plane 0; plane p lies 128 p below
     uint32_t pos = sh + hdr;                      // next record byte in the buffer
-    int p = w - 1;
-    while (p >= 0) {
-        const uint32_t src = kPlOff + (uint32_t)(T::W - 1 - p) * 128u;
-        if ((dense_mask >> p) & 1ull) {
-            // a run of dense rows p, p-1, ..., q: contiguous in the plane buffer when rows
-            // are 128 bytes long, so one move copies the whole run
-            int q = p;
-            if (row_bytes == 128u) {
-                const uint64_t below = (p >= 63) ? ~0ull : ((2ull << p) - 1ull);
-                const uint64_t holes = ~dense_mask & below;               // sparse rows <= p
-                q = holes ? 64 - __clzll((long long)holes) : 0;           // lowest row of the run
-            }
-            const uint32_t rows = (uint32_t)(p - q + 1);
-            smem_move_down(buf, pos, src, rows * row_bytes, lane);
-            pos += rows * row_bytes;
-            p = q - 1;
-        } else {
-            const uint32_t x = *reinterpret_cast<const uint32_t *>(buf + src + 4 * lane);
-            __syncwarp();
-            pos += sparse_row(buf, pos, x, lane, nact);
-            --p;
+    auto header = [&]() {
+        // record header: byte `lane` (branch-free: every lane computes its byte, lanes < hdr store it)
+        const int i = lane;
+        const uint32_t zb = (uint32_t)((uint64_t)z1 >> ((8 * (i - 2)) & 63)) & 0xFFu;
+        const uint32_t fb = (uint32_t)(dense >> ((8u * (flag_bytes - 1u - (uint32_t)(i - 3 - T::Z1B))) & 63u)) & 0xFFu;
+        uint32_t byte = i < 2 + T::Z1B ? zb : ((i == 2 + T::Z1B) ? (uint32_t)w : fb);
+        byte = i == 0 ? (uint32_t)alpha_byte : (i == 1 ? (uint32_t)beta_hat : byte);
+        if ((uint32_t)lane < hdr) buf[sh + i] = (uint8_t)byte;
+    };
+    uint32_t sgn = 0;
+    const bool two = D == kD64 && w > 32;
+    constexpr int R = T::W < 32 ? T::W : 32;
+    uint32_t a[32];
+    if constexpr (D == kD64) {
+        if (two) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) a[j] = (uint32_t)(v[j ^ 7] >> 32);
+            transpose32(a);
+            sgn = a[31];
+#pragma unroll
+            for (int p = 0; p < 31; ++p) *reinterpret_cast<uint32_t *>(dst - (p + 1) * 128) = a[p] ^ sgn;
         }
     }
-    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) a[j] = (uint32_t)v[j ^ 7];
+    transpose32(a);
+    if (!two) sgn = a[R - 1];
+    if (two) *reinterpret_cast<uint32_t *>(dst) = a[31] ^ sgn;
+    auto low_planes = [&]() {
+        *reinterpret_cast<uint32_t *>(dst) = sgn;
+#pragma unroll
+        for (int p = 0; p < R - 1; ++p) *reinterpret_cast<uint32_t *>(dst - (p + 1) * 128) = a[p] ^ sgn;
+    };
+    auto half_rows = [&](int h) {
+        const int wh = w - 32 * h;
+        emit_rows(buf, slots, pos, wh >= 32 ? ~0u : (1u << wh) - 1u, (uint32_t)(dense >> (32 * h)), row_bytes,
+                  bm_bytes, seltab, lane);
+        __syncwarp();
+    };
+    if constexpr (D == kD64) {
+        if (lane == 0) bulk_wait_read();          // the previous record has left the buffer
+        __syncwarp();
+        header();
+        // one copy of the row code for both halves (the low half's planes wait in registers): with
+        // two, instruction fetch made every phase of the kernel slower (485 -> 452 us)
+#pragma unroll 1
+        for (int h = two ? 1 : 0; h >= 0; --h) {
+            if (h == 0) low_planes();
+            __syncwarp();
+            half_rows(h);
+        }
+    } else {
+        low_planes();
+        if (lane == 0) bulk_wait_read();
+        __syncwarp();
+        next();                                   // v and vx are free
+        header();
+        half_rows(0);
+    }
 
     // to global memory: the 16-byte units entirely inside the record with one bulk copy
     // (lane 0), the partial units at its ends (shared with the neighbouring records) bytewise
@@ -728,7 +925,6 @@ __device__ __forceinline__ void analyse_loop(const Job *__restrict__ jobs, int n
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     uint8_t *wbase = smem + warp * kAnalyseWarpBytes;
-    uint8_t *scratch = wbase + kBuf;
     __shared__ Job s_single;                      // the single job, read from shared memory
     if (threadIdx.x == 0) s_single = single;
     __syncthreads();
@@ -748,12 +944,12 @@ __device__ __forceinline__ void analyse_loop(const Job *__restrict__ jobs, int n
         };
         const Job &job = job_of(jobs, njobs, s_single, t);
         const uint64_t c = t - job.chunk_begin;
-        if constexpr (kDt == kDtF64) analyse_chunk<kD64>(job, c, wbase, scratch, lane, next);
-        else if constexpr (kDt == kDtF32) analyse_chunk<kD32>(job, c, wbase, scratch, lane, next);
-        else if constexpr (kDt == kDtF16) analyse_chunk<kD16>(job, c, wbase, scratch, lane, next);
-        else if (job.dtype == 0) analyse_chunk<kD64>(job, c, wbase, scratch, lane, next);
-        else if (job.dtype == 1) analyse_chunk<kD32>(job, c, wbase, scratch, lane, next);
-        else analyse_chunk<kD16>(job, c, wbase, scratch, lane, next);
+        if constexpr (kDt == kDtF64) analyse_chunk<kD64>(job, c, wbase, lane, next);
+        else if constexpr (kDt == kDtF32) analyse_chunk<kD32>(job, c, wbase, lane, next);
+        else if constexpr (kDt == kDtF16) analyse_chunk<kD16>(job, c, wbase, lane, next);
+        else if (job.dtype == 0) analyse_chunk<kD64>(job, c, wbase, lane, next);
+        else if (job.dtype == 1) analyse_chunk<kD32>(job, c, wbase, lane, next);
+        else analyse_chunk<kD16>(job, c, wbase, lane, next);
         __syncwarp();
         if (tn >= total_chunks) break;
         t = tn;
@@ -802,21 +998,29 @@ __device__ void finish_job(const Job &job, int lane) {
 // records before c take < 2^31 bytes (33 * 4096 records of at most 9235 bytes) and one 32-bit
 // reduction adds the lanes' shares.  Beyond that (more than 128 M values at block 1024) the
 // further groups are read when resolving and added in 64 bits.
-struct EmitInfo {
-    unsigned long long meta, dense;
+template <bool k64> struct EmitInfo {
+    uint32_t meta_hi;                 // the analysis word's upper half
+    uint32_t dense_lo, dense_hi[1]; // dense-row mask (planes 32 and up: FP64 only)
     uint32_t g0, t0, t1, s0, s1;      // this lane's group sum, two tile sums, two record sizes
     uint32_t size;                    // c's record size
 };
 
-__device__ __forceinline__ EmitInfo load_info(const Job &job, uint64_t c, int lane) {
+template <bool k64>
+__device__ __forceinline__ EmitInfo<k64> load_info(const Job &job, uint64_t c, int lane) {
     const uint64_t nc = job.nchunks;
     const uint32_t *sizes = reinterpret_cast<const uint32_t *>(job.out + 32);
     const uint32_t *tsum = reinterpret_cast<const uint32_t *>(job.flags + 2 * nc);   // low words
     const uint32_t *gsum = tsum + 2 * tile_count(nc);
     const uint64_t g = c / kGroup, t = c / kTile, tb = g * (kGroup / kTile), cb = t * kTile;
-    EmitInfo e;
-    e.meta = job.flags[c];
-    e.dense = job.flags[nc + c];
+    EmitInfo<k64> e;
+    e.meta_hi = reinterpret_cast<const uint32_t *>(job.flags + c)[1];
+    if constexpr (k64) {
+        const uint2 d = *reinterpret_cast<const uint2 *>(job.flags + nc + c);
+        e.dense_lo = d.x;
+        e.dense_hi[0] = d.y;
+    } else {
+        e.dense_lo = *reinterpret_cast<const uint32_t *>(job.flags + nc + c);
+    }
     e.size = sizes[c];
     e.g0 = (uint64_t)lane < g ? gsum[2 * lane] : 0u;
     e.t0 = tb + (uint64_t)lane < t ? tsum[2 * (tb + lane)] : 0u;
@@ -825,7 +1029,8 @@ __device__ __forceinline__ EmitInfo load_info(const Job &job, uint64_t c, int la
     e.s1 = cb + 32u + (uint64_t)lane < c ? sizes[cb + 32u + lane] : 0u;
     return e;
 }
-__device__ __forceinline__ uint64_t resolve_info(const Job &job, uint64_t c, const EmitInfo &e, int lane) {
+template <bool k64>
+__device__ __forceinline__ uint64_t resolve_info(const Job &job, uint64_t c, const EmitInfo<k64> &e, int lane) {
     const uint32_t p = e.g0 + e.t0 + e.t1 + e.s0 + e.s1;
     const uint64_t g = c / kGroup;
     if (g <= 32u) return __reduce_add_sync(kFull, p);
@@ -843,7 +1048,9 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
                                           uint64_t total_chunks, Control *ctl, uint8_t *smem) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    uint8_t *wbase = smem + warp * EmitLayout<kWide>::kBytes;
+    constexpr int DL = kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64);
+    uint8_t *wbase = smem + warp * EmitLayout<DL, kWide>::kBytes;
+    const uint32_t seltab = compact_sel((uint32_t)lane & 15u);
     if (blockIdx.x == 0 && warp == 0) {          // jobs without chunks: header and length only
         if (jobs == nullptr) {
             if (s_single.nchunks == 0) finish_job(s_single, lane);
@@ -861,52 +1068,54 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
     // the FP32 and FP16 forms keep the values of the chunk after the current one in registers
     // (kPre); the FP64 form has no registers to spare for them
     constexpr bool kPre = kDt == kDtF32 || kDt == kDtF16;
-    constexpr int DP = kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64);
-    typename Traits<DP>::U v[32], vx;
+    typename Traits<DL>::U v[32], vx;
     uint64_t t = ticket_of(take_ticket(ctl, kTicketEmit, lane));
     if (t >= total_chunks) return;
     uint64_t tn = ticket_of(take_ticket(ctl, kTicketEmit, lane));
-    EmitInfo info;
+    constexpr bool k64 = kDt == kDtF64 || kDt == kDtMixed;
+    EmitInfo<k64> info;
     {
         const Job &j0 = job_of(jobs, njobs, s_single, t);
-        info = load_info(j0, t - j0.chunk_begin, lane);
-        if constexpr (kPre) load_chunk<DP>(j0, t - j0.chunk_begin, lane, v, vx);
+        info = load_info<k64>(j0, t - j0.chunk_begin, lane);
+        if constexpr (kPre) load_chunk<DL>(j0, t - j0.chunk_begin, lane, v, vx);
     }
     for (;;) {
         // the ticket after tn, read at the next iteration; tn's workspace words are fetched now
         const unsigned long long raw = tn < total_chunks ? take_ticket(ctl, kTicketEmit, lane) : 0ull;
-        EmitInfo next{};
+        EmitInfo<k64> next{};
         if (tn < total_chunks) {
             if constexpr (!kPre) prefetch_chunk(jobs, njobs, s_single, tn, lane);
             const Job &jn = job_of(jobs, njobs, s_single, tn);
-            next = load_info(jn, tn - jn.chunk_begin, lane);
+            next = load_info<k64>(jn, tn - jn.chunk_begin, lane);
         }
         const Job &job = job_of(jobs, njobs, s_single, t);
         const uint64_t c = t - job.chunk_begin;
         const uint64_t rel = resolve_info(job, c, info, lane);
         if (c == 0) finish_job(job, lane);
+        uint64_t dense = info.dense_lo;
+        if constexpr (k64) dense |= (uint64_t)info.dense_hi[0] << 32;
         auto load_next = [&]() {
             if constexpr (kPre) {
                 if (tn < total_chunks) {
                     const Job &jn = job_of(jobs, njobs, s_single, tn);
-                    load_chunk<DP>(jn, tn - jn.chunk_begin, lane, v, vx);
+                    load_chunk<DL>(jn, tn - jn.chunk_begin, lane, v, vx);
                 }
             }
         };
         if constexpr (kPre) {
-            emit_chunk<DP, kWide, true>(job, c, wbase, lane, info.meta, info.dense, info.size, rel, v, vx, load_next);
+            emit_chunk<DL, kWide, true>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, v, vx, load_next);
         } else if constexpr (kDt == kDtF64) {
             uint64_t u[32], ux;
-            emit_chunk<kD64, kWide, false>(job, c, wbase, lane, info.meta, info.dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD64, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
         } else if (job.dtype == 0) {
             uint64_t u[32], ux;
-            emit_chunk<kD64, kWide, false>(job, c, wbase, lane, info.meta, info.dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD64, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
         } else if (job.dtype == 1) {
             uint32_t u[32], ux;
-            emit_chunk<kD32, kWide, false>(job, c, wbase, lane, info.meta, info.dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD32, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
         } else {
             uint16_t u[32], ux;
-            emit_chunk<kD16, kWide, false>(job, c, wbase, lane, info.meta, info.dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD16, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
         }
         __syncwarp();
         if (tn >= total_chunks) break;
@@ -956,7 +1165,7 @@ void launch_analyse(const Job *d_jobs, int njobs, const Job &single, uint64_t to
 template <bool kWide, int kDt>
 void launch_emit(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, Control *ctl,
                  cudaStream_t stream) {
-    const int w = g_cta_warps[0], smem = w * EmitLayout<kWide>::kBytes;
+    const int w = g_cta_warps[0], smem = w * (int)EmitLayout<kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64), kWide>::kBytes;
     if constexpr (kDt == kDtF32 || kDt == kDtF16) {
         const int g = persistent_grid_of(reinterpret_cast<const void *>(emit_kernel_narrow<kWide, kDt>), w, smem,
                                          g_ctas_per_sm[0], total_chunks);
@@ -1005,7 +1214,7 @@ int persistent_grid_size(const void *kernel, int warps, int smem_bytes, int lim,
 int compress_grid(uint64_t total_chunks) {
     const int w = g_cta_warps[0];
     return persistent_grid_of(reinterpret_cast<const void *>(emit_kernel<false, kDtMixed>), w,
-                              w * EmitLayout<false>::kBytes, g_ctas_per_sm[0], total_chunks);
+                              w * (int)EmitLayout<kD64, false>::kBytes, g_ctas_per_sm[0], total_chunks);
 }
 
 cudaError_t launch_compress(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks,

@@ -199,6 +199,36 @@ __device__ __forceinline__ void transpose32(uint32_t (&a)[32]) {
 #undef FALCON_TSTEP
 }
 
+// 32x32 bit transpose across the warp: afterwards bit l of lane p's word = old bit p of lane l's.
+// The 16- and 8-lane exchanges are one byte permute each, the others a rotate and a bitwise select.
+struct LaneTranspose {
+    uint32_t sel16, sel8;                         // byte-permute selectors
+    uint32_t r4, r2, r1, m4, m2, m1;              // rotations and the bits kept
+};
+__device__ __forceinline__ LaneTranspose lane_transpose_of(int lane) {
+    LaneTranspose t;
+    t.sel16 = (lane & 16) ? 0x3276u : 0x5410u;
+    t.sel8 = (lane & 8) ? 0x3715u : 0x6240u;
+    t.r4 = (lane & 4) ? 28u : 4u;
+    t.r2 = (lane & 2) ? 30u : 2u;
+    t.r1 = (lane & 1) ? 31u : 1u;
+    t.m4 = (lane & 4) ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
+    t.m2 = (lane & 2) ? 0xCCCCCCCCu : 0x33333333u;
+    t.m1 = (lane & 1) ? 0xAAAAAAAAu : 0x55555555u;
+    return t;
+}
+__device__ __forceinline__ uint32_t lane_transpose(uint32_t a, const LaneTranspose &t) {
+    uint32_t b;
+    a = __byte_perm(a, __shfl_xor_sync(kFull, a, 16), t.sel16);
+    a = __byte_perm(a, __shfl_xor_sync(kFull, a, 8), t.sel8);
+    b = __shfl_xor_sync(kFull, a, 4);
+    a = (a & t.m4) | (__funnelshift_l(b, b, t.r4) & ~t.m4);
+    b = __shfl_xor_sync(kFull, a, 2);
+    a = (a & t.m2) | (__funnelshift_l(b, b, t.r2) & ~t.m2);
+    b = __shfl_xor_sync(kFull, a, 1);
+    return (a & t.m1) | (__funnelshift_l(b, b, t.r1) & ~t.m1);
+}
+
 // --------------------------------------------------------------------------------------
 // Shared-memory staging of a chunk's values, swizzled so that lane l's 16-byte units
 // (values 32l .. 32l+31) are read conflict-free: unit u of lane L sits at L*UNITS + (u^(L&7)).
@@ -255,10 +285,9 @@ __device__ __forceinline__ void stage_values_async(const uint8_t *src, uint32_t 
     }
 }
 
-// Lane reads its 32 values (indices 32*lane + k); indices >= m read as +0.
+// Lane reads its 32 values (indices 32*lane + k).
 template <int D>
-__device__ __forceinline__ void read_own(const uint8_t *wsm, int lane, uint32_t m,
-                                         typename Traits<D>::U (&v)[32]) {
+__device__ __forceinline__ void read_own(const uint8_t *wsm, int lane, typename Traits<D>::U (&v)[32]) {
     using U = typename Traits<D>::U;
     constexpr int UN = Traits<D>::UNITS;
     constexpr int PER = 32 / UN;
@@ -281,11 +310,6 @@ __device__ __forceinline__ void read_own(const uint8_t *wsm, int lane, uint32_t 
             v[PER * u + 2] = q.z;
             v[PER * u + 3] = q.w;
         }
-    }
-    if (m < 1024u) {                              // a tail chunk: values past m read as +0
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-            if ((uint32_t)(32 * lane + k) >= m) v[k] = 0;
     }
 }
 
@@ -447,14 +471,16 @@ __device__ __forceinline__ int first_pass_f32(uint32_t u, int atop) {
 // scaled), so an approximation of X closer than 3/8 rounds to g: with m and 5^a both
 // normalised to 64 bits, mulhi(m 2^11, 5^a 2^(63-d)) = floor(X 2^sh), sh = F + 10 - d >= 13,
 // is X within 2^-13, and rounding it at bit sh gives g.  One 64-bit high product per value.
+__device__ __forceinline__ uint64_t case1_round(uint64_t m, uint64_t norm, int sh) {
+    const uint64_t t = __umul64hi(m << 11, norm);
+    return ((t >> (sh - 1)) + 1ull) >> 1;
+}
 __device__ __forceinline__ uint64_t case1_g(uint64_t u, int a) {
     const uint64_t au = u & 0x7FFFFFFFFFFFFFFFull;
     if (au == 0) return 0;
     const int E = (int)(au >> 52) - 1075;
     const uint64_t m = (au & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-    const int sh = -(E + a) + 10 - (int)FALCON_LOG2_POW5[a];
-    const uint64_t t = __umul64hi(m << 11, FALCON_POW5_NORM[a]);
-    const uint64_t N = ((t >> (sh - 1)) + 1ull) >> 1;
+    const uint64_t N = case1_round(m, FALCON_POW5_NORM[a], -(E + a) + 10 - (int)FALCON_LOG2_POW5[a]);
     return (u >> 63) ? (0ull - N) : N;
 }
 __device__ __forceinline__ uint32_t case1_g(uint32_t u, int a) {
