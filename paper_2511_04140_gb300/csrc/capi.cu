@@ -213,7 +213,7 @@ int falcon_compress(const void *d_in, uint64_t n, int dtype, uint32_t block_size
     const size_t ws_bytes = falcon_workspace_bytes(nc);
     void *ws = nullptr;
     if ((st = get_workspace(s, ws_bytes, &ws))) return st;
-    if (cudaMemsetAsync(ws, 0, ws_bytes, s) != cudaSuccess) return FALCON_ERR_CUDA;
+    if (cudaMemsetAsync(ws, 0, sizeof(Control), s) != cudaSuccess) return FALCON_ERR_CUDA;
     uint8_t *w8 = static_cast<uint8_t *>(ws);
     uint64_t *result = reinterpret_cast<uint64_t *>(w8 + kResultOffset);
     const Job j = make_compress_job(d_in, n, dtype, block_size, d_out, out_capacity, w8 + kControlBytes, result);
@@ -257,8 +257,8 @@ int falcon_compress_variant_async(const void *d_in, uint64_t n, int dtype, uint3
         (uintptr_t)d_result % 8 != 0)
         return FALCON_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(d_workspace, 0, need, s) != cudaSuccess) return FALCON_ERR_CUDA;
-    if (cudaMemsetAsync(d_result, 0, 16, s) != cudaSuccess) return FALCON_ERR_CUDA;
+    // the chunk tickets; the launches write every other word they read, and the result
+    if (cudaMemsetAsync(d_workspace, 0, sizeof(Control), s) != cudaSuccess) return FALCON_ERR_CUDA;
     uint8_t *w8 = static_cast<uint8_t *>(d_workspace);
     Job j = make_compress_job(d_in, n, dtype, block_size, d_out, out_capacity, w8 + kControlBytes, d_result);
     j.variant = (uint32_t)variant;
@@ -283,7 +283,6 @@ int falcon_decompress(const void *d_in, size_t in_bytes, void *d_out, size_t out
     const size_t ws_bytes = falcon_workspace_bytes(h.nchunks);
     void *ws = nullptr;
     if ((st = get_workspace(s, ws_bytes, &ws))) return st;
-    if (cudaMemsetAsync(ws, 0, ws_bytes, s) != cudaSuccess) return FALCON_ERR_CUDA;
     uint8_t *w8 = static_cast<uint8_t *>(ws);
     uint64_t *result = reinterpret_cast<uint64_t *>(w8 + kResultOffset);
     const Job j = make_decompress_job(d_in, in_bytes, h, d_out, out_capacity_bytes, w8 + kControlBytes, result);
@@ -310,8 +309,6 @@ int falcon_decompress_async(const void *d_in, size_t in_bytes, const void *h_hea
         (uintptr_t)d_result % 8 != 0)
         return FALCON_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(d_workspace, 0, need, s) != cudaSuccess) return FALCON_ERR_CUDA;
-    if (cudaMemsetAsync(d_result, 0, 16, s) != cudaSuccess) return FALCON_ERR_CUDA;
     uint8_t *w8 = static_cast<uint8_t *>(d_workspace);
     const Job j = make_decompress_job(d_in, in_bytes, h, d_out, out_capacity_bytes, w8 + kControlBytes, d_result);
     if (launch_decompress(nullptr, 1, j, h.nchunks, reinterpret_cast<Control *>(d_workspace), s) != cudaSuccess)
@@ -333,7 +330,6 @@ int falcon_aggregate_async(const void *d_in, size_t in_bytes, const void *h_head
         (uintptr_t)d_stats % 8 != 0)
         return FALCON_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(d_workspace, 0, need, s) != cudaSuccess) return FALCON_ERR_CUDA;
     uint8_t *w8 = static_cast<uint8_t *>(d_workspace);
     // no values are stored: the job has no output; its status word sits in the control region
     uint64_t *result = reinterpret_cast<uint64_t *>(w8 + kResultOffset);
@@ -392,8 +388,6 @@ struct BatchPlan {
     int direction;
     int count;
     uint64_t total_chunks;
-    size_t reset_bytes;       // control block + workspace words, zeroed before each launch
-    uint64_t *d_results;
 };
 std::mutex g_plan_mu;
 std::unordered_map<uintptr_t, BatchPlan> g_plans;
@@ -470,7 +464,7 @@ int falcon_batch_plan(int direction, const falcon_series *h_series, int count, v
         cudaMemcpyAsync(w8 + kControlBytes, jobs.data(), sizeof(Job) * (size_t)count, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return FALCON_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return FALCON_ERR_CUDA;   // the host table is freed below
-    BatchPlan plan{direction, count, total, kControlBytes + table + 8 * words, d_results};
+    BatchPlan plan{direction, count, total};
     std::lock_guard<std::mutex> lk(g_plan_mu);
     g_plans[(uintptr_t)d_workspace] = plan;
     return FALCON_OK;
@@ -486,14 +480,7 @@ int falcon_batch_launch(void *d_workspace, void *stream) {
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t *w8 = static_cast<uint8_t *>(d_workspace);
-    // the control block and the workspace words; the job table in between is kept
-    const size_t table = align256(sizeof(Job) * (size_t)plan.count);
-    if (cudaMemsetAsync(w8, 0, kControlBytes, s) != cudaSuccess) return FALCON_ERR_CUDA;
-    if (plan.reset_bytes > kControlBytes + table &&
-        cudaMemsetAsync(w8 + kControlBytes + table, 0, plan.reset_bytes - kControlBytes - table, s) != cudaSuccess)
-        return FALCON_ERR_CUDA;
-    if (plan.count > 0 && cudaMemsetAsync(plan.d_results, 0, 16 * (size_t)plan.count, s) != cudaSuccess)
-        return FALCON_ERR_CUDA;
+    if (plan.direction == FALCON_COMPRESS && cudaMemsetAsync(w8, 0, sizeof(Control), s) != cudaSuccess) return FALCON_ERR_CUDA;
     if (plan.count == 0) return FALCON_OK;
     const Job *d_jobs = reinterpret_cast<const Job *>(w8 + kControlBytes);
     Control *ctl = reinterpret_cast<Control *>(w8);

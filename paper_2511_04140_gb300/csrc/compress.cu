@@ -1,5 +1,5 @@
 // Falcon compression (Sec. 3 of the paper; the work of Alg. 3 CmpKernel) for sm_103a, as
-// two launches, neither of which waits on another warp:
+// two or three launches, none of which waits on another warp:
 //   1. analyse: each warp takes its chunks by ticket (its one shared-memory value buffer
 //      receives the next chunk by cp.async, swizzled, as soon as the current one is in registers)
 //      and computes
@@ -12,10 +12,11 @@
 //      - the ORs of |Z| (Eq. 5) over 8-column groups, the bit width w, and from those ORs,
 //        transposed across the warp, the non-zero bytes of every row (Sec. 3.3 lambda) without
 //        forming the bit planes; sparse/dense per row; the record size, which goes
-//        into the stream's size array and is added to its 64-chunk tile's and 4096-chunk
-//        group's sums (the size synchronisation of Sec. 3.4); alpha, beta_hat, w and the
-//        dense-row mask, which go into the workspace;
-//   2. emit: each chunk's record offset from those sums, the values again (straight from
+//        into the stream's size array; alpha, beta_hat, w and the dense-row mask, which go into the
+//        workspace;
+//   2. offsets (decompress.cu; the size synchronisation of Sec. 3.4): every record's position into
+//      the workspace.  Streams of at most 1024 chunks skip it, their emit warps add up the sizes;
+//   3. emit: the values again (straight from
 //      global memory, a whole sector per lane and load, not kept in L1: FP64 with the next chunk
 //      prefetched into L2, FP32 and FP16 with the next chunk's values loaded into registers during
 //      the current record), G, the deltas' bit planes (32x32 register transposes, one 32-bit word per
@@ -29,13 +30,16 @@
 // per-value zigzags and bit-sliced counts).  2^26 segment values: FP64 520 -> 453 us, FP32 270 -> 242 us;
 // Case-1 FP64 of 40 M values in 1025-value chunks 622 -> 453 us.  Slower, and left out: two copies of the
 // row code (FP64 485 us: instruction fetch), a transpose shared by both halves in a loop (475 us), dense
-// rows moved in 16-byte units (FP64 461, FP32 238 us), values kept in L1 (483 us).
+// rows moved in 16-byte units (FP64 461, FP32 238 us), values kept in L1 (483 us).  The offsets launch in
+// place of per-tile and per-group sums (two atomics per chunk in the analysis, five loads and a
+// reduction per chunk in the emit, a reset of the workspace): FP64 452 -> 441 us, 2^20-value walk 40 -> 37 us.
 // The paper resolves offsets inside one launch with a decoupled look-back; with about 1800
 // resident warps on a GB300 the waits of that look-back took half of every warp's time, while
 // the analysis recomputed by the emit launch costs less.
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "falcon_device.cuh"
 
@@ -532,11 +536,11 @@ __device__ __forceinline__ void issue_chunk(const Job *jobs, int njobs, const Jo
 }
 
 // Workspace words of a job (job.flags), written by the analysis launch:
-//   flags[c]            alpha byte (5 bits) | beta_hat (5) | w (7), in bits 47..63;
-//   flags[nchunks + c]  the dense-row mask (bit p: plane p is stored dense);
-//   flags[2 nchunks + j]                       the sum of the record sizes of 64-chunk tile j,
-//   flags[2 nchunks + tile_count(nchunks) + g]  and of 4096-chunk group g (atomic adds).
+//   flags[c]            alpha byte (5 bits) | beta_hat (5) | w (7), in bits 47..63; the offsets launch
+//                       adds the record's position (from the first record) below;
+//   flags[nchunks + c]  the dense-row mask (bit p: plane p is stored dense).
 constexpr int kMetaShift = 47;
+static_assert(kMetaShift == kOffsetBits, "the offsets launch fills the bits below");
 
 __device__ __forceinline__ unsigned long long pack_meta(int alpha_byte, int beta_hat, int w) {
     return (unsigned long long)(((uint32_t)alpha_byte << 12) | ((uint32_t)beta_hat << 7) | (uint32_t)w) << kMetaShift;
@@ -661,9 +665,6 @@ __device__ __forceinline__ void analyse_chunk(const Job &job, uint64_t c, uint8_
         reinterpret_cast<uint32_t *>(job.out + 32)[c] = size;
         job.flags[c] = pack_meta(case1 ? alpha : T::A_SENT, beta_hat, w);
         job.flags[job.nchunks + c] = dense_mask;
-        unsigned long long *tsum = job.flags + 2 * job.nchunks;
-        atomicAdd(tsum + c / kTile, (unsigned long long)size);
-        atomicAdd(tsum + tile_count(job.nchunks) + c / kGroup, (unsigned long long)size);
     }
 }
 
@@ -742,10 +743,9 @@ __device__ __forceinline__ void load_own(const uint8_t *src, bool window, int la
     }
 }
 
-// Asks for chunk t's values to be brought into L2 (one prefetch per 128-byte line).
-__device__ __forceinline__ void prefetch_chunk(const Job *jobs, int njobs, const Job &single, uint64_t t, int lane) {
-    const Job &job = (jobs == nullptr) ? single : jobs[find_job(jobs, njobs, t)];
-    const uint64_t first = (t - job.chunk_begin) * (uint64_t)job.block;
+// Asks for a chunk's values to be brought into L2 (one prefetch per 128-byte line).
+__device__ __forceinline__ void prefetch_chunk(const Job &job, uint64_t c, int lane) {
+    const uint64_t first = c * (uint64_t)job.block;
     const uint32_t m = (uint32_t)((job.n - first) < job.block ? (job.n - first) : job.block);
     const uint32_t s = job.dtype == 0 ? 8u : (job.dtype == 1 ? 4u : 2u);
     const uint8_t *src = job.in + first * s;
@@ -776,7 +776,7 @@ __device__ __forceinline__ void load_chunk(const Job &job, uint64_t c, int lane,
 // this record is assembled); otherwise the values are loaded here and `next` does nothing.
 template <int D, bool kWide, bool kPre, class Next>
 __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *buf, uint32_t seltab, int lane,
-                                           uint32_t meta_hi, uint64_t dense, uint32_t size, uint64_t rel,
+                                           uint64_t word, uint64_t dense, uint32_t size, uint64_t rel,
                                            typename Traits<D>::U (&v)[32], typename Traits<D>::U &vx, Next &&next) {
     using T = Traits<D>;
     using U = typename T::U;
@@ -785,7 +785,7 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     const uint64_t first = c * (uint64_t)B;
     const uint32_t m = (uint32_t)((job.n - first) < B ? (job.n - first) : B);
     const uint64_t data_start = 32ull + 4ull * job.nchunks;
-    const uint32_t mb = meta_hi >> (kMetaShift - 32);
+    const uint32_t mb = (uint32_t)(word >> kMetaShift);
     const int alpha_byte = (int)(mb >> 12), beta_hat = (int)((mb >> 7) & 31u), w = (int)(mb & 127u);
     const uint64_t rec_off = data_start + rel;
     if (rec_off + size > job.out_cap) {          // the job's first chunk reports the capacity error
@@ -905,16 +905,21 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     __syncwarp();
 }
 
+// The hot kernels come in four forms by dtype: kDt = 0 (every job FP64), 1 (every job FP32),
+// 3 (every job FP16) or 2 (any, per job: batches and the server).  A single-dtype form carries
+// a third of the code, which the instruction caches notice, and serves a single stream, whose job
+// it reads from shared memory.
+constexpr int kDtF64 = 0, kDtF32 = 1, kDtMixed = 2, kDtF16 = 3;
+
+// Single streams of at most this many chunks need no offsets launch: their emit warps read at most
+// 4 KB of sizes each, one round trip, where the launch costs about 3 us.
+constexpr uint64_t kDirectChunks = 1024;
+
 __device__ __forceinline__ const Job &job_of(const Job *jobs, int njobs, const Job &single, uint64_t t) {
     return (jobs == nullptr) ? single : jobs[find_job(jobs, njobs, t)];
 }
 
 }  // namespace
-
-// The hot kernels come in four forms by dtype: kDt = 0 (every job FP64), 1 (every job FP32),
-// 3 (every job FP16) or 2 (any, per job: batches and the server).  A single-dtype form carries
-// a third of the code, which the instruction caches notice.
-constexpr int kDtF64 = 0, kDtF32 = 1, kDtMixed = 2, kDtF16 = 3;
 
 // Launch 1: analysis of every chunk (chunks by ticket; the next chunk is copied into
 // the warp's one value buffer while the current one is finished).
@@ -971,73 +976,60 @@ analyse_kernel_narrow(const Job *__restrict__ jobs, int njobs, Job single, uint6
     analyse_loop<kDt>(jobs, njobs, single, total_chunks, ctl);
 }
 
-// Stream header, stream length and capacity check of one job (one warp): the length is the
-// header, the size array and the records, whose sizes the analysis added up per group.
-__device__ void finish_job(const Job &job, int lane) {
+// Where a chunk's record starts, relative to the first record, is in its workspace word (the offsets
+// launch, Sec. 3.4's size synchronisation), or, for a single stream of at most kDirectChunks chunks
+// (`direct`), the sum of the sizes before it, added up here.
+__device__ __forceinline__ uint64_t sizes_before(const Job &job, uint64_t c, int lane) {
+    const uint32_t *sizes = reinterpret_cast<const uint32_t *>(job.out + 32);
+    uint32_t part = 0;                            // at most 1024 records of 9235 bytes
+#pragma unroll 4
+    for (uint32_t i = 4u * (uint32_t)lane; i + 4u <= (uint32_t)c; i += 128u) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(sizes + i);
+        part += q.x + q.y + q.z + q.w;
+    }
+    if ((uint32_t)lane < ((uint32_t)c & 3u)) part += sizes[((uint32_t)c & ~3u) + (uint32_t)lane];
+    return __reduce_add_sync(kFull, part);
+}
+constexpr uint64_t kOffsetMask = (1ull << kOffsetBits) - 1ull;
+
+// Stream header, stream length and status of one job (one warp): the length is the header, the size
+// array and the records.
+__device__ void finish_job(const Job &job, bool direct, int lane) {
     const uint64_t nc = job.nchunks;
-    const unsigned long long *gsum = job.flags + 2 * nc + tile_count(nc);
-    uint64_t part = 0;
-    for (uint64_t g = (uint64_t)lane; g < group_count(nc); g += 32) part += gsum[g];
-    const uint64_t total = warp_sum_u64(part);
+    uint64_t total = 0;
+    if (nc > 0) {
+        total = direct ? sizes_before(job, nc - 1u, lane) : (job.flags[nc - 1u] & kOffsetMask);
+        total += reinterpret_cast<const uint32_t *>(job.out + 32)[nc - 1u];
+    }
     if (lane == 0) {
         const uint64_t bytes = 32ull + 4ull * nc + total;
         job.result[0] = bytes;
-        if (bytes > job.out_cap) set_status(job.result, kErrCapacity);
+        job.result[1] = bytes > job.out_cap ? kErrCapacity : kOk;
         uint4 *dst = reinterpret_cast<uint4 *>(job.out);
         dst[0] = make_uint4(0x4E434C46u, 1u | (job.dtype << 8), job.block, 0u);
         dst[1] = make_uint4((uint32_t)job.n, (uint32_t)(job.n >> 32), (uint32_t)nc, (uint32_t)(nc >> 32));
     }
 }
 
-// Where chunk c's record starts, relative to the first record (Sec. 3.4's size synchronisation,
-// from the analysis' sums): the groups before c's group, the tiles of its group before its tile
-// and the chunks of its tile before it.  load_info issues the loads one chunk ahead (every lane:
-// one group sum, two tile sums, two sizes) and keeps the raw words, so that nothing waits on them
-// until resolve_info adds them up a chunk later.  A group's records take < 2^26 bytes and a
-// tile's < 2^20, so their low 32-bit words are the sums; with at most 32 groups before c the
-// records before c take < 2^31 bytes (33 * 4096 records of at most 9235 bytes) and one 32-bit
-// reduction adds the lanes' shares.  Beyond that (more than 128 M values at block 1024) the
-// further groups are read when resolving and added in 64 bits.
-template <bool k64> struct EmitInfo {
-    uint32_t meta_hi;                 // the analysis word's upper half
-    uint32_t dense_lo, dense_hi[1]; // dense-row mask (planes 32 and up: FP64 only)
-    uint32_t g0, t0, t1, s0, s1;      // this lane's group sum, two tile sums, two record sizes
-    uint32_t size;                    // c's record size
+// A chunk to emit: its workspace words and record size, loaded a chunk ahead (unconditionally: a
+// ticket past the last chunk reads the last chunk's, so nothing waits for the loads).
+template <bool kTable, class Mask> struct EmitInfo {
+    const Job *job;
+    uint64_t c;                                   // chunk of the job
+    unsigned long long word;
+    Mask dense;                                   // 32 bits in the narrow kinds' forms
+    uint32_t size;
 };
-
-template <bool k64>
-__device__ __forceinline__ EmitInfo<k64> load_info(const Job &job, uint64_t c, int lane) {
-    const uint64_t nc = job.nchunks;
-    const uint32_t *sizes = reinterpret_cast<const uint32_t *>(job.out + 32);
-    const uint32_t *tsum = reinterpret_cast<const uint32_t *>(job.flags + 2 * nc);   // low words
-    const uint32_t *gsum = tsum + 2 * tile_count(nc);
-    const uint64_t g = c / kGroup, t = c / kTile, tb = g * (kGroup / kTile), cb = t * kTile;
-    EmitInfo<k64> e;
-    e.meta_hi = reinterpret_cast<const uint32_t *>(job.flags + c)[1];
-    if constexpr (k64) {
-        const uint2 d = *reinterpret_cast<const uint2 *>(job.flags + nc + c);
-        e.dense_lo = d.x;
-        e.dense_hi[0] = d.y;
-    } else {
-        e.dense_lo = *reinterpret_cast<const uint32_t *>(job.flags + nc + c);
-    }
-    e.size = sizes[c];
-    e.g0 = (uint64_t)lane < g ? gsum[2 * lane] : 0u;
-    e.t0 = tb + (uint64_t)lane < t ? tsum[2 * (tb + lane)] : 0u;
-    e.t1 = tb + 32u + (uint64_t)lane < t ? tsum[2 * (tb + 32u + lane)] : 0u;
-    e.s0 = cb + (uint64_t)lane < c ? sizes[cb + lane] : 0u;
-    e.s1 = cb + 32u + (uint64_t)lane < c ? sizes[cb + 32u + lane] : 0u;
+template <bool kTable, class Mask>
+__device__ __forceinline__ EmitInfo<kTable, Mask> load_info(const Job *jobs, int njobs, const Job &single, uint64_t t, uint64_t total_chunks) {
+    EmitInfo<kTable, Mask> e;
+    t = t < total_chunks ? t : total_chunks - 1u;
+    e.job = kTable ? jobs + find_job(jobs, njobs, t) : &single;
+    e.c = kTable ? t - e.job->chunk_begin : t;
+    e.word = e.job->flags[e.c];
+    e.dense = *reinterpret_cast<const Mask *>(e.job->flags + e.job->nchunks + e.c);
+    e.size = reinterpret_cast<const uint32_t *>(e.job->out + 32)[e.c];
     return e;
-}
-template <bool k64>
-__device__ __forceinline__ uint64_t resolve_info(const Job &job, uint64_t c, const EmitInfo<k64> &e, int lane) {
-    const uint32_t p = e.g0 + e.t0 + e.t1 + e.s0 + e.s1;
-    const uint64_t g = c / kGroup;
-    if (g <= 32u) return __reduce_add_sync(kFull, p);
-    const unsigned long long *gsum = job.flags + 2 * job.nchunks + tile_count(job.nchunks);
-    uint64_t part = p;
-    for (uint64_t j = 32u + (uint64_t)lane; j < g; j += 32) part += gsum[j];
-    return warp_sum_u64(part);
 }
 
 // Launch 2: the records (chunks by ticket; the next chunk's values are loaded into registers
@@ -1045,22 +1037,23 @@ __device__ __forceinline__ uint64_t resolve_info(const Job &job, uint64_t c, con
 // either-dtype forms).
 template <bool kWide, int kDt>
 __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njobs, const Job &s_single,
-                                          uint64_t total_chunks, Control *ctl, uint8_t *smem) {
+                                          uint64_t total_chunks, bool direct, Control *ctl, uint8_t *smem) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
+    constexpr bool kTable = kDt == kDtMixed;
     constexpr int DL = kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64);
     uint8_t *wbase = smem + warp * EmitLayout<DL, kWide>::kBytes;
     const uint32_t seltab = compact_sel((uint32_t)lane & 15u);
     if (blockIdx.x == 0 && warp == 0) {          // jobs without chunks: header and length only
-        if (jobs == nullptr) {
-            if (s_single.nchunks == 0) finish_job(s_single, lane);
+        if constexpr (!kTable) {
+            if (s_single.nchunks == 0) finish_job(s_single, false, lane);
         } else {
             for (int j0 = 0; j0 < njobs; j0 += 32) {
                 unsigned empty = __ballot_sync(kFull, j0 + lane < njobs && jobs[j0 + lane].nchunks == 0);
                 while (empty) {
                     const int j = j0 + __ffs(empty) - 1;
                     empty &= empty - 1;
-                    finish_job(jobs[j], lane);
+                    finish_job(jobs[j], false, lane);
                 }
             }
         }
@@ -1071,56 +1064,44 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
     typename Traits<DL>::U v[32], vx;
     uint64_t t = ticket_of(take_ticket(ctl, kTicketEmit, lane));
     if (t >= total_chunks) return;
-    uint64_t tn = ticket_of(take_ticket(ctl, kTicketEmit, lane));
-    constexpr bool k64 = kDt == kDtF64 || kDt == kDtMixed;
-    EmitInfo<k64> info;
-    {
-        const Job &j0 = job_of(jobs, njobs, s_single, t);
-        info = load_info<k64>(j0, t - j0.chunk_begin, lane);
-        if constexpr (kPre) load_chunk<DL>(j0, t - j0.chunk_begin, lane, v, vx);
-    }
+    using Mask = typename std::conditional<kPre, uint32_t, unsigned long long>::type;
+    auto info = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
+    if constexpr (kPre) load_chunk<DL>(*info.job, info.c, lane, v, vx);
+    t = ticket_of(take_ticket(ctl, kTicketEmit, lane));          // of the next chunk
     for (;;) {
-        // the ticket after tn, read at the next iteration; tn's workspace words are fetched now
-        const unsigned long long raw = tn < total_chunks ? take_ticket(ctl, kTicketEmit, lane) : 0ull;
-        EmitInfo<k64> next{};
-        if (tn < total_chunks) {
-            if constexpr (!kPre) prefetch_chunk(jobs, njobs, s_single, tn, lane);
-            const Job &jn = job_of(jobs, njobs, s_single, tn);
-            next = load_info<k64>(jn, tn - jn.chunk_begin, lane);
+        // the ticket after t, read at the next iteration; t's workspace words are fetched now
+        const unsigned long long raw = take_ticket(ctl, kTicketEmit, lane);
+        const auto next = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
+        if constexpr (!kPre) {
+            if (t < total_chunks) prefetch_chunk(*next.job, next.c, lane);
         }
-        const Job &job = job_of(jobs, njobs, s_single, t);
-        const uint64_t c = t - job.chunk_begin;
-        const uint64_t rel = resolve_info(job, c, info, lane);
-        if (c == 0) finish_job(job, lane);
-        uint64_t dense = info.dense_lo;
-        if constexpr (k64) dense |= (uint64_t)info.dense_hi[0] << 32;
+        const Job &job = *info.job;
+        const bool dir = !kTable && direct;
+        const uint64_t rel = dir ? sizes_before(job, info.c, lane) : (info.word & kOffsetMask);
+        if (info.c == 0) finish_job(job, dir, lane);
         auto load_next = [&]() {
             if constexpr (kPre) {
-                if (tn < total_chunks) {
-                    const Job &jn = job_of(jobs, njobs, s_single, tn);
-                    load_chunk<DL>(jn, tn - jn.chunk_begin, lane, v, vx);
-                }
+                if (t < total_chunks) load_chunk<DL>(*next.job, next.c, lane, v, vx);
             }
         };
         if constexpr (kPre) {
-            emit_chunk<DL, kWide, true>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, v, vx, load_next);
+            emit_chunk<DL, kWide, true>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, v, vx, load_next);
         } else if constexpr (kDt == kDtF64) {
             uint64_t u[32], ux;
-            emit_chunk<kD64, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD64, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
         } else if (job.dtype == 0) {
             uint64_t u[32], ux;
-            emit_chunk<kD64, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD64, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
         } else if (job.dtype == 1) {
             uint32_t u[32], ux;
-            emit_chunk<kD32, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD32, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
         } else {
             uint16_t u[32], ux;
-            emit_chunk<kD16, kWide, false>(job, c, wbase, seltab, lane, info.meta_hi, dense, info.size, rel, u, ux, load_next);
+            emit_chunk<kD16, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
         }
         __syncwarp();
-        if (tn >= total_chunks) break;
-        t = tn;
-        tn = ticket_of(raw);
+        if (t >= total_chunks) break;
+        t = ticket_of(raw);
         info = next;
     }
     if (lane == 0) bulk_wait();
@@ -1129,24 +1110,24 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
 // FP64 and either-dtype forms (up to 128 registers, 16 warps per SM)
 template <bool kWide, int kDt>
 __global__ void __launch_bounds__(32 * kMaxCompressWarps, 1)
-emit_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
+emit_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, bool direct, Control *ctl) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ Job s_single;
     if (threadIdx.x == 0) s_single = single;
     __syncthreads();
-    emit_loop<kWide, kDt>(jobs, njobs, s_single, total_chunks, ctl, smem);
+    emit_loop<kWide, kDt>(jobs, njobs, s_single, total_chunks, direct, ctl, smem);
 }
 
 // FP32 and FP16 forms: held to 96 registers (FP32 needs 96 without spilling), so that 20 warps
 // fit an SM
 template <bool kWide, int kDt>
 __global__ void __maxnreg__(96)
-emit_kernel_narrow(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
+emit_kernel_narrow(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, bool direct, Control *ctl) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ Job s_single;
     if (threadIdx.x == 0) s_single = single;
     __syncthreads();
-    emit_loop<kWide, kDt>(jobs, njobs, s_single, total_chunks, ctl, smem);
+    emit_loop<kWide, kDt>(jobs, njobs, s_single, total_chunks, direct, ctl, smem);
 }
 
 namespace {
@@ -1163,17 +1144,17 @@ void launch_analyse(const Job *d_jobs, int njobs, const Job &single, uint64_t to
     kernel<<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
 }
 template <bool kWide, int kDt>
-void launch_emit(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, Control *ctl,
-                 cudaStream_t stream) {
+void launch_emit(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, bool direct,
+                 Control *ctl, cudaStream_t stream) {
     const int w = g_cta_warps[0], smem = w * (int)EmitLayout<kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64), kWide>::kBytes;
     if constexpr (kDt == kDtF32 || kDt == kDtF16) {
         const int g = persistent_grid_of(reinterpret_cast<const void *>(emit_kernel_narrow<kWide, kDt>), w, smem,
                                          g_ctas_per_sm[0], total_chunks);
-        emit_kernel_narrow<kWide, kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
+        emit_kernel_narrow<kWide, kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, direct, ctl);
     } else {
         const int g = persistent_grid_of(reinterpret_cast<const void *>(emit_kernel<kWide, kDt>), w, smem,
                                          g_ctas_per_sm[0], total_chunks);
-        emit_kernel<kWide, kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
+        emit_kernel<kWide, kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, direct, ctl);
     }
 }
 
@@ -1229,14 +1210,17 @@ cudaError_t launch_compress(const Job *d_jobs, int njobs, const Job &single, uin
         else if (kind == kDtF16) launch_analyse<kDtF16>(d_jobs, njobs, single, total_chunks, ctl, stream);
         else launch_analyse<kDtMixed>(d_jobs, njobs, single, total_chunks, ctl, stream);
     }
+    // a stream of a few chunks: each emit warp adds up the sizes before its record itself
+    const bool direct = d_jobs == nullptr && single.nchunks <= kDirectChunks;
+    if (!direct) launch_offsets(d_jobs, njobs, single, kOffsetsOfOutput, ctl, stream);
     {   // the emit launch also writes the header and length of every job, chunks or none
-        if (wide && kind == kDtF64) launch_emit<true, kDtF64>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else if (wide && kind == kDtF32) launch_emit<true, kDtF32>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else if (wide) launch_emit<true, kDtF16>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else if (kind == kDtF64) launch_emit<false, kDtF64>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else if (kind == kDtF32) launch_emit<false, kDtF32>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else if (kind == kDtF16) launch_emit<false, kDtF16>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else launch_emit<false, kDtMixed>(d_jobs, njobs, single, total_chunks, ctl, stream);
+        if (wide && kind == kDtF64) launch_emit<true, kDtF64>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
+        else if (wide && kind == kDtF32) launch_emit<true, kDtF32>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
+        else if (wide) launch_emit<true, kDtF16>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
+        else if (kind == kDtF64) launch_emit<false, kDtF64>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
+        else if (kind == kDtF32) launch_emit<false, kDtF32>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
+        else if (kind == kDtF16) launch_emit<false, kDtF16>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
+        else launch_emit<false, kDtMixed>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
     }
     return cudaGetLastError();
 }

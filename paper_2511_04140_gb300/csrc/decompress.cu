@@ -542,21 +542,29 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, uint8_t *smem, uint3
 // adds up every size before its share first (at most 152 CTAs reading at most the whole array, from
 // L2), then scans its share 1024 chunks at a time, so no CTA waits for another.
 __global__ void __launch_bounds__(1024)
-offsets_kernel(const Job *__restrict__ jobs, Job single, uint32_t parts) {
+offsets_kernel(const Job *__restrict__ jobs, Job single, uint32_t parts, int which, Control *ctl) {
     __shared__ uint64_t warp_sums[33];
     const Job &job = (jobs == nullptr) ? single : jobs[blockIdx.x / parts];
     const uint32_t part = blockIdx.x % parts;
     const uint64_t nc = job.nchunks;
+    if (which == kOffsetsOfInput && threadIdx.x == 0) {          // ready for the decode
+        if (blockIdx.x == 0) *ctl = Control{};
+        if (part == 0) {
+            job.result[0] = job.n;
+            job.result[1] = kOk;
+        }
+    }
     const uint64_t share = ((nc + parts - 1) / parts + 1023u) & ~1023ull;
     const uint64_t begin = part * share, end = begin + share < nc ? begin + share : nc;
     if (begin >= nc) return;
-    const uint32_t *sizes = reinterpret_cast<const uint32_t *>(job.in + 32);      // 16-byte aligned
+    // 16-byte aligned
+    const uint32_t *sizes = reinterpret_cast<const uint32_t *>((which == kOffsetsOfInput ? job.in : job.out) + 32);
     uint64_t carry = 0;
     if (begin > 0) {                              // begin is a multiple of 1024
         const uint4 *q = reinterpret_cast<const uint4 *>(sizes);
         uint64_t sum = 0;
         for (uint64_t i = threadIdx.x; i < begin / 4u; i += 1024u) {
-            const uint4 x = __ldg(q + i);
+            const uint4 x = q[i];
             sum += (uint64_t)x.x + x.y + x.z + x.w;
         }
         (void)block_exclusive_scan(sum, carry, warp_sums);
@@ -565,7 +573,10 @@ offsets_kernel(const Job *__restrict__ jobs, Job single, uint32_t parts) {
         const uint64_t c = b + threadIdx.x;
         uint64_t total;
         const uint64_t ex = block_exclusive_scan(c < end ? sizes[c] : 0u, total, warp_sums);
-        if (c < end) job.flags[c] = carry + ex;
+        if (c < end) {
+            if (which == kOffsetsOfInput) job.flags[c] = carry + ex;
+            else job.flags[c] = ((job.flags[c] >> kOffsetBits) << kOffsetBits) | (carry + ex);
+        }
         carry += total;
     }
 }
@@ -591,12 +602,6 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
     if (threadIdx.x == 0) s_single = single;
     if (threadIdx.x < kZeroBytes / 16u) reinterpret_cast<uint4 *>(smem)[threadIdx.x] = make_uint4(0, 0, 0, 0);
     __syncthreads();
-    const uint64_t gw = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-    const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    for (uint64_t j = gw; j < (uint64_t)((jobs != nullptr) ? njobs : 1); j += nw) {
-        const Job &jb = (jobs != nullptr) ? jobs[j] : s_single;
-        if (lane == 0) jb.result[0] = jb.n;
-    }
     // chunk tickets two deep: while one chunk is decoded the next one's record is fetched, and the
     // ticket of the one after that is on its way (read, and its position loads issued, when this
     // chunk is done)
@@ -682,17 +687,17 @@ void launch_decode(const Job *d_jobs, int njobs, const Job &single, uint64_t tot
 }  // namespace
 
 // One CTA per 1024 chunks up to 152 for a single stream; a table's many jobs get one each.
-static void launch_offsets(const Job *d_jobs, int njobs, const Job &single, cudaStream_t stream) {
+void launch_offsets(const Job *d_jobs, int njobs, const Job &single, int which, Control *ctl, cudaStream_t stream) {
     uint32_t parts = 1;
     if (d_jobs == nullptr) {
         const uint64_t steps = (single.nchunks + 1023u) / 1024u;
         parts = steps < 1u ? 1u : (steps > 152u ? 152u : (uint32_t)steps);
     }
-    offsets_kernel<<<(unsigned)njobs * parts, 1024, 0, stream>>>(d_jobs, single, parts);
+    offsets_kernel<<<(unsigned)njobs * parts, 1024, 0, stream>>>(d_jobs, single, parts, which, ctl);
 }
 
 cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cudaStream_t stream) {
-    launch_offsets(nullptr, 1, single, stream);
+    launch_offsets(nullptr, 1, single, kOffsetsOfInput, ctl, stream);
     if (single.nchunks > 0) {
         if (single.dtype == 0) launch_decode<kDtF64, true>(nullptr, 1, single, single.nchunks, ctl, stream);
         else if (single.dtype == 1) launch_decode<kDtF32, true>(nullptr, 1, single, single.nchunks, ctl, stream);
@@ -704,7 +709,7 @@ cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cud
 
 cudaError_t launch_decompress(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks,
                               Control *ctl, cudaStream_t stream) {
-    launch_offsets(d_jobs, njobs, single, stream);
+    launch_offsets(d_jobs, njobs, single, kOffsetsOfInput, ctl, stream);
     if (d_jobs != nullptr) launch_decode<kDtMixed>(d_jobs, njobs, single, total_chunks, ctl, stream);
     else if (single.dtype == 0) launch_decode<kDtF64>(d_jobs, njobs, single, total_chunks, ctl, stream);
     else if (single.dtype == 1) launch_decode<kDtF32>(d_jobs, njobs, single, total_chunks, ctl, stream);

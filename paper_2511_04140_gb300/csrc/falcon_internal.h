@@ -41,7 +41,8 @@ struct Job {
 // row dense, Elf's trial-and-error decimal place).  All write the same record layout.
 enum : uint32_t { kVariantFalcon = 0, kVariantSparse = 1, kVariantDense = 2, kVariantElf = 3 };
 
-// Per-launch control block at the start of the workspace (zeroed before each set of launches):
+// Per-launch control block at the start of the workspace (zero before the analysis: the callers of
+// launch_compress reset it; reset by the offsets launch for decompression):
 // the chunk tickets of the persistent kernels.  A warp takes its next chunk with one atomic
 // add on its kernel's counter (analysis, emit, decode), so warps that met cheaper chunks take
 // more of them and a launch ends with its average warp, not its unluckiest one.
@@ -56,10 +57,10 @@ static_assert(sizeof(Control) == 64, "control block is 64 bytes");
 
 constexpr size_t kControlBytes = 256;   // control block region (keeps flags 256-aligned)
 
-// Workspace words of a job: compression keeps two per chunk (the analysis results and the
-// dense-row mask), then one per 64-chunk tile and one per 4096-chunk group (the sums of their
-// record sizes, which the analysis adds up); decompression keeps the record offset of each chunk
-// in the first words (the aggregate its chunk sums in the next).
+// Workspace words of a job: compression keeps two per chunk (the analysis results with the record
+// offset, and the dense-row mask); decompression keeps the record offset of each chunk in the first
+// words (the aggregate its chunk sums in the next).  The size also counts a word per 64-chunk tile
+// and per 4096-chunk group, which nothing uses now (callers' workspaces keep their size).
 // value kinds of the stream format: 0 FP64, 1 FP32, 2 FP16 (binary16)
 inline bool dtype_valid(int dtype) { return dtype >= 0 && dtype <= 2; }
 inline size_t dtype_bytes(int dtype) { return dtype == 0 ? 8 : (dtype == 1 ? 4 : 2); }
@@ -74,6 +75,12 @@ __host__ __device__ constexpr uint64_t workspace_words(uint64_t nchunks) {
 
 cudaError_t launch_compress(const Job *d_jobs, int njobs, const Job &single,
                             uint64_t total_chunks, Control *ctl, cudaStream_t stream);
+// Record offsets (exclusive prefix of the size array) of every job into its first workspace words:
+// of the streams in `in` (decompression, which also resets the control block and the results), or of
+// the streams being written to `out` (compression: into the low kOffsetBits of the analysis' words).
+enum { kOffsetsOfInput = 0, kOffsetsOfOutput = 1 };
+constexpr int kOffsetBits = 47;
+void launch_offsets(const Job *d_jobs, int njobs, const Job &single, int which, Control *ctl, cudaStream_t stream);
 cudaError_t launch_decompress(const Job *d_jobs, int njobs, const Job &single,
                               uint64_t total_chunks, Control *ctl, cudaStream_t stream);
 // analytics on compressed data: the decode without the stores, then the aggregate into
