@@ -237,23 +237,44 @@ __device__ __forceinline__ uint64_t test_g(uint64_t u, const Case1At &c, bool &o
     ok &= pass;
     return (hi >> 31) ? 0ull - N : N;
 }
+// the same for |g| < 10^8 and 5^a < 2^32
+__device__ __forceinline__ uint64_t test_g(uint64_t u, const Case1At &c, const Case1Narrow &q, bool &ok) {
+    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
+    const uint32_t N = case1_n_narrow(hi, lo, q);
+    const int F = c.f0 - (int)((hi >> 20) & 0x7FFu);
+    const uint32_t p5 = (uint32_t)c.p5, lim = p5 >> 1;
+    bool pass;
+    if (F > 62) {
+        pass = q_test(u, c.a);
+    } else {                                      // F >= 26: |v 10^a| < 2^27 and m 5^a >= 2^52
+        const uint64_t P = (uint64_t)lo * p5 + ((uint64_t)(((hi & 0xFFFFFu) | 0x100000u) * p5) << 32);
+        pass = P - ((uint64_t)N << F) + lim <= 2u * lim;
+    }
+    ok &= pass;
+    const uint32_t s = (uint32_t)((int32_t)hi >> 31);
+    return (uint64_t)(int64_t)(int32_t)((N ^ s) - s);
+}
 template <class U> __device__ __forceinline__ U test_g_narrow(U u, int a, bool &ok) {
     ok &= q_test(u, a);
     return case1_g(u, a);
 }
 
 // all_pass that leaves every value's g in the staging buffer in its place (rolled: small code).
-template <int D>
+// kNarrow (FP64): |v 10^a| < 10^8 for every value.
+template <int D, bool kNarrow = false>
 __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, int a) {
     using U = typename Traits<D>::U;
     constexpr int UN = Traits<D>::UNITS, PER = 32 / UN;
     bool ok = true;
     Case1At c{};
     if constexpr (D == kD64) c = case1_at(a);
+    Case1Narrow cn{};
+    if constexpr (kNarrow) cn = case1_narrow_of(a);
     auto one = [&](U u, uint32_t i) {
         bool pass = true;
         U g;
-        if constexpr (D == kD64) g = test_g(u, c, pass);
+        if constexpr (kNarrow) g = test_g(u, c, cn, pass);
+        else if constexpr (D == kD64) g = test_g(u, c, pass);
         else g = test_g_narrow(u, a, pass);
         ok &= pass || i >= m;
         return g;
@@ -442,7 +463,8 @@ __device__ __forceinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int
         alpha = alpha_bound<D>(buf, lane, m, atop);
         if (alpha < 0) return -1;
         if constexpr (D == kD64) {               // no value can stop early (Thm 4)
-            if (pass_to_g<D>(buf, lane, m, alpha)) return alpha;
+            const bool narrow = alpha + e_max + 1 <= kNarrowBeta && alpha <= 13;
+            if (narrow ? pass_to_g<D, true>(buf, lane, m, alpha) : pass_to_g<D>(buf, lane, m, alpha)) return alpha;
             __syncwarp();
             stage_values_async<D>(src, m, buf, lane);        // the values again
             cp_async_commit();
@@ -793,23 +815,6 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
         return;
     }
 
-    // ---- G (Eq. 4) and its deltas (Eq. 5) -------------------------------------------------------
-    if constexpr (!kPre) load_chunk<D>(job, c, lane, v, vx);
-    if (alpha_byte != T::A_SENT) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = case1_g(v[k], alpha_byte);
-        vx = case1_g(vx, alpha_byte);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = zigzag(v[k]);
-        vx = zigzag(vx);
-    }
-    const U z1 = shfl_x(v[0], 0);
-    U nxt = shfl_down_x(v[0], 1);
-    if (lane == 31) nxt = vx;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = (U)((k < 31 ? v[k + 1] : nxt) - v[k]);
-
     // ---- planes (Sec. 3.3) and record -----------------------------------------------------------
     // The zigzag is done on the planes: plane p of Z is plane p - 1 of the deltas XOR their sign
     // plane, plane 0 is the sign plane (one XOR per plane instead of five operations per value).
@@ -824,6 +829,7 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     uint8_t *slots = buf + L::kRec - (32u - L::kRows) * 128u;         // plane p of a half: 128 (31 - p) further
     uint8_t *dst = slots + 31 * 128 + 4 * lane;                      // plane 0; plane p lies 128 p below
     uint32_t pos = sh + hdr;                      // next record byte in the buffer
+    U z1;
     auto header = [&]() {
         // record header: byte `lane` (branch-free: every lane computes its byte, lanes < hdr store it)
         const int i = lane;
@@ -836,19 +842,49 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     uint32_t sgn = 0;
     const bool two = D == kD64 && w > 32;
     constexpr int R = T::W < 32 ? T::W : 32;
-    uint32_t a[32];
-    if constexpr (D == kD64) {
-        if (two) {
+    uint32_t a[32];                               // the deltas' low words, transposed below
+    // G (Eq. 4) and its deltas (Eq. 5)
+    if constexpr (!kPre) load_chunk<D>(job, c, lane, v, vx);
+    if (D == kD64 && alpha_byte != T::A_SENT && beta_hat <= kNarrowBeta) {
+        // Case 1 with |g| < 10^8: 32-bit arithmetic throughout (and w <= 32)
+        const Case1Narrow q = case1_narrow_of(alpha_byte);
+        uint32_t g[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) a[j] = (uint32_t)(v[j ^ 7] >> 32);
-            transpose32(a);
-            sgn = a[31];
+        for (int k = 0; k < 32; ++k) g[k] = case1_g_narrow((uint64_t)v[k], q);
+        const uint32_t gx = case1_g_narrow((uint64_t)vx, q);
+        z1 = (U)(int64_t)(int32_t)__shfl_sync(kFull, g[0], 0);
+        uint32_t nxt = __shfl_down_sync(kFull, g[0], 1);
+        if (lane == 31) nxt = gx;
 #pragma unroll
-            for (int p = 0; p < 31; ++p) *reinterpret_cast<uint32_t *>(dst - (p + 1) * 128) = a[p] ^ sgn;
+        for (int j = 0; j < 32; ++j) a[j] = ((j ^ 7) < 31 ? g[(j ^ 7) < 31 ? (j ^ 7) + 1 : 0] : nxt) - g[j ^ 7];
+    } else {
+        if (alpha_byte != T::A_SENT) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) v[k] = case1_g(v[k], alpha_byte);
+            vx = case1_g(vx, alpha_byte);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) v[k] = zigzag(v[k]);
+            vx = zigzag(vx);
         }
-    }
+        z1 = shfl_x(v[0], 0);
+        U nxt = shfl_down_x(v[0], 1);
+        if (lane == 31) nxt = vx;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) a[j] = (uint32_t)v[j ^ 7];
+        for (int k = 0; k < 32; ++k) v[k] = (U)((k < 31 ? v[k + 1] : nxt) - v[k]);
+        if constexpr (D == kD64) {
+            if (two) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) a[j] = (uint32_t)(v[j ^ 7] >> 32);
+                transpose32(a);
+                sgn = a[31];
+#pragma unroll
+                for (int p = 0; p < 31; ++p) *reinterpret_cast<uint32_t *>(dst - (p + 1) * 128) = a[p] ^ sgn;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 32; ++j) a[j] = (uint32_t)v[j ^ 7];
+    }
     transpose32(a);
     if (!two) sgn = a[R - 1];
     if (two) *reinterpret_cast<uint32_t *>(dst) = a[31] ^ sgn;

@@ -483,6 +483,32 @@ __device__ __forceinline__ uint64_t case1_g(uint64_t u, int a) {
     const uint64_t N = case1_round(m, FALCON_POW5_NORM[a], -(E + a) + 10 - (int)FALCON_LOG2_POW5[a]);
     return (u >> 63) ? (0ull - N) : N;
 }
+// The same for values with |g| < 10^8 (beta_hat <= kNarrowBeta): one 32-bit high product.  The top
+// words of m and 5^a, both normalised, give t >= 2^30 within three of X 2^sh, and X < 10^8 makes
+// sh >= 4, so t 2^-sh is within 3/16 of X, itself within X 2^-53 of g.
+constexpr int kNarrowBeta = 8;
+struct Case1Narrow {
+    uint32_t norm;                                // top word of 5^a normalised
+    int c;                                        // sh - 1 = c - exponent field
+};
+__device__ __forceinline__ Case1Narrow case1_narrow_of(int a) {
+    return {(uint32_t)(FALCON_POW5_NORM[a] >> 32), 1075 - a + 10 - (int)FALCON_LOG2_POW5[a] - 32 - 1};
+}
+// shifts that give 0 past 31 (a value of +0 has the largest)
+__device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t n) {
+    uint32_t r;
+    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
+__device__ __forceinline__ uint32_t case1_n_narrow(uint32_t hi, uint32_t lo, const Case1Narrow &q) {      // |g|
+    const uint32_t top = __funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 11);
+    const uint32_t sh = (uint32_t)(q.c - (int)((hi >> 20) & 0x7FFu));
+    return (shr_clamp(__umulhi(top, q.norm), sh) + 1u) >> 1;
+}
+__device__ __forceinline__ uint32_t case1_g_narrow(uint64_t u, const Case1Narrow &q) {
+    const uint32_t hi = (uint32_t)(u >> 32), s = (uint32_t)((int32_t)hi >> 31);
+    return (case1_n_narrow(hi, (uint32_t)u, q) ^ s) - s;
+}
 __device__ __forceinline__ uint32_t case1_g(uint32_t u, int a) {
     const uint32_t au = u & 0x7FFFFFFFu;
     if (au == 0) return 0;
