@@ -254,34 +254,83 @@ __device__ __forceinline__ uint64_t test_g(uint64_t u, const Case1At &c, const C
     const uint32_t s = (uint32_t)((int32_t)hi >> 31);
     return (uint64_t)(int64_t)(int32_t)((N ^ s) - s);
 }
-template <class U> __device__ __forceinline__ U test_g_narrow(U u, int a, bool &ok) {
-    ok &= q_test(u, a);
-    return case1_g(u, a);
+// FP32: the round trip |m 5^a - g 2^F| <= 5^a / 2 as in q_test (past F = 62 only +0 passes)
+__device__ __forceinline__ uint32_t test_g(uint32_t u, const Case1F32 &q, bool &ok) {
+    const uint32_t N = case1_n(u, q), e = (u >> 23) & 0xFFu;
+    const int F = q.f0 - (int)e;
+    const uint64_t P = (uint64_t)((u & 0x007FFFFFu) | 0x00800000u) * q.p5;
+    const uint32_t lim = q.p5 >> 1;
+    const bool near = P - ((uint64_t)N << (F & 63)) + lim <= 2u * lim;
+    ok &= F <= 0 || (F > 62 ? (u << 1) == 0u : near);
+    const uint32_t s = (uint32_t)((int32_t)u >> 31);
+    return (N ^ s) - s;
+}
+__device__ __forceinline__ uint16_t test_g(uint16_t u, const Scale16 &q, bool &ok) {
+    bool rt;
+    (void)alg2_step_f16(u, q, rt);
+    ok &= rt;
+    return case1_g(u, q);
 }
 
+// FP32 chunks at beta_hat = 7 (R14) and FP16 chunks at beta_hat = 3 (R18): Alg. 2, value by
+// value, stops at the first decimal place where eps <= mu passes, and if the round trip fails
+// there the value is an exception.  That can happen below a value's own decimal place k only if
+// |v| 10^k >= 2^(p-1) / 1.5 (p = 24 or 11 significand bits): with d / 10^k its shortest decimal,
+// v 10^a (a < k) lies at least 10^-(k-a) - |v| 10^a 2^-p from every integer, more than
+// mu = |v 10^a| 2^-(p-1) below that bound (checked exhaustively over every decimal below it).
+// k <= alpha, so a value can stop early only if |v| 10^alpha reaches the bound.  FP32 tests
+// 3 |v| 10^alpha >= 2^23 (half the bound, as a margin: the bound was checked exhaustively only
+// up to that point); FP16 tests the bound itself, 3 |v| 10^alpha >= 2^11, checked over all
+// 65,536 patterns.  Only those values go through Alg. 2, and none when v_max is below.
+__device__ __forceinline__ bool may_stop_early(uint32_t u, int a) {
+    const uint32_t au = u & 0x7FFFFFFFu;
+    if (au == 0) return false;
+    if (au < 0x00800000u) return true;          // subnormal: take the full test
+    const int E = (int)(au >> 23) - 150;
+    const uint64_t p = 3ull * ((au & 0x007FFFFFu) | 0x00800000u) * FALCON_POW5[a];   // < 2^50
+    const int s = 23 - E - a;                    // 3 m 5^a 2^(E+a) >= 2^23  <=>  p >= 2^s
+    return s <= 0 || (s < 50 && p >= (1ull << s));
+}
+__device__ __forceinline__ bool may_stop_early(uint16_t u, int a) {
+    const uint32_t au = u & 0x7FFFu;
+    if (au == 0) return false;
+    if (au < 0x0400u) return true;
+    const int E = (int)(au >> 10) - 25;
+    const uint32_t p = 3u * ((au & 0x3FFu) | 0x400u) * (uint32_t)FALCON_POW5[a];     // < 2^22
+    const int s = 11 - E - a;                    // 3 m 5^a 2^(E+a) >= 2^11  <=>  p >= 2^s
+    return s <= 0 || (s < 32 && p >= (1u << s));
+}
+__device__ __forceinline__ int first_pass(uint32_t u, int atop) { return first_pass_f32(u, atop); }
+__device__ __forceinline__ int first_pass(uint16_t u, int atop) { return first_pass_f16(u, atop); }
+
 // all_pass that leaves every value's g in the staging buffer in its place (rolled: small code).
-// kNarrow (FP64): |v 10^a| < 10^8 for every value.
+// kNarrow (FP64): |v 10^a| < 10^8 for every value.  With `watch` (FP32, FP16 at the largest beta_hat)
+// `stop` tells whether some value stops early, which counts when all pass.
 template <int D, bool kNarrow = false>
-__device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, int a) {
+__device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, int a, bool watch, bool &stop) {
     using U = typename Traits<D>::U;
     constexpr int UN = Traits<D>::UNITS, PER = 32 / UN;
-    bool ok = true;
+    bool ok = true, early = false;
     Case1At c{};
     if constexpr (D == kD64) c = case1_at(a);
     Case1Narrow cn{};
     if constexpr (kNarrow) cn = case1_narrow_of(a);
-    auto one = [&](U u, uint32_t i) {
-        bool pass = true;
-        U g;
-        if constexpr (kNarrow) g = test_g(u, c, cn, pass);
-        else if constexpr (D == kD64) g = test_g(u, c, pass);
-        else g = test_g_narrow(u, a, pass);
-        ok &= pass || i >= m;
-        return g;
+    Case1F32 cf{};
+    if constexpr (D == kD32) cf = case1_f32_of(a);
+    Scale16 ch{};
+    if constexpr (D == kD16) ch = scale16_of(a);
+    auto one = [&](U u) {
+        if constexpr (D != kD64) {
+            if (watch && may_stop_early(u, a)) early |= first_pass(u, a) < 0;
+        }
+        if constexpr (kNarrow) return test_g(u, c, cn, ok);
+        else if constexpr (D == kD64) return test_g(u, c, ok);
+        else if constexpr (D == kD32) return test_g(u, cf, ok);
+        else return test_g(u, ch, ok);
     };
     if (m > 1024u && lane == 31) {
         U *e = reinterpret_cast<U *>(buf + phys_elem_byte<D>(1024));
-        *e = one(*e, 1024);
+        *e = one(*e);
     }
 #pragma unroll 1
     for (int u = 0; u < UN; ++u) {
@@ -289,9 +338,10 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
         union { uint4 w; U e[PER]; } x;
         x.w = *q;
 #pragma unroll
-        for (int k = 0; k < PER; ++k) x.e[k] = one(x.e[k], 32u * lane + u * PER + k);
+        for (int k = 0; k < PER; ++k) x.e[k] = one(x.e[k]);
         *q = x.w;
     }
+    stop = __any_sync(kFull, early);
     return __all_sync(kFull, ok);
 }
 
@@ -333,53 +383,6 @@ __device__ __forceinline__ int alpha_above(const uint8_t *buf, int lane, uint32_
         if (hi_ok && lo >= hi) return hi;
         a = (lo + hi) >> 1;                     // lo <= a < hi once atop has passed
     }
-}
-
-// FP32 chunks at beta_hat = 7 (R14) and FP16 chunks at beta_hat = 3 (R18): Alg. 2, value by
-// value, stops at the first decimal place where eps <= mu passes, and if the round trip fails
-// there the value is an exception.  That can happen below a value's own decimal place k only if
-// |v| 10^k >= 2^(p-1) / 1.5 (p = 24 or 11 significand bits): with d / 10^k its shortest decimal,
-// v 10^a (a < k) lies at least 10^-(k-a) - |v| 10^a 2^-p from every integer, more than
-// mu = |v 10^a| 2^-(p-1) below that bound (checked exhaustively over every decimal below it).
-// k <= alpha, so a value can stop early only if |v| 10^alpha reaches the bound.  FP32 tests
-// 3 |v| 10^alpha >= 2^23 (half the bound, as a margin: the bound was checked exhaustively only
-// up to that point); FP16 tests the bound itself, 3 |v| 10^alpha >= 2^11, checked over all
-// 65,536 patterns.  Only those values go through Alg. 2, and none when v_max is below.
-__device__ __forceinline__ bool may_stop_early(uint32_t u, int a) {
-    const uint32_t au = u & 0x7FFFFFFFu;
-    if (au == 0) return false;
-    if (au < 0x00800000u) return true;          // subnormal: take the full test
-    const int E = (int)(au >> 23) - 150;
-    const uint64_t p = 3ull * ((au & 0x007FFFFFu) | 0x00800000u) * FALCON_POW5[a];   // < 2^50
-    const int s = 23 - E - a;                    // 3 m 5^a 2^(E+a) >= 2^23  <=>  p >= 2^s
-    return s <= 0 || (s < 50 && p >= (1ull << s));
-}
-__device__ __forceinline__ bool may_stop_early(uint16_t u, int a) {
-    const uint32_t au = u & 0x7FFFu;
-    if (au == 0) return false;
-    if (au < 0x0400u) return true;
-    const int E = (int)(au >> 10) - 25;
-    const uint32_t p = 3u * ((au & 0x3FFu) | 0x400u) * (uint32_t)FALCON_POW5[a];     // < 2^22
-    const int s = 11 - E - a;                    // 3 m 5^a 2^(E+a) >= 2^11  <=>  p >= 2^s
-    return s <= 0 || (s < 32 && p >= (1u << s));
-}
-__device__ __forceinline__ int first_pass(uint32_t u, int atop) { return first_pass_f32(u, atop); }
-__device__ __forceinline__ int first_pass(uint16_t u, int atop) { return first_pass_f16(u, atop); }
-
-// True if some value of the chunk stops early (the chunk then takes Case 2); alpha is the
-// search's alpha_max, at which every value round-trips.
-template <int D>
-__device__ __forceinline__ bool early_stop(const uint8_t *buf, int lane, uint32_t m, typename Traits<D>::U vx,
-                                           bool has_vx, typename Traits<D>::U vmax, int alpha) {
-    if (!may_stop_early(vmax, alpha)) return false;
-    bool bad = has_vx && may_stop_early(vx, alpha) && first_pass(vx, alpha) < 0;
-#pragma unroll 1
-    for (int k = 0; k < 32; ++k) {
-        if (32u * lane + k >= m) break;
-        const typename Traits<D>::U u = lane_value<D>(buf, lane, k);
-        if (may_stop_early(u, alpha)) bad |= first_pass(u, alpha) < 0;
-    }
-    return __any_sync(kFull, bad);
 }
 
 // Fal._Elf's decimal place of one value (Sec. 1's trial and error, ablation of Sec. 5.4.2):
@@ -455,33 +458,37 @@ __device__ __forceinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int
     using U = typename T::U;
     const bool has_vx = m > 1024u && lane == 31;
     const U vx = has_vx ? read_elem<D>(buf, 1024) : (U)0;
-    int alpha;
-    if (elf) {
-        alpha = alpha_elf<D>(buf, lane, m, vx, has_vx, e_max);
-        if (alpha < 0) return -1;
-    } else {
-        alpha = alpha_bound<D>(buf, lane, m, atop);
-        if (alpha < 0) return -1;
-        if constexpr (D == kD64) {               // no value can stop early (Thm 4)
-            const bool narrow = alpha + e_max + 1 <= kNarrowBeta && alpha <= 13;
-            if (narrow ? pass_to_g<D, true>(buf, lane, m, alpha) : pass_to_g<D>(buf, lane, m, alpha)) return alpha;
-            __syncwarp();
-            stage_values_async<D>(src, m, buf, lane);        // the values again
-            cp_async_commit();
-            cp_async_wait_none();
-            __syncwarp();
-            pad_values<D>(buf, m, lane);
-            alpha = alpha_above<D>(buf, lane, m, vx, alpha, atop);
-        } else {
-            if (!all_pass<D>(buf, lane, m, vx, alpha)) alpha = alpha_above<D>(buf, lane, m, vx, alpha, atop);
-            // FP32 (R14), FP16 (R18): below beta_hat = B_MAX no value can stop early
-            // (see early_stop), so Alg. 2 value by value gives the same alpha_max
-            if (alpha >= 0 && alpha + e_max + 1 == T::B_MAX && early_stop<D>(buf, lane, m, vx, has_vx, vmax, alpha))
-                alpha = -1;
+    auto restage = [&]() {                        // the values again
+        __syncwarp();
+        stage_values_async<D>(src, m, buf, lane);
+        cp_async_commit();
+        cp_async_wait_none();
+        __syncwarp();
+        pad_values<D>(buf, m, lane);
+    };
+    // FP32 (R14), FP16 (R18): below beta_hat = B_MAX no value can stop early, so Alg. 2 value by value
+    // gives the same alpha_max.  FP64: no value can (Thm 4).
+    bool stop = false;
+    auto pass = [&](int a) {
+        bool watch = false;
+        if constexpr (D != kD64) watch = !elf && a + e_max + 1 == T::B_MAX && may_stop_early(vmax, a);
+        if constexpr (D == kD64) {
+            if (a + e_max + 1 <= kNarrowBeta && a <= 13) return pass_to_g<D, true>(buf, lane, m, a, false, stop);
         }
+        return pass_to_g<D>(buf, lane, m, a, watch, stop);
+    };
+    int alpha = elf ? alpha_elf<D>(buf, lane, m, vx, has_vx, e_max) : alpha_bound<D>(buf, lane, m, atop);
+    if (alpha < 0) return -1;
+    if (!pass(alpha)) {
+        restage();
+        alpha = alpha_above<D>(buf, lane, m, vx, alpha, atop);
         if (alpha < 0) return -1;
+        (void)pass(alpha);
     }
-    (void)pass_to_g<D>(buf, lane, m, alpha);
+    if (stop) {
+        restage();
+        return -1;
+    }
     return alpha;
 }
 

@@ -76,8 +76,19 @@ __device__ __forceinline__ uint32_t expand_sel(uint32_t n) {
 __device__ __forceinline__ double div_pow10(int64_t g, int a) {
     return __ddiv_rn(__ll2double_rn(g), __longlong_as_double((long long)FALCON_P10_F64[a - FALCON_P10_F64_LO]));
 }
-__device__ __forceinline__ float div_pow10(int32_t g, int a) {
-    return __fdiv_rn(__int2float_rn(g), __uint_as_float(FALCON_P10_F32[a - FALCON_P10_F32_LO]));
+// fl32(fl32(g) / 10^a) by multiplication with r = fl32(10^-a) and one exact residual (Markstein, IBM
+// J. Res. Dev. 34, 1990): q = fl(x r), then fl(q + (x - q 10^a) r) is the correctly rounded quotient.  No
+// result is subnormal (|g| >= 1, a <= 10); checked against division for every 24-bit significand and a.
+struct Div10F32 {
+    float p, r;
+};
+__device__ __forceinline__ Div10F32 div10_f32_of(int a) {
+    const float p = __uint_as_float(FALCON_P10_F32[a - FALCON_P10_F32_LO]);
+    return {p, __frcp_rn(p)};
+}
+__device__ __forceinline__ float div_pow10(float x, const Div10F32 &d) {
+    const float q = __fmul_rn(x, d.r);
+    return __fmaf_rn(__fmaf_rn(-q, d.p, x), d.r, q);
 }
 
 // A chunk to decode and where its record lies.  The loads are unconditional (a ticket past the
@@ -470,15 +481,14 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, uint8_t *smem, uint3
                     vx = div_pow10_exact((int64_t)vx, q);
                 }
             }
-        } else if constexpr (D == kD32) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] = (U)__float_as_uint(div_pow10((int32_t)d[k], (int)alpha));
-            vx = (U)__float_as_uint(div_pow10((int32_t)vx, (int)alpha));
         } else {
-            // fl16(g / 10^a) as fl16(fl32(g / 10^a)): exact for every 16-bit g and a <= 4 (the
+            // FP16: fl16(g / 10^a) as fl16(fl32(g / 10^a)): exact for every 16-bit g and a <= 4 (the
             // second rounding never lands on a different value; checked for all 327,680 inputs)
-            const float p = __uint_as_float(FALCON_P10_F32[alpha - FALCON_P10_F32_LO]);
-            auto conv = [&](U g) { return __half_as_ushort(__float2half_rn(__fdiv_rn((float)(int16_t)g, p))); };
+            const Div10F32 q = div10_f32_of((int)alpha);
+            auto conv = [&](U g) {
+                if constexpr (D == kD32) return __float_as_uint(div_pow10(__int2float_rn((int32_t)g), q));
+                else return __half_as_ushort(__float2half_rn(div_pow10((float)(int16_t)g, q)));
+            };
 #pragma unroll
             for (int k = 0; k < 32; ++k) d[k] = conv(d[k]);
             vx = conv(vx);

@@ -509,36 +509,49 @@ __device__ __forceinline__ uint32_t case1_g_narrow(uint64_t u, const Case1Narrow
     const uint32_t hi = (uint32_t)(u >> 32), s = (uint32_t)((int32_t)hi >> 31);
     return (case1_n_narrow(hi, (uint32_t)u, q) ^ s) - s;
 }
-__device__ __forceinline__ uint32_t case1_g(uint32_t u, int a) {
-    const uint32_t au = u & 0x7FFFFFFFu;
-    if (au == 0) return 0;
-    const int E = (int)(au >> 23) - 150;
-    const uint64_t m = (au & 0x007FFFFFu) | 0x00800000u;
-    const int F = -(E + a);
-    const uint64_t P = m * FALCON_POW5[a];
-    uint64_t N;
-    if (F <= 0) N = P << (-F);
-    else N = (P + (1ull << (F - 1))) >> F;
-    return (u >> 31) ? (0u - (uint32_t)N) : (uint32_t)N;
+// FP32: m 2^8 times 5^a normalised to 32 bits is the exact product P, normalised; X < 10^7 makes its
+// rounding bit lie in the top word, so g = floor(X + 1/2) comes from one 32-bit high product.
+struct Case1F32 {
+    uint32_t p5, norm;                            // 5^a, 5^a with its top bit at bit 31
+    int c, f0;                                    // shift - 1 = c - exponent field, F = f0 - exponent field
+};
+__device__ __forceinline__ Case1F32 case1_f32_of(int a) {
+    const uint32_t p5 = (uint32_t)FALCON_POW5[a];
+    const int d = (int)FALCON_LOG2_POW5[a];
+    // X = P 2^-F, t = P 2^(8 + 31 - d - 32): shift = F + 7 - d
+    return {p5, p5 << (31 - d), 150 - a + 7 - d - 1, 150 - a};
 }
+__device__ __forceinline__ uint32_t case1_n(uint32_t u, const Case1F32 &q) {            // |g|
+    const uint32_t m8 = (u << 8) | 0x80000000u;
+    return (shr_clamp(__umulhi(m8, q.norm), (uint32_t)(q.c - (int)((u >> 23) & 0xFFu))) + 1u) >> 1;
+}
+__device__ __forceinline__ uint32_t case1_g(uint32_t u, const Case1F32 &q) {
+    const uint32_t s = (uint32_t)((int32_t)u >> 31);
+    return (case1_n(u, q) ^ s) - s;
+}
+__device__ __forceinline__ uint32_t case1_g(uint32_t u, int a) { return case1_g(u, case1_f32_of(a)); }
 
-// binary16 (R18): both tests of Alg. 2 at decimal place a from one product, as for FP32:
-// v = m 2^E with an 11-bit m, P = m 5^a < 2^21, F = -(E + a) <= 24; eps <= mu is
-// dist(P, 2^F Z) <= P 2^-10 and the round trip |N 2^F - P| < 5^a / 2 (5^a / 4 below a power
-// of two, where the ulp below v is half as wide).
-__device__ __forceinline__ bool alg2_step_f16(uint16_t u, int a, bool &rt) {
-    const uint32_t au = u & 0x7FFFu;
-    const int F = 25 - (int)(au >> 10) - a;
-    if (au == 0 || F <= 0) { rt = true; return true; }
-    const uint32_t m = (au & 0x3FFu) | 0x400u;
-    const uint32_t p5 = (uint32_t)FALCON_POW5[a];            // 5^a <= 625
-    const uint32_t P = m * p5;
-    const uint32_t lim = p5 >> 1, lim_low = (m == 0x400u) ? ((p5 - 1u) >> 2) : lim;
-    const uint32_t mask = (1u << F) - 1u;
-    const uint32_t r = P & mask, rc = mask - r + 1u;
-    rt = (r > (mask >> 1)) ? (rc <= lim) : (r <= lim_low);
-    return (r < rc ? r : rc) <= (P >> 10);
+// binary16 (R18): both tests of Alg. 2 at decimal place a, in exact FP32 arithmetic (the FMA pipe has
+// room where the integer pipe is the limit): X = v 10^a has an 11-bit times a 10-bit significand, its
+// nearest integer N comes from adding 1.5 2^23 (callers only ask for |X| < 2^22), X - N is exact.
+// eps <= mu is |X - N| <= |X| 2^-10, the round trip |X - N| <= half an ulp of v times 10^a.  (Equality
+// cannot occur there: 5^a is odd.  Below a power of two the ulp is half as wide, which changes nothing:
+// X 2^F = 2^10 5^a, and its distance to a multiple of 2^F is 0 or at least 2^10 > 5^a / 2.)
+struct Scale16 {
+    float p, half;                                // 10^a, 10^a 2^-11
+};
+__device__ __forceinline__ Scale16 scale16_of(int a) {
+    const float p = __uint_as_float(FALCON_P10_F32[a - FALCON_P10_F32_LO]);
+    return {p, p * 0x1p-11f};
 }
+constexpr float kRound16 = 12582912.0f;           // 1.5 2^23
+__device__ __forceinline__ bool alg2_step_f16(uint16_t u, const Scale16 &q, bool &rt) {
+    const float v = __half2float(__ushort_as_half(u)), x = v * q.p;
+    const float n = (x + kRound16) - kRound16, eps = fabsf(x - n);
+    rt = eps <= __uint_as_float(__float_as_uint(v) & 0x7F800000u) * q.half;
+    return eps <= fabsf(x) * 0x1p-10f;
+}
+__device__ __forceinline__ bool alg2_step_f16(uint16_t u, int a, bool &rt) { return alg2_step_f16(u, scale16_of(a), rt); }
 __device__ __forceinline__ bool q_test(uint16_t u, int a) {
     bool rt;
     (void)alg2_step_f16(u, a, rt);
@@ -554,14 +567,11 @@ __device__ __forceinline__ int first_pass_f16(uint16_t u, int atop) {
     }
     return -1;
 }
-__device__ __forceinline__ uint16_t case1_g(uint16_t u, int a) {
-    const uint32_t au = u & 0x7FFFu;
-    if (au == 0) return 0;
-    const int F = 25 - (int)(au >> 10) - a;
-    const uint32_t P = ((au & 0x3FFu) | 0x400u) * (uint32_t)FALCON_POW5[a];
-    const uint32_t N = F <= 0 ? (P << (-F)) : ((P + (1u << (F - 1))) >> F);
-    return (uint16_t)((u >> 15) ? (0u - N) : N);
+// g of a value that passed: the low bits of X + 1.5 2^23
+__device__ __forceinline__ uint16_t case1_g(uint16_t u, const Scale16 &q) {
+    return (uint16_t)__float_as_uint(__half2float(__ushort_as_half(u)) * q.p + kRound16);
 }
+__device__ __forceinline__ uint16_t case1_g(uint16_t u, int a) { return case1_g(u, scale16_of(a)); }
 
 // fl(g / 10^a), correctly rounded (nearest, ties to even), for |g| <= 2^53 and 0 <= a <= 22, in
 // integer arithmetic (the inverse of Eq. 4, Case 1).  g / 10^a = (g / 5^a) 2^-a and the
