@@ -14,14 +14,15 @@
 //         G (inverse Eq. 5), Case 1 divides by 10^alpha (correctly rounded) and Case 2 undoes the
 //         zigzag of the IEEE bits (inverse Eq. 4),
 //      c. whole 32-byte sectors per lane (aligned FP64) or staged, coalesced stores.
-// What bounds it: latency and integer issue together (FP64 segments: ALU pipe 55 %, L1 data pipe
-// 53 %, issue 51 % of cycles at 16 warps per SM; HBM 40 %).  Reading the dense rows in place
-// instead of copying them to a plane buffer took the kernel from 4302 to 2880 warp instructions
-// per FP64 chunk and its shared memory from 17.6 to 13.6 KB per warp (12 to 16 warps per SM).
-// Measured, 2^26 segment values (both launches): FP64 420 -> 322 us, FP32 216 -> 152 us; Case-1
-// FP64 of 40 M values in 1025-value chunks 547 -> 307 us.  Slower, and left out: a TMA bulk copy of
-// the record on an mbarrier (-1 %), tickets for groups of 4 to 8 chunks (-7 to -15 %: the window of
-// memory in use grows with the group), more registers with fewer warps (144: -6 %).
+// What bounds it: integer issue and latency together (FP64 segments: ALU pipe 56 %, L1 data pipe
+// 55 %, issue 52 % of cycles at 16 warps per SM; HBM 45 %), and the instruction stream's length: code is
+// kept short (both FP64 halves run one copy, Case 1 divides in rolled loops on the way out), which
+// took FP64 segments from 310 to 288 us and Case-1 values from 304 to 191 us (40 M in 1025-value chunks).
+// Reading the dense rows in place instead of copying them to a plane buffer took the kernel from 4302 to
+// 2880 warp instructions per FP64 chunk and its shared memory from 17.6 to 13.7 KB per warp (12 to 16
+// warps per SM).  Both launches, 2^26 segment values: FP64 420 -> 288 us, FP32 216 -> 149 us.  Slower, and
+// left out: a TMA bulk copy of the record on an mbarrier (-1 %), tickets for groups of 4 to 8 chunks (-7
+// to -15 %: the window of memory in use grows with the group), more registers with fewer warps (144: -6 %).
 // Every read of a record is bounds-checked against its size; a malformed record sets
 // FALCON_ERR_CORRUPT and writes nothing.
 #include "falcon.h"
@@ -38,7 +39,8 @@ namespace {
 //   - 128-byte slots for the expanded sparse rows of 32 planes at a time (FP64 runs its two
 //     halves one after the other through the same slots), later the staging of a chunk whose
 //     output is not 32-byte aligned,
-//   - where each of those 32 planes' rows lies: (word address, bit shift) pairs.
+//   - where each of those 32 planes' rows lies: (word address, bit shift) pairs,
+//   - what the chunk's last steps need again (ChunkNote).
 // Dense rows are read where they lie in the record, so no plane buffer is kept: 13.6 KB per FP64
 // warp instead of 17.6 KB, 16 resident warps per SM instead of 12.
 constexpr uint32_t kZeroBytes = 144;
@@ -47,8 +49,18 @@ template <int D> struct DecLayout {
     static constexpr uint32_t kRows = Traits<D>::W < 32 ? Traits<D>::W : 32;
     static constexpr uint32_t kSlots = kRows * 128;
     static constexpr uint32_t kTab = 32 * 8;
-    static constexpr uint32_t kWarpBytes = kBuf + kSlots + kTab;
+    static constexpr uint32_t kNote = kBuf + kSlots + kTab;
+    static constexpr uint32_t kWarpBytes = kNote + 32;
 };
+
+// Header fields and place of the chunk being decoded, written down while its planes take the registers
+// (kept in registers they were spilled, and with them the ticket in flight, which is then waited for).
+struct ChunkNote {
+    uint64_t c, z1;
+    const Job *job;
+    uint32_t alpha, beta_hat;
+};
+static_assert(sizeof(ChunkNote) == 32, "ChunkNote is 32 bytes of each warp's shared memory");
 
 // The 32-bit word at any byte offset of the CTA's dynamic shared memory.
 __device__ __forceinline__ uint32_t lds_any(const uint8_t *smem, uint32_t off) {
@@ -243,25 +255,34 @@ __device__ __forceinline__ uint64_t pair64(uint16_t const (&d)[32], int i) {
     return ((uint64_t)hi << 32) | lo;
 }
 
-// The chunk's m values (lane l holds 32 l .. 32 l + 31 in d, lane 31 value 1024 in vx) to dst.  A
-// whole FP64 chunk at a 32-byte aligned address: each lane stores its contiguous values in whole
-// sectors.  Otherwise they pass through the slots (swizzled; FP64 half the lanes at a time) and
-// leave as coalesced 16-byte units, or single values where dst is not 16-byte aligned.  (Whole
-// sectors against staging: FP64 segments 325 / 332 us, FP32 170 / 162 us, so FP32 and FP16, whose
-// values pass the slots once, always stage.)
-template <int D>
-__device__ __forceinline__ void store_values(uint8_t *dst, uint32_t m, uint8_t *slots,
-                                             const typename Traits<D>::U (&d)[32], typename Traits<D>::U vx, int lane) {
+// The chunk's m values (lane l holds 32 l .. 32 l + 31 in d, lane 31 value 1024 in vx) to dst, whole
+// sectors per lane: a whole FP64 chunk at a 32-byte aligned address.
+template <class U>
+__device__ __forceinline__ void store_sectors(uint8_t *dst, uint32_t m, const U (&d)[32], U vx, int lane) {
+    constexpr int S = sizeof(U);
+    if (m > 1024u && lane == 31) *reinterpret_cast<U *>(dst + 1024 * S) = vx;
+    uint8_t *mine = dst + lane * (32 * S);
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+        store32(mine + 32 * i, pair64(d, 4 * i), pair64(d, 4 * i + 1), pair64(d, 4 * i + 2), pair64(d, 4 * i + 3));
+}
+
+// The same at any alignment: the values pass through the slots (swizzled; FP64 half the lanes at a time)
+// and leave as coalesced 16-byte units, or single values where dst is not 16-byte aligned.  `conv`
+// maps what is staged to values in place, on the way out (kRolled: it is long, so the loops are rolled);
+// the whole warp calls it.  (Whole sectors against staging: FP64 segments 325 / 332 us, FP32
+// 170 / 162 us, so FP32 and FP16, whose values pass the slots once, always stage.)
+template <int D, bool kRolled, class Conv>
+__device__ __forceinline__ void store_staged(uint8_t *dst, uint32_t m, uint8_t *slots,
+                                             const typename Traits<D>::U (&d)[32], typename Traits<D>::U vx, int lane,
+                                             Conv &&conv) {
     using T = Traits<D>;
     using U = typename T::U;
     constexpr int S = T::S, UN = T::UNITS, PER = 16 / S;
-    if (m > 1024u && lane == 31) *reinterpret_cast<U *>(dst + 1024 * S) = vx;
-    if (D == kD64 && m >= 1024u && (reinterpret_cast<uintptr_t>(dst) & 31u) == 0) {
-        uint8_t *mine = dst + lane * (32 * S);
-#pragma unroll
-        for (int i = 0; i < S; ++i)
-            store32(mine + 32 * i, pair64(d, 4 * i), pair64(d, 4 * i + 1), pair64(d, 4 * i + 2), pair64(d, 4 * i + 3));
-        return;
+    if (m > 1024u) {
+        U e[1] = {vx};
+        conv(e);
+        if (lane == 31) *reinterpret_cast<U *>(dst + 1024 * S) = e[0];
     }
     constexpr int kPasses = D == kD64 ? 2 : 1, kLanes = 32 / kPasses;
     const bool al16 = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0;
@@ -280,38 +301,67 @@ __device__ __forceinline__ void store_values(uint8_t *dst, uint32_t m, uint8_t *
         }
         __syncwarp();
         uint8_t *out = dst + v0 * S;
-        uint32_t done = 0;
-        if (cnt == (uint32_t)(kLanes * 32)) {     // whole pass: fixed trip counts
+        auto unit = [&](uint32_t q, bool store) {
+            union { uint4 w; U e[PER]; } x;
+            x.w = *reinterpret_cast<const uint4 *>(slots + phys_unit<D>(q) * 16u);
+            conv(x.e);
+            if (store) *reinterpret_cast<uint4 *>(out + 16u * q) = x.w;
+        };
+        auto one = [&](uint32_t i, bool store) {
+            U e[1] = {*reinterpret_cast<const U *>(slots + phys_elem_byte<D>(i))};
+            conv(e);
+            if (store) *reinterpret_cast<U *>(out + i * S) = e[0];
+        };
+        if (!kRolled && cnt == (uint32_t)(kLanes * 32)) {        // whole pass: fixed trip counts
             if (al16) {
 #pragma unroll
-                for (int i = 0; i < kLanes * UN / 32; ++i) {
-                    const uint32_t q = 32u * i + lane;
-                    *reinterpret_cast<uint4 *>(out + 16u * q) = *reinterpret_cast<const uint4 *>(slots + phys_unit<D>(q) * 16u);
-                }
+                for (int i = 0; i < kLanes * UN / 32; ++i) unit(32u * i + lane, true);
             } else {
 #pragma unroll
-                for (int i = 0; i < kLanes; ++i) {
-                    const uint32_t e = 32u * i + lane;
-                    *reinterpret_cast<U *>(out + e * S) = *reinterpret_cast<const U *>(slots + phys_elem_byte<D>(e));
-                }
+                for (int i = 0; i < kLanes; ++i) one(32u * i + lane, true);
             }
-            __syncwarp();
-            continue;
+        } else {
+            uint32_t done = 0;
+            if (al16) {
+                done = cnt * S >> 4;
+#pragma unroll 1
+                for (uint32_t q = 0; q < done; q += 32) unit(min(q + lane, done - 1u), q + lane < done);
+                done *= PER;
+            }
+#pragma unroll 1
+            for (uint32_t i = done; i < cnt; i += 32) one(min(i + lane, cnt - 1u), i + lane < cnt);
         }
-        if (al16) {
-            const uint32_t nunits = cnt * S >> 4;
-#pragma unroll 4
-            for (uint32_t q = lane; q < nunits; q += 32)
-                *reinterpret_cast<uint4 *>(out + 16u * q) = *reinterpret_cast<const uint4 *>(slots + phys_unit<D>(q) * 16u);
-            done = nunits * PER;
-        }
-        // value 32 i + lane of the pass belongs to its lane i, unit lane / PER
-#pragma unroll 8
-        for (uint32_t e = done + lane; e < cnt; e += 32)
-            *reinterpret_cast<U *>(out + e * S) = *reinterpret_cast<const U *>(slots + phys_elem_byte<D>(e));
         __syncwarp();
     }
 }
+
+// FP64 Case 1: g to fl(g / 10^alpha).  Values of a warp that all fit 32 bits (the common case) take the
+// 96-bit reciprocal, others the exact division, |g| > 2^53 (only in streams no encoder writes) the
+// FP64 divide.
+struct ConvF64 {
+    Div10Narrow qn;
+    int alpha;
+    __device__ __forceinline__ explicit ConvF64(int a) : qn(div10_narrow_of(a < kDiv10NarrowMax ? a : kDiv10NarrowMax)), alpha(a) {}
+    template <int N> __device__ __forceinline__ void operator()(uint64_t (&g)[N]) const {
+        uint32_t wide = alpha > kDiv10NarrowMax ? 1u : 0u;
+#pragma unroll
+        for (int i = 0; i < N; ++i) wide |= (uint32_t)(g[i] >> 32) ^ (uint32_t)((int32_t)(uint32_t)g[i] >> 31);
+        if (!__any_sync(kFull, wide)) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const uint32_t s = (uint32_t)((int32_t)(uint32_t)g[i] >> 31);
+                g[i] = div_pow10_exact32(((uint32_t)g[i] ^ s) - s, s, qn);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const uint32_t hi = (uint32_t)(g[i] >> 32), mag = hi ^ (uint32_t)((int32_t)hi >> 31);
+                g[i] = mag >= (1u << 21) ? (uint64_t)__double_as_longlong(div_pow10((int64_t)g[i], alpha))
+                                         : div_pow10_exact((int64_t)g[i], div10_of(alpha));
+            }
+        }
+    }
+};
 
 // A value's exact FP64 value, and its key in IEEE 754 totalOrder (for min / max of non-NaN values).
 __device__ __forceinline__ double value_f64(uint64_t b) { return __longlong_as_double((long long)b); }
@@ -329,32 +379,36 @@ __device__ __forceinline__ uint64_t order_key(double x) {
 // (NaN count, totalOrder min / max, their sum: each lane its 32 values in index order, then a
 // butterfly over the lanes, identical in every lane since FP addition commutes); the chunk's
 // sum goes to sums[c], the rest into the control block by atomics.
-template <int D, class L, bool kAgg, class Next>
-__device__ __forceinline__ void decode_chunk(const Rec &r0, uint8_t *smem, uint32_t wofs, uint32_t seltab, int lane,
+template <int D, class L, bool kAgg, bool kTable, class Next>
+__device__ __forceinline__ void decode_chunk(const Rec &r0, const Job &single, uint8_t *smem, uint32_t wofs, uint32_t seltab, int lane,
                                              Next &&next, Control *ctl) {
     using T = Traits<D>;
     using U = typename T::U;
     const uint32_t slots = wofs + L::kBuf, tab = slots + L::kSlots;
-    const Job &job = *r0.job;
-    const uint64_t c = r0.c;
-    const uint32_t B = job.block;
-    const uint64_t first = c * (uint64_t)B;
-    const uint32_t m = (uint32_t)((job.n - first) < B ? (job.n - first) : B);
-    const uint32_t cols = chunk_cols(m);
+    ChunkNote &note = *reinterpret_cast<ChunkNote *>(smem + wofs + L::kNote);
+    auto values_in = [](const Job &job, uint64_t c) {
+        const uint64_t left = job.n - c * (uint64_t)job.block;
+        return (uint32_t)(left < job.block ? left : job.block);
+    };
+    const uint32_t cols = chunk_cols(values_in(kTable ? *r0.job : single, r0.c));
     const uint32_t row_bytes = cols / 8u, bm_bytes = cols / 64u;
     const uint32_t rec = wofs + (r0.phase & 15u);
 
     // ---- a. header and flags ------------------------------------------------------------------
     bool bad = r0.phase == kBadRecord;
-    const uint32_t h0 = lds_any(smem, rec);
-    const uint32_t alpha = h0 & 0xFFu, beta_hat = (h0 >> 8) & 0xFFu;
-    U z1;
-    if constexpr (D == kD64) z1 = ((uint64_t)lds_any(smem, rec + 6) << 32) | lds_any(smem, rec + 2);
-    else if constexpr (D == kD32) z1 = lds_any(smem, rec + 2);
-    else z1 = (uint16_t)(h0 >> 16);
+    if (lane == 0) {
+        const uint32_t h0 = lds_any(smem, rec);
+        note.c = r0.c;
+        if (kTable) note.job = r0.job;
+        note.alpha = h0 & 0xFFu;
+        note.beta_hat = (h0 >> 8) & 0xFFu;
+        if constexpr (D == kD64) note.z1 = ((uint64_t)lds_any(smem, rec + 6) << 32) | lds_any(smem, rec + 2);
+        else if constexpr (D == kD32) note.z1 = lds_any(smem, rec + 2);
+        else note.z1 = h0 >> 16;
+    }
     const uint32_t w = smem[rec + 2 + T::Z1B];
     const uint32_t hdr = 3u + T::Z1B + (w + 7u) / 8u;
-    if (w > (uint32_t)T::W || (m <= 1u && w != 0u) || hdr > r0.size) bad = true;
+    if (w > (uint32_t)T::W || (cols == 0u && w != 0u) || hdr > r0.size) bad = true;
     // the flags' last w bits, big-endian: bit p is plane p's
     const uint32_t rows_lo = w >= 32u ? ~0u : (1u << w) - 1u;
     const uint32_t dense_lo = bswap(lds_any(smem, rec + hdr - 4u)) & rows_lo;
@@ -374,62 +428,71 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, uint8_t *smem, uint3
     // Lanes past the row's bytes (tail chunks) gather stale bytes; their columns lie past the
     // chunk's values, are never stored, and only feed the scan of later lanes.
     U d[32];
-    uint32_t top0 = 0;                            // FP64: plane 32's word
     if constexpr (D == kD64) {
-        if (!bad && w > 32u) {
-            const uint32_t rows_hi = w >= 64u ? ~0u : (1u << (w - 32u)) - 1u;
-            const uint32_t dense_hi = bswap(lds_any(smem, rec + hdr - 8u)) & rows_hi;
-            place_rows(smem, slots, tab, cur, rows_hi, dense_hi, row_bytes, bm_bytes, rl, lane);
-            __syncwarp();
-            uint32_t a[32];
-            {
+        // both halves run one copy of this code (a third of the kernel's instructions otherwise)
+        uint32_t hi[32], a[32], top = 0, sgn = 0;         // top: plane 32's word, the low half's last row
+#pragma unroll
+        for (int k = 0; k < 32; ++k) hi[k] = 0;
+        if (!bad) {
+#pragma unroll 1
+            for (int h = w > 32u ? 1 : 0; h >= 0; --h) {
+                const uint32_t wh = w - 32u * (uint32_t)h, rows = wh >= 32u ? ~0u : (1u << wh) - 1u;
+                const uint32_t dense = bswap(lds_any(smem, rec + hdr - 4u - 4u * (uint32_t)h)) & rows;
+                place_rows(smem, slots, tab, cur, rows, dense, row_bytes, bm_bytes, rl, lane);
+                __syncwarp();
                 uint32_t r[32];
                 gather_rows<32>(smem, tab, lane, r);
-                top0 = r[0];
+                sgn = h ? 0u : r[0];
 #pragma unroll
-                for (int i = 0; i < 31; ++i) a[i] = r[i + 1];
-                a[31] = 0;
+                for (int i = 0; i < 31; ++i) a[i] = r[i + 1] ^ sgn;
+                a[31] = top ^ sgn;
+                top = r[0];
+                __syncwarp();
+                if (h == 0) next();               // the record has been read
+                transpose32(a);
+                if (h) {
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) hi[k] = a[k ^ 7];
+                }
             }
-            transpose32(a);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] = (U)a[k ^ 7] << 32;
-            __syncwarp();
+            bad = cur - rec != r0.size;
+            if (bad && lane == 0) set_status((kTable ? *r0.job : single).result, kErrCorrupt);
+            if (bad) return;
         } else {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) d[k] = 0;
+            if (lane == 0) set_status((kTable ? *r0.job : single).result, kErrCorrupt);
+            __syncwarp();
+            next();
+            return;
         }
-    }
-    if (!bad) {
-        place_rows(smem, slots, tab, cur, rows_lo, dense_lo, row_bytes, bm_bytes, rl, lane);
-        bad = cur - rec != r0.size;
-    }
-    if (bad) {
-        if (lane == 0) set_status(job.result, kErrCorrupt);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            const uint32_t s = (uint32_t)((int32_t)(sgn << (31 - (k ^ 7))) >> 31);
+            d[k] = (U)(((uint64_t)(hi[k] ^ s) << 32) | a[k ^ 7]);
+        }
+    } else {
+        if (!bad) {
+            place_rows(smem, slots, tab, cur, rows_lo, dense_lo, row_bytes, bm_bytes, rl, lane);
+            bad = cur - rec != r0.size;
+        }
         __syncwarp();
-        next();
-        return;
-    }
-    __syncwarp();
-    {
+        if (bad) {
+            if (lane == 0) set_status((kTable ? *r0.job : single).result, kErrCorrupt);
+            next();
+            return;
+        }
         constexpr int R = T::W < 32 ? T::W : 32;
         uint32_t a[32], r[R];
         gather_rows<R>(smem, tab, lane, r);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) a[i] = i + 1 < R ? r[i + 1] ^ r[0] : (i + 1 == R ? top0 ^ r[0] : 0u);
+        for (int i = 0; i < 32; ++i) a[i] = i + 1 < R ? r[i + 1 < R ? i + 1 : 0] ^ r[0] : (i + 1 == R ? r[0] : 0u);
         __syncwarp();
         next();                                   // the record has been read
         transpose32(a);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            if constexpr (D == kD64) {
-                const uint32_t s = (uint32_t)((int32_t)(r[0] << (31 - (k ^ 7))) >> 31);
-                d[k] = ((uint64_t)((uint32_t)(d[k] >> 32) ^ s) << 32) | a[k ^ 7];
-            } else {
-                d[k] = (U)a[k ^ 7];
-            }
-        }
+        for (int k = 0; k < 32; ++k) d[k] = (U)a[k ^ 7];
     }
     // ---- c. G (inverse Eq. 5): lane l's values 32 l .. 32 l + 31 -------------------------------
+    const U z1 = (U)note.z1;
     U run = 0;
 #pragma unroll
     for (int k = 0; k < 32; ++k) run += d[k];
@@ -442,44 +505,33 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, uint8_t *smem, uint3
         run += t;
     }
     U vx = run;                                   // lane 31: value 1024
+    const Job &job = kTable ? *note.job : single;
+    const uint64_t c = note.c;
+    const uint32_t m = values_in(job, c), alpha = note.alpha, beta_hat = note.beta_hat;
+    uint8_t *dst = job.out + c * (uint64_t)job.block * T::S;
     // ---- d. values (inverse Eq. 4) ---------------------------------------------------------------
     if (alpha <= (uint32_t)T::A_MAX && beta_hat <= (uint32_t)T::B_MAX) {
         if constexpr (D == kD64) {
-            // every g fits 32 bits (|g| <= 2^31): the common case
-            uint32_t wide = 0;
-            auto hi = [](uint64_t g) { return (uint32_t)(g >> 32); };
-            auto sgn = [](uint32_t x) { return (uint32_t)((int32_t)x >> 31); };
-#pragma unroll
-            for (int k = 0; k < 32; ++k) wide |= hi(d[k]) ^ sgn((uint32_t)d[k]);
-            wide |= hi(vx) ^ sgn((uint32_t)vx);
-            if (alpha <= (uint32_t)kDiv10NarrowMax && !__any_sync(kFull, wide)) {
-                const Div10Narrow q = div10_narrow_of((int)alpha);
-                auto conv = [&](uint32_t g) {
-                    const uint32_t s = sgn(g);
-                    return div_pow10_exact32((g ^ s) - s, s, q);
-                };
-#pragma unroll
-                for (int k = 0; k < 32; ++k) d[k] = conv((uint32_t)d[k]);
-                vx = conv((uint32_t)vx);
-            } else {
-                uint32_t big = hi(vx) ^ sgn(hi(vx));
-#pragma unroll
-                for (int k = 0; k < 32; ++k) big |= hi(d[k]) ^ sgn(hi(d[k]));
-                if (__any_sync(kFull, big >= (1u << 21))) {       // some |g| > 2^53: only in streams no encoder writes
+            const ConvF64 conv((int)alpha);
+            if constexpr (kAgg) {                 // the values are wanted in registers
 #pragma unroll 1
-                    for (int i = 0; i < 32; ++i) {          // rolled (small code): the values rotate through d[0]
-                        const U v = (U)__double_as_longlong(div_pow10((int64_t)d[0], (int)alpha));
+                for (int i = 0; i < 32; i += 2) {       // rolled (small code): the values rotate through d[0], d[1]
+                    U e[2] = {d[0], d[1]};
+                    conv(e);
 #pragma unroll
-                        for (int k = 0; k < 31; ++k) d[k] = d[k + 1];
-                        d[31] = v;
-                    }
-                    vx = (U)__double_as_longlong(div_pow10((int64_t)vx, (int)alpha));
-                } else {
-                    const Div10 q = div10_of((int)alpha);
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) d[k] = div_pow10_exact((int64_t)d[k], q);
-                    vx = div_pow10_exact((int64_t)vx, q);
+                    for (int k = 0; k < 30; ++k) d[k] = d[k + 2];
+                    d[30] = e[0];
+                    d[31] = e[1];
                 }
+                U e[1] = {vx};
+                conv(e);
+                vx = e[0];
+            } else {
+                // divided on the way out, in rolled loops: unrolled over the 32 registers, the
+                // division cost every chunk spills and instruction fetch (2^26 segments 309 -> 296 us
+                // without, 2^25 decimal values 206 -> 160 us)
+                store_staged<D, true>(dst, m, smem + slots, d, vx, lane, conv);
+                return;
             }
         } else {
             // FP16: fl16(g / 10^a) as fl16(fl32(g / 10^a)): exact for every 16-bit g and a <= 4 (the
@@ -542,7 +594,8 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, uint8_t *smem, uint3
         return;
     }
 
-    store_values<D>(job.out + first * T::S, m, smem + slots, d, vx, lane);
+    if (D == kD64 && m >= 1024u && (reinterpret_cast<uintptr_t>(dst) & 31u) == 0) store_sectors(dst, m, d, vx, lane);
+    else store_staged<D, false>(dst, m, smem + slots, d, vx, lane, [](auto &) {});
 }
 
 }  // namespace
@@ -632,12 +685,12 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
             if (tn < total_chunks) rn = issue_record(ln, wbase, lane);
             cp_async_commit();
         };
-        if constexpr (kDt == kDtF64) decode_chunk<kD64, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
-        else if constexpr (kDt == kDtF32) decode_chunk<kD32, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
-        else if constexpr (kDt == kDtF16) decode_chunk<kD16, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
-        else if (rec.job->dtype == 0) decode_chunk<kD64, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
-        else if (rec.job->dtype == 1) decode_chunk<kD32, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
-        else decode_chunk<kD16, L, kAgg>(rec, smem, wofs, seltab, lane, next, ctl);
+        if constexpr (kDt == kDtF64) decode_chunk<kD64, L, kAgg, kTable>(rec, s_single, smem, wofs, seltab, lane, next, ctl);
+        else if constexpr (kDt == kDtF32) decode_chunk<kD32, L, kAgg, kTable>(rec, s_single, smem, wofs, seltab, lane, next, ctl);
+        else if constexpr (kDt == kDtF16) decode_chunk<kD16, L, kAgg, kTable>(rec, s_single, smem, wofs, seltab, lane, next, ctl);
+        else if (rec.job->dtype == 0) decode_chunk<kD64, L, kAgg, kTable>(rec, s_single, smem, wofs, seltab, lane, next, ctl);
+        else if (rec.job->dtype == 1) decode_chunk<kD32, L, kAgg, kTable>(rec, s_single, smem, wofs, seltab, lane, next, ctl);
+        else decode_chunk<kD16, L, kAgg, kTable>(rec, s_single, smem, wofs, seltab, lane, next, ctl);
         if (tn >= total_chunks) break;
         rec = rn;
         tn = ticket_of(raw);
