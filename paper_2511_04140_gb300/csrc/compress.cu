@@ -47,8 +47,8 @@ namespace falcon {
 
 namespace {
 
-constexpr int kBuf = 8288;                  // one chunk of values / one record (+32 readable)
-constexpr int kAnalyseWarpBytes = kBuf;     // analysis: one value buffer
+// one chunk of values (1025, swizzled) of a kind
+template <int D> constexpr int kAnalyseWarpBytes = 1024 * Traits<D>::S + 32;
 
 // The emit launch's per-warp buffers: the record, assembled at the output's 16-byte phase, and
 // 128-byte slots for the rows of 32 planes at a time, top plane first (FP64 runs its two halves one
@@ -450,9 +450,10 @@ __device__ __noinline__ int alpha_elf(const uint8_t *buf, int lane, uint32_t m, 
 
 // Case 1's alpha_max of a chunk that may be Case 1 (no special value, the test value passes at
 // atop), or -1.  On success the staging buffer holds G (Eq. 4) in place of the values, otherwise
-// the values.
+// the values.  Out of line, over the staged values: many workloads' chunks never get here, and its code
+// stays out of the others' instruction stream.
 template <int D>
-__device__ __forceinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, int e_max, int atop,
+__device__ __noinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, int e_max, int atop,
                                            typename Traits<D>::U vmax, bool elf) {
     using T = Traits<D>;
     using U = typename T::U;
@@ -507,21 +508,25 @@ template <int D> struct Mag {
 
 // Case decision (Eq. 4) of a chunk whose keys have maximum `top` (kmax: this lane's) and, if
 // `low`, some value with a zero exponent field.  Returns alpha_max | beta_hat << 8, alpha_max = 31
-// in Case 2; the staging buffer holds G on a Case 1 return, the values otherwise.  Out of line,
-// over the staged values, with none of them in registers: the code of the rarer decisions stays out
-// of the hot path's instruction stream.
+// in Case 2; the staging buffer holds G on a Case 1 return, the values otherwise.
 constexpr int kCase2 = 31;
 template <int D>
-__device__ __noinline__ int case_decision(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, uint32_t kmax,
-                                          uint32_t top, bool low, bool elf) {
+__device__ __forceinline__ int case_decision(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, uint32_t kmax,
+                                             uint32_t top, bool low, bool elf) {
     using T = Traits<D>;
     using U = typename T::U;
     constexpr U ABS = Mag<D>::ABS;
     constexpr int kNone = kCase2 | (T::B_SENT << 8);
     if (low) {                                    // +0 or a special value (-0, subnormal)
+        constexpr int PER = 16 / T::S;
         bool s = m > 1024u && lane == 31 && is_special(read_elem<D>(buf, 1024));
-#pragma unroll 4
-        for (int k = 0; k < 32; ++k) s |= is_special(lane_value<D>(buf, lane, k));
+#pragma unroll 2
+        for (int u = 0; u < T::UNITS; ++u) {
+            union { uint4 w; U e[PER]; } x;
+            x.w = *reinterpret_cast<const uint4 *>(buf + (lane * T::UNITS + unit_swizzle<D>(lane, u)) * 16);
+#pragma unroll
+            for (int k = 0; k < PER; ++k) s |= Mag<D>::key(x.e[k], 0) < Mag<D>::kExpOne && x.e[k] != 0;
+        }
         if (__any_sync(kFull, s)) return kNone;
     }
     // the largest magnitude (FP64: one that shares its key's top bits)
@@ -624,35 +629,42 @@ __device__ __forceinline__ void analyse_chunk(const Job &job, uint64_t c, uint8_
     }
     const bool case1 = alpha != kCase2;
 
-    // ---- 2. G ---------------------------------------------------------------------------------
-    U v[32];
-    read_own<D>(buf, lane, v);
-    U vx = m > 1024u && lane == 31 ? read_elem<D>(buf, 1024) : v[31];        // no further value: no further delta
-    __syncwarp();
-    next();                                     // the staged values have been read
-    if (!case1) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = zigzag(v[k]);
-        vx = zigzag(vx);
-    }
-
-    // ---- 3. |Z| by 8-column groups, w -----------------------------------------------------------
-    U nxt = shfl_down_x(v[0], 1);
-    if (lane == 31) nxt = vx;
-    // OR of the Z of columns 8 i .. 8 i + 7: Z = (x ^ s) << 1 | (s & 1) for the delta x with sign s
-    U o[4];
-#pragma unroll
+    // ---- 2. G and |Z| by 8-column groups, w ----------------------------------------------------
+    // o[i]: OR of the Z of columns 8 i .. 8 i + 7; Z = (x ^ s) << 1 | (s & 1) for the delta x with
+    // sign s.  One group at a time (nine values in registers, not 32): 80 registers and 24 warps per SM.
+    U o[4] = {0, 0, 0, 0};
+    constexpr int GU = UN / 4;                   // 16-byte units per group
+#pragma unroll 1
     for (int i = 0; i < 4; ++i) {
+        U g[9];
+#pragma unroll
+        for (int u = 0; u < GU; ++u) {
+            union { uint4 w; U e[PER]; } x;
+            x.w = *reinterpret_cast<const uint4 *>(buf + (lane * UN + unit_swizzle<D>(lane, i * GU + u)) * 16);
+#pragma unroll
+            for (int k = 0; k < PER; ++k) g[u * PER + k] = x.e[k];
+        }
+        // the value after the group; past the chunk's last value there is no further delta
+        g[8] = (i == 3 && lane == 31 && m <= 1024u) ? g[7] : read_elem<D>(buf, 32u * lane + 8u * i + 8u);
+        if (!case1) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) g[k] = zigzag(g[k]);
+        }
         U mag = 0, neg = 0;
 #pragma unroll
-        for (int k = 8 * i; k < 8 * i + 8; ++k) {
-            const U x = (U)((k < 31 ? v[k + 1] : nxt) - v[k]);
+        for (int k = 0; k < 8; ++k) {
+            const U x = (U)(g[k + 1] - g[k]);
             const U s = sign_mask(x);
             mag |= x ^ s;
             neg |= s;
         }
-        o[i] = (U)((U)(mag << 1) | (neg & 1u));
+        o[0] = o[1];                             // the loop is rolled: the groups move up
+        o[1] = o[2];
+        o[2] = o[3];
+        o[3] = (U)((U)(mag << 1) | (neg & 1u));
     }
+    __syncwarp();
+    next();                                     // the staged values have been read
     const U zor = warp_or_x((U)(o[0] | o[1] | o[2] | o[3]));
     const int w = zor ? ((D == 0) ? 64 - __clzll((long long)zor) : 32 - __clz((int)zor)) : 0;
 
@@ -972,7 +984,7 @@ __device__ __forceinline__ void analyse_loop(const Job *__restrict__ jobs, int n
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    uint8_t *wbase = smem + warp * kAnalyseWarpBytes;
+    uint8_t *wbase = smem + warp * kAnalyseWarpBytes<kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64)>;
     __shared__ Job s_single;                      // the single job, read from shared memory
     if (threadIdx.x == 0) s_single = single;
     __syncthreads();
@@ -1005,17 +1017,10 @@ __device__ __forceinline__ void analyse_loop(const Job *__restrict__ jobs, int n
     cp_async_wait_none();
 }
 
-// FP64, FP16 and either-dtype forms (up to 128 registers, 16 warps per SM)
+// Held to 80 registers, 24 warps per SM (either-dtype form: 96 and 20).
 template <int kDt>
-__global__ void __launch_bounds__(32 * kMaxCompressWarps, 1)
+__global__ void __maxnreg__(kDt == kDtMixed ? 96 : 80)
 analyse_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
-    analyse_loop<kDt>(jobs, njobs, single, total_chunks, ctl);
-}
-
-// FP32 form: held to 96 registers, so that 20 warps fit an SM
-template <int kDt>
-__global__ void __maxnreg__(96)
-analyse_kernel_narrow(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
     analyse_loop<kDt>(jobs, njobs, single, total_chunks, ctl);
 }
 
@@ -1179,12 +1184,9 @@ int persistent_grid_of(const void *kernel, int warps, int smem_bytes, int lim, u
 template <int kDt>
 void launch_analyse(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, Control *ctl,
                     cudaStream_t stream) {
-    const int w = g_cta_warps[0], smem = w * kAnalyseWarpBytes;
-    void (*kernel)(const Job *, int, Job, uint64_t, Control *);
-    if constexpr (kDt == kDtF32) kernel = analyse_kernel_narrow<kDt>;
-    else kernel = analyse_kernel<kDt>;
-    const int g = persistent_grid_of(reinterpret_cast<const void *>(kernel), w, smem, g_ctas_per_sm[0], total_chunks);
-    kernel<<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
+    const int w = g_cta_warps[0], smem = w * kAnalyseWarpBytes<kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64)>;
+    const int g = persistent_grid_of(reinterpret_cast<const void *>(analyse_kernel<kDt>), w, smem, g_ctas_per_sm[0], total_chunks);
+    analyse_kernel<kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
 }
 template <bool kWide, int kDt>
 void launch_emit(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, bool direct,
