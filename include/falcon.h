@@ -108,6 +108,16 @@ int falcon_compress(const void *d_in, uint64_t n, int dtype, uint32_t block_size
 int falcon_decompress(const void *d_in, size_t in_bytes, void *d_out, size_t out_capacity_bytes,
                       uint64_t *n_out, void *stream);
 
+/* Reads the 32-byte header of the stream at d_in (device) into h_header (host): one copy on `stream`,
+ * which is synchronised.  FALCON_ERR_CORRUPT for a stream shorter than a header; the header itself is
+ * not judged (falcon_stream_info does). */
+int falcon_read_header(const void *d_in, size_t in_bytes, void *h_header, void *stream);
+
+/* falcon_decompress for a caller that has the stream's first 32 bytes on the host already (h_header),
+ * and sized d_out from them: saves the header's read back. */
+int falcon_decompress_known(const void *d_in, size_t in_bytes, const void *h_header, void *d_out,
+                            size_t out_capacity_bytes, uint64_t *n_out, void *stream);
+
 /* Device workspace (bytes) needed by the asynchronous entry points for a stream of
  * num_chunks chunks.  Must be 256-byte aligned device memory. */
 size_t falcon_workspace_bytes(uint64_t num_chunks);

@@ -65,6 +65,48 @@ int get_workspace(cudaStream_t stream, size_t bytes, void **out) {
     return FALCON_OK;
 }
 
+// Page-locked 64-byte slots for the small device-to-host reads of the synchronous entry points
+// (headers, results): a pageable target costs the driver a staging step on each.  One slab of 64
+// slots, freed by falcon_release once none is in use; a call that finds none reads into pageable memory.
+struct HostSlots {
+    std::mutex mu;
+    uint8_t *slab = nullptr;
+    uint64_t used = 0;
+} g_slots;
+
+class HostSlot {
+  public:
+    HostSlot() {
+        std::lock_guard<std::mutex> lk(g_slots.mu);
+        if (!g_slots.slab) {
+            void *p = nullptr;
+            if (cudaHostAlloc(&p, 64 * 64, cudaHostAllocPortable) == cudaSuccess) g_slots.slab = static_cast<uint8_t *>(p);
+            else (void)cudaGetLastError();
+        }
+        if (g_slots.slab && ~g_slots.used) {
+            at_ = __builtin_ctzll(~g_slots.used);
+            g_slots.used |= 1ull << at_;
+        }
+    }
+    ~HostSlot() {
+        if (at_ < 0) return;
+        std::lock_guard<std::mutex> lk(g_slots.mu);
+        g_slots.used &= ~(1ull << at_);
+    }
+    HostSlot(const HostSlot &) = delete;
+    HostSlot &operator=(const HostSlot &) = delete;
+    // bytes (at most 64) from the device, waited for; nullptr on a CUDA error
+    const void *read(const void *d_src, size_t bytes, cudaStream_t s) {
+        void *dst = at_ >= 0 ? static_cast<void *>(g_slots.slab + 64 * at_) : own_;
+        if (cudaMemcpyAsync(dst, d_src, bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) return nullptr;
+        return cudaStreamSynchronize(s) == cudaSuccess ? dst : nullptr;
+    }
+
+  private:
+    int at_ = -1;
+    uint64_t own_[8];
+};
+
 struct Header {
     uint64_t n, nchunks;
     uint32_t block;
@@ -148,9 +190,9 @@ Job make_decompress_job(const void *d_in, size_t in_bytes, const Header &h, void
 }
 
 int finish_sync(cudaStream_t stream, const void *d_result, uint64_t *value) {
-    uint64_t h[2] = {0, 0};
-    if (cudaMemcpyAsync(h, d_result, sizeof h, cudaMemcpyDeviceToHost, stream) != cudaSuccess) return FALCON_ERR_CUDA;
-    if (cudaStreamSynchronize(stream) != cudaSuccess) return FALCON_ERR_CUDA;
+    HostSlot slot;
+    const uint64_t *h = static_cast<const uint64_t *>(slot.read(d_result, 16, stream));
+    if (!h) return FALCON_ERR_CUDA;
     if (h[1] != 0) return (int)h[1];
     *value = h[0];
     return FALCON_OK;
@@ -267,17 +309,24 @@ int falcon_compress_variant_async(const void *d_in, uint64_t n, int dtype, uint3
     return FALCON_OK;
 }
 
-int falcon_decompress(const void *d_in, size_t in_bytes, void *d_out, size_t out_capacity_bytes,
-                      uint64_t *n_out, void *stream) {
-    if (!d_in || !n_out) return FALCON_ERR_INVALID;
+int falcon_read_header(const void *d_in, size_t in_bytes, void *h_header, void *stream) {
+    if (!d_in || !h_header) return FALCON_ERR_INVALID;
+    if (in_bytes < FALCON_HEADER_BYTES) return FALCON_ERR_CORRUPT;
+    HostSlot slot;
+    const void *h = slot.read(d_in, FALCON_HEADER_BYTES, static_cast<cudaStream_t>(stream));
+    if (!h) return FALCON_ERR_CUDA;
+    std::memcpy(h_header, h, FALCON_HEADER_BYTES);
+    return FALCON_OK;
+}
+
+int falcon_decompress_known(const void *d_in, size_t in_bytes, const void *h_header, void *d_out,
+                            size_t out_capacity_bytes, uint64_t *n_out, void *stream) {
+    if (!d_in || !h_header || !n_out) return FALCON_ERR_INVALID;
     if ((uintptr_t)d_in % 16 != 0) return FALCON_ERR_INVALID;
     if (in_bytes < FALCON_HEADER_BYTES) return FALCON_ERR_CORRUPT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    uint8_t hdr[FALCON_HEADER_BYTES];
-    if (cudaMemcpyAsync(hdr, d_in, sizeof hdr, cudaMemcpyDeviceToHost, s) != cudaSuccess) return FALCON_ERR_CUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return FALCON_ERR_CUDA;
     Header h;
-    int st = parse_header(hdr, sizeof hdr, &h);
+    int st = parse_header(static_cast<const uint8_t *>(h_header), FALCON_HEADER_BYTES, &h);
     if (st) return st;
     if ((st = decompress_args(d_in, in_bytes, h, d_out, out_capacity_bytes))) return st;
     const size_t ws_bytes = falcon_workspace_bytes(h.nchunks);
@@ -293,6 +342,16 @@ int falcon_decompress(const void *d_in, size_t in_bytes, void *d_out, size_t out
     if (st) return st;
     *n_out = v;
     return FALCON_OK;
+}
+
+int falcon_decompress(const void *d_in, size_t in_bytes, void *d_out, size_t out_capacity_bytes,
+                      uint64_t *n_out, void *stream) {
+    if (!d_in || !n_out) return FALCON_ERR_INVALID;
+    if ((uintptr_t)d_in % 16 != 0) return FALCON_ERR_INVALID;
+    uint8_t hdr[FALCON_HEADER_BYTES];
+    const int st = falcon_read_header(d_in, in_bytes, hdr, stream);
+    if (st) return st;
+    return falcon_decompress_known(d_in, in_bytes, hdr, d_out, out_capacity_bytes, n_out, stream);
 }
 
 int falcon_decompress_async(const void *d_in, size_t in_bytes, const void *h_header, void *d_out,
@@ -345,20 +404,19 @@ int falcon_aggregate(const void *d_in, size_t in_bytes, falcon_stats *h_stats, v
     if (in_bytes < FALCON_HEADER_BYTES) return FALCON_ERR_CORRUPT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t hdr[FALCON_HEADER_BYTES];
-    if (cudaMemcpyAsync(hdr, d_in, sizeof hdr, cudaMemcpyDeviceToHost, s) != cudaSuccess) return FALCON_ERR_CUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return FALCON_ERR_CUDA;
     Header h;
-    int st = parse_header(hdr, sizeof hdr, &h);
-    if (st) return st;
+    int st = falcon_read_header(d_in, in_bytes, hdr, stream);
+    if (st || (st = parse_header(hdr, sizeof hdr, &h))) return st;
     // the workspace, then one falcon_stats after it, in the cached buffer
     const size_t ws_bytes = falcon_workspace_bytes(h.nchunks);
     void *ws = nullptr;
     if ((st = get_workspace(s, ws_bytes + 256, &ws))) return st;
     falcon_stats *d_stats = reinterpret_cast<falcon_stats *>(static_cast<uint8_t *>(ws) + ws_bytes);
     if ((st = falcon_aggregate_async(d_in, in_bytes, hdr, ws, ws_bytes, d_stats, stream))) return st;
-    if (cudaMemcpyAsync(h_stats, d_stats, sizeof(falcon_stats), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return FALCON_ERR_CUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return FALCON_ERR_CUDA;
+    HostSlot slot;
+    const void *got = slot.read(d_stats, sizeof(falcon_stats), s);
+    if (!got) return FALCON_ERR_CUDA;
+    std::memcpy(h_stats, got, sizeof(falcon_stats));
     return (int)h_stats->status;
 }
 
@@ -374,6 +432,13 @@ int falcon_release(void) {
     }
     g_ws.clear();
     cudaSetDevice(cur);
+    {
+        std::lock_guard<std::mutex> slots(g_slots.mu);
+        if (g_slots.slab && g_slots.used == 0) {
+            cudaFreeHost(g_slots.slab);
+            g_slots.slab = nullptr;
+        }
+    }
     falcon_pipeline_release();
     falcon_noalloc_release();
     return FALCON_OK;

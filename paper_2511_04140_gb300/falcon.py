@@ -78,6 +78,10 @@ def _load():
             L.falcon_compress.argtypes = [vp, u64, ci, u32, vp, sz, c.POINTER(sz), vp]
             L.falcon_decompress.restype = ci
             L.falcon_decompress.argtypes = [vp, sz, vp, sz, c.POINTER(u64), vp]
+            L.falcon_read_header.restype = ci
+            L.falcon_read_header.argtypes = [vp, sz, vp, vp]
+            L.falcon_decompress_known.restype = ci
+            L.falcon_decompress_known.argtypes = [vp, sz, vp, vp, sz, c.POINTER(u64), vp]
             L.falcon_workspace_bytes.restype = sz
             L.falcon_workspace_bytes.argtypes = [u64]
             L.falcon_compress_async.restype = ci
@@ -200,15 +204,21 @@ def decompress(s: torch.Tensor, out: torch.Tensor | None = None, stream=None) ->
     """Decompresses a uint8 CUDA tensor holding one stream; returns the values."""
     if not s.is_cuda or s.dtype != torch.uint8:
         raise ValueError("s must be a uint8 CUDA tensor")
-    hdr = s[:HEADER_BYTES].cpu().numpy().tobytes() if s.numel() >= HEADER_BYTES else b""
-    if len(hdr) < HEADER_BYTES:
+    if s.numel() < HEADER_BYTES:
         raise FalconError(ERR_CORRUPT, "decompress")
+    L, here = _load(), _stream_ptr(None)
+    if stream is None or stream.cuda_stream == here:
+        buf = ctypes.create_string_buffer(HEADER_BYTES)
+        _check(L.falcon_read_header(s.data_ptr(), s.numel(), buf, here), "decompress")
+        hdr = buf.raw
+    else:                                        # also waits for what the current stream still has to write
+        hdr = s[:HEADER_BYTES].cpu().numpy().tobytes()
     n, code, _, _ = stream_info(hdr)
     dtype = torch_dtype(code)
     if out is None:
         out = torch.empty(max(n, 1), dtype=dtype, device=s.device)
     n_out = ctypes.c_uint64()
-    _check(_load().falcon_decompress(s.data_ptr(), s.numel(), out.data_ptr(), out.numel() * out.element_size(),
+    _check(L.falcon_decompress_known(s.data_ptr(), s.numel(), hdr, out.data_ptr(), out.numel() * out.element_size(),
                                      ctypes.byref(n_out), _stream_ptr(stream)), "decompress")
     return out[:n_out.value]
 

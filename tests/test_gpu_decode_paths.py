@@ -66,3 +66,36 @@ def test_record_positions_over_shares(F, oracle, chunks):
     vals = synth.random_walk(2 * chunks - 1, seed=chunks % 11, dtype=np.float32)
     s = torch.frombuffer(bytearray(oracle.compress(vals, 2)), dtype=torch.uint8).cuda()
     assert np.array_equal(_u(F.decompress(s).cpu().numpy()), _u(vals))
+
+
+def test_synchronous_calls_on_other_streams_and_many_threads(F, oracle):
+    """The synchronous calls on streams of their own, from several threads at once: every result is the
+    one-thread result."""
+    import threading
+    vals = synth.random_walk(3000, seed=1)
+    want = oracle.compress(vals, 1024)
+    x = torch.from_numpy(vals).cuda()
+    y = F.decompress(F.compress(x, 1024, stream=torch.cuda.Stream()), stream=torch.cuda.Stream())
+    assert np.array_equal(_u(y.cpu().numpy()), _u(vals))
+    torch.cuda.synchronize()
+    bad = []
+
+    streams = {s.cuda_stream: s for s in (torch.cuda.Stream() for _ in range(24))}    # distinct ones
+
+    def work(st):
+        with torch.cuda.stream(st):
+            for _ in range(10):
+                s = F.compress(x, 1024)
+                if s.cpu().numpy().tobytes() != want or not torch.equal(F.decompress(s), x):
+                    bad.append(1)
+
+    threads = [threading.Thread(target=work, args=(st,)) for st in streams.values()]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+    s = torch.frombuffer(bytearray(want[:20]), dtype=torch.uint8).cuda()
+    with pytest.raises(F.FalconError) as e:
+        F.decompress(s)
+    assert e.value.status == F.ERR_CORRUPT
