@@ -255,7 +255,6 @@ int falcon_compress(const void *d_in, uint64_t n, int dtype, uint32_t block_size
     const size_t ws_bytes = falcon_workspace_bytes(nc);
     void *ws = nullptr;
     if ((st = get_workspace(s, ws_bytes, &ws))) return st;
-    if (cudaMemsetAsync(ws, 0, sizeof(Control), s) != cudaSuccess) return FALCON_ERR_CUDA;
     uint8_t *w8 = static_cast<uint8_t *>(ws);
     uint64_t *result = reinterpret_cast<uint64_t *>(w8 + kResultOffset);
     const Job j = make_compress_job(d_in, n, dtype, block_size, d_out, out_capacity, w8 + kControlBytes, result);
@@ -299,8 +298,6 @@ int falcon_compress_variant_async(const void *d_in, uint64_t n, int dtype, uint3
         (uintptr_t)d_result % 8 != 0)
         return FALCON_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the chunk tickets; the launches write every other word they read, and the result
-    if (cudaMemsetAsync(d_workspace, 0, sizeof(Control), s) != cudaSuccess) return FALCON_ERR_CUDA;
     uint8_t *w8 = static_cast<uint8_t *>(d_workspace);
     Job j = make_compress_job(d_in, n, dtype, block_size, d_out, out_capacity, w8 + kControlBytes, d_result);
     j.variant = (uint32_t)variant;
@@ -545,7 +542,6 @@ int falcon_batch_launch(void *d_workspace, void *stream) {
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t *w8 = static_cast<uint8_t *>(d_workspace);
-    if (plan.direction == FALCON_COMPRESS && cudaMemsetAsync(w8, 0, sizeof(Control), s) != cudaSuccess) return FALCON_ERR_CUDA;
     if (plan.count == 0) return FALCON_OK;
     const Job *d_jobs = reinterpret_cast<const Job *>(w8 + kControlBytes);
     Control *ctl = reinterpret_cast<Control *>(w8);

@@ -987,18 +987,20 @@ __device__ __forceinline__ void analyse_loop(const Job *__restrict__ jobs, int n
     uint8_t *wbase = smem + warp * kAnalyseWarpBytes<kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64)>;
     __shared__ Job s_single;                      // the single job, read from shared memory
     if (threadIdx.x == 0) s_single = single;
+    pdl_trigger();
     __syncthreads();
-    uint64_t t = ticket_of(take_ticket(ctl, kTicketAnalyse, lane));
+    const Tickets tickets{ctl, kTicketAnalyse, total_chunks};
+    uint64_t t = tickets.first();
     if (t >= total_chunks) return;
     issue_chunk(jobs, njobs, s_single, t, wbase, lane);
     cp_async_commit();
     for (;;) {
-        const unsigned long long raw = take_ticket(ctl, kTicketAnalyse, lane);   // the chunk after t
+        const unsigned long long raw = tickets.draw(lane);       // the chunk after t
         uint64_t tn = total_chunks;
         cp_async_wait_none();                    // the current chunk has landed
         __syncwarp();
         auto next = [&]() {
-            tn = ticket_of(raw);
+            tn = tickets.chunk(raw);
             if (tn < total_chunks) issue_chunk(jobs, njobs, s_single, tn, wbase, lane);
             cp_async_commit();
         };
@@ -1110,15 +1112,16 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
     // (kPre); the FP64 form has no registers to spare for them
     constexpr bool kPre = kDt == kDtF32 || kDt == kDtF16;
     typename Traits<DL>::U v[32], vx;
-    uint64_t t = ticket_of(take_ticket(ctl, kTicketEmit, lane));
+    const Tickets tickets{ctl, kTicketEmit, total_chunks};
+    uint64_t t = tickets.first();
     if (t >= total_chunks) return;
     using Mask = typename std::conditional<kPre, uint32_t, unsigned long long>::type;
     auto info = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
     if constexpr (kPre) load_chunk<DL>(*info.job, info.c, lane, v, vx);
-    t = ticket_of(take_ticket(ctl, kTicketEmit, lane));          // of the next chunk
+    t = tickets.chunk(tickets.draw(lane));       // the next chunk
     for (;;) {
         // the ticket after t, read at the next iteration; t's workspace words are fetched now
-        const unsigned long long raw = take_ticket(ctl, kTicketEmit, lane);
+        const unsigned long long raw = tickets.draw(lane);
         const auto next = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
         if constexpr (!kPre) {
             if (t < total_chunks) prefetch_chunk(*next.job, next.c, lane);
@@ -1149,7 +1152,7 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
         }
         __syncwarp();
         if (t >= total_chunks) break;
-        t = ticket_of(raw);
+        t = tickets.chunk(raw);
         info = next;
     }
     if (lane == 0) bulk_wait();
@@ -1163,6 +1166,7 @@ emit_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_
     __shared__ Job s_single;
     if (threadIdx.x == 0) s_single = single;
     __syncthreads();
+    pdl_wait();
     emit_loop<kWide, kDt>(jobs, njobs, s_single, total_chunks, direct, ctl, smem);
 }
 
@@ -1175,32 +1179,52 @@ emit_kernel_narrow(const Job *__restrict__ jobs, int njobs, Job single, uint64_t
     __shared__ Job s_single;
     if (threadIdx.x == 0) s_single = single;
     __syncthreads();
+    pdl_wait();
     emit_loop<kWide, kDt>(jobs, njobs, s_single, total_chunks, direct, ctl, smem);
 }
 
 namespace {
 int persistent_grid_of(const void *kernel, int warps, int smem_bytes, int lim, uint64_t total_chunks);
 
-template <int kDt>
-void launch_analyse(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, Control *ctl,
-                    cudaStream_t stream) {
-    const int w = g_cta_warps[0], smem = w * kAnalyseWarpBytes<kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64)>;
-    const int g = persistent_grid_of(reinterpret_cast<const void *>(analyse_kernel<kDt>), w, smem, g_ctas_per_sm[0], total_chunks);
-    analyse_kernel<kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
+template <int kDt> constexpr int kind_of() { return kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64); }
+
+// A kernel of a form with its launch shape: pointer, threads, dynamic shared memory, grid.
+template <class K> struct Shape {
+    K kernel;
+    int threads, smem, grid;
+};
+template <int kDt> auto analyse_shape(uint64_t total_chunks) {
+    const int w = g_cta_warps[0], smem = w * kAnalyseWarpBytes<kind_of<kDt>()>;
+    auto *k = analyse_kernel<kDt>;
+    return Shape<decltype(k)>{k, 32 * w, smem,
+                              persistent_grid_of(reinterpret_cast<const void *>(k), w, smem, g_ctas_per_sm[0], total_chunks)};
 }
+template <bool kWide, int kDt> auto emit_shape(uint64_t total_chunks) {
+    const int w = g_cta_warps[0], smem = w * (int)EmitLayout<kind_of<kDt>(), kWide>::kBytes;
+    auto *k = [] {
+        if constexpr (kDt == kDtF32 || kDt == kDtF16) return emit_kernel_narrow<kWide, kDt>;
+        else return emit_kernel<kWide, kDt>;
+    }();
+    return Shape<decltype(k)>{k, 32 * w, smem,
+                              persistent_grid_of(reinterpret_cast<const void *>(k), w, smem, g_ctas_per_sm[0], total_chunks)};
+}
+
 template <bool kWide, int kDt>
-void launch_emit(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, bool direct,
-                 Control *ctl, cudaStream_t stream) {
-    const int w = g_cta_warps[0], smem = w * (int)EmitLayout<kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64), kWide>::kBytes;
-    if constexpr (kDt == kDtF32 || kDt == kDtF16) {
-        const int g = persistent_grid_of(reinterpret_cast<const void *>(emit_kernel_narrow<kWide, kDt>), w, smem,
-                                         g_ctas_per_sm[0], total_chunks);
-        emit_kernel_narrow<kWide, kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, direct, ctl);
-    } else {
-        const int g = persistent_grid_of(reinterpret_cast<const void *>(emit_kernel<kWide, kDt>), w, smem,
-                                         g_ctas_per_sm[0], total_chunks);
-        emit_kernel<kWide, kDt><<<g, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, direct, ctl);
-    }
+cudaError_t launch_form(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks, Control *ctl,
+                        cudaStream_t stream) {
+    const auto an = analyse_shape<kDt>(total_chunks);
+    const auto em = emit_shape<kWide, kDt>(total_chunks);
+    // the chunk tickets, unless both grids have a warp for every chunk
+    if (((uint64_t)an.grid * an.threads / 32u < total_chunks || (uint64_t)em.grid * em.threads / 32u < total_chunks) &&
+        cudaMemsetAsync(ctl, 0, sizeof(Control), stream) != cudaSuccess)
+        return cudaGetLastError();
+    if (total_chunks > 0) an.kernel<<<an.grid, an.threads, an.smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
+    // a stream of a few chunks: each emit warp adds up the sizes before its record itself
+    const bool direct = d_jobs == nullptr && single.nchunks <= kDirectChunks;
+    if (!direct) launch_offsets(d_jobs, njobs, single, kOffsetsOfOutput, ctl, stream);
+    // the emit launch also writes the header and length of every job, chunks or none
+    (void)launch_after(em.kernel, em.grid, em.threads, em.smem, stream, d_jobs, njobs, single, total_chunks, direct, ctl);
+    return cudaGetLastError();
 }
 
 // Resident CTAs per SM of a persistent kernel at one CTA shape, looked up once per (kernel,
@@ -1245,29 +1269,16 @@ int compress_grid(uint64_t total_chunks) {
 
 cudaError_t launch_compress(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks,
                             Control *ctl, cudaStream_t stream) {
+    if (d_jobs != nullptr) return launch_form<false, kDtMixed>(d_jobs, njobs, single, total_chunks, ctl, stream);
     // the every-row-sparse ablation writes records larger than the plane slots hold
-    const bool wide = d_jobs == nullptr && single.variant == kVariantSparse;
-    const int kind = d_jobs != nullptr ? kDtMixed
-                                       : (single.dtype == 0 ? kDtF64 : (single.dtype == 1 ? kDtF32 : kDtF16));
-    if (total_chunks > 0) {
-        if (kind == kDtF64) launch_analyse<kDtF64>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else if (kind == kDtF32) launch_analyse<kDtF32>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else if (kind == kDtF16) launch_analyse<kDtF16>(d_jobs, njobs, single, total_chunks, ctl, stream);
-        else launch_analyse<kDtMixed>(d_jobs, njobs, single, total_chunks, ctl, stream);
+    if (single.variant == kVariantSparse) {
+        if (single.dtype == 0) return launch_form<true, kDtF64>(d_jobs, njobs, single, total_chunks, ctl, stream);
+        if (single.dtype == 1) return launch_form<true, kDtF32>(d_jobs, njobs, single, total_chunks, ctl, stream);
+        return launch_form<true, kDtF16>(d_jobs, njobs, single, total_chunks, ctl, stream);
     }
-    // a stream of a few chunks: each emit warp adds up the sizes before its record itself
-    const bool direct = d_jobs == nullptr && single.nchunks <= kDirectChunks;
-    if (!direct) launch_offsets(d_jobs, njobs, single, kOffsetsOfOutput, ctl, stream);
-    {   // the emit launch also writes the header and length of every job, chunks or none
-        if (wide && kind == kDtF64) launch_emit<true, kDtF64>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
-        else if (wide && kind == kDtF32) launch_emit<true, kDtF32>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
-        else if (wide) launch_emit<true, kDtF16>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
-        else if (kind == kDtF64) launch_emit<false, kDtF64>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
-        else if (kind == kDtF32) launch_emit<false, kDtF32>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
-        else if (kind == kDtF16) launch_emit<false, kDtF16>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
-        else launch_emit<false, kDtMixed>(d_jobs, njobs, single, total_chunks, direct, ctl, stream);
-    }
-    return cudaGetLastError();
+    if (single.dtype == 0) return launch_form<false, kDtF64>(d_jobs, njobs, single, total_chunks, ctl, stream);
+    if (single.dtype == 1) return launch_form<false, kDtF32>(d_jobs, njobs, single, total_chunks, ctl, stream);
+    return launch_form<false, kDtF16>(d_jobs, njobs, single, total_chunks, ctl, stream);
 }
 
 }  // namespace falcon

@@ -607,6 +607,8 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, const Job &single, u
 __global__ void __launch_bounds__(1024)
 offsets_kernel(const Job *__restrict__ jobs, Job single, uint32_t parts, int which, Control *ctl) {
     __shared__ uint64_t warp_sums[33];
+    pdl_trigger();
+    pdl_wait();                                   // compression: the analysis' sizes
     const Job &job = (jobs == nullptr) ? single : jobs[blockIdx.x / parts];
     const uint32_t part = blockIdx.x % parts;
     const uint64_t nc = job.nchunks;
@@ -665,18 +667,21 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
     if (threadIdx.x == 0) s_single = single;
     if (threadIdx.x < kZeroBytes / 16u) reinterpret_cast<uint4 *>(smem)[threadIdx.x] = make_uint4(0, 0, 0, 0);
     __syncthreads();
+    if constexpr (kAgg) pdl_trigger();            // the finish launch
+    pdl_wait();                                   // the offsets, and everything before them
     // chunk tickets two deep: while one chunk is decoded the next one's record is fetched, and the
     // ticket of the one after that is on its way (read, and its position loads issued, when this
     // chunk is done)
     constexpr bool kTable = kDt == kDtMixed;
-    uint64_t tn = ticket_of(take_ticket(ctl, kTicketDecode, lane));
+    const Tickets tickets{ctl, kTicketDecode, total_chunks};
+    uint64_t tn = tickets.first();
     if (tn >= total_chunks) return;
     Rec rec = issue_record(locate<kTable>(jobs, njobs, s_single, tn, total_chunks), wbase, lane);
     cp_async_commit();
-    tn = ticket_of(take_ticket(ctl, kTicketDecode, lane));
+    tn = tickets.chunk(tickets.draw(lane));
     Loc ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks);
     for (;;) {
-        const unsigned long long raw = take_ticket(ctl, kTicketDecode, lane);
+        const unsigned long long raw = tickets.draw(lane);
         cp_async_wait_none();                    // the current record has landed
         __syncwarp();
         // the next record goes into the same buffer once this one has been read
@@ -693,7 +698,7 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
         else decode_chunk<kD16, L, kAgg, kTable>(rec, s_single, smem, wofs, seltab, lane, next, ctl);
         if (tn >= total_chunks) break;
         rec = rn;
-        tn = ticket_of(raw);
+        tn = tickets.chunk(raw);
         ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks);
     }
     cp_async_wait_none();
@@ -713,6 +718,7 @@ int decompress_grid(uint64_t total_chunks) {
 __global__ void __launch_bounds__(1024)
 aggregate_finish_kernel(Job single, Control *ctl, falcon_stats *out) {
     __shared__ double part[1024];
+    pdl_wait();
     const uint64_t nc = single.nchunks;
     const double *sums = reinterpret_cast<const double *>(single.flags + nc);
     const uint64_t c0 = nc * threadIdx.x / 1024u, c1 = nc * (threadIdx.x + 1u) / 1024u;
@@ -745,7 +751,7 @@ void launch_decode(const Job *d_jobs, int njobs, const Job &single, uint64_t tot
     const int w = g_cta_warps[1], smem = (int)(kZeroBytes + w * DecLayout<layout_kind<kDt>()>::kWarpBytes);
     const int grid = persistent_grid_size(reinterpret_cast<const void *>(decompress_kernel<kDt, kAgg>), w, smem,
                                           g_ctas_per_sm[1], total_chunks);
-    decompress_kernel<kDt, kAgg><<<grid, 32 * w, smem, stream>>>(d_jobs, njobs, single, total_chunks, ctl);
+    (void)launch_after(decompress_kernel<kDt, kAgg>, grid, 32 * w, smem, stream, d_jobs, njobs, single, total_chunks, ctl);
 }
 }  // namespace
 
@@ -756,7 +762,10 @@ void launch_offsets(const Job *d_jobs, int njobs, const Job &single, int which, 
         const uint64_t steps = (single.nchunks + 1023u) / 1024u;
         parts = steps < 1u ? 1u : (steps > 152u ? 152u : (uint32_t)steps);
     }
-    offsets_kernel<<<(unsigned)njobs * parts, 1024, 0, stream>>>(d_jobs, single, parts, which, ctl);
+    // compression's follows the analysis; decompression's is the first launch of the call, after whatever
+    // the caller has enqueued
+    if (which == kOffsetsOfOutput) (void)launch_after(offsets_kernel, njobs * (int)parts, 1024, 0, stream, d_jobs, single, parts, which, ctl);
+    else offsets_kernel<<<(unsigned)njobs * parts, 1024, 0, stream>>>(d_jobs, single, parts, which, ctl);
 }
 
 cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cudaStream_t stream) {
@@ -766,7 +775,7 @@ cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cud
         else if (single.dtype == 1) launch_decode<kDtF32, true>(nullptr, 1, single, single.nchunks, ctl, stream);
         else launch_decode<kDtF16, true>(nullptr, 1, single, single.nchunks, ctl, stream);
     }
-    aggregate_finish_kernel<<<1, 1024, 0, stream>>>(single, ctl, static_cast<falcon_stats *>(d_stats));
+    (void)launch_after(aggregate_finish_kernel, 1, 1024, 0, stream, single, ctl, static_cast<falcon_stats *>(d_stats));
     return cudaGetLastError();
 }
 

@@ -76,6 +76,12 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_none() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+// Programmatic dependent launch: a kernel launched with launch_after (falcon_internal.h) may start once
+// every CTA of the kernel before it has called pdl_trigger or ended; after pdl_wait that kernel, and
+// with it all before it, has completed and its writes are visible.  Nothing global is touched earlier.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Bulk (TMA) copy of `bytes` from shared to global memory, both 16-byte aligned, bytes a
 // multiple of 16, tracked in the issuing thread's bulk groups.  The writers of the shared
 // bytes must have executed fence_proxy_async() first.
@@ -670,21 +676,30 @@ __device__ __forceinline__ int find_job(const Job *jobs, int njobs, uint64_t t) 
     return lo;
 }
 
-// Chunk tickets (Control): take_ticket issues lane 0's atomic add and returns its raw result
-// (valid in lane 0 only); ticket_of broadcasts it.  Issuing the atomic a chunk before its result
-// is read hides the atomic's latency behind the current chunk; the add is predicated on lane 0
-// into a register zeroed beforehand, so no instruction selects between the two and waits for it.
-__device__ __forceinline__ unsigned long long take_ticket(Control *ctl, int which, int lane) {
-    unsigned long long r;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %1, 0;\n\tmov.b64 %0, 0;\n\t"
-        "@p atom.global.add.u64 %0, [%2], 1;\n\t}"
-        : "=l"(r)
-        : "r"(lane), "l"(&ctl->ticket[which])
-        : "memory");
-    return r;
-}
-__device__ __forceinline__ uint64_t ticket_of(unsigned long long raw) { return shfl_u64(raw, 0); }
+// Chunk hand-out (Control).  A warp's first chunk is the one of its own number; tickets, drawn by
+// one atomic add each, hand out the rest, so a grid with a warp for every chunk draws none (and nobody
+// has to reset its counter).  draw issues lane 0's atomic and returns its raw result (valid in lane 0
+// only); chunk broadcasts it.  Issuing the atomic a chunk before its result is read hides its latency
+// behind the current chunk; the add is predicated into a register set beforehand, so no instruction
+// selects between the two and waits for it.
+struct Tickets {
+    Control *ctl;
+    int which;
+    uint64_t total;
+    __device__ __forceinline__ uint32_t warps() const { return gridDim.x * (blockDim.x >> 5); }
+    __device__ __forceinline__ uint64_t first() const { return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
+    __device__ __forceinline__ unsigned long long draw(int lane) const {
+        unsigned long long r;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %1, 0;\n\tmov.b64 %0, %3;\n\t"
+            "@p atom.global.add.u64 %0, [%2], 1;\n\t}"
+            : "=l"(r)
+            : "r"((int)(lane == 0 && warps() < total)), "l"(&ctl->ticket[which]), "l"(total)
+            : "memory");
+        return r;
+    }
+    __device__ __forceinline__ uint64_t chunk(unsigned long long raw) const { return warps() + shfl_u64(raw, 0); }
+};
 
 __device__ __forceinline__ uint32_t chunk_cols(uint32_t m) { return m <= 1 ? 0u : ((m - 1u + 63u) & ~63u); }
 

@@ -41,8 +41,9 @@ struct Job {
 // row dense, Elf's trial-and-error decimal place).  All write the same record layout.
 enum : uint32_t { kVariantFalcon = 0, kVariantSparse = 1, kVariantDense = 2, kVariantElf = 3 };
 
-// Per-launch control block at the start of the workspace (zero before the analysis: the callers of
-// launch_compress reset it; reset by the offsets launch for decompression):
+// Per-launch control block at the start of the workspace (reset by launch_compress where its launches
+// draw tickets, by the offsets launch for decompression; the launches write every other word they read,
+// and the results):
 // the chunk tickets of the persistent kernels.  A warp takes its next chunk with one atomic
 // add on its kernel's counter (analysis, emit, decode), so warps that met cheaper chunks take
 // more of them and a launch ends with its average warp, not its unluckiest one.
@@ -101,6 +102,23 @@ extern int g_cta_warps[2];
 // Persistent grid of a kernel with `warps` warps per CTA and smem_bytes dynamic shared memory:
 // as many CTAs as fit (at most lim per SM when lim > 0), fewer when there is less work.
 int persistent_grid_size(const void *kernel, int warps, int smem_bytes, int lim, uint64_t total_chunks);
+
+// Launches a kernel whose CTAs may be placed, and run up to their pdl_wait, while the kernel enqueued
+// before it on the stream drains: the launch's latency and the first instruction fetches overlap it.
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), int grid, int threads, int smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 // Grid size used for a launch over total_chunks work items (persistent, occupancy-bound).
 int compress_grid(uint64_t total_chunks);

@@ -279,7 +279,6 @@ struct falcon_server {
         if (cudaStreamWaitEvent(cs, s.up, 0) != cudaSuccess) return FALCON_ERR_CUDA;
         if (cudaMemcpyAsync(d_jobs(s), s.h_jobs, sizeof(Job) * (size_t)count, cudaMemcpyHostToDevice, cs) != cudaSuccess)
             return FALCON_ERR_CUDA;
-        if (g.op == FALCON_COMPRESS && cudaMemsetAsync(s.d_area, 0, sizeof(Control), cs) != cudaSuccess) return FALCON_ERR_CUDA;
         Job dummy{};
         auto *ctl = reinterpret_cast<Control *>(s.d_area);
         const cudaError_t e = g.op == FALCON_COMPRESS ? launch_compress(d_jobs(s), count, dummy, total, ctl, cs)
