@@ -151,8 +151,8 @@ __device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, ui
             if (have[i] && (uint32_t)lane < p[i]) mine = sum;
             if (have[i] && maps) bm[at] = (uint8_t)(pair >> (8 * i));
             const uint32_t packed = __byte_perm(x[i], 0u, __shfl_sync(kFull, seltab, (int)(nibs >> (8 * i))));
-            const uint32_t n = (c >> (8 * i)) & 7u;
             uint8_t *q = rec + at + bm_bytes + ((excl >> (8 * i)) & 255u);
+            const uint32_t n = (c >> (8 * i)) & 7u;
 #pragma unroll
             for (int t = 0; t < 4; ++t)
                 if (n > (uint32_t)t) q[t] = (uint8_t)(packed >> (8 * t));
@@ -809,16 +809,12 @@ __device__ __forceinline__ void load_chunk(const Job &job, uint64_t c, int lane,
     vx = (m > 1024u && lane == 31) ? __ldg(reinterpret_cast<const U *>(src) + 1024) : v[31];
 }
 
-// Launch 2, one chunk: G, Z and the plane words again (alpha and w from the analysis), then
-// the record at its offset.  meta / dense: the chunk's workspace words; size: its record size;
-// rel: its record offset relative to the first record.  With kPre the chunk's values arrive in
-// v / vx, loaded during the previous chunk, and `next` loads the following chunk's into them
-// as soon as the plane words are in shared memory (the register loads then complete while
-// this record is assembled); otherwise the values are loaded here and `next` does nothing.
-template <int D, bool kWide, bool kPre, class Next>
+// Emit, one chunk: G and its deltas again (alpha and w from the analysis), their planes, and the record at
+// its offset.  word / dense: the chunk's workspace words; size: its record size; rel: its record offset
+// relative to the first record.
+template <int D, bool kWide>
 __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *buf, uint32_t seltab, int lane,
-                                           uint64_t word, uint64_t dense, uint32_t size, uint64_t rel,
-                                           typename Traits<D>::U (&v)[32], typename Traits<D>::U &vx, Next &&next) {
+                                           uint64_t word, uint64_t dense, uint32_t size, uint64_t rel) {
     using T = Traits<D>;
     using U = typename T::U;
     using L = EmitLayout<D, kWide>;
@@ -829,10 +825,7 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     const uint32_t mb = (uint32_t)(word >> kMetaShift);
     const int alpha_byte = (int)(mb >> 12), beta_hat = (int)((mb >> 7) & 31u), w = (int)(mb & 127u);
     const uint64_t rec_off = data_start + rel;
-    if (rec_off + size > job.out_cap) {          // the job's first chunk reports the capacity error
-        next();
-        return;
-    }
+    if (rec_off + size > job.out_cap) return;    // the job's first chunk reports the capacity error
 
     // ---- planes (Sec. 3.3) and record -----------------------------------------------------------
     // The zigzag is done on the planes: plane p of Z is plane p - 1 of the deltas XOR their sign
@@ -863,7 +856,8 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     constexpr int R = T::W < 32 ? T::W : 32;
     uint32_t a[32];                               // the deltas' low words, transposed below
     // G (Eq. 4) and its deltas (Eq. 5)
-    if constexpr (!kPre) load_chunk<D>(job, c, lane, v, vx);
+    U v[32], vx;
+    load_chunk<D>(job, c, lane, v, vx);
     if (D == kD64 && alpha_byte != T::A_SENT && beta_hat <= kNarrowBeta) {
         // Case 1 with |g| < 10^8: 32-bit arithmetic throughout (and w <= 32)
         const Case1Narrow q = case1_narrow_of(alpha_byte);
@@ -934,7 +928,6 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
         low_planes();
         if (lane == 0) bulk_wait_read();
         __syncwarp();
-        next();                                   // v and vx are free
         header();
         half_rows(0);
     }
@@ -1082,9 +1075,8 @@ __device__ __forceinline__ EmitInfo<kTable, Mask> load_info(const Job *jobs, int
     return e;
 }
 
-// Launch 2: the records (chunks by ticket; the next chunk's values are loaded into registers
-// during the current one in the FP32 and FP16 forms, prefetched into L2 in the FP64 and
-// either-dtype forms).
+// The records (chunks by ticket; the next chunk's values are prefetched into L2: FP32 loading them into
+// registers during the current record left 20 warps per SM instead of 24 and took 234 us against 225).
 template <bool kWide, int kDt>
 __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njobs, const Job &s_single,
                                           uint64_t total_chunks, bool direct, Control *ctl, uint8_t *smem) {
@@ -1108,48 +1100,28 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
             }
         }
     }
-    // the FP32 and FP16 forms keep the values of the chunk after the current one in registers
-    // (kPre); the FP64 form has no registers to spare for them
-    constexpr bool kPre = kDt == kDtF32 || kDt == kDtF16;
-    typename Traits<DL>::U v[32], vx;
     const Tickets tickets{ctl, kTicketEmit, total_chunks};
     uint64_t t = tickets.first();
     if (t >= total_chunks) return;
-    using Mask = typename std::conditional<kPre, uint32_t, unsigned long long>::type;
+    using Mask = typename std::conditional<DL == kD64, unsigned long long, uint32_t>::type;
     auto info = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
-    if constexpr (kPre) load_chunk<DL>(*info.job, info.c, lane, v, vx);
     t = tickets.chunk(tickets.draw(lane));       // the next chunk
     for (;;) {
         // the ticket after t, read at the next iteration; t's workspace words are fetched now
         const unsigned long long raw = tickets.draw(lane);
         const auto next = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
-        if constexpr (!kPre) {
-            if (t < total_chunks) prefetch_chunk(*next.job, next.c, lane);
-        }
+        if (t < total_chunks) prefetch_chunk(*next.job, next.c, lane);
         const Job &job = *info.job;
         const bool dir = !kTable && direct;
         const uint64_t rel = dir ? sizes_before(job, info.c, lane) : (info.word & kOffsetMask);
         if (info.c == 0) finish_job(job, dir, lane);
-        auto load_next = [&]() {
-            if constexpr (kPre) {
-                if (t < total_chunks) load_chunk<DL>(*next.job, next.c, lane, v, vx);
-            }
+        auto emit = [&](auto kind) {
+            emit_chunk<decltype(kind)::value, kWide>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel);
         };
-        if constexpr (kPre) {
-            emit_chunk<DL, kWide, true>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, v, vx, load_next);
-        } else if constexpr (kDt == kDtF64) {
-            uint64_t u[32], ux;
-            emit_chunk<kD64, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
-        } else if (job.dtype == 0) {
-            uint64_t u[32], ux;
-            emit_chunk<kD64, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
-        } else if (job.dtype == 1) {
-            uint32_t u[32], ux;
-            emit_chunk<kD32, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
-        } else {
-            uint16_t u[32], ux;
-            emit_chunk<kD16, kWide, false>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel, u, ux, load_next);
-        }
+        if constexpr (!kTable) emit(std::integral_constant<int, DL>{});
+        else if (job.dtype == 0) emit(std::integral_constant<int, kD64>{});
+        else if (job.dtype == 1) emit(std::integral_constant<int, kD32>{});
+        else emit(std::integral_constant<int, kD16>{});
         __syncwarp();
         if (t >= total_chunks) break;
         t = tickets.chunk(raw);
@@ -1158,23 +1130,10 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
     if (lane == 0) bulk_wait();
 }
 
-// FP64 and either-dtype forms (up to 128 registers, 16 warps per SM)
+// FP64 and either-dtype forms: 128 registers, 16 warps per SM; FP32 and FP16: 80 and 24.
 template <bool kWide, int kDt>
-__global__ void __launch_bounds__(32 * kMaxCompressWarps, 1)
+__global__ void __maxnreg__(kDt == kDtF32 || kDt == kDtF16 ? 80 : 128)
 emit_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, bool direct, Control *ctl) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ Job s_single;
-    if (threadIdx.x == 0) s_single = single;
-    __syncthreads();
-    pdl_wait();
-    emit_loop<kWide, kDt>(jobs, njobs, s_single, total_chunks, direct, ctl, smem);
-}
-
-// FP32 and FP16 forms: held to 96 registers (FP32 needs 96 without spilling), so that 20 warps
-// fit an SM
-template <bool kWide, int kDt>
-__global__ void __maxnreg__(96)
-emit_kernel_narrow(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, bool direct, Control *ctl) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ Job s_single;
     if (threadIdx.x == 0) s_single = single;
@@ -1201,10 +1160,7 @@ template <int kDt> auto analyse_shape(uint64_t total_chunks) {
 }
 template <bool kWide, int kDt> auto emit_shape(uint64_t total_chunks) {
     const int w = g_cta_warps[0], smem = w * (int)EmitLayout<kind_of<kDt>(), kWide>::kBytes;
-    auto *k = [] {
-        if constexpr (kDt == kDtF32 || kDt == kDtF16) return emit_kernel_narrow<kWide, kDt>;
-        else return emit_kernel<kWide, kDt>;
-    }();
+    auto *k = emit_kernel<kWide, kDt>;
     return Shape<decltype(k)>{k, 32 * w, smem,
                               persistent_grid_of(reinterpret_cast<const void *>(k), w, smem, g_ctas_per_sm[0], total_chunks)};
 }

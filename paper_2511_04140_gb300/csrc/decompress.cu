@@ -654,7 +654,7 @@ template <int kDt> constexpr int layout_kind() { return kDt == kDtF32 ? kD32 : (
 // Registers: 128 (FP64, either-dtype: 16 warps per SM), 80 (FP32, FP16: 24 warps; 96 registers and
 // 20 warps: 1.3 % slower).  The aggregate forms keep FP64 sums as well and take 168.
 template <int kDt, bool kAgg = false>
-__global__ void __maxnreg__((kDt == kDtF32 || kDt == kDtF16) && !kAgg ? 80 : (kAgg ? 168 : 128))
+__global__ void __maxnreg__((kDt == kDtF32 || kDt == kDtF16) && !kAgg ? 80 : (kAgg ? (kDt == kDtF64 ? 168 : 128) : 128))
 decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
