@@ -340,9 +340,10 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
 #pragma unroll
         for (int k = 0; k < PER; ++k) x.e[k] = one(x.e[k]);
         *q = x.w;
+        if (!__all_sync(kFull, ok)) return false;
     }
     stop = __any_sync(kFull, early);
-    return __all_sync(kFull, ok);
+    return true;
 }
 
 // Smallest a in [0, atop] at which every value passes the round-trip test, or -1 (Case 2).
@@ -510,6 +511,11 @@ template <int D> struct Mag {
 // `low`, some value with a zero exponent field.  Returns alpha_max | beta_hat << 8, alpha_max = 31
 // in Case 2; the staging buffer holds G on a Case 1 return, the values otherwise.
 constexpr int kCase2 = 31;
+// the value a lane's FP64 key stands for
+template <int D>
+__device__ __forceinline__ typename Traits<D>::U lane_max(const uint8_t *buf, int lane, uint32_t key) {
+    return read_elem<D>(buf, 32u * (uint32_t)lane + (key & 63u)) & Mag<D>::ABS;
+}
 template <int D>
 __device__ __forceinline__ int case_decision(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, uint32_t kmax,
                                              uint32_t top, bool low, bool elf) {
@@ -551,9 +557,15 @@ __device__ __forceinline__ int case_decision(const uint8_t *src, uint8_t *buf, i
         }
     }
     const int atop = min(T::A_MAX, T::B_MAX - 1 - e_max);
-    // quick rejection: Alg. 2's round trip on the largest magnitude first (the test reads
-    // only |v|, so it runs on vmax itself, the same in every lane)
-    if (!elf && (atop < 0 || !q_test(vmax, atop))) return kNone;
+    // quick rejection: Alg. 2's round trip on every lane's largest magnitude first (the test reads only
+    // |v|).  One outlier that happens to pass does not send its chunk through the search: a few such
+    // chunks, each worth a hundred others, made a launch's tail (2^24 values: 55 us of analysis against 33).
+    if (!elf) {
+        U own;
+        if constexpr (D == kD64) own = lane_max<D>(buf, lane, kmax);
+        else own = (U)kmax;
+        if (atop < 0 || !__all_sync(kFull, q_test(own, atop))) return kNone;
+    }
     const int alpha = case1_alpha<D>(src, buf, lane, m, e_max, atop, vmax, elf);
     return alpha < 0 ? kNone : alpha | ((alpha + e_max + 1) << 8);
 }
@@ -600,17 +612,29 @@ __device__ __forceinline__ void analyse_chunk(const Job &job, uint64_t c, uint8_
     // Three-input maxima and minima over the keys settle the special values: exponent all ones iff
     // the maximum says so; a zero exponent field (rare but for zeros) is looked at again.
     pad_values<D>(buf, m, lane);
-    constexpr int UN = T::UNITS, PER = 32 / UN;
-    uint32_t kmax = 0, kmin = ~0u;
-#pragma unroll 4
-    for (int u = 0; u < UN; ++u) {
-        union { uint4 w; U e[PER]; } x;
-        x.w = *reinterpret_cast<const uint4 *>(buf + (lane * UN + unit_swizzle<D>(lane, u)) * 16);
+    constexpr int UN = T::UNITS, PER = 32 / UN, GU = UN / 4;         // 16-byte units; of 8 values
+    // unit GU i + u of this lane: the swizzle splits into a part for i and one for u
+    const uint32_t key_bits = D == kD16 ? ((uint32_t)lane >> 1) & 3u : (uint32_t)lane & 7u;
+    const uint8_t *own = buf + lane * (UN * 16);
+    auto group = [&](int i) { return ((GU * (uint32_t)i) ^ (key_bits & ~(GU - 1u))) * 16u; };
+    uint32_t low_unit[GU];
 #pragma unroll
-        for (int k = 0; k < PER; k += 2) {
-            const uint32_t a = Mag<D>::key(x.e[k], u * PER + k), b = Mag<D>::key(x.e[k + 1], u * PER + k + 1);
-            kmax = __vimax3_u32(kmax, a, b);
-            kmin = __vimin3_u32(kmin, a, b);
+    for (int u = 0; u < GU; ++u) low_unit[u] = ((uint32_t)u ^ (key_bits & (GU - 1u))) * 16u;
+    uint32_t kmax = 0, kmin = ~0u;
+#pragma unroll 2
+    for (int i = 0; i < 4; ++i) {
+        const uint8_t *at = own + group(i);
+#pragma unroll
+        for (int u = 0; u < GU; ++u) {
+            union { uint4 w; U e[PER]; } x;
+            x.w = *reinterpret_cast<const uint4 *>(at + low_unit[u]);
+#pragma unroll
+            for (int k = 0; k < PER; k += 2) {
+                const uint32_t n = (uint32_t)(8 * i + u * PER + k);
+                const uint32_t a = Mag<D>::key(x.e[k], n), b = Mag<D>::key(x.e[k + 1], n + 1);
+                kmax = __vimax3_u32(kmax, a, b);
+                kmin = __vimin3_u32(kmin, a, b);
+            }
         }
     }
     if (m > 1024u && lane == 31) {
@@ -632,36 +656,54 @@ __device__ __forceinline__ void analyse_chunk(const Job &job, uint64_t c, uint8_
     // ---- 2. G and |Z| by 8-column groups, w ----------------------------------------------------
     // o[i]: OR of the Z of columns 8 i .. 8 i + 7; Z = (x ^ s) << 1 | (s & 1) for the delta x with
     // sign s.  One group at a time (nine values in registers, not 32): 80 registers and 24 warps per SM.
+    // From the last group to the first, so that each hands its first value's G to the one before.
     U o[4] = {0, 0, 0, 0};
-    constexpr int GU = UN / 4;                   // 16-byte units per group
+    // the value after lane 31's last group: past the chunk's last value there is no further delta
+    U after = (lane == 31 && m <= 1024u) ? read_elem<D>(buf, 1023) : read_elem<D>(buf, 32u * lane + 32u);
+    if (!case1) after = zigzag(after);
 #pragma unroll 1
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 3; i >= 0; --i) {
+        const uint8_t *at = own + group(i);
         U g[9];
 #pragma unroll
         for (int u = 0; u < GU; ++u) {
             union { uint4 w; U e[PER]; } x;
-            x.w = *reinterpret_cast<const uint4 *>(buf + (lane * UN + unit_swizzle<D>(lane, i * GU + u)) * 16);
+            x.w = *reinterpret_cast<const uint4 *>(at + low_unit[u]);
 #pragma unroll
             for (int k = 0; k < PER; ++k) g[u * PER + k] = x.e[k];
         }
-        // the value after the group; past the chunk's last value there is no further delta
-        g[8] = (i == 3 && lane == 31 && m <= 1024u) ? g[7] : read_elem<D>(buf, 32u * lane + 8u * i + 8u);
         if (!case1) {
 #pragma unroll
-            for (int k = 0; k < 9; ++k) g[k] = zigzag(g[k]);
+            for (int k = 0; k < 8; ++k) g[k] = zigzag(g[k]);
         }
-        U mag = 0, neg = 0;
+        g[8] = after;
+        after = g[0];
+        uint32_t neg = 0;
+        o[3] = o[2];                             // the loop is rolled: the groups move up
+        o[2] = o[1];
+        o[1] = o[0];
+        if constexpr (D == kD64) {
+            uint32_t lo = 0, hi = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const U x = (U)(g[k + 1] - g[k]);
-            const U s = sign_mask(x);
-            mag |= x ^ s;
-            neg |= s;
+            for (int k = 0; k < 8; ++k) {
+                const uint64_t x = g[k + 1] - g[k];
+                const uint32_t xh = (uint32_t)(x >> 32), sg = (uint32_t)((int32_t)xh >> 31);
+                lo |= (uint32_t)x ^ sg;
+                hi |= xh ^ sg;
+                neg |= sg;
+            }
+            o[0] = ((uint64_t)__funnelshift_l(lo, hi, 1) << 32) | ((lo << 1) | (neg & 1u));
+        } else {
+            U mag = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const U x = (U)(g[k + 1] - g[k]);
+                const U sg = sign_mask(x);
+                mag |= x ^ sg;
+                neg |= sg;
+            }
+            o[0] = (U)((U)(mag << 1) | (neg & 1u));
         }
-        o[0] = o[1];                             // the loop is rolled: the groups move up
-        o[1] = o[2];
-        o[2] = o[3];
-        o[3] = (U)((U)(mag << 1) | (neg & 1u));
     }
     __syncwarp();
     next();                                     // the staged values have been read
