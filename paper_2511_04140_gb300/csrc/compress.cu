@@ -570,14 +570,18 @@ __device__ __forceinline__ int case_decision(const uint8_t *src, uint8_t *buf, i
     return alpha < 0 ? kNone : alpha | ((alpha + e_max + 1) << 8);
 }
 
-__device__ __forceinline__ void issue_chunk(const Job *jobs, int njobs, const Job &single, uint64_t t,
-                                            uint8_t *buf, int lane) {
-    const Job &job = (jobs == nullptr) ? single : jobs[find_job(jobs, njobs, t)];
-    const uint64_t c = t - job.chunk_begin;
+__device__ __forceinline__ uint32_t values_in(const Job &job, uint64_t c) {
+    const uint64_t left = job.n - c * (uint64_t)job.block;
+    return (uint32_t)(left < job.block ? left : job.block);
+}
+
+// Starts the copy of chunk c's values; kD: the kind, or -1 for the job's own.
+template <int kD>
+__device__ __forceinline__ void issue_chunk(const Job &job, uint64_t c, uint8_t *buf, int lane) {
     const uint64_t first = c * (uint64_t)job.block;
-    const uint32_t m = (uint32_t)((job.n - first) < job.block ? (job.n - first) : job.block);
-    if (job.dtype == 0) stage_values_async<kD64>(job.in + first * 8u, m, buf, lane);
-    else if (job.dtype == 1) stage_values_async<kD32>(job.in + first * 4u, m, buf, lane);
+    const uint32_t m = values_in(job, c);
+    if (kD == kD64 || (kD < 0 && job.dtype == 0)) stage_values_async<kD64>(job.in + first * 8u, m, buf, lane);
+    else if (kD == kD32 || (kD < 0 && job.dtype == 1)) stage_values_async<kD32>(job.in + first * 4u, m, buf, lane);
     else stage_values_async<kD16>(job.in + first * 2u, m, buf, lane);
 }
 
@@ -1005,10 +1009,6 @@ constexpr int kDtF64 = 0, kDtF32 = 1, kDtMixed = 2, kDtF16 = 3;
 // 4 KB of sizes each, one round trip, where the launch costs about 3 us.
 constexpr uint64_t kDirectChunks = 1024;
 
-__device__ __forceinline__ const Job &job_of(const Job *jobs, int njobs, const Job &single, uint64_t t) {
-    return (jobs == nullptr) ? single : jobs[find_job(jobs, njobs, t)];
-}
-
 }  // namespace
 
 // Launch 1: analysis of every chunk (chunks by ticket; the next chunk is copied into
@@ -1024,32 +1024,40 @@ __device__ __forceinline__ void analyse_loop(const Job *__restrict__ jobs, int n
     if (threadIdx.x == 0) s_single = single;
     pdl_trigger();
     __syncthreads();
+    constexpr bool kTable = kDt == kDtMixed;
+    constexpr int kD = kTable ? -1 : (kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64));
     const Tickets tickets{ctl, kTicketAnalyse, total_chunks};
     uint64_t t = tickets.first();
     if (t >= total_chunks) return;
-    issue_chunk(jobs, njobs, s_single, t, wbase, lane);
+    const Job *job = kTable ? find_job(jobs, njobs, t, lane) : &s_single;
+    issue_chunk<kD>(*job, kTable ? t - job->chunk_begin : t, wbase, lane);
     cp_async_commit();
     for (;;) {
         const unsigned long long raw = tickets.draw(lane);       // the chunk after t
         uint64_t tn = total_chunks;
+        const Job *jn = job;
         cp_async_wait_none();                    // the current chunk has landed
         __syncwarp();
         auto next = [&]() {
             tn = tickets.chunk(raw);
-            if (tn < total_chunks) issue_chunk(jobs, njobs, s_single, tn, wbase, lane);
+            if (tn < total_chunks) {
+                if (kTable) jn = find_job(jobs, njobs, tn, lane);
+                issue_chunk<kD>(kTable ? *jn : s_single, kTable ? tn - jn->chunk_begin : tn, wbase, lane);
+            }
             cp_async_commit();
         };
-        const Job &job = job_of(jobs, njobs, s_single, t);
-        const uint64_t c = t - job.chunk_begin;
-        if constexpr (kDt == kDtF64) analyse_chunk<kD64>(job, c, wbase, lane, next);
-        else if constexpr (kDt == kDtF32) analyse_chunk<kD32>(job, c, wbase, lane, next);
-        else if constexpr (kDt == kDtF16) analyse_chunk<kD16>(job, c, wbase, lane, next);
-        else if (job.dtype == 0) analyse_chunk<kD64>(job, c, wbase, lane, next);
-        else if (job.dtype == 1) analyse_chunk<kD32>(job, c, wbase, lane, next);
-        else analyse_chunk<kD16>(job, c, wbase, lane, next);
+        if constexpr (!kTable) {
+            analyse_chunk<kD>(s_single, t, wbase, lane, next);
+        } else {
+            const uint64_t c = t - job->chunk_begin;
+            if (job->dtype == 0) analyse_chunk<kD64>(*job, c, wbase, lane, next);
+            else if (job->dtype == 1) analyse_chunk<kD32>(*job, c, wbase, lane, next);
+            else analyse_chunk<kD16>(*job, c, wbase, lane, next);
+        }
         __syncwarp();
         if (tn >= total_chunks) break;
         t = tn;
+        job = jn;
     }
     cp_async_wait_none();
 }
@@ -1106,10 +1114,11 @@ template <bool kTable, class Mask> struct EmitInfo {
     uint32_t size;
 };
 template <bool kTable, class Mask>
-__device__ __forceinline__ EmitInfo<kTable, Mask> load_info(const Job *jobs, int njobs, const Job &single, uint64_t t, uint64_t total_chunks) {
+__device__ __forceinline__ EmitInfo<kTable, Mask> load_info(const Job *jobs, int njobs, const Job &single, uint64_t t, uint64_t total_chunks,
+                                                            int lane) {
     EmitInfo<kTable, Mask> e;
     t = t < total_chunks ? t : total_chunks - 1u;
-    e.job = kTable ? jobs + find_job(jobs, njobs, t) : &single;
+    e.job = kTable ? find_job(jobs, njobs, t, lane) : &single;
     e.c = kTable ? t - e.job->chunk_begin : t;
     e.word = e.job->flags[e.c];
     e.dense = *reinterpret_cast<const Mask *>(e.job->flags + e.job->nchunks + e.c);
@@ -1146,12 +1155,12 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
     uint64_t t = tickets.first();
     if (t >= total_chunks) return;
     using Mask = typename std::conditional<DL == kD64, unsigned long long, uint32_t>::type;
-    auto info = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
+    auto info = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks, lane);
     t = tickets.chunk(tickets.draw(lane));       // the next chunk
     for (;;) {
         // the ticket after t, read at the next iteration; t's workspace words are fetched now
         const unsigned long long raw = tickets.draw(lane);
-        const auto next = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks);
+        const auto next = load_info<kTable, Mask>(jobs, njobs, s_single, t, total_chunks, lane);
         if (t < total_chunks) prefetch_chunk(*next.job, next.c, lane);
         const Job &job = *info.job;
         const bool dir = !kTable && direct;

@@ -115,10 +115,11 @@ struct Loc {
 // Forms for one job (a single stream) read it from shared memory; the either-dtype form finds
 // the ticket's job in the table.
 template <bool kTable>
-__device__ __forceinline__ Loc locate(const Job *jobs, int njobs, const Job &single, uint64_t t, uint64_t total_chunks) {
+__device__ __forceinline__ Loc locate(const Job *jobs, int njobs, const Job &single, uint64_t t, uint64_t total_chunks,
+                                      int lane) {
     Loc l;
     t = t < total_chunks ? t : total_chunks - 1u;
-    l.job = kTable ? jobs + find_job(jobs, njobs, t) : &single;
+    l.job = kTable ? find_job(jobs, njobs, t, lane) : &single;
     l.c = kTable ? t - l.job->chunk_begin : t;
     l.off = l.job->flags[l.c];
     l.size = reinterpret_cast<const uint32_t *>(l.job->in + 32)[l.c];
@@ -676,10 +677,10 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
     const Tickets tickets{ctl, kTicketDecode, total_chunks};
     uint64_t tn = tickets.first();
     if (tn >= total_chunks) return;
-    Rec rec = issue_record(locate<kTable>(jobs, njobs, s_single, tn, total_chunks), wbase, lane);
+    Rec rec = issue_record(locate<kTable>(jobs, njobs, s_single, tn, total_chunks, lane), wbase, lane);
     cp_async_commit();
     tn = tickets.chunk(tickets.draw(lane));
-    Loc ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks);
+    Loc ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks, lane);
     for (;;) {
         const unsigned long long raw = tickets.draw(lane);
         cp_async_wait_none();                    // the current record has landed
@@ -699,7 +700,7 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
         if (tn >= total_chunks) break;
         rec = rn;
         tn = tickets.chunk(raw);
-        ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks);
+        ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks, lane);
     }
     cp_async_wait_none();
 }

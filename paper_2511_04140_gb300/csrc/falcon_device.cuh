@@ -665,15 +665,18 @@ __device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t &t
     return r;
 }
 
-// Finds the job that owns global ticket t (jobs sorted by chunk_begin).
-__device__ __forceinline__ int find_job(const Job *jobs, int njobs, uint64_t t) {
-    int lo = 0, hi = njobs - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (jobs[mid].chunk_begin <= t) lo = mid;
-        else hi = mid - 1;
+// Finds the job that owns global chunk t (jobs sorted by chunk_begin), the whole warp probing 32
+// places at a time: two dependent loads for a thousand jobs instead of ten.
+__device__ __forceinline__ const Job *find_job(const Job *jobs, int njobs, uint64_t t, int lane) {
+    int lo = 0, n = njobs;                        // the owner lies in [lo, lo + n)
+    while (n > 1) {
+        const int step = (n + 31) / 32, i = lane * step;
+        const unsigned le = __ballot_sync(kFull, i < n && jobs[lo + (i < n ? i : 0)].chunk_begin <= t);
+        const int k = (31 - __clz((int)le)) * step;       // the last probe that begins at or before t
+        lo += k;
+        n = min(step, n - k);
     }
-    return lo;
+    return jobs + lo;
 }
 
 // Chunk hand-out (Control).  A warp's first chunk is the one of its own number; tickets, drawn by
