@@ -178,53 +178,53 @@ __device__ __forceinline__ Rec issue_record(const Loc &l, uint8_t *rbuf, int lan
 // one unaligned word, spread by one byte permute.  No position is checked: a row takes at most
 // 16 + 128 bytes, so every read stays in the record buffer whatever the bytes say, and the caller's
 // size check rejects a malformed record before anything is stored.
+// `line` is where plane 0's row would lie if every row below the sparse ones met so far were dense, so
+// plane q's row is at line - row_bytes * q and a sparse row moves it by its length less row_bytes.
 struct RowLane {                                  // per-lane constants of a chunk's row walk
-    uint32_t keep;                                // bitmap bits of this lane's group that exist
+    uint32_t keep;                                // bits of this lane's bitmap word that exist
     uint32_t before;                              // those of the lanes before this one
     uint32_t seltab;                              // expand_sel(lane & 15)
 };
 __device__ __forceinline__ void place_rows(uint8_t *smem, uint32_t slots, uint32_t tab, uint32_t &cur, uint32_t rows,
                                            uint32_t dense, uint32_t row_bytes, uint32_t bm_bytes, const RowLane &rl,
                                            int lane) {
-    const uint32_t start = cur;
-    const uint32_t group = (uint32_t)lane >> 3, gshift = 8u * group, nshift = 28u - 4u * ((uint32_t)lane & 7u);
+    // bitmap word of 8 lanes as it lies in memory: byte k covers lanes 2 k (high nibble) and 2 k + 1
+    const uint32_t group = (uint32_t)lane >> 3, gshift = 8u * group;
+    const uint32_t nshift = 8u * (((uint32_t)lane & 7u) >> 1) + ((lane & 1) ? 0u : 4u);
     const uint32_t presel = group ? 0x443Fu + group : 0x4444u;
+    const uint32_t step = bm_bytes - row_bytes;
     uint32_t sparse = rows & ~dense;
-    uint32_t sum = 0, mine = 0;                   // sparse bytes so far; above this lane's plane
-    uint32_t above = 32u - (uint32_t)__clz((int)rows);
+    uint32_t line = cur + row_bytes * ((uint32_t)__popc(rows) - 1u), mine = line;       // mine: for this lane's plane
+    uint8_t *own = smem + slots + 4u * lane;
     // the row before: its two words, shift, selector and slot (its store waits for none of this
     // row's loads; the first iteration stores zeros where the second puts the first row)
     uint32_t w0 = 0, w1 = 0, wsh = 0, sel = 0x4444u;
-    uint8_t *slot = smem + slots + 128u * (31u - (uint32_t)__clz((int)sparse)) + 4u * lane;
+    uint8_t *slot = own + 128u * (31u - (uint32_t)__clz((int)sparse));
     const bool any = sparse != 0u;
 #pragma unroll 1
     while (sparse) {
         const uint32_t p = 31u - (uint32_t)__clz((int)sparse);
         sparse ^= 1u << p;
-        cur += row_bytes * (above - 1u - p);      // the dense rows in between
-        above = p;
-        const uint32_t b = cur + 4u * group;
+        const uint32_t at = line - row_bytes * p, b = at + 4u * group;
         const uint32_t *bw = reinterpret_cast<const uint32_t *>(smem + (b & ~3u));
         const uint32_t b0 = bw[0], b1 = bw[1];
         *reinterpret_cast<uint32_t *>(slot) = __byte_perm(__funnelshift_r(w0, w1, wsh), 0u, sel);
-        const uint32_t W = bswap(__funnelshift_r(b0, b1, b * 8u)) & rl.keep;   // first row byte at bit 31
+        const uint32_t W = __funnelshift_r(b0, b1, b * 8u) & rl.keep;
         const uint32_t incl = __reduce_or_sync(kFull, (uint32_t)__popc(W) << gshift) * 0x01010101u;
-        const uint32_t total = incl >> 24;        // at most 128
-        const uint32_t at = cur + bm_bytes + __byte_perm(incl, 0u, presel) + (uint32_t)__popc(W & rl.before);
+        line += step + (incl >> 24);              // at most 128
+        const uint32_t q = at + bm_bytes + __byte_perm(incl, 0u, presel) + (uint32_t)__popc(W & rl.before);
         sel = __shfl_sync(kFull, rl.seltab, (int)(W >> nshift));
-        const uint32_t *aw = reinterpret_cast<const uint32_t *>(smem + (at & ~3u));
+        const uint32_t *aw = reinterpret_cast<const uint32_t *>(smem + (q & ~3u));
         w0 = aw[0];
         w1 = aw[1];
-        wsh = at * 8u;
-        slot = smem + slots + 128u * p + 4u * lane;
-        cur += bm_bytes + total;
-        sum += bm_bytes + total;
-        if ((uint32_t)lane < p) mine = sum;
+        wsh = q * 8u;
+        slot = own + 128u * p;
+        if ((uint32_t)lane < p) mine = line;
     }
     if (any) *reinterpret_cast<uint32_t *>(slot) = __byte_perm(__funnelshift_r(w0, w1, wsh), 0u, sel);
-    cur += row_bytes * above;
+    cur = line + row_bytes;
     const bool mine_dense = (dense >> lane) & 1u, exists = (rows >> lane) & 1u;
-    uint32_t a = start + row_bytes * (uint32_t)__popc((dense >> lane) >> 1) + mine;
+    uint32_t a = mine - row_bytes * (uint32_t)lane;
     a = mine_dense ? a : (exists ? slots + 128u * (uint32_t)lane : 0u);
     *reinterpret_cast<uint2 *>(smem + tab + 8u * lane) = make_uint2(a & ~3u, a * 8u);
 }
@@ -417,8 +417,9 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, const Job &single, u
     {
         const uint32_t nact = cols / 32u, g8 = (uint32_t)lane & ~7u;
         const uint32_t have = nact > g8 ? min(nact - g8, 8u) : 0u;          // lanes of this group with row bytes
-        rl.keep = have ? 0xFFFFFFFFu << (32u - 4u * have) : 0u;
-        rl.before = (lane & 7) ? 0xFFFFFFFFu << (32u - 4u * ((uint32_t)lane & 7u)) : 0u;
+        const uint32_t k8 = 8u * (((uint32_t)lane & 7u) >> 1);
+        rl.keep = have == 8u ? 0xFFFFFFFFu : (1u << (4u * have)) - 1u;       // `have` is even
+        rl.before = ((1u << k8) - 1u) | ((lane & 1) ? 0xF0u << k8 : 0u);
         rl.seltab = seltab;
     }
     uint32_t cur = rec + hdr;
