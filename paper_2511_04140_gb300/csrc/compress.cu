@@ -210,58 +210,73 @@ __device__ __forceinline__ bool all_pass(const uint8_t *buf, int lane, uint32_t 
 
 // Test and g of one value at decimal place a together (Eq. 4, Case 1): g = round(v 10^a) from one
 // 64-bit high product, then the exact distance |m 5^a - g 2^F| against 5^a / 2, modulo 2^64 (exact
-// while F <= 62, since g lies within one of v 10^a; smaller values take q_test).  Below a power of
-// two the interval is half as wide, which changes nothing: there m 5^a = 2^52 5^a, and its distance
-// to a multiple of 2^F is 0 or at least 2^52 > 5^a / 2.
+// while F <= 62, since g lies within one of v 10^a).  Below a power of two the interval is half as
+// wide, which changes nothing: there m 5^a = 2^52 5^a, and its distance to a multiple of 2^F is 0 or
+// at least 2^52 > 5^a / 2.  Other values but +0 (which passes, and whose g is 0 as the shift says) set
+// `slow` and are left to q_test, which stays out of the loop over the values.
 struct Case1At {                                  // constants of a decimal place
     uint64_t p5, norm;                            // 5^a, 5^a with its top bit at bit 63
     int f0, sh0;                                  // F = f0 - exponent field, shift = F + sh0
-    int a;
 };
 __device__ __forceinline__ Case1At case1_at(int a) {
-    return {FALCON_POW5[a], FALCON_POW5_NORM[a], 1075 - a, 10 - (int)FALCON_LOG2_POW5[a], a};
+    return {FALCON_POW5[a], FALCON_POW5_NORM[a], 1075 - a, 10 - (int)FALCON_LOG2_POW5[a]};
 }
-__device__ __forceinline__ uint64_t test_g(uint64_t u, const Case1At &c, bool &ok) {
+__device__ __forceinline__ uint64_t test_g(uint64_t u, const Case1At &c, bool &ok, uint32_t &slow) {
     const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
     const int F = c.f0 - (int)((hi >> 20) & 0x7FFu);
     const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
-    uint64_t N = case1_round(m, c.norm, F + c.sh0);
-    bool pass;
+    const uint64_t N = (shr_clamp64(__umul64hi(m << 11, c.norm), (uint32_t)(F + c.sh0 - 1)) + 1ull) >> 1;
     if (F > 62 || F <= 0) {
-        pass = q_test(u, c.a);
-        if ((u << 1) == 0) N = 0;
+        slow |= (hi << 1) | lo;
     } else {
         const uint64_t lim = c.p5 >> 1;
-        pass = (m * c.p5 - (N << F)) + lim <= 2u * lim;
+        ok &= (m * c.p5 - (N << F)) + lim <= 2u * lim;
     }
-    ok &= pass;
     return (hi >> 31) ? 0ull - N : N;
 }
-// the same for |g| < 10^8 and 5^a < 2^32
-__device__ __forceinline__ uint64_t test_g(uint64_t u, const Case1At &c, const Case1Narrow &q, bool &ok) {
-    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
-    const uint32_t N = case1_n_narrow(hi, lo, q);
-    const int F = c.f0 - (int)((hi >> 20) & 0x7FFu);
-    const uint32_t p5 = (uint32_t)c.p5, lim = p5 >> 1;
-    bool pass;
-    if (F > 62) {
-        pass = q_test(u, c.a);
-    } else {                                      // F >= 26: |v 10^a| < 2^27 and m 5^a >= 2^52
-        const uint64_t P = (uint64_t)lo * p5 + ((uint64_t)(((hi & 0xFFFFFu) | 0x100000u) * p5) << 32);
-        pass = P - ((uint64_t)N << F) + lim <= 2u * lim;
-    }
-    ok &= pass;
-    const uint32_t s = (uint32_t)((int32_t)hi >> 31);
-    return (uint64_t)(int64_t)(int32_t)((N ^ s) - s);
+// The same for |g| < 10^8 and 5^a < 2^31.  The product is scaled by 2^t so that F + t >= 32 (X < 10^8
+// and m >= 2^52 give F >= 26 + 2.3 a), which leaves g 2^F out of its low word; modulo 2^64 it is exact
+// while F + t <= 64: g then is the only multiple in reach.  (With q_test out of line, 40 M decimal values
+// at block 1025 compress in 367 us against 389 with both tests per value in 64-bit shifts; q_test in
+// line again: 379.)
+struct TestNarrow {
+    Case1Narrow g;
+    uint32_t p5, lim;                             // 2^t 5^a, 2^t floor(5^a / 2)
+    int c;                                        // F + t - 32 = c - exponent field
+};
+__device__ __forceinline__ TestNarrow test_narrow_of(int a) {
+    const int t = a < 3 ? 6 : 0;
+    const uint32_t p5 = (uint32_t)FALCON_POW5[a];
+    return {case1_narrow_of(a), p5 << t, (p5 >> 1) << t, 1075 - a + t - 32};
 }
-// FP32: the round trip |m 5^a - g 2^F| <= 5^a / 2 as in q_test (past F = 62 only +0 passes)
-__device__ __forceinline__ uint32_t test_g(uint32_t u, const Case1F32 &q, bool &ok) {
-    const uint32_t N = case1_n(u, q), e = (u >> 23) & 0xFFu;
-    const int F = q.f0 - (int)e;
-    const uint64_t P = (uint64_t)((u & 0x007FFFFFu) | 0x00800000u) * q.p5;
-    const uint32_t lim = q.p5 >> 1;
-    const bool near = P - ((uint64_t)N << (F & 63)) + lim <= 2u * lim;
-    ok &= F <= 0 || (F > 62 ? (u << 1) == 0u : near);
+__device__ __forceinline__ uint64_t test_g(uint64_t u, const TestNarrow &q, bool &ok, uint32_t &slow) {
+    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
+    const uint32_t N = case1_n_narrow(hi, lo, q.g);
+    const uint32_t f = (uint32_t)(q.c - (int)((hi >> 20) & 0x7FFu));
+    const uint64_t P = (uint64_t)lo * q.p5 + ((uint64_t)(((hi & 0xFFFFFu) | 0x100000u) * q.p5 - shl_clamp(N, f)) << 32);
+    if (f > 32u) slow |= (hi << 1) | lo;
+    else ok &= P + q.lim <= 2u * q.lim;
+    // a negative value with g = 0 has failed
+    const uint32_t s = (uint32_t)((int32_t)hi >> 31);
+    return ((uint64_t)s << 32) | ((N ^ s) - s);
+}
+// FP32: the round trip |m 5^a - g 2^F| <= 5^a / 2 as in q_test, on the normalised product m 2^8 5^a
+// 2^(31-d) that g comes from (g 2^F scaled alike is a multiple of 2^32, and exact modulo 2^64 up to
+// 2^64: past that, |v 10^a| < 1/2 and only +0 passes).
+struct TestF32 {
+    Case1F32 g;
+    uint64_t lim;                                 // floor(5^a / 2) scaled alike
+};
+__device__ __forceinline__ TestF32 test_f32_of(int a) {
+    const Case1F32 g = case1_f32_of(a);
+    return {g, (uint64_t)(g.p5 >> 1) << (39 - (int)FALCON_LOG2_POW5[a])};
+}
+__device__ __forceinline__ uint32_t test_g(uint32_t u, const TestF32 &q, bool &ok) {
+    const uint64_t P = (uint64_t)((u << 8) | 0x80000000u) * q.g.norm;
+    const uint32_t sh = (uint32_t)(q.g.c - (int)((u >> 23) & 0xFFu));        // the shift - 1, as in case1_n
+    const uint32_t N = (shr_clamp((uint32_t)(P >> 32), sh) + 1u) >> 1;
+    const bool near = P - ((uint64_t)shl_clamp(N, sh + 1u) << 32) + q.lim <= 2u * q.lim;
+    ok &= (near && sh < 32u) || (u << 1) == 0u;
     const uint32_t s = (uint32_t)((int32_t)u >> 31);
     return (N ^ s) - s;
 }
@@ -303,6 +318,9 @@ __device__ __forceinline__ bool may_stop_early(uint16_t u, int a) {
 __device__ __forceinline__ int first_pass(uint32_t u, int atop) { return first_pass_f32(u, atop); }
 __device__ __forceinline__ int first_pass(uint16_t u, int atop) { return first_pass_f16(u, atop); }
 
+// q_test of a 16-byte unit's values, out of the loop over them (instruction fetch)
+__device__ __noinline__ bool unit_pass(uint64_t x, uint64_t y, int a) { return q_test(x, a) && q_test(y, a); }
+
 // all_pass that leaves every value's g in the staging buffer in its place (rolled: small code).
 // kNarrow (FP64): |v 10^a| < 10^8 for every value.  With `watch` (FP32, FP16 at the largest beta_hat)
 // `stop` tells whether some value stops early, which counts when all pass.
@@ -311,35 +329,44 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
     using U = typename Traits<D>::U;
     constexpr int UN = Traits<D>::UNITS, PER = 32 / UN;
     bool ok = true, early = false;
+    uint32_t slow = 0;
     Case1At c{};
-    if constexpr (D == kD64) c = case1_at(a);
-    Case1Narrow cn{};
-    if constexpr (kNarrow) cn = case1_narrow_of(a);
-    Case1F32 cf{};
-    if constexpr (D == kD32) cf = case1_f32_of(a);
+    if constexpr (D == kD64 && !kNarrow) c = case1_at(a);
+    TestNarrow cn{};
+    if constexpr (kNarrow) cn = test_narrow_of(a);
+    TestF32 cf{};
+    if constexpr (D == kD32) cf = test_f32_of(a);
     Scale16 ch{};
     if constexpr (D == kD16) ch = scale16_of(a);
     auto one = [&](U u) {
         if constexpr (D != kD64) {
             if (watch && may_stop_early(u, a)) early |= first_pass(u, a) < 0;
         }
-        if constexpr (kNarrow) return test_g(u, c, cn, ok);
-        else if constexpr (D == kD64) return test_g(u, c, ok);
+        if constexpr (kNarrow) return test_g(u, cn, ok, slow);
+        else if constexpr (D == kD64) return test_g(u, c, ok, slow);
         else if constexpr (D == kD32) return test_g(u, cf, ok);
         else return test_g(u, ch, ok);
     };
     if (m > 1024u && lane == 31) {
         U *e = reinterpret_cast<U *>(buf + phys_elem_byte<D>(1024));
-        *e = one(*e);
+        const U x = *e;
+        *e = one(x);
+        if constexpr (D == kD64) {
+            if (slow) ok &= unit_pass(x, x, a);
+        }
     }
 #pragma unroll 1
     for (int u = 0; u < UN; ++u) {
         uint4 *q = reinterpret_cast<uint4 *>(buf + (lane * UN + unit_swizzle<D>(lane, u)) * 16);
-        union { uint4 w; U e[PER]; } x;
+        union { uint4 w; U e[PER]; } x, g;
         x.w = *q;
+        slow = 0;
 #pragma unroll
-        for (int k = 0; k < PER; ++k) x.e[k] = one(x.e[k]);
-        *q = x.w;
+        for (int k = 0; k < PER; ++k) g.e[k] = one(x.e[k]);
+        *q = g.w;
+        if constexpr (D == kD64) {
+            if (slow) ok &= unit_pass(x.e[0], x.e[1], a);
+        }
         if (!__all_sync(kFull, ok)) return false;
     }
     stop = __any_sync(kFull, early);

@@ -516,6 +516,16 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t n) {
     asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
     return r;
 }
+__device__ __forceinline__ uint64_t shr_clamp64(uint64_t x, uint32_t n) {
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+    return r;
+}
+__device__ __forceinline__ uint32_t shl_clamp(uint32_t x, uint32_t n) {
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
 __device__ __forceinline__ uint32_t case1_n_narrow(uint32_t hi, uint32_t lo, const Case1Narrow &q) {      // |g|
     const uint32_t top = __funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 11);
     const uint32_t sh = (uint32_t)(q.c - (int)((hi >> 20) & 0x7FFu));

@@ -57,6 +57,20 @@ def test_largest_value_at_a_power_of_ten(F, oracle, k):
             check(F, oracle, synth.decimal_to_f64(d, min(places, 22)), 1024)
 
 
+@pytest.mark.parametrize("dtype,digits", [(np.float64, 8), (np.float64, 9), (np.float64, 14), (np.float32, 6), (np.float32, 7)])
+@pytest.mark.parametrize("places", [0, 1, 2, 3, 4, 6, 9, 13, 14])
+def test_decimals_of_every_size(F, oracle, dtype, digits, places):
+    """Decimals of 0 to `digits` digits in one chunk (zeros, the smallest, both sides of the 32-bit
+    arithmetic's limit), then chunks with one value an ulp beside its decimal."""
+    rng = np.random.default_rng(places + 100 * digits)
+    d = np.trunc(rng.choice([-1.0, 1.0], 4 * 1025) * 10.0 ** rng.uniform(-0.5, digits, 4 * 1025)).astype(np.int64)
+    vals = (d.astype(np.float64) / 10.0 ** places).astype(dtype) + dtype(0)         # no -0
+    for i, at in ((1, 5), (2, 1024), (3, 700)):
+        vals[1025 * i + at] = np.nextafter(vals[1025 * i + at], dtype(np.inf if i == 1 else -np.inf))
+    vals += dtype(0)
+    check(F, oracle, vals, 1025)
+
+
 @pytest.mark.parametrize("dtype", [np.float64, np.float32, np.float16])
 @pytest.mark.parametrize("block", [64, 65, 1000, 1024, 1025])
 def test_row_mixes(F, oracle, dtype, block):
