@@ -113,14 +113,15 @@ __device__ __forceinline__ void copy_rows(uint8_t *dst, const uint8_t *src, uint
 // Sparse rows go four at a time: their nibbles in the bytes of one word, so one shuffle serves four
 // bitmaps, and their byte counts in the bytes of another, so one prefix scan serves four rows (a
 // row has at most 128 non-zero bytes); what used to be a chain of ballots and reductions per row
-// has four rows' work to overlap.  Then runs of dense rows are copied.
+// has four rows' work to overlap.  Then runs of dense rows are copied.  `line` is where plane 0's row
+// would lie if every row below the sparse ones met so far were dense: plane q's row is at
+// line - row_bytes * q, and a sparse row moves it by its length less row_bytes.
 __device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, uint32_t &cur, uint32_t rows,
                                           uint32_t dense, uint32_t row_bytes, uint32_t bm_bytes, uint32_t seltab, int lane) {
-    const uint32_t start = cur;
     const bool maps = !(lane & 1) && (uint32_t)lane < 2u * bm_bytes;      // this lane stores a bitmap byte
     uint32_t sparse = rows & ~dense;
-    uint32_t sum = 0, mine = 0;                   // sparse bytes so far; above this lane's plane
-    uint32_t above = 32u - (uint32_t)__clz((int)rows);
+    const uint32_t step = bm_bytes - row_bytes;
+    uint32_t line = cur + row_bytes * ((uint32_t)__popc(rows) - 1u), mine = line;       // mine: for this lane's plane
     uint8_t *bm = rec + (lane >> 1);
 #pragma unroll 1
     while (sparse) {
@@ -142,13 +143,9 @@ __device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, ui
         const uint32_t pair = (nibs << 4) | __shfl_down_sync(kFull, nibs, 1);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const uint32_t gap = have[i] ? row_bytes * (above - 1u - p[i]) : 0u;   // the dense rows in between
-            const uint32_t len = have[i] ? bm_bytes + ((tot >> (8 * i)) & 255u) : 0u;
-            const uint32_t at = cur + gap;
-            above = have[i] ? p[i] : above;
-            cur = at + len;
-            sum += len;
-            if (have[i] && (uint32_t)lane < p[i]) mine = sum;
+            const uint32_t at = line - row_bytes * p[i];
+            if (have[i]) line += step + ((tot >> (8 * i)) & 255u);
+            if ((uint32_t)lane < p[i]) mine = line;
             if (have[i] && maps) bm[at] = (uint8_t)(pair >> (8 * i));
             const uint32_t packed = __byte_perm(x[i], 0u, __shfl_sync(kFull, seltab, (int)(nibs >> (8 * i))));
             uint8_t *q = rec + at + bm_bytes + ((excl >> (8 * i)) & 255u);
@@ -158,8 +155,8 @@ __device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, ui
                 if (n > (uint32_t)t) q[t] = (uint8_t)(packed >> (8 * t));
         }
     }
-    cur += row_bytes * above;
-    const uint32_t place = start + row_bytes * (uint32_t)__popc((dense >> lane) >> 1) + mine;   // of dense plane `lane`
+    cur = line + row_bytes;
+    const uint32_t place = mine - row_bytes * (uint32_t)lane;              // of dense plane `lane`
     uint32_t dm = dense;
 #pragma unroll 1
     while (dm) {
