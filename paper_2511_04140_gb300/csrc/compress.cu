@@ -119,7 +119,10 @@ __device__ __forceinline__ void copy_rows(uint8_t *dst, const uint8_t *src, uint
 __device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, uint32_t &cur, uint32_t rows,
                                           uint32_t dense, uint32_t row_bytes, uint32_t bm_bytes, uint32_t seltab, int lane) {
     const bool maps = !(lane & 1) && (uint32_t)lane < 2u * bm_bytes;      // this lane stores a bitmap byte
-    uint32_t sparse = rows & ~dense;
+    // through a reduction, so that the mask and the totals are known to be the warp's: the arithmetic on
+    // them leaves the integer pipe (2^26 FP32 211.5 -> 208.2 us, 2^24 FP16 83.8 -> 82.6, FP64 -0.3 %; the
+    // addresses as well: 1 % slower)
+    uint32_t sparse = __reduce_or_sync(kFull, rows & ~dense);
     const uint32_t step = bm_bytes - row_bytes;
     uint32_t line = cur + row_bytes * ((uint32_t)__popc(rows) - 1u), mine = line;       // mine: for this lane's plane
     uint8_t *bm = rec + (lane >> 1);
@@ -139,7 +142,7 @@ __device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, ui
         uint32_t c = nibs - ((nibs >> 1) & 0x05050505u);             // set bits of every nibble
         c = (c & 0x03030303u) + ((c >> 2) & 0x03030303u);
         const uint32_t incl = warp_inclusive(c);
-        const uint32_t tot = __shfl_sync(kFull, incl, 31), excl = incl - c;
+        const uint32_t tot = __reduce_add_sync(kFull, c), excl = incl - c;
         const uint32_t pair = (nibs << 4) | __shfl_down_sync(kFull, nibs, 1);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
