@@ -308,10 +308,10 @@ __device__ __forceinline__ void store_staged(uint8_t *dst, uint32_t m, uint8_t *
             conv(x.e);
             if (store) *reinterpret_cast<uint4 *>(out + 16u * q) = x.w;
         };
-        auto one = [&](uint32_t i, bool store) {
+        auto one = [&](uint32_t i) {
             U e[1] = {*reinterpret_cast<const U *>(slots + phys_elem_byte<D>(i))};
             conv(e);
-            if (store) *reinterpret_cast<U *>(out + i * S) = e[0];
+            *reinterpret_cast<U *>(out + i * S) = e[0];
         };
         if (!kRolled && cnt == (uint32_t)(kLanes * 32)) {        // whole pass: fixed trip counts
             if (al16) {
@@ -319,7 +319,7 @@ __device__ __forceinline__ void store_staged(uint8_t *dst, uint32_t m, uint8_t *
                 for (int i = 0; i < kLanes * UN / 32; ++i) unit(32u * i + lane, true);
             } else {
 #pragma unroll
-                for (int i = 0; i < kLanes; ++i) one(32u * i + lane, true);
+                for (int i = 0; i < kLanes; ++i) one(32u * i + lane);
             }
         } else {
             uint32_t done = 0;
@@ -329,8 +329,16 @@ __device__ __forceinline__ void store_staged(uint8_t *dst, uint32_t m, uint8_t *
                 for (uint32_t q = 0; q < done; q += 32) unit(min(q + lane, done - 1u), q + lane < done);
                 done *= PER;
             }
+            // two values at a time, whose divisions overlap (b = 1025: 179.2 -> 172.6 us; four: 182.1)
 #pragma unroll 1
-            for (uint32_t i = done; i < cnt; i += 32) one(min(i + lane, cnt - 1u), i + lane < cnt);
+            for (uint32_t i = done + lane; i - lane < cnt; i += 64) {
+                const uint32_t j = i + 32u;
+                auto at = [&](uint32_t k) { return *reinterpret_cast<const U *>(slots + phys_elem_byte<D>(min(k, cnt - 1u))); };
+                U e[2] = {at(i), at(j)};
+                conv(e);
+                if (i < cnt) *reinterpret_cast<U *>(out + i * S) = e[0];
+                if (j < cnt) *reinterpret_cast<U *>(out + j * S) = e[1];
+            }
         }
         __syncwarp();
     }
