@@ -16,23 +16,22 @@
 //        workspace;
 //   2. offsets (decompress.cu; the size synchronisation of Sec. 3.4): every record's position into
 //      the workspace.  Streams of at most 1024 chunks skip it, their emit warps add up the sizes;
-//   3. emit: the values again (straight from
-//      global memory, a whole sector per lane and load, not kept in L1: FP64 with the next chunk
-//      prefetched into L2, FP32 and FP16 with the next chunk's values loaded into registers during
-//      the current record), G, the deltas' bit planes (32x32 register transposes, one 32-bit word per
-//      plane: 4 row bytes per lane), zigzagged by one XOR with the sign plane, through 128-byte slots
-//      into the record, assembled in shared memory at the output's 16-byte phase and sent to
-//      its offset with one TMA bulk copy;
+//   3. emit: the values again (straight from global memory, a whole sector per lane and load, not kept in
+//      L1, the next chunk prefetched into L2), G, the deltas' bit planes (32x32 register transposes, one
+//      32-bit word per plane: 4 row bytes per lane), zigzagged by one XOR with the sign plane, through
+//      128-byte slots into the record, assembled in shared memory at the output's 16-byte phase and
+//      sent to its offset with one TMA bulk copy;
 //      the warp of each job's first chunk writes the header and the stream length and checks
 //      the capacity.
-// Both are bound by integer issue (FP64 segments: ALU pipe 59 % and 66 % of active cycles, 1559 and
-// 3018 warp instructions per chunk, against 1801 and 3590 with ballots and reductions per sparse row,
-// per-value zigzags and bit-sliced counts).  2^26 segment values: FP64 520 -> 453 us, FP32 270 -> 242 us;
-// Case-1 FP64 of 40 M values in 1025-value chunks 622 -> 453 us.  Slower, and left out: two copies of the
-// row code (FP64 485 us: instruction fetch), a transpose shared by both halves in a loop (475 us), dense
-// rows moved in 16-byte units (FP64 461, FP32 238 us), values kept in L1 (483 us).  The offsets launch in
-// place of per-tile and per-group sums (two atomics per chunk in the analysis, five loads and a
-// reduction per chunk in the emit, a reset of the workspace): FP64 452 -> 441 us, 2^20-value walk 40 -> 37 us.
+// Both are bound by integer issue (FP64 segments: ALU pipe 74 % and 66 % of active cycles, 1217 and 2734
+// warp instructions per chunk, against 1801 and 3590 with ballots and reductions per sparse row,
+// per-value zigzags and bit-sliced counts) and, where chunks take different paths, by instruction fetch.
+// 2^26 segment values: FP64 520 -> 370 us, FP32 273 -> 211 us; Case-1 FP64 of 40 M values in 1025-value
+// chunks 622 -> 320 us.  Slower, and left out (each measured when the rest stood at about 450 us): two
+// copies of the row code (FP64 485 us: instruction fetch), a transpose shared by both halves in a loop
+// (475 us), dense rows moved in 16-byte units (FP64 461, FP32 238 us), values kept in L1 (483 us).  The
+// offsets launch in place of per-tile and per-group sums (two atomics per chunk in the analysis, five loads
+// and a reduction per chunk in the emit, a reset of the workspace): FP64 452 -> 441 us, 2^20-value walk 40 -> 37 us.
 // The paper resolves offsets inside one launch with a decoupled look-back; with about 1800
 // resident warps on a GB300 the waits of that look-back took half of every warp's time, while
 // the analysis recomputed by the emit launch costs less.
@@ -315,11 +314,44 @@ __device__ __forceinline__ bool may_stop_early(uint16_t u, int a) {
     const int s = 11 - E - a;                    // 3 m 5^a 2^(E+a) >= 2^11  <=>  p >= 2^s
     return s <= 0 || (s < 32 && p >= (1u << s));
 }
+// A magnitude no larger than the smallest that may stop early at a (chunks here hold no subnormals), so
+// that a unit's largest magnitude tells whether any of its values is to be looked at: the bound over
+// 3 10^a, rounded down.  (may_stop_early of every value instead: 2^24 FP16 segments 83.0 us against 78.7,
+// 2^25 FP32 decimals 212.6 against 206.6, 2^25 FP32 walk 144.6 against 142.8.)
+template <int D> __device__ __forceinline__ uint32_t early_floor(int a) {
+    const float p10 = (float)(FALCON_POW5[a] << a);             // exact: a <= 10
+    if constexpr (D == kD32) return __float_as_uint(__fdiv_rd(2796202.5f, p10));          // below 2^23 / 3
+    else return __half_as_ushort(__float2half_rd(__fdiv_rd(682.5f, p10)));                // below 2^11 / 3
+}
 __device__ __forceinline__ int first_pass(uint32_t u, int atop) { return first_pass_f32(u, atop); }
 __device__ __forceinline__ int first_pass(uint16_t u, int atop) { return first_pass_f16(u, atop); }
 
+// Classification of a chunk's magnitudes: FP64 by a key that keeps the top 25 bits of the high word
+// and carries the value's index below, FP32 and FP16 by the magnitude itself.
+template <int D> struct Mag {
+    using U = typename Traits<D>::U;
+    static constexpr U ABS = (U)((U)~(U)0 >> 1);                 // every bit but the sign
+    static constexpr uint32_t kExpAll = D == kD64 ? 0x7FF00000u : (D == kD32 ? 0x7F800000u : 0x7C00u);
+    static constexpr uint32_t kExpOne = D == kD64 ? 0x00100000u : (D == kD32 ? 0x00800000u : 0x0400u);
+    static __device__ __forceinline__ uint32_t key(U u, uint32_t k) {
+        if constexpr (D == kD64) return ((uint32_t)(u >> 32) & 0x7FFFFFC0u) | k;
+        else return (uint32_t)(u & ABS);
+    }
+};
+
 // q_test of a 16-byte unit's values, out of the loop over them (instruction fetch)
 __device__ __noinline__ bool unit_pass(uint64_t x, uint64_t y, int a) { return q_test(x, a) && q_test(y, a); }
+
+// whether Alg. 2 stops early on a value of a 16-byte unit (those from floor_bits on can)
+template <int D> __device__ __noinline__ bool unit_stops(uint4 w, int a, uint32_t floor_bits) {
+    union { uint4 w; typename Traits<D>::U e[16 / Traits<D>::S]; } x;
+    x.w = w;
+    bool early = false;
+#pragma unroll
+    for (int k = 0; k < 16 / Traits<D>::S; ++k)
+        if ((uint32_t)(x.e[k] & Mag<D>::ABS) >= floor_bits) early |= first_pass(x.e[k], a) < 0;
+    return early;
+}
 
 // all_pass that leaves every value's g in the staging buffer in its place (rolled: small code).
 // kNarrow (FP64): |v 10^a| < 10^8 for every value.  With `watch` (FP32, FP16 at the largest beta_hat)
@@ -338,10 +370,9 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
     if constexpr (D == kD32) cf = test_f32_of(a);
     Scale16 ch{};
     if constexpr (D == kD16) ch = scale16_of(a);
+    uint32_t floor_bits = 0;
+    if constexpr (D != kD64) floor_bits = early_floor<D>(a);
     auto one = [&](U u) {
-        if constexpr (D != kD64) {
-            if (watch && may_stop_early(u, a)) early |= first_pass(u, a) < 0;
-        }
         if constexpr (kNarrow) return test_g(u, cn, ok, slow);
         else if constexpr (D == kD64) return test_g(u, c, ok, slow);
         else if constexpr (D == kD32) return test_g(u, cf, ok);
@@ -353,6 +384,8 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
         *e = one(x);
         if constexpr (D == kD64) {
             if (slow) ok &= unit_pass(x, x, a);
+        } else {
+            if (watch && (uint32_t)(x & Mag<D>::ABS) >= floor_bits) early = first_pass(x, a) < 0;
         }
     }
 #pragma unroll 1
@@ -366,6 +399,11 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
         *q = g.w;
         if constexpr (D == kD64) {
             if (slow) ok &= unit_pass(x.e[0], x.e[1], a);
+        } else if (watch) {
+            uint32_t top = 0;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) top = max(top, (uint32_t)(x.e[k] & Mag<D>::ABS));
+            if (top >= floor_bits) early |= unit_stops<D>(x.w, a, floor_bits);
         }
         if (!__all_sync(kFull, ok)) return false;
     }
@@ -520,19 +558,6 @@ __device__ __noinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int la
     }
     return alpha;
 }
-
-// Classification of a chunk's magnitudes: FP64 by a key that keeps the top 25 bits of the high word
-// and carries the value's index below, FP32 and FP16 by the magnitude itself.
-template <int D> struct Mag {
-    using U = typename Traits<D>::U;
-    static constexpr U ABS = (U)((U)~(U)0 >> 1);                 // every bit but the sign
-    static constexpr uint32_t kExpAll = D == kD64 ? 0x7FF00000u : (D == kD32 ? 0x7F800000u : 0x7C00u);
-    static constexpr uint32_t kExpOne = D == kD64 ? 0x00100000u : (D == kD32 ? 0x00800000u : 0x0400u);
-    static __device__ __forceinline__ uint32_t key(U u, uint32_t k) {
-        if constexpr (D == kD64) return ((uint32_t)(u >> 32) & 0x7FFFFFC0u) | k;
-        else return (uint32_t)(u & ABS);
-    }
-};
 
 // Case decision (Eq. 4) of a chunk whose keys have maximum `top` (kmax: this lane's) and, if
 // `low`, some value with a zero exponent field.  Returns alpha_max | beta_hat << 8, alpha_max = 31
