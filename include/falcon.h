@@ -10,8 +10,8 @@
  *   - delta + zigzag coding (Eq. 5);
  *   - the adaptive sparse/dense bit-plane encoding of Sec. 3.3 (Fig. 8);
  *   - the compressed-size synchronisation and chunk writing of Sec. 3.4 (Alg. 3): the record
- *     sizes and their sums per 64- and 4096-chunk group, then every record written at its
- *     offset (two kernel launches on the caller's stream, none waiting on another warp);
+ *     sizes, their prefix sums, then every record written at its offset (two or three kernel
+ *     launches on the caller's stream, no warp waiting on another);
  * and decompression (Sec. 4) is its exact inverse.  FP32 follows the same steps with
  * alpha <= 10, beta <= 7 and 32-bit integers; FP16 (binary16, FALCON_F16; Sec. 2.1 extends
  * the method to other precisions, this library fixes its constants) with alpha <= 4,
@@ -122,7 +122,7 @@ int falcon_decompress_known(const void *d_in, size_t in_bytes, const void *h_hea
  * num_chunks chunks.  Must be 256-byte aligned device memory. */
 size_t falcon_workspace_bytes(uint64_t num_chunks);
 
-/* Asynchronous compression: enqueues a workspace reset and the kernels on `stream` and
+/* Asynchronous compression: enqueues the kernels (and a small reset) on `stream` and
  * returns without synchronising, so it can be captured in a CUDA graph.
  * d_result (device, 2 x uint64): [0] = stream length in bytes, [1] = falcon_status of the
  * device-side work (the host return value only covers argument checks and launch).
@@ -166,7 +166,7 @@ typedef struct {
 /* Asynchronous aggregate of the stream at d_in (device, in_bytes; h_header a host copy of
  * its first 32 bytes) into d_stats (device, one falcon_stats).  d_workspace:
  * falcon_workspace_bytes(number of chunks) bytes of 256-byte aligned device memory owned by
- * the caller.  Enqueues four launches on `stream` and returns without synchronising
+ * the caller.  Enqueues three launches on `stream` and returns without synchronising
  * (capturable).  Errors as falcon_decompress_async. */
 int falcon_aggregate_async(const void *d_in, size_t in_bytes, const void *h_header, void *d_workspace,
                            size_t workspace_bytes, falcon_stats *d_stats, void *stream);
@@ -264,8 +264,8 @@ size_t falcon_batch_workspace_bytes(int direction, const falcon_series *h_series
 int falcon_batch_plan(int direction, const falcon_series *h_series, int count, void *d_workspace,
                       size_t workspace_bytes, uint64_t *d_results, void *stream);
 
-/* Enqueues one execution of the plan held by d_workspace on `stream` (workspace and result
- * reset, then the persistent kernel): no host synchronisation, capturable in a CUDA graph. */
+/* Enqueues one execution of the plan held by d_workspace on `stream` (the launches of one
+ * direction over all series): no host synchronisation, capturable in a CUDA graph. */
 int falcon_batch_launch(void *d_workspace, void *stream);
 
 /* Drops the host-side record of the plan held by d_workspace. */

@@ -14,15 +14,16 @@
 //         G (inverse Eq. 5), Case 1 divides by 10^alpha (correctly rounded) and Case 2 undoes the
 //         zigzag of the IEEE bits (inverse Eq. 4),
 //      c. whole 32-byte sectors per lane (aligned FP64) or staged, coalesced stores.
-// What bounds it: integer issue and latency together (FP64 segments: ALU pipe 56 %, L1 data pipe
-// 55 %, issue 52 % of cycles at 16 warps per SM; HBM 45 %), and the instruction stream's length: code is
-// kept short (both FP64 halves run one copy, Case 1 divides in rolled loops on the way out), which
-// took FP64 segments from 310 to 288 us and Case-1 values from 304 to 191 us (40 M in 1025-value chunks).
+// What bounds it: integer issue and latency together (FP64 Case-1 values: ALU pipe 66 %, issue 64 % of cycles
+// at 16 warps per SM; HBM 45 % on FP64 segments), and the instruction stream's length: code is kept short
+// (both FP64 halves run one copy, Case 1 divides in rolled loops on the way out), which took FP64 segments
+// from 310 to 288 us and Case-1 values from 304 to 191 us (40 M in 1025-value chunks).
 // Reading the dense rows in place instead of copying them to a plane buffer took the kernel from 4302 to
 // 2880 warp instructions per FP64 chunk and its shared memory from 17.6 to 13.7 KB per warp (12 to 16
-// warps per SM).  Both launches, 2^26 segment values: FP64 420 -> 288 us, FP32 216 -> 149 us.  Slower, and
-// left out: a TMA bulk copy of the record on an mbarrier (-1 %), tickets for groups of 4 to 8 chunks (-7
-// to -15 %: the window of memory in use grows with the group), more registers with fewer warps (144: -6 %).
+// warps per SM).  Both launches, 2^26 segment values: FP64 420 -> 274 us, FP32 216 -> 139 us; the Case-1
+// values 550 -> 172 us.  Slower, and left out: a TMA bulk copy of the record on an mbarrier (-1 %), tickets
+// for groups of 4 to 8 chunks (-7 to -15 %: the window of memory in use grows with the group), more
+// registers with fewer warps (144: -6 %).
 // Every read of a record is bounds-checked against its size; a malformed record sets
 // FALCON_ERR_CORRUPT and writes nothing.
 #include "falcon.h"

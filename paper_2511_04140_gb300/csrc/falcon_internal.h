@@ -6,13 +6,12 @@
 namespace falcon {
 
 // Warps per CTA of the persistent kernels: a launch parameter (falcon_set_cta_warps) that
-// changes no output byte; every warp works on its own chunks.  The launch bounds keep the
-// register budget of the default shape (4 warps, 4 CTAs per SM for compression; 3 CTAs per SM
-// of 4 warps for decompression) at every allowed shape.
+// changes no output byte; every warp works on its own chunks.  The kernels' register budgets
+// (80 to 168 per thread, set per kernel) hold at every allowed shape.
 constexpr int kWarpsPerCta = 4;                 // default
 constexpr int kThreads = 32 * kWarpsPerCta;
-constexpr int kMaxCompressWarps = 16;           // 512 threads: 128 registers per thread
-constexpr int kMaxDecompressWarps = 12;         // 384 threads: 170 registers per thread
+constexpr int kMaxCompressWarps = 16;           // 512 threads of up to 128 registers
+constexpr int kMaxDecompressWarps = 12;         // 384 threads of up to 168 registers
 constexpr uint32_t kMaxBlock = 1025;
 
 // Status codes (identical numbering to falcon_status in include/falcon.h).

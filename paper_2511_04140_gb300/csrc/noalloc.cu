@@ -54,8 +54,7 @@ extern "C" int falcon_compress_noalloc(const void *d_in, uint64_t n, int dtype, 
     if (chunks > FALCON_NOALLOC_MAX_CHUNKS) return FALCON_ERR_UNSUPPORTED;
     void *scratch = nullptr;
     if ((st = scratch_address(&scratch))) return st;
-    // zeroes, on `stream`, the control block, the per-chunk words this call uses and
-    // d_result, then enqueues the three compression launches
+    // enqueues, on `stream`, the compression launches, which write every word of the scratch they read
     return falcon_compress_async(d_in, n, dtype, block_size, d_out, out_capacity, scratch, kScratchBytes, d_result,
                                  stream);
 }
