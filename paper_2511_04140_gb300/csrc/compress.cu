@@ -26,7 +26,7 @@
 // Both are bound by integer issue (FP64 segments: ALU pipe 75 % and 66 % of active cycles, 1236 and 2751
 // warp instructions per chunk, against 1801 and 3590 with ballots and reductions per sparse row,
 // per-value zigzags and bit-sliced counts) and, where chunks take different paths, by instruction fetch.
-// 2^26 segment values: FP64 520 -> 370 us, FP32 273 -> 211 us; Case-1 FP64 of 40 M values in 1025-value
+// 2^26 segment values: FP64 520 -> 366 us, FP32 273 -> 209 us; Case-1 FP64 of 40 M values in 1025-value
 // chunks 622 -> 320 us.  Slower, and left out (each measured when the rest stood at about 450 us): two
 // copies of the row code (FP64 485 us: instruction fetch), a transpose shared by both halves in a loop
 // (475 us), dense rows moved in 16-byte units (FP64 461, FP32 238 us), values kept in L1 (483 us).  The
@@ -74,11 +74,11 @@ __device__ __forceinline__ uint32_t compact_sel(uint32_t n) {
     return sel;
 }
 
-// non-zero nibble of x (bit 3 - i set iff byte i is non-zero): the bytes' high-bit flags moved to
-// bits 32..35 by one high multiply
-__device__ __forceinline__ uint32_t nz_nibble(uint32_t x) {
+// 128 times the non-zero nibble of x (bit 3 - i set iff byte i is non-zero): the bytes' high-bit flags
+// weighted and added by one four-way dot product (by a high multiply: 2^26 FP64 361 us against 356.5)
+__device__ __forceinline__ uint32_t nz_nibble128(uint32_t x) {
     const uint32_t y = (((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
-    return __umulhi(y, 0x10080402u) & 15u;
+    return __dp4a(y, 0x01020408u, 0u);
 }
 
 // inclusive prefix sum over the warp (the shuffle's own predicate says which lanes add)
@@ -136,7 +136,8 @@ __device__ __forceinline__ void emit_rows(uint8_t *rec, const uint8_t *slots, ui
             sparse &= ~(1u << p[i]);
             x[i] = *reinterpret_cast<const uint32_t *>(slots + 128u * (31u - p[i]) + 4u * lane);
             if (i > 0) x[i] = have[i] ? x[i] : 0u;
-            nibs |= nz_nibble(x[i]) << (8 * i);
+            const uint32_t n = nz_nibble128(x[i]);
+            nibs = i == 0 ? n >> 7 : nibs + (n << (8 * i - 7));
         }
         uint32_t c = nibs - ((nibs >> 1) & 0x05050505u);             // set bits of every nibble
         c = (c & 0x03030303u) + ((c >> 2) & 0x03030303u);
