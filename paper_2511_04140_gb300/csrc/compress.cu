@@ -23,7 +23,7 @@
 //      sent to its offset with one TMA bulk copy;
 //      the warp of each job's first chunk writes the header and the stream length and checks
 //      the capacity.
-// Both are bound by integer issue (FP64 segments: ALU pipe 75 % and 66 % of active cycles, 1236 and 2751
+// Both are bound by integer issue (FP64 segments: ALU pipe 75 % and 66 % of active cycles, 1236 and 2741
 // warp instructions per chunk, against 1801 and 3590 with ballots and reductions per sparse row,
 // per-value zigzags and bit-sliced counts) and, where chunks take different paths, by instruction fetch.
 // 2^26 segment values: FP64 520 -> 366 us, FP32 273 -> 209 us; Case-1 FP64 of 40 M values in 1025-value
