@@ -20,7 +20,7 @@
 // from 310 to 288 us and Case-1 values from 304 to 191 us (40 M in 1025-value chunks).
 // Reading the dense rows in place instead of copying them to a plane buffer took the kernel from 4302 to
 // 2880 warp instructions per FP64 chunk and its shared memory from 17.6 to 13.7 KB per warp (12 to 16
-// warps per SM).  Both launches, 2^26 segment values: FP64 420 -> 274 us, FP32 216 -> 139 us; the Case-1
+// warps per SM).  Both launches, 2^26 segment values: FP64 420 -> 273 us, FP32 216 -> 139 us; the Case-1
 // values 550 -> 172 us.  Slower, and left out: a TMA bulk copy of the record on an mbarrier (-1 %), tickets
 // for groups of 4 to 8 chunks (-7 to -15 %: the window of memory in use grows with the group), more
 // registers with fewer warps (144: -6 %).
