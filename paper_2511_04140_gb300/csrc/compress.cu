@@ -53,11 +53,22 @@ template <int D> constexpr int kAnalyseWarpBytes = 1024 * Traits<D>::S + 32;
 // 128-byte slots for the rows of 32 planes at a time, top plane first (FP64 runs its two halves one
 // after the other through the same slots).  A row takes at most 128 bytes of the record, 16 more in
 // an every-row-sparse one (Sec. 5.4.2 ablation, the wide layout).
+// A chunk's planes go into the slots while the bulk copy of the warp's previous record may still be
+// reading its buffer, so the slots lie past the longest record of any kind the warp meets: the form's
+// layout places them, for every kind it runs.  (Placed by the chunk's own kind in the either-dtype form,
+// the slots of an FP32 or FP16 chunk were inside the FP64 record before it.)
 template <int D, bool kWide> struct EmitLayout {
     static constexpr uint32_t W = Traits<D>::W;
     static constexpr uint32_t kRec = (3u + Traits<D>::Z1B + W / 8u + W * (kWide ? 144u : 128u) + 15u + 15u) / 16u * 16u;
     static constexpr uint32_t kRows = W < 32u ? W : 32u;
     static constexpr uint32_t kBytes = kRec + kRows * 128u + 16u;         // + 16 readable past any slot
+    // where kind K's chunks have their slots in this form's buffer
+    template <int K> static constexpr uint32_t slots_of() {
+        using Own = EmitLayout<K, kWide>;
+        static_assert(Own::kRec <= kRec && kRec + Own::kRows * 128u + 16u <= kBytes,
+                      "a chunk's slots would overlap a record that is still being copied out, or the next warp's buffer");
+        return kRec;
+    }
 };
 
 // Byte-permute selector that moves a word's non-zero bytes to its front, by nibble n (bit 3 - i: byte
@@ -927,12 +938,12 @@ __device__ __forceinline__ void map_rolled(U (&v)[32], F &&f) {
 // Emit, one chunk: G and its deltas again (alpha and w from the analysis), their planes, and the record at
 // its offset.  word / dense: the chunk's workspace words; size: its record size; rel: its record offset
 // relative to the first record.
-template <int D, bool kWide>
+// L: the form's buffer layout.
+template <int D, class L>
 __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *buf, uint32_t seltab, int lane,
                                            uint64_t word, uint64_t dense, uint32_t size, uint64_t rel) {
     using T = Traits<D>;
     using U = typename T::U;
-    using L = EmitLayout<D, kWide>;
     const uint32_t B = job.block;
     const uint64_t first = c * (uint64_t)B;
     const uint32_t m = (uint32_t)((job.n - first) < B ? (job.n - first) : B);
@@ -953,7 +964,8 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(gdst) & 15u);
     const uint32_t flag_bytes = ((uint32_t)w + 7u) / 8u;
     const uint32_t hdr = 3u + T::Z1B + flag_bytes;
-    uint8_t *slots = buf + L::kRec - (32u - L::kRows) * 128u;         // plane p of a half: 128 (31 - p) further
+    constexpr int R = T::W < 32 ? T::W : 32;
+    uint8_t *slots = buf + L::template slots_of<D>() - (32u - R) * 128u;      // plane p of a half: 128 (31 - p) further
     uint8_t *dst = slots + 31 * 128 + 4 * lane;                      // plane 0; plane p lies 128 p below
     uint32_t pos = sh + hdr;                      // next record byte in the buffer
     U z1;
@@ -968,7 +980,6 @@ __device__ __forceinline__ void emit_chunk(const Job &job, uint64_t c, uint8_t *
     };
     uint32_t sgn = 0;
     const bool two = D == kD64 && w > 32;
-    constexpr int R = T::W < 32 ? T::W : 32;
     uint32_t a[32];                               // the deltas' low words, transposed below
     // G (Eq. 4) and its deltas (Eq. 5).  FP64's two Case 1 conversions are rolled: unrolled over the 32
     // values they are 7 and 18 KB of code, and warps on chunks of both kinds waited for instructions
@@ -1212,7 +1223,8 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
     const int warp = threadIdx.x >> 5;
     constexpr bool kTable = kDt == kDtMixed;
     constexpr int DL = kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64);
-    uint8_t *wbase = smem + warp * EmitLayout<DL, kWide>::kBytes;
+    using L = EmitLayout<DL, kWide>;
+    uint8_t *wbase = smem + warp * L::kBytes;
     const uint32_t seltab = compact_sel((uint32_t)lane & 15u);
     if (blockIdx.x == 0 && warp == 0) {          // jobs without chunks: header and length only
         if constexpr (!kTable) {
@@ -1244,7 +1256,7 @@ __device__ __forceinline__ void emit_loop(const Job *__restrict__ jobs, int njob
         const uint64_t rel = dir ? sizes_before(job, info.c, lane) : (info.word & kOffsetMask);
         if (info.c == 0) finish_job(job, dir, lane);
         auto emit = [&](auto kind) {
-            emit_chunk<decltype(kind)::value, kWide>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel);
+            emit_chunk<decltype(kind)::value, L>(job, info.c, wbase, seltab, lane, info.word, info.dense, info.size, rel);
         };
         if constexpr (!kTable) emit(std::integral_constant<int, DL>{});
         else if (job.dtype == 0) emit(std::integral_constant<int, kD64>{});
