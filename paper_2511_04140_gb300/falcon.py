@@ -201,25 +201,28 @@ def compress(x: torch.Tensor, block: int = 1024, out: torch.Tensor | None = None
 
 
 def decompress(s: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    """Decompresses a uint8 CUDA tensor holding one stream; returns the values."""
+    """Decompresses a uint8 CUDA tensor holding one stream; returns the values.  On another stream than
+    the current one, the call also waits for what the current stream still has to do."""
     if not s.is_cuda or s.dtype != torch.uint8:
         raise ValueError("s must be a uint8 CUDA tensor")
     if s.numel() < HEADER_BYTES:
         raise FalconError(ERR_CORRUPT, "decompress")
-    L, here = _load(), _stream_ptr(None)
-    if stream is None or stream.cuda_stream == here:
-        buf = ctypes.create_string_buffer(HEADER_BYTES)
-        _check(L.falcon_read_header(s.data_ptr(), s.numel(), buf, here), "decompress")
-        hdr = buf.raw
-    else:                                        # also waits for what the current stream still has to write
-        hdr = s[:HEADER_BYTES].cpu().numpy().tobytes()
+    L, at = _load(), _stream_ptr(stream)
+    if stream is not None:
+        here = torch.cuda.current_stream(s.device)
+        if here.cuda_stream != at:               # s, or memory that `out` takes over, may still be in use there
+            here.synchronize()
+    # read in the launch's order: the launch takes the header as it is read here
+    buf = ctypes.create_string_buffer(HEADER_BYTES)
+    _check(L.falcon_read_header(s.data_ptr(), s.numel(), buf, at), "decompress")
+    hdr = buf.raw
     n, code, _, _ = stream_info(hdr)
     dtype = torch_dtype(code)
     if out is None:
         out = torch.empty(max(n, 1), dtype=dtype, device=s.device)
     n_out = ctypes.c_uint64()
     _check(L.falcon_decompress_known(s.data_ptr(), s.numel(), hdr, out.data_ptr(), out.numel() * out.element_size(),
-                                     ctypes.byref(n_out), _stream_ptr(stream)), "decompress")
+                                     ctypes.byref(n_out), at), "decompress")
     return out[:n_out.value]
 
 
