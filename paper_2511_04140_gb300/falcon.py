@@ -207,6 +207,8 @@ def decompress(s: torch.Tensor, out: torch.Tensor | None = None, stream=None) ->
         raise ValueError("s must be a uint8 CUDA tensor")
     if s.numel() < HEADER_BYTES:
         raise FalconError(ERR_CORRUPT, "decompress")
+    if not s.is_contiguous():                    # a strided view whose own bytes start no stream
+        stream_info(s[:HEADER_BYTES].cpu().numpy().tobytes())
     L, at = _load(), _stream_ptr(stream)
     if stream is not None:
         here = torch.cuda.current_stream(s.device)
