@@ -406,6 +406,13 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, const Job &single, u
 
     // ---- a. header and flags ------------------------------------------------------------------
     bool bad = r0.phase == kBadRecord;
+    // a malformed record: its chunk adds nothing to the aggregate, whose finish reads every chunk's sum
+    auto reject = [&]() {
+        if (lane != 0) return;
+        const Job &job = kTable ? *note.job : single;
+        set_status(job.result, kErrCorrupt);
+        if constexpr (kAgg) reinterpret_cast<double *>(job.flags + job.nchunks)[note.c] = 0.0;
+    };
     if (lane == 0) {
         const uint32_t h0 = lds_any(smem, rec);
         note.c = r0.c;
@@ -467,10 +474,12 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, const Job &single, u
                 }
             }
             bad = cur - rec != r0.size;
-            if (bad && lane == 0) set_status((kTable ? *r0.job : single).result, kErrCorrupt);
-            if (bad) return;
+            if (bad) {
+                reject();
+                return;
+            }
         } else {
-            if (lane == 0) set_status((kTable ? *r0.job : single).result, kErrCorrupt);
+            reject();
             __syncwarp();
             next();
             return;
@@ -487,7 +496,7 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, const Job &single, u
         }
         __syncwarp();
         if (bad) {
-            if (lane == 0) set_status((kTable ? *r0.job : single).result, kErrCorrupt);
+            reject();
             next();
             return;
         }
