@@ -26,6 +26,8 @@
 // registers with fewer warps (144: -6 %).
 // Every read of a record is bounds-checked against its size; a malformed record sets
 // FALCON_ERR_CORRUPT and writes nothing.
+#include <algorithm>
+
 #include "falcon.h"
 #include "falcon_device.cuh"
 
@@ -621,31 +623,24 @@ __device__ __forceinline__ void decode_chunk(const Rec &r0, const Job &single, u
 }  // namespace
 
 // The position of every record (exclusive prefix of the u32 size array) of every job into the
-// first words of job.flags.  `parts` CTAs per job, each over its own share of the chunks: a CTA
+// first words of job.flags.  A single stream: `parts` CTAs, each over its own share of the chunks; a CTA
 // adds up every size before its share first (at most 152 CTAs reading at most the whole array, from
-// L2), then scans its share 1024 chunks at a time, so no CTA waits for another.
-__global__ void __launch_bounds__(1024)
-offsets_kernel(const Job *__restrict__ jobs, Job single, uint32_t parts, int which, Control *ctl) {
-    __shared__ uint64_t warp_sums[33];
-    pdl_trigger();
-    pdl_wait();                                   // compression: the analysis' sizes
-    const Job &job = (jobs == nullptr) ? single : jobs[blockIdx.x / parts];
-    const uint32_t part = blockIdx.x % parts;
-    const uint64_t nc = job.nchunks;
-    if (which == kOffsetsOfInput && threadIdx.x == 0) {          // ready for the decode
-        if (blockIdx.x == 0) *ctl = Control{};
-        if (part == 0) {
-            job.result[0] = job.n;
-            job.result[1] = kOk;
-        }
-    }
-    const uint64_t share = ((nc + parts - 1) / parts + 1023u) & ~1023ull;
-    const uint64_t begin = part * share, end = begin + share < nc ? begin + share : nc;
-    if (begin >= nc) return;
-    // 16-byte aligned
-    const uint32_t *sizes = reinterpret_cast<const uint32_t *>((which == kOffsetsOfInput ? job.in : job.out) + 32);
+// L2), then scans its share 1024 chunks at a time, so no CTA waits for another.  A table: `per` jobs per
+// CTA, each by a warp of its own when it has at most 32 `per` chunks (a warp scans 32 chunks in about the
+// time the CTA takes for a job), the longer ones by the whole CTA in turn.
+// 16,000 FP32 series of 10 values, one CTA each: compressed in 366 us, decompressed in 172; so 231 and 52.
+__device__ __forceinline__ void put_position(const Job &job, int which, uint64_t c, uint64_t at) {
+    if (which == kOffsetsOfInput) job.flags[c] = at;
+    else job.flags[c] = ((job.flags[c] >> kOffsetBits) << kOffsetBits) | at;
+}
+__device__ __forceinline__ const uint32_t *sizes_of(const Job &job, int which) {          // 16-byte aligned
+    return reinterpret_cast<const uint32_t *>((which == kOffsetsOfInput ? job.in : job.out) + 32);
+}
+// chunks [begin, end) by the whole CTA; begin a multiple of 1024
+__device__ __forceinline__ void scan_by_cta(const Job &job, int which, uint64_t begin, uint64_t end, uint64_t *warp_sums) {
+    const uint32_t *sizes = sizes_of(job, which);
     uint64_t carry = 0;
-    if (begin > 0) {                              // begin is a multiple of 1024
+    if (begin > 0) {
         const uint4 *q = reinterpret_cast<const uint4 *>(sizes);
         uint64_t sum = 0;
         for (uint64_t i = threadIdx.x; i < begin / 4u; i += 1024u) {
@@ -658,12 +653,58 @@ offsets_kernel(const Job *__restrict__ jobs, Job single, uint32_t parts, int whi
         const uint64_t c = b + threadIdx.x;
         uint64_t total;
         const uint64_t ex = block_exclusive_scan(c < end ? sizes[c] : 0u, total, warp_sums);
-        if (c < end) {
-            if (which == kOffsetsOfInput) job.flags[c] = carry + ex;
-            else job.flags[c] = ((job.flags[c] >> kOffsetBits) << kOffsetBits) | (carry + ex);
-        }
+        if (c < end) put_position(job, which, c, carry + ex);
         carry += total;
     }
+}
+// a short job by one warp
+__device__ __forceinline__ void scan_by_warp(const Job &job, int which, int lane) {
+    const uint32_t *sizes = sizes_of(job, which);
+    const uint32_t nc = (uint32_t)job.nchunks;
+    uint64_t carry = 0;
+    uint32_t size = (uint32_t)lane < nc ? sizes[lane] : 0u;
+    for (uint32_t b = 0; b < nc; b += 32u) {
+        const uint32_t c = b + (uint32_t)lane, mine = size;
+        size = c + 32u < nc ? sizes[c + 32u] : 0u;
+        const uint64_t incl = mine + warp_exclusive_u64(mine, lane);
+        if (c < nc) put_position(job, which, c, carry + incl - mine);
+        carry += shfl_u64(incl, 31);
+    }
+}
+__device__ __forceinline__ void start_decode(const Job &job) {            // the results, ready for the decode
+    job.result[0] = job.n;
+    job.result[1] = kOk;
+}
+__global__ void __launch_bounds__(1024, 2)
+offsets_kernel(Job single, uint32_t parts, int which, Control *ctl) {
+    __shared__ uint64_t warp_sums[33];
+    pdl_trigger();
+    pdl_wait();                                   // compression: the analysis' sizes
+    const uint64_t nc = single.nchunks;
+    if (which == kOffsetsOfInput && blockIdx.x == 0 && threadIdx.x == 0) {
+        *ctl = Control{};
+        start_decode(single);
+    }
+    const uint64_t share = ((nc + parts - 1) / parts + 1023u) & ~1023ull;
+    const uint64_t begin = blockIdx.x * share, end = begin + share < nc ? begin + share : nc;
+    if (begin < nc) scan_by_cta(single, which, begin, end, warp_sums);
+}
+__global__ void __launch_bounds__(1024, 2)
+table_offsets_kernel(const Job *__restrict__ jobs, int njobs, uint32_t per, int which, Control *ctl) {
+    __shared__ uint64_t warp_sums[33];
+    pdl_trigger();
+    pdl_wait();
+    if (which == kOffsetsOfInput && blockIdx.x == 0 && threadIdx.x == 0) *ctl = Control{};
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Job *mine = jobs + (size_t)blockIdx.x * per;
+    const int count = min((int)per, njobs - (int)(blockIdx.x * per));
+    auto is_short = [&](const Job &job) { return per > 1u && job.nchunks <= 32u * per; };
+    if (warp < count) {
+        if (which == kOffsetsOfInput && lane == 0) start_decode(mine[warp]);
+        if (is_short(mine[warp])) scan_by_warp(mine[warp], which, lane);
+    }
+    for (int i = 0; i < count; ++i)
+        if (!is_short(mine[i])) scan_by_cta(mine[i], which, 0, mine[i].nchunks, warp_sums);
 }
 
 // Forms by dtype: kDt = 0 (every job FP64), 1 (every job FP32), 2 (either, per job).
@@ -775,17 +816,23 @@ void launch_decode(const Job *d_jobs, int njobs, const Job &single, uint64_t tot
 }
 }  // namespace
 
-// One CTA per 1024 chunks up to 152 for a single stream; a table's many jobs get one each.
+// A single stream: one CTA per 1024 chunks, up to 152.  A table: one CTA per job up to 304 jobs (two
+// CTAs of 1024 threads to an SM), beyond that up to 32 jobs share a CTA, so that many short jobs do
+// not take their CTAs' launches in turn.
+// Compression's follows the analysis; decompression's is the first launch of the call, after whatever
+// the caller has enqueued.
 void launch_offsets(const Job *d_jobs, int njobs, const Job &single, int which, Control *ctl, cudaStream_t stream) {
-    uint32_t parts = 1;
+    const bool after = which == kOffsetsOfOutput;
     if (d_jobs == nullptr) {
         const uint64_t steps = (single.nchunks + 1023u) / 1024u;
-        parts = steps < 1u ? 1u : (steps > 152u ? 152u : (uint32_t)steps);
+        const uint32_t parts = steps < 1u ? 1u : (steps > 152u ? 152u : (uint32_t)steps);
+        if (after) (void)launch_after(offsets_kernel, (int)parts, 1024, 0, stream, single, parts, which, ctl);
+        else offsets_kernel<<<parts, 1024, 0, stream>>>(single, parts, which, ctl);
+        return;
     }
-    // compression's follows the analysis; decompression's is the first launch of the call, after whatever
-    // the caller has enqueued
-    if (which == kOffsetsOfOutput) (void)launch_after(offsets_kernel, njobs * (int)parts, 1024, 0, stream, d_jobs, single, parts, which, ctl);
-    else offsets_kernel<<<(unsigned)njobs * parts, 1024, 0, stream>>>(d_jobs, single, parts, which, ctl);
+    const uint32_t per = std::min(((uint32_t)njobs + 303u) / 304u, 32u), ctas = ((uint32_t)njobs + per - 1u) / per;
+    if (after) (void)launch_after(table_offsets_kernel, (int)ctas, 1024, 0, stream, d_jobs, njobs, per, which, ctl);
+    else table_offsets_kernel<<<ctas, 1024, 0, stream>>>(d_jobs, njobs, per, which, ctl);
 }
 
 cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cudaStream_t stream) {
