@@ -354,25 +354,27 @@ template <int D> struct Mag {
 // q_test of a 16-byte unit's values, out of the loop over them (instruction fetch)
 __device__ __noinline__ bool unit_pass(uint64_t x, uint64_t y, int a) { return q_test(x, a) && q_test(y, a); }
 
-// whether Alg. 2 stops early on a value of a 16-byte unit (those from floor_bits on can)
-template <int D> __device__ __noinline__ bool unit_stops(uint4 w, int a, uint32_t floor_bits) {
+// whether Alg. 2 stops early on one of the first `count` values of a 16-byte unit (those from floor_bits
+// on can)
+template <int D> __device__ __noinline__ bool unit_stops(uint4 w, int a, uint32_t floor_bits, uint32_t count) {
     union { uint4 w; typename Traits<D>::U e[16 / Traits<D>::S]; } x;
     x.w = w;
     bool early = false;
 #pragma unroll
     for (int k = 0; k < 16 / Traits<D>::S; ++k)
-        if ((uint32_t)(x.e[k] & Mag<D>::ABS) >= floor_bits) early |= first_pass(x.e[k], a) < 0;
+        if ((uint32_t)k < count && (uint32_t)(x.e[k] & Mag<D>::ABS) >= floor_bits) early |= first_pass(x.e[k], a) < 0;
     return early;
 }
 
 // all_pass that leaves every value's g in the staging buffer in its place (rolled: small code).
-// kNarrow (FP64): |v 10^a| < 10^8 for every value.  With `watch` (FP32, FP16 at the largest beta_hat)
-// `stop` tells whether some value stops early, which counts when all pass.
+// kNarrow (FP64): |v 10^a| < 10^8 for every value.  With `watch` (FP32, FP16 at the largest beta_hat) no
+// value may stop early either; that test reads the chunk's own values, not a tail's
+// padding (one FP32 value of seven digits and its 1023 copies: 37 us for the call, 14 so).
 template <int D, bool kNarrow = false>
-__device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, int a, bool watch, bool &stop) {
+__device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, int a, bool watch) {
     using U = typename Traits<D>::U;
     constexpr int UN = Traits<D>::UNITS, PER = 32 / UN;
-    bool ok = true, early = false;
+    bool ok = true;
     uint32_t slow = 0;
     Case1At c{};
     if constexpr (D == kD64 && !kNarrow) c = case1_at(a);
@@ -397,7 +399,7 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
         if constexpr (D == kD64) {
             if (slow) ok &= unit_pass(x, x, a);
         } else {
-            if (watch && (uint32_t)(x & Mag<D>::ABS) >= floor_bits) early = first_pass(x, a) < 0;
+            if (watch && (uint32_t)(x & Mag<D>::ABS) >= floor_bits) ok &= first_pass(x, a) >= 0;
         }
     }
 #pragma unroll 1
@@ -409,17 +411,17 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
 #pragma unroll
         for (int k = 0; k < PER; ++k) g.e[k] = one(x.e[k]);
         *q = g.w;
+        const uint32_t first = 32u * (uint32_t)lane + (uint32_t)(u * PER);        // the unit's first value
         if constexpr (D == kD64) {
             if (slow) ok &= unit_pass(x.e[0], x.e[1], a);
-        } else if (watch) {
+        } else if (watch && first < m) {
             uint32_t top = 0;
 #pragma unroll
             for (int k = 0; k < PER; ++k) top = max(top, (uint32_t)(x.e[k] & Mag<D>::ABS));
-            if (top >= floor_bits) early |= unit_stops<D>(x.w, a, floor_bits);
+            if (top >= floor_bits) ok &= !unit_stops<D>(x.w, a, floor_bits, m - first);
         }
         if (!__all_sync(kFull, ok)) return false;
     }
-    stop = __any_sync(kFull, early);
     return true;
 }
 
@@ -530,9 +532,10 @@ __device__ __noinline__ int alpha_elf(const uint8_t *buf, int lane, uint32_t m, 
 // atop), or -1.  On success the staging buffer holds G (Eq. 4) in place of the values, otherwise
 // the values.  Out of line, over the staged values: many workloads' chunks never get here, and its code
 // stays out of the others' instruction stream.
+// vmax: the chunk's largest magnitude; own: this lane's (FP32 and FP16 only).
 template <int D>
 __device__ __noinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int lane, uint32_t m, int e_max, int atop,
-                                           typename Traits<D>::U vmax, bool elf) {
+                                           typename Traits<D>::U vmax, uint32_t own, bool elf) {
     using T = Traits<D>;
     using U = typename T::U;
     const bool has_vx = m > 1024u && lane == 31;
@@ -546,25 +549,30 @@ __device__ __noinline__ int case1_alpha(const uint8_t *src, uint8_t *buf, int la
         pad_values<D>(buf, m, lane);
     };
     // FP32 (R14), FP16 (R18): below beta_hat = B_MAX no value can stop early, so Alg. 2 value by value
-    // gives the same alpha_max.  FP64: no value can (Thm 4).
-    bool stop = false;
+    // gives the same alpha_max.  At B_MAX (a = atop) a chunk with an early stop is Case 2, as one with a
+    // failing value is; in data full of them every lane's largest value tells most chunks (1023 FP32
+    // decimals of seven digits: 43 us for the call, 12 so).  FP64: no value can stop (Thm 4).
     auto pass = [&](int a) {
         bool watch = false;
-        if constexpr (D != kD64) watch = !elf && a + e_max + 1 == T::B_MAX && may_stop_early(vmax, a);
-        if constexpr (D == kD64) {
-            if (a + e_max + 1 <= kNarrowBeta && a <= 13) return pass_to_g<D, true>(buf, lane, m, a, false, stop);
+        if constexpr (D != kD64) {
+            watch = !elf && a + e_max + 1 == T::B_MAX && may_stop_early(vmax, a);
+            if (watch && __any_sync(kFull, first_pass((U)own, a) < 0)) return false;
         }
-        return pass_to_g<D>(buf, lane, m, a, watch, stop);
+        if constexpr (D == kD64) {
+            if (a + e_max + 1 <= kNarrowBeta && a <= 13) return pass_to_g<D, true>(buf, lane, m, a, false);
+        }
+        return pass_to_g<D>(buf, lane, m, a, watch);
     };
     int alpha = elf ? alpha_elf<D>(buf, lane, m, vx, has_vx, e_max) : alpha_bound<D>(buf, lane, m, atop);
     if (alpha < 0) return -1;
-    if (!pass(alpha)) {
+    bool ok = pass(alpha);
+    if (!ok) {
         restage();
         alpha = alpha_above<D>(buf, lane, m, vx, alpha, atop);
         if (alpha < 0) return -1;
-        (void)pass(alpha);
+        ok = pass(alpha);
     }
-    if (stop) {
+    if (D != kD64 && !ok) {                       // every value passes, but some value stops early
         restage();
         return -1;
     }
@@ -630,7 +638,7 @@ __device__ __forceinline__ int case_decision(const uint8_t *src, uint8_t *buf, i
         else own = (U)kmax;
         if (atop < 0 || !__all_sync(kFull, q_test(own, atop))) return kNone;
     }
-    const int alpha = case1_alpha<D>(src, buf, lane, m, e_max, atop, vmax, elf);
+    const int alpha = case1_alpha<D>(src, buf, lane, m, e_max, atop, vmax, D == kD64 ? 0u : kmax, elf);
     return alpha < 0 ? kNone : alpha | ((alpha + e_max + 1) << 8);
 }
 
