@@ -1327,7 +1327,7 @@ cudaError_t launch_form(const Job *d_jobs, int njobs, const Job &single, uint64_
     const bool direct = d_jobs == nullptr && single.nchunks <= kDirectChunks;
     if (!direct) launch_offsets(d_jobs, njobs, single, kOffsetsOfOutput, ctl, stream);
     // the emit launch also writes the header and length of every job, chunks or none
-    (void)launch_after(em.kernel, em.grid, em.threads, em.smem, stream, d_jobs, njobs, single, total_chunks, direct, ctl);
+    (void)launch_after(g_ctas_per_sm[0] == 0, em.kernel, em.grid, em.threads, em.smem, stream, d_jobs, njobs, single, total_chunks, direct, ctl);
     return cudaGetLastError();
 }
 

@@ -812,7 +812,8 @@ void launch_decode(const Job *d_jobs, int njobs, const Job &single, uint64_t tot
     const int w = g_cta_warps[1], smem = (int)(kZeroBytes + w * DecLayout<layout_kind<kDt>()>::kWarpBytes);
     const int grid = persistent_grid_size(reinterpret_cast<const void *>(decompress_kernel<kDt, kAgg>), w, smem,
                                           g_ctas_per_sm[1], total_chunks);
-    (void)launch_after(decompress_kernel<kDt, kAgg>, grid, 32 * w, smem, stream, d_jobs, njobs, single, total_chunks, ctl);
+    (void)launch_after(g_ctas_per_sm[1] == 0, decompress_kernel<kDt, kAgg>, grid, 32 * w, smem, stream, d_jobs, njobs, single,
+                       total_chunks, ctl);
 }
 }  // namespace
 
@@ -826,12 +827,12 @@ void launch_offsets(const Job *d_jobs, int njobs, const Job &single, int which, 
     if (d_jobs == nullptr) {
         const uint64_t steps = (single.nchunks + 1023u) / 1024u;
         const uint32_t parts = steps < 1u ? 1u : (steps > 152u ? 152u : (uint32_t)steps);
-        if (after) (void)launch_after(offsets_kernel, (int)parts, 1024, 0, stream, single, parts, which, ctl);
+        if (after) (void)launch_after(true, offsets_kernel, (int)parts, 1024, 0, stream, single, parts, which, ctl);
         else offsets_kernel<<<parts, 1024, 0, stream>>>(single, parts, which, ctl);
         return;
     }
     const uint32_t per = std::min(((uint32_t)njobs + 303u) / 304u, 32u), ctas = ((uint32_t)njobs + per - 1u) / per;
-    if (after) (void)launch_after(table_offsets_kernel, (int)ctas, 1024, 0, stream, d_jobs, njobs, per, which, ctl);
+    if (after) (void)launch_after(true, table_offsets_kernel, (int)ctas, 1024, 0, stream, d_jobs, njobs, per, which, ctl);
     else table_offsets_kernel<<<ctas, 1024, 0, stream>>>(d_jobs, njobs, per, which, ctl);
 }
 
@@ -842,7 +843,7 @@ cudaError_t launch_aggregate(const Job &single, Control *ctl, void *d_stats, cud
         else if (single.dtype == 1) launch_decode<kDtF32, true>(nullptr, 1, single, single.nchunks, ctl, stream);
         else launch_decode<kDtF16, true>(nullptr, 1, single, single.nchunks, ctl, stream);
     }
-    (void)launch_after(aggregate_finish_kernel, 1, 1024, 0, stream, single, ctl, static_cast<falcon_stats *>(d_stats));
+    (void)launch_after(true, aggregate_finish_kernel, 1, 1024, 0, stream, single, ctl, static_cast<falcon_stats *>(d_stats));
     return cudaGetLastError();
 }
 

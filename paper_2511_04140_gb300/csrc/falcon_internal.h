@@ -104,8 +104,12 @@ int persistent_grid_size(const void *kernel, int warps, int smem_bytes, int lim,
 
 // Launches a kernel whose CTAs may be placed, and run up to their pdl_wait, while the kernel enqueued
 // before it on the stream drains: the launch's latency and the first instruction fetches overlap it.
+// `early` false: placed once that kernel has ended, for persistent grids that g_ctas_per_sm caps.  CTAs
+// placed early go where the draining kernel leaves room, several to an SM while others get none, which a
+// grid of all the CTAs that fit evens out and a capped one does not (2^24 normal FP32 values compressed
+// with one CTA per SM: 194 us placed early, 134 not).
 template <class... P, class... A>
-cudaError_t launch_after(void (*kernel)(P...), int grid, int threads, int smem, cudaStream_t stream, A... args) {
+cudaError_t launch_after(bool early, void (*kernel)(P...), int grid, int threads, int smem, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
@@ -115,7 +119,7 @@ cudaError_t launch_after(void (*kernel)(P...), int grid, int threads, int smem, 
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
