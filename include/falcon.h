@@ -212,7 +212,8 @@ int falcon_compress_variant_async(const void *d_in, uint64_t n, int dtype, uint3
  *   - Allocates nothing: no cudaMalloc, cudaFree or allocating library routine.
  *   - The first call on a device looks the array's address up (cudaGetSymbolAddress, with
  *     that device current) and keeps it; make that first call before any stream capture.
- *   - Zeroes, on `stream`, the scratch words it uses and d_result before the kernels.
+ *   - The kernels write every scratch word that they read, and d_result (a small reset of the control
+ *     block is enqueued before them where they draw chunk tickets).
  *   - Every call on a device uses the same array: calls that overlap in time (two streams,
  *     or two host threads without ordering) race and corrupt each other's output; order
  *     them on one stream.

@@ -425,13 +425,12 @@ __device__ __forceinline__ bool pass_to_g(uint8_t *buf, int lane, uint32_t m, in
     return true;
 }
 
-// Smallest a in [0, atop] at which every value passes the round-trip test, or -1 (Case 2).
-// For chunks of valid values the predicate is monotone in a (Thm 4 with Thm 3), and its
-// smallest true point is the largest decimal place of the values; a failure at atop means
-// some value is an exception or needs alpha > atop.  Each lane's first value is tested at
-// atop (a failure settles Case 2), then its own decimal place is found; the warp's maximum
-// is a lower bound, and for most chunks the answer: one all-value test confirms it (`lb_ok`: the
-// caller has already made it).  Otherwise the answer lies above it (test atop, then bisect).
+// alpha_max is the smallest a in [0, atop] at which every value passes the round-trip test (none: Case
+// 2).  For chunks of valid values the predicate is monotone in a (Thm 4 with Thm 3), and its smallest
+// true point is the largest decimal place of the values; a failure at atop means some value is an
+// exception or needs alpha > atop.  A lower bound: each lane's first value is tested at atop (a failure
+// settles Case 2: -1), then its own decimal place is found, and the warp's maximum is returned.  For most
+// chunks it is the answer, which the caller's test of every value confirms; otherwise alpha_above goes on.
 template <int D>
 __device__ __forceinline__ int alpha_bound(const uint8_t *buf, int lane, uint32_t m, int atop) {
     using U = typename Traits<D>::U;
@@ -442,7 +441,7 @@ __device__ __forceinline__ int alpha_bound(const uint8_t *buf, int lane, uint32_
     while (a0 < atop && !q_test(v0, a0)) ++a0;
     return (int)__reduce_max_sync(kFull, (uint32_t)a0);
 }
-// the answer above a lower bound that failed
+// the answer above a lower bound that failed (test atop, then bisect), or -1
 template <int D>
 __device__ __forceinline__ int alpha_above(const uint8_t *buf, int lane, uint32_t m, typename Traits<D>::U vx,
                                            int lb, int atop) {
@@ -1158,7 +1157,8 @@ __device__ __forceinline__ void analyse_loop(const Job *__restrict__ jobs, int n
 }
 
 // FP32 and FP16 in 80 registers, 24 warps per SM; FP64 and the either-dtype form in 96 and 20 warps (FP64
-// in 80 spills 16 bytes: 2^24 walk 104.8 us against 102.3, 40 M decimal values 367.0 against 364.8).
+// in 80 spills 16 bytes: 2^24 walk 104.8 us against 102.3, 40 M decimal values 367.0 against 364.8; the
+// either-dtype form spills 12 bytes in 96).
 template <int kDt>
 __global__ void __maxnreg__(kDt == kDtF32 || kDt == kDtF16 ? 80 : 96)
 analyse_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
@@ -1363,12 +1363,6 @@ int persistent_grid_of(const void *kernel, int warps, int smem_bytes, int lim, u
 
 int persistent_grid_size(const void *kernel, int warps, int smem_bytes, int lim, uint64_t total_chunks) {
     return persistent_grid_of(kernel, warps, smem_bytes, lim, total_chunks);
-}
-
-int compress_grid(uint64_t total_chunks) {
-    const int w = g_cta_warps[0];
-    return persistent_grid_of(reinterpret_cast<const void *>(emit_kernel<false, kDtMixed>), w,
-                              w * (int)EmitLayout<kD64, false>::kBytes, g_ctas_per_sm[0], total_chunks);
 }
 
 cudaError_t launch_compress(const Job *d_jobs, int njobs, const Job &single, uint64_t total_chunks,

@@ -713,7 +713,8 @@ constexpr int kDtF64 = 0, kDtF32 = 1, kDtMixed = 2, kDtF16 = 3;
 template <int kDt> constexpr int layout_kind() { return kDt == kDtF32 ? kD32 : (kDt == kDtF16 ? kD16 : kD64); }
 
 // Registers: 128 (FP64, either-dtype: 16 warps per SM), 80 (FP32, FP16: 24 warps; 96 registers and
-// 20 warps: 1.3 % slower).  The aggregate forms keep FP64 sums as well and take 168.
+// 20 warps: 1.3 % slower).  The aggregate forms keep every value and the FP64 sums in registers: 168
+// (FP64: 12 warps) and 128.
 template <int kDt, bool kAgg = false>
 __global__ void __maxnreg__((kDt == kDtF32 || kDt == kDtF16) && !kAgg ? 80 : (kAgg ? (kDt == kDtF64 ? 168 : 128) : 128))
 decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t total_chunks, Control *ctl) {
@@ -763,13 +764,6 @@ decompress_kernel(const Job *__restrict__ jobs, int njobs, Job single, uint64_t 
         ln = locate<kTable>(jobs, njobs, s_single, tn, total_chunks, lane);
     }
     cp_async_wait_none();
-}
-
-int decompress_grid(uint64_t total_chunks) {
-    const int w = g_cta_warps[1];
-    return persistent_grid_size(reinterpret_cast<const void *>(decompress_kernel<kDtMixed>), w,
-                                (int)(kZeroBytes + w * DecLayout<kD64>::kWarpBytes),
-                                g_ctas_per_sm[1], total_chunks);
 }
 
 // The aggregate's last step (one CTA): thread t adds the chunk sums of its contiguous share in

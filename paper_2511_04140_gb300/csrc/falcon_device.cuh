@@ -72,8 +72,6 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// wait until at most the most recently committed group is still in flight
-__device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_none() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // Programmatic dependent launch: a kernel launched with launch_after (falcon_internal.h) may start once
@@ -126,20 +124,11 @@ __device__ __forceinline__ uint32_t shfl_x(uint32_t v, int src) { return __shfl_
 __device__ __forceinline__ uint64_t shfl_x(uint64_t v, int src) { return shfl_u64(v, src); }
 __device__ __forceinline__ uint32_t shfl_down_x(uint32_t v, int d) { return __shfl_down_sync(kFull, v, d); }
 __device__ __forceinline__ uint64_t shfl_down_x(uint64_t v, int d) { return shfl_down_u64(v, d); }
-__device__ __forceinline__ uint32_t shfl_up_x(uint32_t v, int d) { return __shfl_up_sync(kFull, v, d); }
-__device__ __forceinline__ uint64_t shfl_up_x(uint64_t v, int d) { return shfl_up_u64(v, d); }
 __device__ __forceinline__ uint16_t shfl_x(uint16_t v, int src) { return (uint16_t)__shfl_sync(kFull, (uint32_t)v, src); }
 __device__ __forceinline__ uint16_t shfl_down_x(uint16_t v, int d) {
     return (uint16_t)__shfl_down_sync(kFull, (uint32_t)v, d);
 }
-__device__ __forceinline__ uint16_t shfl_up_x(uint16_t v, int d) { return (uint16_t)__shfl_up_sync(kFull, (uint32_t)v, d); }
 
-__device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += ((uint64_t)__shfl_xor_sync(kFull, (uint32_t)(v >> 32), o) << 32) |
-                                          __shfl_xor_sync(kFull, (uint32_t)v, o);
-    return v;
-}
 __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
     uint32_t hi = __reduce_max_sync(kFull, (uint32_t)(v >> 32));
     uint32_t lo = __reduce_max_sync(kFull, ((uint32_t)(v >> 32) == hi) ? (uint32_t)v : 0u);
@@ -302,34 +291,6 @@ __device__ __forceinline__ void stage_values_async(const uint8_t *src, uint32_t 
         else if constexpr (D == kD32) cp_async4(base + phys_elem_byte<D>(e), src + (size_t)e * S);
         else                                     // no 2-byte cp.async: a plain copy (visible at the next __syncwarp)
             *reinterpret_cast<uint16_t *>(wsm + phys_elem_byte<D>(e)) = *reinterpret_cast<const uint16_t *>(src + (size_t)e * S);
-    }
-}
-
-// Lane reads its 32 values (indices 32*lane + k).
-template <int D>
-__device__ __forceinline__ void read_own(const uint8_t *wsm, int lane, typename Traits<D>::U (&v)[32]) {
-    using U = typename Traits<D>::U;
-    constexpr int UN = Traits<D>::UNITS;
-    constexpr int PER = 32 / UN;
-#pragma unroll
-    for (int u = 0; u < UN; ++u) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(wsm + (lane * UN + unit_swizzle<D>(lane, u)) * 16);
-        if constexpr (D == kD64) {
-            v[PER * u + 0] = ((U)q.y << 32) | q.x;
-            v[PER * u + 1] = ((U)q.w << 32) | q.z;
-        } else if constexpr (D == kD16) {
-            const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                v[PER * u + 2 * h] = (U)(w4[h] & 0xFFFFu);
-                v[PER * u + 2 * h + 1] = (U)(w4[h] >> 16);
-            }
-        } else {
-            v[PER * u + 0] = q.x;
-            v[PER * u + 1] = q.y;
-            v[PER * u + 2] = q.z;
-            v[PER * u + 3] = q.w;
-        }
     }
 }
 

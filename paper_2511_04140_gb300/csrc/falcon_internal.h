@@ -9,7 +9,6 @@ namespace falcon {
 // changes no output byte; every warp works on its own chunks.  The kernels' register budgets
 // (80 to 168 per thread, set per kernel) hold at every allowed shape.
 constexpr int kWarpsPerCta = 4;                 // default
-constexpr int kThreads = 32 * kWarpsPerCta;
 constexpr int kMaxCompressWarps = 16;           // 512 threads of up to 128 registers
 constexpr int kMaxDecompressWarps = 12;         // 384 threads of up to 168 registers
 constexpr uint32_t kMaxBlock = 1025;
@@ -32,7 +31,7 @@ struct Job {
     unsigned long long *flags;     // the job's workspace words (workspace_words(nchunks))
     unsigned long long *result;    // [0] stream bytes (compress) / values (decompress), [1] status
     uint32_t block;
-    uint32_t dtype;                // 0 = FP64, 1 = FP32
+    uint32_t dtype;                // 0 = FP64, 1 = FP32, 2 = FP16
     uint32_t variant;              // compression: kVariant* (decompression: unused)
 };
 
@@ -60,7 +59,8 @@ constexpr size_t kControlBytes = 256;   // control block region (keeps flags 256
 // Workspace words of a job: compression keeps two per chunk (the analysis results with the record
 // offset, and the dense-row mask); decompression keeps the record offset of each chunk in the first
 // words (the aggregate its chunk sums in the next).  The size also counts a word per 64-chunk tile
-// and per 4096-chunk group, which nothing uses now (callers' workspaces keep their size).
+// and per 4096-chunk group: nothing uses them now, but falcon_workspace_bytes is part of the ABI, so
+// workspaces sized by an earlier version stay large enough and the other way round.
 // value kinds of the stream format: 0 FP64, 1 FP32, 2 FP16 (binary16)
 inline bool dtype_valid(int dtype) { return dtype >= 0 && dtype <= 2; }
 inline size_t dtype_bytes(int dtype) { return dtype == 0 ? 8 : (dtype == 1 ? 4 : 2); }
@@ -122,9 +122,5 @@ cudaError_t launch_after(bool early, void (*kernel)(P...), int grid, int threads
     cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
-
-// Grid size used for a launch over total_chunks work items (persistent, occupancy-bound).
-int compress_grid(uint64_t total_chunks);
-int decompress_grid(uint64_t total_chunks);
 
 }  // namespace falcon
