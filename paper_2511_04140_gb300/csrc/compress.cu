@@ -23,11 +23,11 @@
 //      sent to its offset with one TMA bulk copy;
 //      the warp of each job's first chunk writes the header and the stream length and checks
 //      the capacity.
-// Both are bound by integer issue (FP64 segments: ALU pipe 75 % and 66 % of active cycles, 1236 and 2741
+// Both are bound by integer issue (FP64 segments: ALU pipe 75 % and 66 % of active cycles, 1235 and 2741
 // warp instructions per chunk, against 1801 and 3590 with ballots and reductions per sparse row,
 // per-value zigzags and bit-sliced counts) and, where chunks take different paths, by instruction fetch.
-// 2^26 segment values: FP64 521 -> 362 us, FP32 272 -> 207 us; Case-1 FP64 of 40 M values in 1025-value
-// chunks 622 -> 318 us.  Slower, and left out (each measured when the rest stood at about 450 us): two
+// 2^26 segment values: FP64 520 -> 357 us, FP32 270 -> 206 us; Case-1 FP64 of 40 M values in 1025-value
+// chunks 622 -> 317 us.  Slower, and left out (each measured when the rest stood at about 450 us): two
 // copies of the row code (FP64 485 us: instruction fetch), a transpose shared by both halves in a loop
 // (475 us), dense rows moved in 16-byte units (FP64 461, FP32 238 us), values kept in L1 (483 us).  The
 // offsets launch in place of per-tile and per-group sums (two atomics per chunk in the analysis, five loads

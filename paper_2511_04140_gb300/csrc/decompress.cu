@@ -1,6 +1,6 @@
 // Falcon decompression (Sec. 4 of the paper) for sm_103a: two launches per call.
 //
-// 1. offsets_kernel: the chunk-size array is read and its exclusive prefix (the chunk
+// 1. offsets_kernel (a table's: table_offsets_kernel): the chunk-size array is read and its exclusive prefix (the chunk
 //    offset array) is written to the workspace - the step Sec. 4 performs first.
 // 2. decompress_kernel: persistent; each warp takes its chunks by ticket (one atomic add each; no
 //    ordering constraint remains).  Each warp has one record buffer: the cp.async of its
@@ -15,17 +15,17 @@
 //         zigzag of the IEEE bits (inverse Eq. 4),
 //      c. whole 32-byte sectors per lane (aligned FP64) or staged, coalesced stores.
 // What bounds it: integer issue and latency together (FP64 Case-1 values: ALU pipe 66 %, issue 64 % of cycles
-// at 16 warps per SM; HBM 45 % on FP64 segments), and the instruction stream's length: code is kept short
+// at 16 warps per SM; HBM 37 % on FP64 segments), and the instruction stream's length: code is kept short
 // (both FP64 halves run one copy, Case 1 divides in rolled loops on the way out), which took FP64 segments
 // from 310 to 288 us and Case-1 values from 304 to 191 us (40 M in 1025-value chunks).
 // Reading the dense rows in place instead of copying them to a plane buffer took the kernel from 4302 to
-// 2880 warp instructions per FP64 chunk and its shared memory from 17.6 to 13.7 KB per warp (12 to 16
-// warps per SM).  Both launches, 2^26 segment values: FP64 420 -> 273 us, FP32 216 -> 139 us; the Case-1
-// values 550 -> 172 us.  Slower, and left out: a TMA bulk copy of the record on an mbarrier (-1 %), tickets
+// 2709 warp instructions per FP64 chunk and its shared memory from 17.6 to 13.7 KB per warp (12 to 16
+// warps per SM).  Both launches, 2^26 segment values: FP64 419 -> 270 us, FP32 216 -> 137 us; the Case-1
+// values 549 -> 170 us.  Slower, and left out: a TMA bulk copy of the record on an mbarrier (-1 %), tickets
 // for groups of 4 to 8 chunks (-7 to -15 %: the window of memory in use grows with the group), more
 // registers with fewer warps (144: -6 %).
 // Every read of a record is bounds-checked against its size; a malformed record sets
-// FALCON_ERR_CORRUPT and writes nothing.
+// FALCON_ERR_CORRUPT and writes no value.
 #include <algorithm>
 
 #include "falcon.h"
